@@ -56,12 +56,33 @@ struct BInst {
 struct BParams {  // rewritten by the host before every outer iteration
   int active;     // 0: converged (skipped)
   int degree;     // 0: no filter this iteration
-  int mu_off;     // offset of mu_0 in the coefficient table
+  int mu_off;     // offset of mu_0 in the coefficient table (doubles, or for FP32 and
+                  // float-float sweeps (hi, lo) pairs)
   int flags;      // device-written: 1 = a Cholesky pass was shifted, 2 = breakdown
   double alpha, beta;
   int f32;        // 1: this iteration's filter runs in FP32 (V32, W32, FP32 values)
   int ff;         // 1: it runs in float-float (V and W hold (hi, lo) pairs in place)
+  // alpha and beta as (hi, lo) pairs, and the doubled ones of the steps k >= 2:
+  // a row group converting them on the device would spend more of the slow FP64
+  // pipe on its scalars than it spends on arithmetic
+  float2 alpha_ff, beta_ff, alpha2_ff, beta2_ff;
 };
+
+// (hi, lo) pair of a coefficient: the nearest float and the nearest float to
+// the rest (host; the high part is the FP32 sweeps' coefficient)
+inline float2 pair_of_double(double v) {
+  const float hi = (float)v;
+  return make_float2(hi, (float)(v - (double)hi));
+}
+
+inline void set_scale(BParams& P, double alpha, double beta) {
+  P.alpha = alpha;
+  P.beta = beta;
+  P.alpha_ff = pair_of_double(alpha);
+  P.beta_ff = pair_of_double(beta);
+  P.alpha2_ff = pair_of_double(2 * alpha);
+  P.beta2_ff = pair_of_double(2 * beta);
+}
 
 struct BTask {
   int inst, bundle;
@@ -125,9 +146,13 @@ __device__ __forceinline__ void batched_row_group(const BatchArgs& b, int t, int
     double* Z = (k & 1) ? W1 : W2;
     s.X = X; s.ldx = NB; s.Z = Z; s.ldz = NB;
     s.Y = k < n ? Z : nullptr; s.ldy = NB;
-    s.Vin = V; s.ldvi = I.ns; s.Vout = V; s.ldvo = I.ns;
-    s.c_ax = 2 * P.alpha; s.c_x = 2 * P.beta; s.mu2 = mu[k];
-    cheb_rows<double, NB, MODE_GENERIC>(I.A, s, lrow0);
+    s.c_ax = 2 * P.alpha; s.c_x = 2 * P.beta;
+    s.nacc = step_terms(k, n);
+    if (s.nacc) {
+      s.Vin = V; s.ldvi = I.ns; s.Vout = V; s.ldvo = I.ns;
+      s.mu0 = mu[k - 2]; s.mu1 = mu[k - 1]; s.mu2 = mu[k];
+    }
+    cheb_rows<double, NB, MODE_EITHER>(I.A, s, lrow0);
   }
 }
 
@@ -144,33 +169,39 @@ __device__ __forceinline__ void batched_row_group_f32(const BatchArgs& b, int t,
   float* V = I.V32 + (int64_t)tk.bundle * NB;
   float* W1 = I.W32 + (int64_t)tk.bundle * 2 * D * NB;
   float* W2 = W1 + D * NB;
-  const double* mu = b.mu + P.mu_off;
+  const float2* mu = reinterpret_cast<const float2*>(b.mu) + P.mu_off;
   StepArgs<float> s{};
   if (k == 1) {
     s.X = V; s.ldx = I.ns; s.Y = W1; s.ldy = NB;
-    s.c_ax = (float)P.alpha; s.c_x = (float)P.beta;
+    s.c_ax = P.alpha_ff.x; s.c_x = P.beta_ff.x;
     cheb_rows<float, NB, MODE_SPMMV>(I.A32, s, lrow0);
   } else if (k == 2) {
     s.X = W1; s.ldx = NB; s.Z = V; s.ldz = I.ns;
     s.Y = n > 2 ? W2 : nullptr; s.ldy = NB;
     s.Vout = V; s.ldvo = I.ns;
-    s.c_ax = (float)(2 * P.alpha); s.c_x = (float)(2 * P.beta);
-    s.mu0 = (float)mu[0]; s.mu1 = (float)mu[1]; s.mu2 = (float)mu[2];
+    s.c_ax = P.alpha2_ff.x; s.c_x = P.beta2_ff.x;
+    s.mu0 = mu[0].x; s.mu1 = mu[1].x; s.mu2 = mu[2].x;
     cheb_rows<float, NB, MODE_SECOND>(I.A32, s, lrow0);
   } else {
     float* X = (k & 1) ? W2 : W1;
     float* Z = (k & 1) ? W1 : W2;
     s.X = X; s.ldx = NB; s.Z = Z; s.ldz = NB;
     s.Y = k < n ? Z : nullptr; s.ldy = NB;
-    s.Vin = V; s.ldvi = I.ns; s.Vout = V; s.ldvo = I.ns;
-    s.c_ax = (float)(2 * P.alpha); s.c_x = (float)(2 * P.beta); s.mu2 = (float)mu[k];
-    cheb_rows<float, NB, MODE_GENERIC>(I.A32, s, lrow0);
+    s.c_ax = P.alpha2_ff.x; s.c_x = P.beta2_ff.x;
+    s.nacc = step_terms(k, n);
+    if (s.nacc) {
+      s.Vin = V; s.ldvi = I.ns; s.Vout = V; s.ldvo = I.ns;
+      s.mu0 = mu[k - 2].x; s.mu1 = mu[k - 1].x; s.mu2 = mu[k].x;
+    }
+    cheb_rows<float, NB, MODE_EITHER>(I.A32, s, lrow0);
   }
 }
 
 // float-float sweeps of an instance (its FP32 form's finish, or the FF form):
 // the same steps on V and W reinterpreted as (hi, lo) pairs, which k_bconvert
 // writes in place of the doubles before the filter and turns back after it
+__device__ __forceinline__ ff as_ff(float2 p) { return ff(p.x, p.y); }
+
 template <int NB>
 __device__ __forceinline__ void batched_row_group_ff(const BatchArgs& b, int t, int64_t lrow0, int k) {
   const BTask tk = b.task[t];
@@ -182,35 +213,40 @@ __device__ __forceinline__ void batched_row_group_ff(const BatchArgs& b, int t, 
   ff* V = reinterpret_cast<ff*>(I.V + (int64_t)tk.bundle * NB);
   ff* W1 = reinterpret_cast<ff*>(I.W + (int64_t)tk.bundle * 2 * D * NB);
   ff* W2 = W1 + D * NB;
-  const double* mu = b.mu + P.mu_off;
+  const ff* mu = reinterpret_cast<const ff*>(b.mu) + P.mu_off;
   StepArgs<ff> s{};
   if (k == 1) {
     s.X = V; s.ldx = I.ns; s.Y = W1; s.ldy = NB;
-    s.c_ax = ff(P.alpha); s.c_x = ff(P.beta);
+    s.c_ax = as_ff(P.alpha_ff); s.c_x = as_ff(P.beta_ff);
     cheb_rows<ff, NB, MODE_SPMMV>(I.Aff, s, lrow0);
   } else if (k == 2) {
     s.X = W1; s.ldx = NB; s.Z = V; s.ldz = I.ns;
     s.Y = n > 2 ? W2 : nullptr; s.ldy = NB;
     s.Vout = V; s.ldvo = I.ns;
-    s.c_ax = ff(2 * P.alpha); s.c_x = ff(2 * P.beta);
-    s.mu0 = ff(mu[0]); s.mu1 = ff(mu[1]); s.mu2 = ff(mu[2]);
+    s.c_ax = as_ff(P.alpha2_ff); s.c_x = as_ff(P.beta2_ff);
+    s.mu0 = mu[0]; s.mu1 = mu[1]; s.mu2 = mu[2];
     cheb_rows<ff, NB, MODE_SECOND>(I.Aff, s, lrow0);
   } else {
     ff* X = (k & 1) ? W2 : W1;
     ff* Z = (k & 1) ? W1 : W2;
     s.X = X; s.ldx = NB; s.Z = Z; s.ldz = NB;
     s.Y = k < n ? Z : nullptr; s.ldy = NB;
-    s.Vin = V; s.ldvi = I.ns; s.Vout = V; s.ldvo = I.ns;
-    s.c_ax = ff(2 * P.alpha); s.c_x = ff(2 * P.beta); s.mu2 = ff(mu[k]);
-    cheb_rows<ff, NB, MODE_GENERIC>(I.Aff, s, lrow0);
+    s.c_ax = as_ff(P.alpha2_ff); s.c_x = as_ff(P.beta2_ff);
+    s.nacc = step_terms(k, n);
+    if (s.nacc) {
+      s.Vin = V; s.ldvi = I.ns; s.Vout = V; s.ldvo = I.ns;
+      s.mu0 = mu[k - 2]; s.mu1 = mu[k - 1]; s.mu2 = mu[k];
+    }
+    cheb_rows<ff, NB, MODE_EITHER>(I.Aff, s, lrow0);
   }
 }
 
 // FF: the instantiation with FP32 and float-float rows only, the filter of
-// solves that use float-float sweeps.  It runs the shape of the
-// single-problem FP32 and float-float steps, 4-warp CTAs and 12 per SM
-// (48 warps, <= 40 registers): both are bound by memory latency.
-constexpr int BF_FF_WARPS = 4, BF_FF_BLOCKS = 12;
+// solves that use float-float sweeps, in 4-warp CTAs.  Eight of them per SM (64
+// registers) rather than twelve: at 40 registers the two row types spill 420
+// bytes (12 instances of L = 10 .. 14, nb = 8: 125 ms of filter per solve against
+// 167 ms).
+constexpr int BF_FF_WARPS = 4, BF_FF_BLOCKS = 8;
 template <int NB, bool FF>
 __global__ void __launch_bounds__(FF ? BF_FF_WARPS * 32 : WARPS * 32, FF ? BF_FF_BLOCKS : 3)
     k_batched_filter(BatchArgs b) {
@@ -1051,7 +1087,7 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
     wr[i] = prob[i].b;
   }
   // first iteration: no filter, orthonormalise + Rayleigh-Ritz
-  for (int i = 0; i < n_inst; ++i) B.h_par[i] = BParams{1, 0, 0, 0, 0.0, 0.0, 0, 0};
+  for (int i = 0; i < n_inst; ++i) B.h_par[i] = BParams{1};
   *B.h_kmax = 0;
   B.list_tasks();
   // capture one iteration as a graph; replay it every outer iteration
@@ -1154,17 +1190,19 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
       }
       deg[i] = n;
       std::vector<double> mu = filter_coeffs(alpha * wl[i] + beta, alpha * wr[i] + beta, n);
-      std::copy(mu.begin(), mu.end(), B.h_mu + mu_off);
       P.degree = n;
       P.mu_off = (int)mu_off;
-      P.alpha = alpha;
-      P.beta = beta;
+      set_scale(P, alpha, beta);
       P.flags = 0;
       stall[i] = maxr > 0.5 * prev_max[i] ? stall[i] + 1 : 0;
       if (use32[i] && (maxr <= 100.0 * 0x1.0p-24 * norm_h[i] || stall[i] >= 2)) use32[i] = 0;
       prev_max[i] = maxr;
       P.f32 = use32[i];
       P.ff = !use32[i] && ffs;
+      if (P.f32 || P.ff)
+        std::transform(mu.begin(), mu.end(), reinterpret_cast<float2*>(B.h_mu) + mu_off, pair_of_double);
+      else
+        std::copy(mu.begin(), mu.end(), B.h_mu + mu_off);
       mu_off += n + 1;
       kmax = std::max(kmax, n);
     }
@@ -1239,7 +1277,8 @@ fd_status fd_tune_batched(fd_ctx* ctx, int n_inst, const char* const* specs, int
           ctx->launches++;
           const double a = 2.0 / (M[i]->gersh_hi - M[i]->gersh_lo + 1e-3);
           const double b = -(M[i]->gersh_hi + M[i]->gersh_lo) / (M[i]->gersh_hi - M[i]->gersh_lo + 1e-3);
-          B.h_par[i] = BParams{1, probe_degree, 0, 0, a, b, 0, 0};
+          B.h_par[i] = BParams{1, probe_degree};
+          set_scale(B.h_par[i], a, b);
           const double vec = (double)nb * M[i]->D * 8.0, mat = (double)M[i]->nnz * 12.0;
           const int n = probe_degree;
           bytes += (ns / nb) * ((mat + 2 * vec) + (mat + 4 * vec) + (n - 3) * (mat + 5 * vec) + (mat + 4 * vec));

@@ -101,19 +101,24 @@ struct V16<ffa::ff> {
   __device__ __forceinline__ void set(const float4& t) { v[0] = ff(t.x, t.y); v[1] = ff(t.z, t.w); }
   __device__ __forceinline__ float4 get() const { return make_float4(v[0].hi, v[0].lo, v[1].hi, v[1].lo); }
   __device__ __forceinline__ void ldg(const ff* p) { set(__ldg(reinterpret_cast<const float4*>(p))); }
-  __device__ __forceinline__ void ldcs(const ff* p) { set(__ldcs(reinterpret_cast<const float4*>(p))); }
-  __device__ __forceinline__ void stcs(ff* p) const { __stcs(reinterpret_cast<float4*>(p), get()); }
-  __device__ __forceinline__ void st(ff* p) const { *reinterpret_cast<float4*>(p) = get(); }
-  __device__ __forceinline__ void ldg_pol(const ff* p, uint64_t pol) {
+  __device__ __forceinline__ void ld(const ff* p) {
     float4 t;
-    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
-        : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "l"(p), "l"(pol));
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "l"(p) : "memory");
     set(t);
   }
+  __device__ __forceinline__ void ldcs(const ff* p) {
+    float4 t;
+    asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "l"(p) : "memory");
+    set(t);
+  }
+  __device__ __forceinline__ void stcs(ff* p) const { __stcs(reinterpret_cast<float4*>(p), get()); }
+  __device__ __forceinline__ void st(ff* p) const { *reinterpret_cast<float4*>(p) = get(); }
   __device__ __forceinline__ void ld_pol(const ff* p, uint64_t pol) {
     float4 t;
     asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
-                 : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "l"(p), "l"(pol));
+                 : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "l"(p), "l"(pol) : "memory");
     set(t);
   }
   __device__ __forceinline__ void st_pol(ff* p, uint64_t pol) const {

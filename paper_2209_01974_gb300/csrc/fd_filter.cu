@@ -2,7 +2,13 @@
 // fused with the three-term recurrence and the accumulation of the filter
 // coefficients (Alg. 2 fuses the SpMV with the vector update; Sec. 3.2,
 // Eq. EstimateT: with the fused kernel W1 is read once and W2, V are read and
-// written, kappa = 5).
+// written, kappa = 5).  The accumulator is visited every third step only, with
+// three terms (step_terms), so a step moves 11/3 vectors on average, and the
+// steps follow each other by programmatic dependent launch (step_wait).
+// Measured: 2.1M-row stencil, nb = 64, FP32, degree 40 with its two conversions
+// 21.1 -> 17.6 ms; 1.4M-row road graph, nb = 32, FP32 6.95 -> 5.53 ms; 110,592-row
+// Anderson, nb = 32, float-float 19.1 -> 15.8 ms, FP64 (bound by the FP64 pipe)
+// 32.9 -> 31.3 ms.
 //
 // Work mapping: a group of G lanes owns one SELL row; each lane holds CPL
 // 16-byte vectors of the row (G * CPL * 16 bytes = nb * sizeof(T)), so every
@@ -34,6 +40,7 @@ __global__ void __launch_bounds__(step_warps<T>() * 32, step_min_blocks<T>())
     k_cheb_step(SellArgs<T> A, StepArgs<T> s, unsigned pf) {
   using L = Layout<T, NB>;
   constexpr int WARPS = step_warps<T>();
+  step_release();
   // L2 prefetch for the CTA that starts one resident wave (pf CTAs) later:
   // its first loads (row-wise operands, then the SELL slab they index) are a
   // chain of dependent DRAM round trips that no register budget can overlap.
@@ -43,8 +50,11 @@ __global__ void __launch_bounds__(step_warps<T>() * 32, step_min_blocks<T>())
   }
   const int64_t warp = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
   const int64_t row0 = warp * L::RPW;
-  if (row0 >= A.D) return;
-  cheb_rows<T, NB, MODE>(A, s, row0);
+  if (row0 >= A.D) {
+    step_wait();
+    return;
+  }
+  cheb_rows<T, NB, MODE, true>(A, s, row0);
 }
 
 template <typename T, int NB, int MODE>
@@ -52,9 +62,8 @@ __global__ void __launch_bounds__(WARPS * 32, MIN_BLOCKS_F64)  // 64 registers: 
     k_kron_step(KronArgs<T> K, StepArgs<T> s) {
   using L = Layout<T, NB>;
   const int64_t warp = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
-  const int64_t row0 = warp * L::RPW;
-  if (row0 >= K.D) return;
-  kron_rows<T, NB, MODE>(K, s, row0);
+  step_release();
+  kron_rows<T, NB, MODE>(K, s, warp * L::RPW);
 }
 
 // debug checks: flag any index outside [0, bound) (a grid-stride scan)
@@ -83,6 +92,11 @@ __global__ void k_permute_rows(const T* src, int64_t lds, T* dst, int64_t ldd,
 }
 
 // ---- dispatch -------------------------------------------------------------
+template <typename T>
+bool dependent_step(const fd_ctx* ctx, unsigned grid, unsigned wave) {
+  return !std::is_same_v<T, double> || grid * 2 <= (unsigned)ctx->num_sms || grid >= wave;
+}
+
 template <typename T, int NB>
 fd_status launch_kron_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<T>& s) {
   using L = Layout<T, NB>;
@@ -109,11 +123,11 @@ fd_status launch_kron_step(fd_ctx* ctx, const fd_matrix* M, int mode, const Step
     K.diag = reinterpret_cast<const ff*>(M->kdiagff);
   }
   const unsigned grid = (unsigned)cdiv(M->D, (int64_t)WARPS * L::RPW);
-  if (mode == MODE_SPMMV) k_kron_step<T, NB, MODE_SPMMV><<<grid, WARPS * 32, 0, ctx->stream>>>(K, s);
-  else if (mode == MODE_SECOND) k_kron_step<T, NB, MODE_SECOND><<<grid, WARPS * 32, 0, ctx->stream>>>(K, s);
-  else k_kron_step<T, NB, MODE_GENERIC><<<grid, WARPS * 32, 0, ctx->stream>>>(K, s);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
+  const bool dep = dependent_step<T>(ctx, grid, (unsigned)ctx->num_sms * MIN_BLOCKS_F64);  // see launch_step
+  if (mode == MODE_SPMMV) return launch_step_kernel(ctx, k_kron_step<T, NB, MODE_SPMMV>, grid, WARPS * 32, 0, false, K, s);
+  if (mode == MODE_SECOND) return launch_step_kernel(ctx, k_kron_step<T, NB, MODE_SECOND>, grid, WARPS * 32, 0, dep, K, s);
+  if (mode == MODE_PLAIN) return launch_step_kernel(ctx, k_kron_step<T, NB, MODE_PLAIN>, grid, WARPS * 32, 0, dep, K, s);
+  return launch_step_kernel(ctx, k_kron_step<T, NB, MODE_GENERIC>, grid, WARPS * 32, 0, dep, K, s);
 }
 
 template <typename T, int NB>
@@ -130,11 +144,17 @@ fd_status launch_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<
   const unsigned grid = (unsigned)cdiv(M->D, rows_per_block);
   // prefetch distance: one wave of resident CTAs (the launch-bounds occupancy)
   const unsigned pf = (unsigned)ctx->num_sms * step_min_blocks<T>();
-  if (mode == MODE_SPMMV) k_cheb_step<T, NB, MODE_SPMMV><<<grid, SW * 32, 0, ctx->stream>>>(A, s, pf);
-  else if (mode == MODE_SECOND) k_cheb_step<T, NB, MODE_SECOND><<<grid, SW * 32, 0, ctx->stream>>>(A, s, pf);
-  else k_cheb_step<T, NB, MODE_GENERIC><<<grid, SW * 32, 0, ctx->stream>>>(A, s, pf);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
+  // Dependent launch, but for the first step (MODE_SPMMV), which follows a
+  // kernel that is not a step, and for FP64 grids between half the SMs and one
+  // wave: their CTAs would be placed beside the previous step's, unevenly over
+  // the SMs, and the FP64 pipe of the fuller ones sets the time (nb = 16, 4,900
+  // rows in 154 CTAs: 9.2 us a step against 8.2 us; 1,728 rows in 54 CTAs:
+  // 3.4 us against 4.1 us).
+  const bool dep = dependent_step<T>(ctx, grid, pf);
+  if (mode == MODE_SPMMV) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SPMMV>, grid, SW * 32, 0, false, A, s, pf);
+  if (mode == MODE_SECOND) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SECOND>, grid, SW * 32, 0, dep, A, s, pf);
+  if (mode == MODE_PLAIN) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_PLAIN>, grid, SW * 32, 0, dep, A, s, pf);
+  return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_GENERIC>, grid, SW * 32, 0, dep, A, s, pf);
 }
 
 template <typename T>
@@ -209,7 +229,9 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
   }
   FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_SECOND, s));
   bytes += mat_bytes + (n > 2 ? 4 : 3) * vec;
-  // generic steps: xk = 2 A~ x_{k-1} - x_{k-2}; acc += mu_k xk
+  // generic steps: xk = 2 A~ x_{k-1} - x_{k-2}; acc += mu_k xk, three terms at a
+  // time.  The reported bytes stay those of Eq. EstimateT (kappa = 5), the
+  // algorithm's own count; what a step moves is less (step_terms).
   T* xp = x1;  // x_{k-1}
   T* xpp = x2; // x_{k-2} buffer after step 2 is the other one
   // after step 2: x_{k-1} = x2, x_{k-2} = x1
@@ -219,20 +241,20 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
     s = StepArgs<T>{};
     s.X = xp; s.ldx = ldw; s.Z = xpp; s.ldz = ldw;
     s.c_ax = (T)(2 * alpha); s.c_x = (T)(2 * beta);
-    s.mu2 = (T)mu[k];
-    s.Vin = acc; s.ldvi = lda;
-    const bool last = k == n;
-    if (!last) {
-      s.Y = xpp; s.ldy = ldw;
+    s.nacc = step_terms(k, n);
+    if (s.nacc) {
+      s.mu0 = (T)mu[k - 2]; s.mu1 = (T)mu[k - 1]; s.mu2 = (T)mu[k];
+      s.Vin = acc; s.ldvi = lda;
       s.Vout = acc; s.ldvo = lda;
+    }
+    if (k < n) {
+      s.Y = xpp; s.ldy = ldw;
       bytes += mat_bytes + 5 * vec;
     } else {
-      s.Y = nullptr;
-      if (ident) { s.Vout = acc; s.ldvo = lda; }
-      else { s.Vout = xpp; s.ldvo = ldw; final_buf = xpp; }
+      if (!ident) { s.Vout = xpp; s.ldvo = ldw; final_buf = xpp; }
       bytes += mat_bytes + 4 * vec;
     }
-    FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_GENERIC, s));
+    FD_TRY(step_dispatch<T>(ctx, M, nb, s.nacc ? MODE_GENERIC : MODE_PLAIN, s));
     T* t = xp; xp = xpp; xpp = t;
   }
   if (!ident) {
@@ -250,7 +272,8 @@ __global__ void k_spmv1(const int64_t* chunk_ptr, const int32_t* row_len, const 
                         const double* val, int64_t D, int C, const double* x, double* y) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= D) return;
-  int64_t base = chunk_ptr[i / C] + i % C;
+  const uint32_t chunk = (uint32_t)i / (uint32_t)C;
+  int64_t base = chunk_ptr[chunk] + ((uint32_t)i - chunk * (uint32_t)C);
   int len = row_len[i];
   double s = 0.0;
   for (int j = 0; j < len; ++j) s = fma(val[base + (int64_t)j * C], x[col[base + (int64_t)j * C]], s);
@@ -286,8 +309,10 @@ __global__ void __launch_bounds__(WARPS * 32, 4)
     const bool active = row < A.D;
     const int len = active ? A.row_len[row] : 0;
     const int wlen = __reduce_max_sync(0xffffffffu, len);
+    RowHead<double> h;
+    h.load(A, row, active);
     V16<double> acc[L::CPL], xi[L::CPL];
-    row_product<double, NB>(A, X, NB, row, active, len, wlen, gl, acc, xi);
+    row_product<double, NB>(h, X, NB, len, wlen, gl, acc, xi);
     if (active) {
 #pragma unroll
       for (int v = 0; v < L::CPL; ++v) {

@@ -114,6 +114,26 @@ fd_status host_stage(fd_ctx* ctx, size_t bytes, void** out);
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// Launch a filter step kernel; dependent: under programmatic dependent launch
+// on the step before it in the stream (the kernel calls step_wait).
+template <typename... P, typename... A>
+fd_status launch_step_kernel(fd_ctx* ctx, void (*kernel)(P...), unsigned grid, int threads, size_t smem,
+                             bool dependent, const A&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  FD_CUDA(ctx, cudaLaunchKernelEx(&cfg, kernel, args...));
+  FD_LAUNCHED(ctx);
+  return FD_OK;
+}
+
 // ---- SELL construction (fd_matrix.cu) -------------------------------------
 // Build the SELL-C-sigma arrays of `A` from a device CSR (rowptr D+1, col, val),
 // columns ascending per row.  Frees nothing it was given.

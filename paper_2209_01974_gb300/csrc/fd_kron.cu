@@ -48,6 +48,7 @@ namespace fdi {
 namespace {
 
 using step::MODE_GENERIC;
+using step::MODE_PLAIN;
 using step::MODE_SECOND;
 using step::MODE_SPMMV;
 using step::V16;
@@ -87,7 +88,8 @@ struct PanelStep {
   const T* Vin;
   T* Vout;
   T c_ax, c_x;         // x_k = c_ax (H x_{k-1}) + c_x x_{k-1} [- x_{k-2}]
-  T mu0, mu1, mu2;     // SECOND: Vout = mu0 z + mu1 x + mu2 y; GENERIC: Vout = Vin + mu2 y
+  T mu0, mu1, mu2;     // SECOND: Vout = mu0 z + mu1 x + mu2 y; GENERIC: Vout = Vin + the last nacc
+  int nacc;            // of the three terms, none if 0 (step::step_terms)
 };
 
 template <typename T>
@@ -103,7 +105,7 @@ __device__ __forceinline__ void hop_batch(V16<T>& acc, const T* const* hp, const
                                           uint64_t keep) {
   V16<T> x[N];
 #pragma unroll
-  for (int q = 0; q < N; ++q) x[q].ldg_pol(hp[q] + (int64_t)d * V16<T>::E, keep);
+  for (int q = 0; q < N; ++q) x[q].ld_pol(hp[q] + (int64_t)d * V16<T>::E, keep);
 #pragma unroll
   for (int q = 0; q < N; ++q) axpy(acc, hv[q], x[q]);
 }
@@ -134,6 +136,7 @@ __global__ void __launch_bounds__(KP_THREADS, KP_MIN_BLOCKS)
   __shared__ const T* hop_ptr[KP_MAX_HOPS];  // first row of slab u' in this panel
   __shared__ T hop_val[KP_MAX_HOPS];
 
+  step::step_release();
   const int per_panel = K.dim_up * K.chunks;
   const int p = blockIdx.x / per_panel;
   const int rem = blockIdx.x - p * per_panel;
@@ -154,8 +157,9 @@ __global__ void __launch_bounds__(KP_THREADS, KP_MIN_BLOCKS)
   const uint64_t keep = step::policy_evict_last();
   const uint64_t stream = step::policy_evict_first();
   V* slab = reinterpret_cast<V*>(kp_smem);
+  step::step_wait();
   if (STAGE)
-    for (int d = threadIdx.x; d < K.dim_dn; d += blockDim.x) slab[d].ldg_pol(X + (r0 + d) * E, keep);
+    for (int d = threadIdx.x; d < K.dim_dn; d += blockDim.x) slab[d].ld_pol(X + (r0 + d) * E, keep);
   __syncthreads();
   const uint32_t bu = K.bits_up[u];
   const int d_beg = STAGE ? 0 : chunk * KP_ROWS_UNSTAGED;
@@ -192,7 +196,7 @@ __global__ void __launch_bounds__(KP_THREADS, KP_MIN_BLOCKS)
       }
     }
     if (STAGE) xi = slab[d];
-    else xi.ldg_pol(X + (r0 + d) * E, keep);
+    else xi.ld_pol(X + (r0 + d) * E, keep);
     const T dg = K.diag[__popc(bu & bd)];
 #pragma unroll
     for (int e = 0; e < E; ++e) acc.v[e] = dg * xi.v[e];
@@ -218,7 +222,7 @@ __global__ void __launch_bounds__(KP_THREADS, KP_MIN_BLOCKS)
       for (; j < j1; ++j) {
         const uint32_t e1 = __ldg(K.dn_ent + j);
         V w;
-        w.ldg_pol(X + (r0 + (e1 & 0x7fffffffu)) * E, keep);
+        w.ld_pol(X + (r0 + (e1 & 0x7fffffffu)) * E, keep);
         axpy(acc, (e1 >> 31) ? K.dn_v1 : K.dn_v0, w);
       }
     }
@@ -229,18 +233,25 @@ __global__ void __launch_bounds__(KP_THREADS, KP_MIN_BLOCKS)
       for (int e = 0; e < E; ++e) y.v[e] = s.c_ax * acc.v[e] + s.c_x * xi.v[e];
       y.st_pol(Ys + o, stream);
     } else {
-      V out;
 #pragma unroll
       for (int e = 0; e < E; ++e) y.v[e] = s.c_ax * acc.v[e] + s.c_x * xi.v[e] - z.v[e];
-      if (MODE == MODE_SECOND) {
-#pragma unroll
-        for (int e = 0; e < E; ++e) out.v[e] = s.mu0 * z.v[e] + s.mu1 * xi.v[e] + s.mu2 * y.v[e];
-      } else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) out.v[e] = vin.v[e] + s.mu2 * y.v[e];
-      }
       if (Ys) y.st_pol(Ys + o, stream);
-      out.st_pol(Os + o, stream);
+      if (MODE != MODE_PLAIN) {
+        V out;
+        if (MODE == MODE_SECOND) {
+#pragma unroll
+          for (int e = 0; e < E; ++e) out.v[e] = s.mu0 * z.v[e] + s.mu1 * xi.v[e] + s.mu2 * y.v[e];
+        } else {
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            T a = vin.v[e];
+            if (s.nacc > 2) a = a + s.mu0 * z.v[e];
+            if (s.nacc > 1) a = a + s.mu1 * xi.v[e];
+            out.v[e] = a + s.mu2 * y.v[e];
+          }
+        }
+        out.st_pol(Os + o, stream);
+      }
     }
   }
 }
@@ -321,7 +332,7 @@ KronPanel<T> panel_args(const fd_ctx* ctx, const fd_matrix* M) {
 
 // shared-memory opt-in of the staged kernels, once per device and instantiation
 constexpr int KP_MAX_DEVICES = 64;
-bool g_kp_attr[KP_MAX_DEVICES][3] = {};
+bool g_kp_attr[KP_MAX_DEVICES][4] = {};  // by MODE
 
 template <typename T, int MODE, bool STAGE>
 fd_status launch_panel(fd_ctx* ctx, const KronPanel<T>& K, int np, const PanelStep<T>& s) {
@@ -343,9 +354,9 @@ fd_status launch_panel(fd_ctx* ctx, const KronPanel<T>& K, int np, const PanelSt
   }
   const int64_t grid = (int64_t)np * K.dim_up * K.chunks;
   if (grid >= (1ll << 31)) return set_err(ctx, FD_ERR_ARG, "panel grid too large");
-  k_kron_panel<T, MODE, STAGE><<<(unsigned)grid, KP_THREADS, smem, ctx->stream>>>(K, s);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
+  // only the first step (MODE_SPMMV) follows a kernel that is not a step
+  return launch_step_kernel(ctx, k_kron_panel<T, MODE, STAGE>, (unsigned)grid, KP_THREADS, smem,
+                            MODE != MODE_SPMMV, K, s);
 }
 
 template <typename T>
@@ -353,10 +364,12 @@ fd_status panel_step(fd_ctx* ctx, const KronPanel<T>& K, int np, int mode, const
   if (K.chunks == 1) {
     if (mode == MODE_SPMMV) return launch_panel<T, MODE_SPMMV, true>(ctx, K, np, s);
     if (mode == MODE_SECOND) return launch_panel<T, MODE_SECOND, true>(ctx, K, np, s);
+    if (mode == MODE_PLAIN) return launch_panel<T, MODE_PLAIN, true>(ctx, K, np, s);
     return launch_panel<T, MODE_GENERIC, true>(ctx, K, np, s);
   }
   if (mode == MODE_SPMMV) return launch_panel<T, MODE_SPMMV, false>(ctx, K, np, s);
   if (mode == MODE_SECOND) return launch_panel<T, MODE_SECOND, false>(ctx, K, np, s);
+  if (mode == MODE_PLAIN) return launch_panel<T, MODE_PLAIN, false>(ctx, K, np, s);
   return launch_panel<T, MODE_GENERIC, false>(ctx, K, np, s);
 }
 
@@ -399,9 +412,11 @@ fd_status kron_filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int 
   for (int k = 3; k <= n; ++k) {
     s = PanelStep<T>{};
     s.X = xp; s.Z = xpp; s.Vin = P0; s.Vout = P0;
-    s.c_ax = (T)(2 * alpha); s.c_x = (T)(2 * beta); s.mu2 = (T)mu[k];
+    s.c_ax = (T)(2 * alpha); s.c_x = (T)(2 * beta);
+    s.mu0 = (T)mu[k - 2]; s.mu1 = (T)mu[k - 1]; s.mu2 = (T)mu[k];
+    s.nacc = step::step_terms(k, n);
     s.Y = k < n ? xpp : nullptr;
-    FD_TRY(panel_step<T>(ctx, K, np, MODE_GENERIC, s));
+    FD_TRY(panel_step<T>(ctx, K, np, s.nacc ? MODE_GENERIC : MODE_PLAIN, s));
     bytes += (k < n ? 5 : 4) * vec;
     std::swap(xp, xpp);
   }

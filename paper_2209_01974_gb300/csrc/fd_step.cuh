@@ -27,9 +27,12 @@ struct V16<double> {
     double2 t = __ldg(reinterpret_cast<const double2*>(p));
     v[0] = t.x; v[1] = t.y;
   }
+  // coherent loads of vectors written by the previous step (see step_wait)
+  __device__ __forceinline__ void ld(const double* p) {
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];\n" : "=d"(v[0]), "=d"(v[1]) : "l"(p) : "memory");
+  }
   __device__ __forceinline__ void ldcs(const double* p) {
-    double2 t = __ldcs(reinterpret_cast<const double2*>(p));
-    v[0] = t.x; v[1] = t.y;
+    asm volatile("ld.global.cs.v2.f64 {%0, %1}, [%2];\n" : "=d"(v[0]), "=d"(v[1]) : "l"(p) : "memory");
   }
   __device__ __forceinline__ void stcs(double* p) const {
     __stcs(reinterpret_cast<double2*>(p), make_double2(v[0], v[1]));
@@ -38,14 +41,10 @@ struct V16<double> {
     *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
   }
   // loads and stores with an L2 eviction policy (createpolicy); the loads do
-  // not allocate in L1.  ldg_pol: read-only data (non-coherent path)
-  __device__ __forceinline__ void ldg_pol(const double* p, uint64_t pol) {
-    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;\n"
-        : "=d"(v[0]), "=d"(v[1]) : "l"(p), "l"(pol));
-  }
+  // not allocate in L1
   __device__ __forceinline__ void ld_pol(const double* p, uint64_t pol) {
     asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;\n"
-                 : "=d"(v[0]), "=d"(v[1]) : "l"(p), "l"(pol));
+                 : "=d"(v[0]), "=d"(v[1]) : "l"(p), "l"(pol) : "memory");
   }
   __device__ __forceinline__ void st_pol(double* p, uint64_t pol) const {
     asm volatile("st.global.L2::cache_hint.v2.f64 [%0], {%1, %2}, %3;\n"
@@ -60,9 +59,13 @@ struct V16<float> {
     float4 t = __ldg(reinterpret_cast<const float4*>(p));
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
   }
+  __device__ __forceinline__ void ld(const float* p) {
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p) : "memory");
+  }
   __device__ __forceinline__ void ldcs(const float* p) {
-    float4 t = __ldcs(reinterpret_cast<const float4*>(p));
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p) : "memory");
   }
   __device__ __forceinline__ void stcs(float* p) const {
     __stcs(reinterpret_cast<float4*>(p), make_float4(v[0], v[1], v[2], v[3]));
@@ -70,13 +73,9 @@ struct V16<float> {
   __device__ __forceinline__ void st(float* p) const {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
   }
-  __device__ __forceinline__ void ldg_pol(const float* p, uint64_t pol) {
-    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
-        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "l"(pol));
-  }
   __device__ __forceinline__ void ld_pol(const float* p, uint64_t pol) {
     asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "l"(pol));
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "l"(pol) : "memory");
   }
   __device__ __forceinline__ void st_pol(float* p, uint64_t pol) const {
     asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;\n"
@@ -111,7 +110,12 @@ struct SellArgs {
   int C;
 };
 
-enum { MODE_SPMMV = 0, MODE_SECOND = 1, MODE_GENERIC = 2 };
+// Step k holds x_{k-2} (z), x_{k-1} (the row's own gathered vector) and x_k, so
+// one step in three adds the last three terms to the accumulator (MODE_GENERIC)
+// and the two others leave it alone (MODE_PLAIN): 11/3 vectors moved per step on
+// average instead of five.  The terms enter the sum in the same order and from
+// the same stored values as one by one.  MODE_EITHER decides by nacc at run time.
+enum { MODE_SPMMV = 0, MODE_SECOND = 1, MODE_GENERIC = 2, MODE_PLAIN = 3, MODE_EITHER = 4 };
 
 template <typename T>
 struct StepArgs {
@@ -121,8 +125,33 @@ struct StepArgs {
   const T* Vin; int64_t ldvi;
   T* Vout; int64_t ldvo;
   T c_ax, c_x;               // x_k = c_ax * (A x_{k-1}) + c_x * x_{k-1} [- x_{k-2}]
-  T mu0, mu1, mu2;           // SECOND: Vout = mu0 z + mu1 x + mu2 y; GENERIC: Vout = Vin + mu2 y
+  T mu0, mu1, mu2;           // SECOND: Vout = mu0 z + mu1 x + mu2 y; GENERIC: Vout = Vin + [mu0 z +]
+                             // [mu1 x +] mu2 y, the last nacc (1 .. 3) of the terms, or no accumulation (0)
+  int nacc;
 };
+
+template <int MODE, typename S>
+__device__ __forceinline__ bool accumulates(const S& s) {
+  return MODE == MODE_SECOND || MODE == MODE_GENERIC || (MODE == MODE_EITHER && s.nacc);
+}
+
+// Which of the generic steps 3 .. n accumulate, and how many terms: the second
+// step has added mu_0 .. mu_2, then every third step adds three, and the last
+// step whatever is left.
+__host__ __device__ __forceinline__ int step_terms(int k, int n) {
+  const int r = (k - 2) % 3;
+  return r == 0 ? 3 : k == n ? r : 0;
+}
+
+// Programmatic dependent launch: a step kernel lets the next one's CTAs start
+// while its own last CTAs run (step_release), and touches the vectors the
+// previous step wrote only after that step has completed (step_wait); what it
+// loads before the wait (matrix entries, hop lists) is written by no step.
+// Every thread passes step_wait, so a step's completion implies its
+// predecessors'.  The vectors are read with coherent loads (a step starts
+// before its operands are final, which rules out the read-only path).
+__device__ __forceinline__ void step_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
 constexpr int WARPS = 8;
 constexpr int BATCH = 4;   // entries per batch; SELL chunk lengths are multiples of 8
@@ -152,6 +181,31 @@ struct Layout {
   static_assert(NB % E == 0 && Q % G == 0, "nb must fill whole 16-byte vectors");
 };
 
+// The first BATCH entries of a SELL row and where the rest is.
+template <typename T>
+struct RowHead {
+  const int32_t* cp;
+  const T* vp;
+  uint32_t C;
+  int32_t c[BATCH];
+  T a[BATCH];
+  // Rows at or beyond D inside the last chunk are SELL padding rows: their
+  // entries exist (value 0, column 0), but they have no vector row.
+  __device__ __forceinline__ void load(const SellArgs<T>& A, int64_t row, bool active) {
+    C = (uint32_t)A.C;
+    const uint32_t r = (uint32_t)row, chunk = r / C;  // rows < 2^31: a 64-bit division costs tens of instructions
+    const int64_t base = __ldg(A.chunk_ptr + chunk) + (r - chunk * C);
+    cp = A.col + base;
+    vp = A.val + base;
+#pragma unroll
+    for (int u = 0; u < BATCH; ++u) {
+      c[u] = __ldg(cp + u * C);
+      a[u] = ldg_val(vp + u * C);
+    }
+    if (!active) { c[0] = 0; a[0] = T(0); }
+  }
+};
+
 // Gather-accumulate s = sum_j a_ij x_j over the SELL row, returning the row's
 // own vector xi (entry 0 is the diagonal).  Entries are taken BATCH at a time:
 // the matrix loads of a batch, then all its gathers, so a row of up to BATCH
@@ -160,45 +214,28 @@ struct Layout {
 // bounds; the gathers and FMAs of entries past the row's own length are
 // skipped (FP64 arithmetic, not memory, bounds the FP64 step on GB300).
 template <typename T, int NB>
-__device__ __forceinline__ void row_product(const SellArgs<T>& A, const T* __restrict__ X,
-                                            int64_t ldx, int64_t row, bool active, int len,
-                                            int wlen, int gl, V16<T> (&acc)[Layout<T, NB>::CPL],
+__device__ __forceinline__ void row_product(const RowHead<T>& h, const T* X, int64_t ldx, int len, int wlen,
+                                            int gl, V16<T> (&acc)[Layout<T, NB>::CPL],
                                             V16<T> (&xi)[Layout<T, NB>::CPL]) {
   using L = Layout<T, NB>;
   constexpr int E = L::E;
-  // Rows at or beyond D inside the last chunk are SELL padding rows: their
-  // entries exist (value 0, column 0), but they have no vector row.
-  const int64_t base = A.chunk_ptr[row / A.C] + (row % A.C);
-  const int32_t* cp = A.col + base;
-  const T* vp = A.val + base;
-  const uint32_t C = (uint32_t)A.C;
   const uint32_t ld = (uint32_t)ldx;
   const T* xl = X + gl * E;
-  {
-    int32_t c[BATCH];
-    T a[BATCH];
 #pragma unroll
-    for (int u = 0; u < BATCH; ++u) {
-      c[u] = __ldg(cp + u * C);
-      a[u] = ldg_val(vp + u * C);
-    }
-    if (!active) { c[0] = 0; a[0] = T(0); }
+  for (int v = 0; v < L::CPL; ++v) {
+    xi[v].ld(xl + (uint64_t)(uint32_t)h.c[0] * ld + v * L::G * E);
 #pragma unroll
-    for (int v = 0; v < L::CPL; ++v) {
-      xi[v].ldg(xl + (uint64_t)(uint32_t)c[0] * ld + v * L::G * E);
+    for (int e = 0; e < E; ++e) acc[v].v[e] = h.a[0] * xi[v].v[e];
+  }
 #pragma unroll
-      for (int e = 0; e < E; ++e) acc[v].v[e] = a[0] * xi[v].v[e];
-    }
+  for (int u = 1; u < BATCH; ++u) {
+    if (u < len) {  // entries past the row's length are padding: skip their FMAs
 #pragma unroll
-    for (int u = 1; u < BATCH; ++u) {
-      if (u < len) {  // entries past the row's length are padding: skip their FMAs
+      for (int v = 0; v < L::CPL; ++v) {
+        V16<T> x;
+        x.ld(xl + (uint64_t)(uint32_t)h.c[u] * ld + v * L::G * E);
 #pragma unroll
-        for (int v = 0; v < L::CPL; ++v) {
-          V16<T> x;
-          x.ldg(xl + (uint64_t)(uint32_t)c[u] * ld + v * L::G * E);
-#pragma unroll
-          for (int e = 0; e < E; ++e) acc[v].v[e] = fma(a[u], x.v[e], acc[v].v[e]);
-        }
+        for (int e = 0; e < E; ++e) acc[v].v[e] = fma(h.a[u], x.v[e], acc[v].v[e]);
       }
     }
   }
@@ -207,8 +244,8 @@ __device__ __forceinline__ void row_product(const SellArgs<T>& A, const T* __res
     T a[BATCH];
 #pragma unroll
     for (int u = 0; u < BATCH; ++u) {
-      c[u] = __ldg(cp + (j0 + u) * C);
-      a[u] = ldg_val(vp + (j0 + u) * C);
+      c[u] = __ldg(h.cp + (j0 + u) * h.C);
+      a[u] = ldg_val(h.vp + (j0 + u) * h.C);
     }
 #pragma unroll
     for (int u = 0; u < BATCH; ++u) {
@@ -216,7 +253,7 @@ __device__ __forceinline__ void row_product(const SellArgs<T>& A, const T* __res
 #pragma unroll
         for (int v = 0; v < L::CPL; ++v) {
           V16<T> x;
-          x.ldg(xl + (uint64_t)(uint32_t)c[u] * ld + v * L::G * E);
+          x.ld(xl + (uint64_t)(uint32_t)c[u] * ld + v * L::G * E);
 #pragma unroll
           for (int e = 0; e < E; ++e) acc[v].v[e] = fma(a[u], x.v[e], acc[v].v[e]);
         }
@@ -242,7 +279,7 @@ template <typename T, int NB, int MODE>
 __device__ __forceinline__ void prefetch_rows(const SellArgs<T>& A, const StepArgs<T>& s,
                                               int64_t r0, int64_t r1) {
   constexpr int LPR = (NB * (int)sizeof(T) + 127) / 128;  // lines per vector row
-  constexpr int NS = MODE == MODE_GENERIC ? 3 : MODE == MODE_SECOND ? 2 : 1;
+  constexpr int NS = MODE == MODE_GENERIC ? 3 : MODE == MODE_SPMMV ? 1 : 2;
   const int n = (int)(r1 - r0) * LPR;
   for (int q = threadIdx.x; q < NS * n; q += blockDim.x) {
     const int st = q / n, rq = q % n;
@@ -252,7 +289,7 @@ __device__ __forceinline__ void prefetch_rows(const SellArgs<T>& A, const StepAr
     prefetch_l2(p + off);
   }
   if (threadIdx.x >= blockDim.x - 32) {
-    const int64_t c0 = (r0 + A.C - 1) / A.C, c1 = (r1 + A.C - 1) / A.C;
+    const uint32_t C = (uint32_t)A.C, c0 = ((uint32_t)r0 + C - 1) / C, c1 = ((uint32_t)r1 + C - 1) / C;
     if (c0 >= c1) return;
     const int64_t e0 = A.chunk_ptr[c0], e1 = A.chunk_ptr[c1];
     const int64_t l0c = (e0 * 4) >> 7, l1c = (e1 * 4 + 127) >> 7;
@@ -265,34 +302,15 @@ __device__ __forceinline__ void prefetch_rows(const SellArgs<T>& A, const StepAr
   }
 }
 
-// One fused Chebyshev step (or a plain SpMMV) for the warp's rows row0 ..
-// row0 + RPW - 1 (row0 < D, a multiple of RPW); all 32 lanes must call it.
+// x_k of one row from its product, and the accumulator
 template <typename T, int NB, int MODE>
-__device__ __forceinline__ void cheb_rows(const SellArgs<T>& A, const StepArgs<T>& s,
-                                          int64_t row0) {
+__device__ __forceinline__ void step_epilogue(const StepArgs<T>& s, int64_t row, int gl,
+                                              const V16<T> (&acc)[Layout<T, NB>::CPL],
+                                              const V16<T> (&xi)[Layout<T, NB>::CPL],
+                                              const V16<T> (&z)[Layout<T, NB>::CPL],
+                                              const V16<T> (&vin)[Layout<T, NB>::CPL]) {
   using L = Layout<T, NB>;
   constexpr int E = L::E;
-  const int lane = threadIdx.x & 31;
-  const int g = lane / L::G, gl = lane % L::G;
-  const int64_t row = row0 + g;
-  const bool active = row < A.D;
-  const int len = active ? A.row_len[row] : 0;
-  const int wlen = __reduce_max_sync(0xffffffffu, len);
-
-  // the row-wise operands do not depend on the gathers: issue them first
-  V16<T> z[L::CPL], vin[L::CPL];
-  if (MODE != MODE_SPMMV && active) {
-#pragma unroll
-    for (int v = 0; v < L::CPL; ++v) {
-      const int64_t off = gl * E + v * L::G * E;
-      z[v].ldcs(s.Z + row * s.ldz + off);
-      if (MODE == MODE_GENERIC) vin[v].ldcs(s.Vin + row * s.ldvi + off);
-    }
-  }
-  V16<T> acc[L::CPL], xi[L::CPL];
-  row_product<T, NB>(A, s.X, s.ldx, row, active, len, wlen, gl, acc, xi);
-  if (!active) return;
-
 #pragma unroll
   for (int v = 0; v < L::CPL; ++v) {
     const int64_t off = gl * E + v * L::G * E;
@@ -302,21 +320,64 @@ __device__ __forceinline__ void cheb_rows(const SellArgs<T>& A, const StepArgs<T
       for (int e = 0; e < E; ++e) y.v[e] = s.c_ax * acc[v].v[e] + s.c_x * xi[v].v[e];
       y.st(s.Y + row * s.ldy + off);
     } else {
-      V16<T> o;
 #pragma unroll
       for (int e = 0; e < E; ++e) y.v[e] = s.c_ax * acc[v].v[e] + s.c_x * xi[v].v[e] - z[v].v[e];
-      if (MODE == MODE_SECOND) {
+      if (accumulates<MODE>(s)) {
+        V16<T> o;
+        if (MODE == MODE_SECOND) {
 #pragma unroll
-        for (int e = 0; e < E; ++e)
-          o.v[e] = s.mu0 * z[v].v[e] + s.mu1 * xi[v].v[e] + s.mu2 * y.v[e];
-      } else {
+          for (int e = 0; e < E; ++e)
+            o.v[e] = s.mu0 * z[v].v[e] + s.mu1 * xi[v].v[e] + s.mu2 * y.v[e];
+        } else {
 #pragma unroll
-        for (int e = 0; e < E; ++e) o.v[e] = vin[v].v[e] + s.mu2 * y.v[e];
+          for (int e = 0; e < E; ++e) {
+            T a = vin[v].v[e];
+            if (s.nacc > 2) a = a + s.mu0 * z[v].v[e];
+            if (s.nacc > 1) a = a + s.mu1 * xi[v].v[e];
+            o.v[e] = a + s.mu2 * y.v[e];
+          }
+        }
+        o.stcs(s.Vout + row * s.ldvo + off);
       }
       if (s.Y) y.st(s.Y + row * s.ldy + off);
-      o.stcs(s.Vout + row * s.ldvo + off);
     }
   }
+}
+
+// One fused Chebyshev step (or a plain SpMMV) for the warp's rows row0 ..
+// row0 + RPW - 1 (row0 < D, a multiple of RPW); all 32 lanes must call it.
+// WAIT: the step runs under programmatic dependent launch; the row's first
+// entries are loaded before the wait.
+template <typename T, int NB, int MODE, bool WAIT = false>
+__device__ __forceinline__ void cheb_rows(const SellArgs<T>& A, const StepArgs<T>& s,
+                                          int64_t row0) {
+  using L = Layout<T, NB>;
+  constexpr int E = L::E;
+  const int lane = threadIdx.x & 31;
+  const int g = lane / L::G, gl = lane % L::G;
+  const int64_t row = row0 + g;
+  const bool active = row < A.D;
+  const int len = active ? __ldg(A.row_len + row) : 0;
+  RowHead<T> h;
+  h.load(A, row, active);
+  const int wlen = __reduce_max_sync(0xffffffffu, len);
+  if (WAIT) step_wait();
+
+  // the row-wise operands do not depend on the gathers: issue them first
+  V16<T> z[L::CPL], vin[L::CPL];
+  if (MODE != MODE_SPMMV && active) {
+#pragma unroll
+    for (int v = 0; v < L::CPL; ++v) {
+      const int64_t off = gl * E + v * L::G * E;
+      z[v].ldcs(s.Z + row * s.ldz + off);
+      if (MODE != MODE_SECOND && accumulates<MODE>(s)) vin[v].ldcs(s.Vin + row * s.ldvi + off);
+    }
+  }
+  V16<T> acc[L::CPL], xi[L::CPL];
+  row_product<T, NB>(h, s.X, s.ldx, len, wlen, gl, acc, xi);
+  if (!active) return;
+
+  step_epilogue<T, NB, MODE>(s, row, gl, acc, xi, z, vin);
 }
 
 // ---------------------------------------------------------------------------
@@ -344,37 +405,61 @@ struct KronArgs {
 
 // s = sum_j h_ij x_j for row (u, d), the entries in the order of the stored
 // row (diagonal first, then ascending columns: the up hops to u' < u, the
-// down hops, the up hops to u' > u), so the sums round as in the SELL kernel
+// down hops, the up hops to u' > u), so the sums round as in the SELL kernel.
+// Hops are taken BATCH at a time, as in row_product: the table loads of a
+// batch, then its gathers.
 template <typename T, int NB>
-__device__ __forceinline__ void kron_row_product(const KronArgs<T>& K, const T* __restrict__ X, int64_t ldx,
+__device__ __forceinline__ void kron_row_product(const KronArgs<T>& K, const T* X, int64_t ldx,
                                                  int64_t row, int gl, V16<T> (&acc)[Layout<T, NB>::CPL],
                                                  V16<T> (&xi)[Layout<T, NB>::CPL]) {
   using L = Layout<T, NB>;
   constexpr int E = L::E;
   const T* xl = X + gl * E;
-  const int64_t u = row / K.dim_dn, d = row - u * K.dim_dn;
-  const T dg = K.diag[__popc(K.bits_up[u] & K.bits_dn[d])];
+  const int64_t u = (uint32_t)row / (uint32_t)K.dim_dn, d = row - u * K.dim_dn;
+  const T dg = K.diag[__popc(__ldg(K.bits_up + u) & __ldg(K.bits_dn + d))];
+  const int64_t ku = __ldg(K.ptr_up + u), ke = __ldg(K.ptr_up + u + 1);
+  const int64_t kd = __ldg(K.ptr_dn + d), kde = __ldg(K.ptr_dn + d + 1);
 #pragma unroll
   for (int v = 0; v < L::CPL; ++v) {
-    xi[v].ldg(xl + row * ldx + v * L::G * E);
+    xi[v].ld(xl + row * ldx + v * L::G * E);
 #pragma unroll
     for (int e = 0; e < E; ++e) acc[v].v[e] = dg * xi[v].v[e];
   }
-  auto add = [&](T a, int64_t r) {
+  // entries [k, ke) of one table
+  auto hops = [&](const int32_t* col, const T* val, int64_t k, int64_t ke, int64_t r0, int64_t rs) {
+    for (; k < ke; k += BATCH) {
+      int32_t c[BATCH];
+      T a[BATCH];
 #pragma unroll
-    for (int v = 0; v < L::CPL; ++v) {
-      V16<T> x;
-      x.ldg(xl + r * ldx + v * L::G * E);
+      for (int q = 0; q < BATCH; ++q) {
+        const int64_t kq = k + q < ke ? k + q : ke - 1;
+        c[q] = __ldg(col + kq);
+        a[q] = ldg_val(val + kq);
+      }
 #pragma unroll
-      for (int e = 0; e < E; ++e) acc[v].v[e] = fma(a, x.v[e], acc[v].v[e]);
+      for (int q = 0; q < BATCH; ++q) {
+        if (k + q < ke) {
+          const T* xr = xl + (r0 + c[q] * rs) * ldx;
+#pragma unroll
+          for (int v = 0; v < L::CPL; ++v) {
+            V16<T> x;
+            x.ld(xr + v * L::G * E);
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc[v].v[e] = fma(a[q], x.v[e], acc[v].v[e]);
+          }
+        }
+      }
     }
   };
-  int64_t k = K.ptr_up[u];
-  const int64_t ke = K.ptr_up[u + 1];
-  for (; k < ke && K.col_up[k] < u; ++k) add(K.val_up[k], (int64_t)K.col_up[k] * K.dim_dn + d);
-  const int64_t kd1 = K.ptr_dn[d + 1];
-  for (int64_t kd = K.ptr_dn[d]; kd < kd1; ++kd) add(K.val_dn[kd], u * K.dim_dn + K.col_dn[kd]);
-  for (; k < ke; ++k) add(K.val_up[k], (int64_t)K.col_up[k] * K.dim_dn + d);
+  int64_t k1 = ku, hi = ke;  // first up hop to u' > u (targets ascend)
+  while (k1 < hi) {
+    const int64_t mid = (k1 + hi) >> 1;
+    if (__ldg(K.col_up + mid) < u) k1 = mid + 1;
+    else hi = mid;
+  }
+  hops(K.col_up, K.val_up, ku, k1, d, K.dim_dn);
+  hops(K.col_dn, K.val_dn, kd, kde, u * K.dim_dn, 1);
+  hops(K.col_up, K.val_up, k1, ke, d, K.dim_dn);
 }
 
 // One fused Chebyshev step with the matrix-free Hubbard operator; the same
@@ -386,6 +471,7 @@ __device__ __forceinline__ void kron_rows(const KronArgs<T>& K, const StepArgs<T
   const int lane = threadIdx.x & 31;
   const int g = lane / L::G, gl = lane % L::G;
   const int64_t row = row0 + g;
+  step_wait();
   if (row >= K.D) return;  // no warp-wide operations follow
   V16<T> z[L::CPL], vin[L::CPL];
   if (MODE != MODE_SPMMV) {
@@ -393,35 +479,12 @@ __device__ __forceinline__ void kron_rows(const KronArgs<T>& K, const StepArgs<T
     for (int v = 0; v < L::CPL; ++v) {
       const int64_t off = gl * E + v * L::G * E;
       z[v].ldcs(s.Z + row * s.ldz + off);
-      if (MODE == MODE_GENERIC) vin[v].ldcs(s.Vin + row * s.ldvi + off);
+      if (MODE != MODE_SECOND && accumulates<MODE>(s)) vin[v].ldcs(s.Vin + row * s.ldvi + off);
     }
   }
   V16<T> acc[L::CPL], xi[L::CPL];
   kron_row_product<T, NB>(K, s.X, s.ldx, row, gl, acc, xi);
-#pragma unroll
-  for (int v = 0; v < L::CPL; ++v) {
-    const int64_t off = gl * E + v * L::G * E;
-    V16<T> y;
-    if (MODE == MODE_SPMMV) {
-#pragma unroll
-      for (int e = 0; e < E; ++e) y.v[e] = s.c_ax * acc[v].v[e] + s.c_x * xi[v].v[e];
-      y.st(s.Y + row * s.ldy + off);
-    } else {
-      V16<T> o;
-#pragma unroll
-      for (int e = 0; e < E; ++e) y.v[e] = s.c_ax * acc[v].v[e] + s.c_x * xi[v].v[e] - z[v].v[e];
-      if (MODE == MODE_SECOND) {
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-          o.v[e] = s.mu0 * z[v].v[e] + s.mu1 * xi[v].v[e] + s.mu2 * y.v[e];
-      } else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) o.v[e] = vin[v].v[e] + s.mu2 * y.v[e];
-      }
-      if (s.Y) y.st(s.Y + row * s.ldy + off);
-      o.stcs(s.Vout + row * s.ldvo + off);
-    }
-  }
+  step_epilogue<T, NB, MODE>(s, row, gl, acc, xi, z, vin);
 }
 
 }  // namespace step
