@@ -22,6 +22,7 @@
 #include "fd_internal.cuh"
 #include "fd_step.cuh"
 #include "fd_ff.cuh"
+#include "fd_eig.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -31,7 +32,7 @@ namespace {
 using namespace step;
 using ffa::ff;
 
-constexpr int BMAX_NS = 96;  // single-CTA shared-memory Jacobi / Cholesky limit
+constexpr int BMAX_NS = 96;  // single-CTA shared-memory Cholesky limit
 
 struct BInst {
   SellArgs<double> A;
@@ -513,112 +514,6 @@ __global__ void __launch_bounds__(256) k_brotate(const BInst* insts, const BPara
   }
 }
 
-// cyclic Jacobi on G (n x n, n <= BMAX_NS) in shared memory; eigenvalues
-// ascending into theta, eigenvectors (columns) into Ri
-__global__ void __launch_bounds__(256) k_bjacobi(const BInst* insts, const BParams* par) {
-  const BInst& I = insts[blockIdx.x];
-  const BParams& Pm = par[blockIdx.x];
-  if (!Pm.active || (Pm.flags & 2)) return;
-  const int n = I.ns, np = n + (n & 1), half = np / 2;
-  extern __shared__ double sm[];
-  double* A = sm;              // np x np
-  double* Q = A + np * np;     // np x np
-  double* cs = Q + np * np;    // 2 * half
-  __shared__ double red[256];
-  for (int e = threadIdx.x; e < np * np; e += blockDim.x) {
-    int i = e / np, j = e % np;
-    A[e] = (i < n && j < n) ? I.G[i * n + j] : 0.0;
-    Q[e] = i == j ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  double fro = 0.0;
-  for (int e = threadIdx.x; e < np * np; e += blockDim.x) fro += A[e] * A[e];
-  red[threadIdx.x] = fro;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  const double fro2 = red[0];
-  __syncthreads();
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    double off = 0.0;
-    for (int e = threadIdx.x; e < np * np; e += blockDim.x)
-      if (e / np != e % np) off += A[e] * A[e];
-    red[threadIdx.x] = off;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    const bool done = red[0] <= 1e-28 * fro2;
-    __syncthreads();
-    if (done) break;
-    for (int round = 0; round < np - 1; ++round) {
-      const int m = np - 1;
-      for (int k = threadIdx.x; k < half; k += blockDim.x) {
-        int a = k == 0 ? round % m : (round + k) % m;
-        int b = k == 0 ? m : (round - k + m) % m;
-        int p = min(a, b), q = max(a, b);
-        double apq = A[p * np + q], c = 1.0, s = 0.0;
-        if (apq != 0.0) {
-          double tau = (A[q * np + q] - A[p * np + p]) / (2.0 * apq);
-          double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-          c = 1.0 / sqrt(1.0 + t * t);
-          s = t * c;
-        }
-        cs[2 * k] = c;
-        cs[2 * k + 1] = s;
-      }
-      __syncthreads();
-      // rows: A <- J^T A
-      for (int e = threadIdx.x; e < half * np; e += blockDim.x) {
-        int k = e / np, j = e % np;
-        int a = k == 0 ? round % m : (round + k) % m;
-        int b = k == 0 ? m : (round - k + m) % m;
-        int p = min(a, b), q = max(a, b);
-        double c = cs[2 * k], s = cs[2 * k + 1];
-        double ap = A[p * np + j], aq = A[q * np + j];
-        A[p * np + j] = c * ap - s * aq;
-        A[q * np + j] = s * ap + c * aq;
-      }
-      __syncthreads();
-      // columns: A <- A J, Q <- Q J
-      for (int e = threadIdx.x; e < half * np; e += blockDim.x) {
-        int k = e / np, i = e % np;
-        int a = k == 0 ? round % m : (round + k) % m;
-        int b = k == 0 ? m : (round - k + m) % m;
-        int p = min(a, b), q = max(a, b);
-        double c = cs[2 * k], s = cs[2 * k + 1];
-        double ap = A[i * np + p], aq = A[i * np + q];
-        A[i * np + p] = c * ap - s * aq;
-        A[i * np + q] = s * ap + c * aq;
-        double qp = Q[i * np + p], qq = Q[i * np + q];
-        Q[i * np + p] = c * qp - s * qq;
-        Q[i * np + q] = s * qp + c * qq;
-      }
-      __syncthreads();
-      for (int k = threadIdx.x; k < half; k += blockDim.x) {
-        int a = k == 0 ? round % m : (round + k) % m;
-        int b = k == 0 ? m : (round - k + m) % m;
-        A[a * np + b] = 0.0;
-        A[b * np + a] = 0.0;
-      }
-      __syncthreads();
-    }
-  }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double ai = A[i * np + i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      const double aj = A[j * np + j];
-      rank += (aj < ai) || (aj == ai && j < i);
-    }
-    I.theta[rank] = ai;
-    for (int r = 0; r < n; ++r) I.Ri[r * n + rank] = Q[r * np + i];
-  }
-}
-
 __global__ void k_bresid(const BInst* insts, const BParams* par) {
   const BInst& I = insts[blockIdx.y];
   const BParams& Pm = par[blockIdx.y];
@@ -671,6 +566,9 @@ struct Batch {
   std::vector<int64_t> h_off;
   BInst* d_inst = nullptr;
   BParams* d_par = nullptr;
+  EigTask* d_eig = nullptr;
+  float* d_eig_part = nullptr;
+  std::vector<EigTask> h_eig;
   BTask* d_task = nullptr;
   int64_t* d_off = nullptr;
   double* d_mu = nullptr;
@@ -754,7 +652,7 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
     const size_t nn = (size_t)ns[i] * ns[i];
     off[i] = bytes;
     bytes += sizeof(double) * (2 * D * ns[i] + 2 * D * ns[i] + 3 * nn + GSLICES * nn + 2 * ns[i] +
-                               RBLK * ns[i]);
+                               RBLK * ns[i] + eig_work_doubles(ns[i]));
     bytes = (bytes + 255) & ~(size_t)255;
     if (f32) bytes += sizeof(float) * 3 * D * ns[i] + 256;  // V32 and the bundles' W32
     bytes = (bytes + 255) & ~(size_t)255;
@@ -763,6 +661,7 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
   }
   FD_CUDA(ctx, cudaMalloc(&B.arena, bytes));
   B.h_inst.resize(n);
+  B.h_eig.assign(n, EigTask{});
   for (int i = 0; i < n; ++i) {
     const fd_matrix* M = A[i];
     BInst& I = B.h_inst[i];
@@ -789,12 +688,14 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
     I.W32 = nullptr;
     if (f32) {  // after the FP64 part, 256-byte aligned
       char* q = (char*)B.arena + off[i] +
-                (((sizeof(double) * (4 * D * ns[i] + 3 * nn + GSLICES * nn + 2 * ns[i] + RBLK * ns[i])) + 255) &
+                (((sizeof(double) * (4 * D * ns[i] + 3 * nn + GSLICES * nn + 2 * ns[i] + RBLK * ns[i] +
+                                    eig_work_doubles(ns[i]))) + 255) &
                  ~(size_t)255);
       I.V32 = (float*)q;
       I.W32 = I.V32 + D * ns[i];
     }
-    I.rpart = p;
+    I.rpart = p; p += RBLK * ns[i];
+    eig_task_layout(&B.h_eig[i], ns[i], p);
     for (int b = 0; b < ns[i] / nb; ++b) B.h_task.push_back({i, b});
   }
   B.h_off.assign(B.h_task.size() + 1, 0);
@@ -807,6 +708,16 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
   FD_TRY(workspace(ctx, "batch_desc", sizeof(BInst) * n + sizeof(BParams) * n + sizeof(BTask) * nta +
                                           sizeof(int64_t) * (nta + 1) + sizeof(int) * (nta + 1) + 64, &p));
   char* c = (char*)p;
+  for (int i = 0; i < n; ++i) {  // the parameters' place is known now
+    const BParams* par = (const BParams*)(c + sizeof(BInst) * n) + i;
+    EigTask& E = B.h_eig[i];
+    E.H = B.h_inst[i].G;
+    E.w = B.h_inst[i].theta;
+    E.Qout = B.h_inst[i].Ri;
+    E.active = &par->active;
+    E.flags = &par->flags;
+    E.flag_mask = 2;
+  }
   B.d_inst = (BInst*)c; c += sizeof(BInst) * n;
   B.d_par = (BParams*)c; c += sizeof(BParams) * n;
   B.d_task = (BTask*)c; c += sizeof(BTask) * nta;
@@ -814,6 +725,11 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
   B.d_off = (int64_t*)c; c += sizeof(int64_t) * (nta + 1);
   B.d_tdeg = (int*)c; c += sizeof(int) * nta;
   B.d_ntask = (int*)c;
+  void* pe;
+  FD_TRY(workspace(ctx, "batch_eig", sizeof(EigTask) * n + sizeof(float) * eig_part_floats(ctx, n), &pe));
+  B.d_eig = (EigTask*)pe;
+  B.d_eig_part = (float*)(B.d_eig + n);
+  FD_CUDA(ctx, cudaMemcpyAsync(B.d_eig, B.h_eig.data(), sizeof(EigTask) * n, cudaMemcpyHostToDevice, ctx->stream));
   B.mu_cap = mu_cap;
   FD_TRY(workspace(ctx, "batch_mu", sizeof(double) * mu_cap + 64, &p));
   B.d_mu = (double*)p;
@@ -897,8 +813,6 @@ fd_status launch_ortho_rr(fd_ctx* ctx, Batch& B) {
   const dim3 rgrid((unsigned)cdiv(B.max_D, 16), n);
   const size_t chol_smem = sizeof(double) * (nsm * nsm + 8 * nsm);
   const size_t rot_smem = sizeof(double) * 16 * nsm;
-  const int np = nsm + (nsm & 1);
-  const size_t jac_smem = sizeof(double) * (2 * np * np + np);
   for (int pass = 0; pass < 3; ++pass) {
     const int only_shifted = pass == 2;
     k_bgram_partial<<<ggrid, 256, 0, st>>>(B.d_inst, B.d_par, 0, only_shifted);
@@ -915,8 +829,7 @@ fd_status launch_ortho_rr(fd_ctx* ctx, Batch& B) {
   FD_LAUNCHED(ctx);
   k_bgram_reduce<<<dim3((unsigned)cdiv(nsm * nsm, 256), n), 256, 0, st>>>(B.d_inst, B.d_par, 0);
   FD_LAUNCHED(ctx);
-  k_bjacobi<<<n, 256, jac_smem, st>>>(B.d_inst, B.d_par);
-  FD_LAUNCHED(ctx);
+  FD_TRY(eig_batch(ctx, B.d_eig, n, nsm, 40, B.d_eig_part));
   k_brotate<<<rgrid, 256, rot_smem, st>>>(B.d_inst, B.d_par, 0, 0, 0);
   FD_LAUNCHED(ctx);
   FD_TRY(launch_filter(ctx, B, 1));  // A (V Q) directly, cheaper than rotating AV
@@ -930,11 +843,8 @@ fd_status launch_ortho_rr(fd_ctx* ctx, Batch& B) {
 fd_status set_kernel_smem(fd_ctx* ctx, int nsm) {
   const size_t chol_smem = sizeof(double) * (nsm * nsm + 8 * nsm);
   const size_t rot_smem = sizeof(double) * 16 * nsm;
-  const int np = nsm + (nsm & 1);
-  const size_t jac_smem = sizeof(double) * (2 * np * np + np);
   FD_CUDA(ctx, cudaFuncSetAttribute(k_bchol_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chol_smem));
   FD_CUDA(ctx, cudaFuncSetAttribute(k_brotate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rot_smem));
-  FD_CUDA(ctx, cudaFuncSetAttribute(k_bjacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)jac_smem));
   return FD_OK;
 }
 

@@ -1,7 +1,6 @@
 // Dense FP64 kernels of the FD loop: tall-skinny Gram products, in-place block
-// rotations, Cholesky and triangular inverse (Cholesky-QR, Sec. 2), the
-// parallel cyclic Jacobi eigensolver of the Rayleigh-Ritz step (Sec. 2) and
-// the residual norms rho_i = ||A v_i - theta_i v_i||_2 (Sec. 2, Alg. 1).
+// rotations, Cholesky and triangular inverse (Cholesky-QR, Sec. 2) and the
+// residual norms rho_i = ||A v_i - theta_i v_i||_2 (Sec. 2, Alg. 1).
 //
 // FP64 arithmetic on GB300 runs at about 1.2 TFLOP/s, so these kernels are
 // FP64-ALU bound; they use register tiles fed from shared memory and split the
@@ -260,142 +259,6 @@ __global__ void k_identity(double* A, int n) {
 }
 
 // ---------------------------------------------------------------------------
-// parallel cyclic Jacobi (round-robin pairing), cooperative grid
-// ---------------------------------------------------------------------------
-struct JacobiArgs {
-  double* A0;   // np x np, current
-  double* A1;   // np x np, next
-  double* Q;    // np x np, accumulated rotations
-  double* part; // gridDim.x partial sums
-  int n, np;
-  int max_sweeps;
-  double rel_tol;
-  int* sweeps_out;
-};
-
-__device__ __forceinline__ void pair_of(int round, int k, int np, int* p, int* q) {
-  int a, b;
-  const int m = np - 1;
-  if (k == 0) { a = round % m; b = m; }
-  else { a = (round + k) % m; b = (round - k + m) % m; }
-  *p = min(a, b);
-  *q = max(a, b);
-}
-
-__device__ __forceinline__ void rot_params(const double* A, int np, int p, int q, double* c,
-                                           double* s) {
-  const double apq = A[(int64_t)p * np + q];
-  if (apq == 0.0) { *c = 1.0; *s = 0.0; return; }
-  const double app = A[(int64_t)p * np + p], aqq = A[(int64_t)q * np + q];
-  const double tau = (aqq - app) / (2.0 * apq);
-  const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-  *c = 1.0 / sqrt(1.0 + t * t);
-  *s = t * (*c);
-}
-
-__device__ double grid_sum(cg::grid_group& grid, double v, double* part, double* sh) {
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-  grid.sync();
-  double s = 0.0;
-  for (int b = 0; b < (int)gridDim.x; ++b) s += part[b];  // same order in every CTA
-  grid.sync();  // every CTA has read `part` before it is reused
-  return s;
-}
-
-__global__ void __launch_bounds__(256) k_jacobi(JacobiArgs a) {
-  cg::grid_group grid = cg::this_grid();
-  __shared__ double sh[256];
-  extern __shared__ double cs[];  // np/2 (c, s) pairs for the current round
-  const int np = a.np, half = np / 2;
-  const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
-  double* Acur = a.A0;
-  double* Anext = a.A1;
-  // Frobenius norm of A
-  double f = 0.0;
-  for (int64_t e = gtid; e < (int64_t)np * np; e += gthreads) f += Acur[e] * Acur[e];
-  const double fro2 = grid_sum(grid, f, a.part, sh);
-  int sweep = 0;
-  for (; sweep < a.max_sweeps; ++sweep) {
-    double off = 0.0;
-    for (int64_t e = gtid; e < (int64_t)np * np; e += gthreads)
-      if (e / np != e % np) off += Acur[e] * Acur[e];
-    const double off2 = grid_sum(grid, off, a.part, sh);
-    if (off2 <= a.rel_tol * a.rel_tol * fro2) break;
-    for (int round = 0; round < np - 1; ++round) {
-      for (int k = threadIdx.x; k < half; k += blockDim.x) {
-        int p, q;
-        pair_of(round, k, np, &p, &q);
-        rot_params(Acur, np, p, q, &cs[2 * k], &cs[2 * k + 1]);
-      }
-      __syncthreads();
-      // 2 x 2 blocks (pair k rows) x (pair l cols): B = J_k^T A J_l
-      for (int64_t e = gtid; e < (int64_t)half * half; e += gthreads) {
-        const int k = (int)(e / half), l = (int)(e % half);
-        int p, q, r, s;
-        pair_of(round, k, np, &p, &q);
-        pair_of(round, l, np, &r, &s);
-        const double ck = cs[2 * k], sk = cs[2 * k + 1], cl = cs[2 * l], sl = cs[2 * l + 1];
-        const double apr = Acur[(int64_t)p * np + r], aps = Acur[(int64_t)p * np + s];
-        const double aqr = Acur[(int64_t)q * np + r], aqs = Acur[(int64_t)q * np + s];
-        const double m0r = ck * apr - sk * aqr, m0s = ck * aps - sk * aqs;
-        const double m1r = sk * apr + ck * aqr, m1s = sk * aps + ck * aqs;
-        double bpr = m0r * cl - m0s * sl, bps = m0r * sl + m0s * cl;
-        double bqr = m1r * cl - m1s * sl, bqs = m1r * sl + m1s * cl;
-        if (k == l) { bps = 0.0; bqr = 0.0; }
-        Anext[(int64_t)p * np + r] = bpr; Anext[(int64_t)p * np + s] = bps;
-        Anext[(int64_t)q * np + r] = bqr; Anext[(int64_t)q * np + s] = bqs;
-      }
-      // Q <- Q J (rows independent)
-      for (int64_t e = gtid; e < (int64_t)np * half; e += gthreads) {
-        const int i = (int)(e / half), l = (int)(e % half);
-        int r, s;
-        pair_of(round, l, np, &r, &s);
-        const double cl = cs[2 * l], sl = cs[2 * l + 1];
-        const double qr = a.Q[(int64_t)i * np + r], qs = a.Q[(int64_t)i * np + s];
-        a.Q[(int64_t)i * np + r] = cl * qr - sl * qs;
-        a.Q[(int64_t)i * np + s] = sl * qr + cl * qs;
-      }
-      grid.sync();
-      double* t = Acur; Acur = Anext; Anext = t;
-    }
-  }
-  if (gtid == 0) *a.sweeps_out = sweep;
-  // make the final matrix available in A0
-  if (Acur != a.A0)
-    for (int64_t e = gtid; e < (int64_t)np * np; e += gthreads) a.A0[e] = Acur[e];
-}
-
-// sort eigenpairs ascending (ties by index) and copy the n x n leading block
-__global__ void k_eig_sort(const double* A, const double* Q, int n, int np, double* w,
-                           double* Qout) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double ai = A[(int64_t)i * np + i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      const double aj = A[(int64_t)j * np + j];
-      rank += (aj < ai) || (aj == ai && j < i);
-    }
-    w[rank] = ai;
-    for (int r = 0; r < n; ++r) Qout[(int64_t)r * n + rank] = Q[(int64_t)r * np + i];
-  }
-}
-
-__global__ void k_pad_square(const double* H, int n, int np, double* A, double* Q) {
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)np * np) return;
-  int i = (int)(e / np), j = (int)(e % np);
-  A[e] = (i < n && j < n) ? H[(int64_t)i * n + j] : 0.0;
-  Q[e] = i == j ? 1.0 : 0.0;
-}
-
-// ---------------------------------------------------------------------------
 // residual norms
 // ---------------------------------------------------------------------------
 __global__ void k_resid_partial(const double* V, const double* AV, int64_t ld, int64_t D, int n,
@@ -563,35 +426,6 @@ fd_status tri_inverse(fd_ctx* ctx, const double* R, int n, double* Rinv) {
   if (smem > 48 * 1024)
     FD_CUDA(ctx, cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   k_tri_inverse<<<(unsigned)cdiv(n, 8), 256, smem, ctx->stream>>>(R, n, Rinv);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
-}
-
-fd_status sym_eig(fd_ctx* ctx, double* H, int n, double* w, double* Q, int max_sweeps) {
-  const int np = n + (n & 1);
-  void* p;
-  FD_TRY(workspace(ctx, "jacobi", sizeof(double) * (3 * (size_t)np * np + 4096) + 64, &p));
-  double* A0 = (double*)p;
-  double* A1 = A0 + (size_t)np * np;
-  double* Qw = A1 + (size_t)np * np;
-  double* part = Qw + (size_t)np * np;
-  int* sweeps = (int*)(part + 4096);
-  const int T = 256;
-  k_pad_square<<<(unsigned)cdiv((int64_t)np * np, T), T, 0, ctx->stream>>>(H, n, np, A0, Qw);
-  FD_LAUNCHED(ctx);
-  const size_t smem = sizeof(double) * np;  // np/2 (c, s) pairs
-  int per_sm = 0;
-  FD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi, T, smem));
-  const int64_t work = std::max<int64_t>((int64_t)np * np / 4, (int64_t)np * np / 2);
-  int grid = (int)std::min<int64_t>(cdiv(work, T), (int64_t)per_sm * ctx->num_sms);
-  grid = std::max(1, std::min(grid, 4096));
-  JacobiArgs a;
-  a.A0 = A0; a.A1 = A1; a.Q = Qw; a.part = part; a.n = n; a.np = np;
-  a.max_sweeps = max_sweeps; a.rel_tol = 1e-14; a.sweeps_out = sweeps;
-  void* args[] = {&a};
-  FD_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_jacobi, grid, T, args, smem, ctx->stream));
-  FD_LAUNCHED(ctx);
-  k_eig_sort<<<1, 512, 0, ctx->stream>>>(A0, Qw, n, np, w, Q);
   FD_LAUNCHED(ctx);
   return FD_OK;
 }
