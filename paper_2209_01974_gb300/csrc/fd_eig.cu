@@ -83,8 +83,10 @@ __device__ __forceinline__ void group_sync(int g) {
 // rotation that (nearly) annihilates a_pq: (c, s) orthogonal to FP64 rounding
 __device__ __forceinline__ void angle(double app, double aqq, double apq, double* c, double* s) {
   const float d = (float)(aqq - app), o = 2.0f * (float)apq;
-  // entries are scaled to |a| <= 1 and stay below the order n; not finite: NaN input
-  if (o == 0.0f || !(fabsf(o) < 1e30f) || !(fabsf(d) < 1e30f)) {
+  // entries are scaled to |a| <= 1 and stay below the order n (not finite: NaN
+  // input); what is below 1e-30 is far under the convergence threshold, and its
+  // reciprocal below would overflow for equal diagonal entries
+  if (!(fabsf(o) > 1e-30f && fabsf(o) < 1e30f) || !(fabsf(d) < 1e30f)) {
     *c = 1.0;
     *s = 0.0;
     return;

@@ -66,6 +66,19 @@ def test_clusters(gap):
     _check(csr, ns, 2)
 
 
+@pytest.mark.parametrize("tiny", [1e-320, 1e-300, 1e-45, 1e-40, 1e-36, 1e-31, 1e-20])
+def test_tiny_couplings_of_equal_diagonal_entries(tiny):
+    # V = the first 16 unit vectors: H is the leading block of the matrix
+    D = 40
+    H = np.eye(D)
+    H[0, 9] = H[9, 0] = H[2, 3] = H[3, 2] = tiny
+    ptr = np.arange(0, D * D + 1, D, dtype=np.int64)
+    csr = (ptr, np.tile(np.arange(D, dtype=np.int32), D), H.reshape(-1).copy())
+    theta, resid, V = _ritz(csr, np.eye(D)[:, :16].copy())
+    assert np.abs(theta - 1.0).max() <= 1e-15 and np.abs(V.T @ V - np.eye(16)).max() <= 1e-14
+    assert resid.max() <= 1e-15
+
+
 def test_nan_gives_nan():
     p, c, v = fd_inputs.random_symmetric_csr(120, 5, 3)
     V0 = np.linalg.qr(fd_inputs.random_block(120, 20, 5))[0]
