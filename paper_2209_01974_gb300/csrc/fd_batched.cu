@@ -985,9 +985,11 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
   // largest wanted residual reaches 100 u32 |H| or fails to halve twice in a row
   std::vector<int> use32(n_inst, f32 ? 1 : 0), stall(n_inst, 0);
   std::vector<double> prev_max(n_inst, INFINITY), norm_h(n_inst, 0.0);
+  std::vector<uint64_t> seeds(n_inst);
+  for (int i = 0; i < n_inst; ++i) seeds[i] = prob[i].seed;
+  s = spectral_bounds_batch(ctx, n_inst, A, lsteps, seeds.data(), lam_l.data(), lam_r.data());
+  if (s != FD_OK) { B.release(); return s; }
   for (int i = 0; i < n_inst; ++i) {
-    s = spectral_bounds(ctx, A[i], lsteps, prob[i].seed, &lam_l[i], &lam_r[i]);
-    if (s != FD_OK) { B.release(); return s; }
     widen[i] = 0.01 * (lam_r[i] - lam_l[i]);
     norm_h[i] = std::max(std::fabs(lam_l[i]), std::fabs(lam_r[i]));
     k_bstart<<<(unsigned)cdiv(A[i]->D * ns[i], 256), 256, 0, st>>>(

@@ -267,19 +267,6 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// ---- nb = 1 SpMV (Lanczos), lane per row over the SELL chunk ---------------
-__global__ void k_spmv1(const int64_t* chunk_ptr, const int32_t* row_len, const int32_t* col,
-                        const double* val, int64_t D, int C, const double* x, double* y) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= D) return;
-  const uint32_t chunk = (uint32_t)i / (uint32_t)C;
-  int64_t base = chunk_ptr[chunk] + ((uint32_t)i - chunk * (uint32_t)C);
-  int len = row_len[i];
-  double s = 0.0;
-  for (int j = 0; j < len; ++j) s = fma(val[base + (int64_t)j * C], x[col[base + (int64_t)j * C]], s);
-  y[i] = s;
-}
-
 // ---- KPM: Chebyshev iteration on R random vectors with moment partial sums
 constexpr int KPM_BLOCKS_PER_SM = 8;
 
@@ -505,13 +492,6 @@ fd_status spmmv(fd_ctx* ctx, const fd_matrix* M, fd_prec prec, const void* X, in
     if (wide) FD_TRY(permute<double>(ctx, M, (const double*)ys, nb, (double*)Y, ldy, nb, false));
     else FD_TRY(permute<float>(ctx, M, (const float*)ys, nb, (float*)Y, ldy, nb, false));
   }
-  return FD_OK;
-}
-
-fd_status spmv1(fd_ctx* ctx, const fd_matrix* M, const double* x, double* y) {
-  k_spmv1<<<(unsigned)cdiv(M->D, 256), 256, 0, ctx->stream>>>(M->chunk_ptr, M->row_len, M->col,
-                                                              M->val, M->D, M->C, x, y);
-  FD_LAUNCHED(ctx);
   return FD_OK;
 }
 

@@ -157,8 +157,6 @@ fd_status kron_filter(fd_ctx* ctx, const fd_matrix* A, fd_prec prec, void* V, in
                       void* W1, void* W2, int64_t ldw, double* bytes_out);
 // the panel kernel's tables of A (after the per-species tables exist)
 fd_status kron_panel_tables(fd_ctx* ctx, fd_matrix* A, double t);
-// nb = 1 SpMV in SELL order, FP64: y = A x (x, y dense vectors in SELL order)
-fd_status spmv1(fd_ctx* ctx, const fd_matrix* A, const double* x, double* y);
 // KPM Chebyshev iteration with moment epilogue (fd_filter.cu)
 fd_status kpm(fd_ctx* ctx, const fd_matrix* A, int n_moments, int R, uint64_t seed,
               double alpha, double beta, double* mu_host);
@@ -231,9 +229,14 @@ fd_status lehmann_ritz(fd_ctx* ctx, const double* V, double* AV, int64_t ld, int
                        const double* theta_dev, double rho, std::vector<double>* below,
                        std::vector<double>* above, bool* ok);
 
-// ---- solver pieces (fd_solve.cu) ------------------------------------------
+// ---- inclusion intervals (fd_lanczos.cu) ------------------------------------
 fd_status spectral_bounds(fd_ctx* ctx, const fd_matrix* A, int steps, uint64_t seed,
                           double* lam_l, double* lam_r);
+// the same for n_inst matrices, each with its own seed
+fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const* A, int steps,
+                                const uint64_t* seeds, double* lam_l, double* lam_r);
+
+// ---- solver pieces (fd_solve.cu) ------------------------------------------
 // Jackson-damped window coefficients, p(window centre) = 1 (host arithmetic)
 std::vector<double> filter_coeffs(double x_l, double x_r, int n);
 

@@ -22,53 +22,6 @@
 namespace fdi {
 namespace {
 
-// dot products out[j] = sum_i Q[j * D + i] * w[i], j < k (partials + fixed-order reduce)
-__global__ void k_dots_partial(const double* Q, int k, const double* w, int64_t D, double* P) {
-  __shared__ double sh[256];
-  for (int j = 0; j < k; ++j) {
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < D;
-         i += (int64_t)gridDim.x * blockDim.x)
-      s = fma(Q[(int64_t)j * D + i], w[i], s);
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-      if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) P[(int64_t)j * gridDim.x + blockIdx.x] = sh[0];
-    __syncthreads();
-  }
-}
-__global__ void k_dots_reduce(const double* P, int k, int nb, double* out) {
-  for (int j = threadIdx.x; j < k; j += blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += P[(int64_t)j * nb + b];
-    out[j] = s;
-  }
-}
-// w -= sum_j Q_j c_j
-__global__ void k_sub_proj(const double* Q, int k, const double* c, int64_t D, double* w) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= D) return;
-  double s = w[i];
-  for (int j = 0; j < k; ++j) s -= Q[(int64_t)j * D + i] * c[j];
-  w[i] = s;
-}
-__global__ void k_scale_copy(const double* w, double f, int64_t D, double* q) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < D) q[i] = w[i] * f;
-}
-__global__ void k_lanczos_start(const int64_t* perm, int64_t D, uint64_t key, double* r) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < D) r[i] = fdrng::irwin_hall(key, (uint64_t)perm[i]);
-}
-__global__ void k_tridiag(const double* a, const double* b, int k, double* T) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= k * k) return;
-  int i = e / k, j = e % k;
-  T[e] = i == j ? a[i] : (j == i + 1 ? b[i] : (i == j + 1 ? b[j] : 0.0));
-}
 // start block, original row order: V[i][j] = g(seed, stream 2, i * ns + j)
 __global__ void k_start_block(double* V, int64_t ld, int64_t D, int ns, uint64_t key) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -156,92 +109,6 @@ struct Timer {
 };
 
 }  // namespace
-
-fd_status spectral_bounds(fd_ctx* ctx, const fd_matrix* A, int steps, uint64_t seed,
-                          double* lam_l, double* lam_r) {
-  cudaStream_t st = ctx->stream;
-  const int64_t D = A->D;
-  const int m = (int)std::min<int64_t>(steps, D);
-  const int T = 256;
-  const int nbk = (int)std::min<int64_t>(ctx->num_sms * 2, cdiv(D, T));
-  void* p;
-  FD_TRY(workspace(ctx, "lanczos", sizeof(double) * ((size_t)(m + 2) * D + (size_t)m * nbk + 4 * m + 64 + 4 * (size_t)m * m), &p));
-  double* Q = (double*)p;              // m x D, Lanczos vectors
-  double* w = Q + (size_t)m * D;       // D
-  double* r = w + D;                   // D
-  double* P = r + D;                   // m x nbk partials
-  double* dots = P + (size_t)m * nbk;  // m
-  double* ab = dots + m;               // alpha, beta (2m)
-  double* T2 = ab + 2 * m + 64;        // m x m
-  double* wk = T2 + (size_t)m * m;     // eigenvalues
-  double* Qk = wk + m;                 // m x m eigenvectors
-  k_lanczos_start<<<(unsigned)cdiv(D, T), T, 0, st>>>(A->perm, D, fdrng::key(seed, fdrng::STREAM_LANCZOS), r);
-  FD_LAUNCHED(ctx);
-  auto dot_into = [&](const double* Qm, int k, const double* v) -> fd_status {
-    k_dots_partial<<<nbk, T, 0, st>>>(Qm, k, v, D, P);
-    FD_LAUNCHED(ctx);
-    k_dots_reduce<<<1, 64, 0, st>>>(P, k, nbk, dots);
-    FD_LAUNCHED(ctx);
-    return FD_OK;
-  };
-  FD_TRY(dot_into(r, 1, r));
-  double nrm2 = 0;
-  FD_CUDA(ctx, cudaMemcpyAsync(&nrm2, dots, sizeof(double), cudaMemcpyDeviceToHost, st));
-  FD_CUDA(ctx, cudaStreamSynchronize(st));
-  k_scale_copy<<<(unsigned)cdiv(D, T), T, 0, st>>>(r, 1.0 / std::sqrt(nrm2), D, Q);
-  FD_LAUNCHED(ctx);
-  std::vector<double> alpha, beta;
-  double beta_last = 0.0;
-  for (int j = 0; j < m; ++j) {
-    FD_TRY(spmv1(ctx, A, Q + (size_t)j * D, w));
-    FD_TRY(dot_into(Q + (size_t)j * D, 1, w));
-    double a = 0;
-    FD_CUDA(ctx, cudaMemcpyAsync(&a, dots, sizeof(double), cudaMemcpyDeviceToHost, st));
-    for (int pass = 0; pass < 2; ++pass) {  // full reorthogonalisation, twice
-      FD_TRY(dot_into(Q, j + 1, w));
-      k_sub_proj<<<(unsigned)cdiv(D, T), T, 0, st>>>(Q, j + 1, dots, D, w);
-      FD_LAUNCHED(ctx);
-    }
-    FD_TRY(dot_into(w, 1, w));
-    double b2 = 0;
-    FD_CUDA(ctx, cudaMemcpyAsync(&b2, dots, sizeof(double), cudaMemcpyDeviceToHost, st));
-    FD_CUDA(ctx, cudaStreamSynchronize(st));
-    alpha.push_back(a);
-    beta_last = std::sqrt(b2);
-    if (j == m - 1 || beta_last <= 1e-14 * std::max(1.0, std::fabs(a))) break;
-    beta.push_back(beta_last);
-    k_scale_copy<<<(unsigned)cdiv(D, T), T, 0, st>>>(w, 1.0 / beta_last, D, Q + (size_t)(j + 1) * D);
-    FD_LAUNCHED(ctx);
-  }
-  const int k = (int)alpha.size();
-  std::vector<double> hab(2 * k, 0.0);
-  std::copy(alpha.begin(), alpha.end(), hab.begin());
-  std::copy(beta.begin(), beta.end(), hab.begin() + k);
-  FD_CUDA(ctx, cudaMemcpyAsync(ab, hab.data(), sizeof(double) * 2 * k, cudaMemcpyHostToDevice, st));
-  k_tridiag<<<(unsigned)cdiv(k * k, T), T, 0, st>>>(ab, ab + k, k, T2);
-  FD_LAUNCHED(ctx);
-  double tmin, tmax, smin, smax;
-  if (k == 1) {
-    tmin = tmax = alpha[0];
-    smin = smax = 1.0;
-  } else {
-    FD_TRY(sym_eig(ctx, T2, k, wk, Qk, 40));
-    std::vector<double> hw(k), hq((size_t)k * k);
-    FD_CUDA(ctx, cudaMemcpyAsync(hw.data(), wk, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
-    FD_CUDA(ctx, cudaMemcpyAsync(hq.data(), Qk, sizeof(double) * k * k, cudaMemcpyDeviceToHost, st));
-    FD_CUDA(ctx, cudaStreamSynchronize(st));
-    tmin = hw[0];
-    tmax = hw[k - 1];
-    smin = hq[(size_t)(k - 1) * k + 0];
-    smax = hq[(size_t)(k - 1) * k + (k - 1)];
-  }
-  const double wdt = std::max(tmax - tmin, 1e-10 * std::max({1.0, std::fabs(tmin), std::fabs(tmax)}));
-  double lo = tmin - std::fabs(beta_last * smin) - 0.01 * wdt;
-  double hi = tmax + std::fabs(beta_last * smax) + 0.01 * wdt;
-  *lam_l = std::max(A->gersh_lo, lo);
-  *lam_r = std::min(A->gersh_hi, hi);
-  return FD_OK;
-}
 
 }  // namespace fdi
 

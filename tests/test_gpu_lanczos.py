@@ -1,0 +1,37 @@
+"""Inclusion intervals from the one-launch Lanczos kernel against the oracle:
+few rows, more steps than rows, an invariant start (early stop), permuted rows,
+sizes around the rows of a CTA."""
+import numpy as np
+import pytest
+
+from oracle import lanczos
+from oracle import matrices as mat
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("spec,C,sigma", [
+    ("chain:n=2,t=1", 32, 1), ("chain:n=3,t=1", 32, 1), ("chain:n=63,t=1", 32, 1), ("chain:n=65,t=1", 32, 1),
+    ("anderson3d:L=11,W=3,seed=5", 64, 1), ("chain:n=777,t=1", 96, 8), ("anderson3d:L=24,W=16,seed=2", 32, 1),
+])
+@pytest.mark.parametrize("steps", [1, 2, 20, 50])
+def test_bounds_match_oracle(spec, C, sigma, steps):
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    csr = mat.build(spec)
+    A = fd.fd_build_matrix(ctx, spec, C=C, sigma=sigma)
+    lo, hi = fd.fd_spectral_bounds(ctx, A, steps, 7)
+    olo, ohi = lanczos.inclusion_interval(csr, steps, 7)
+    # extreme Ritz values are well conditioned; the residual bound beta |s| loses
+    # digits only where it is itself far below the interval's width
+    assert max(abs(lo - olo), abs(hi - ohi)) <= 1e-9 * (ohi - olo)
+
+
+def test_early_stop_on_an_invariant_subspace():
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    D = 500
+    d = np.where(np.arange(D) % 3 == 0, -1.0, 2.0)   # two eigenvalues: two steps span everything
+    csr = (np.arange(D + 1, dtype=np.int64), np.arange(D, dtype=np.int32), d)
+    A = fd.fd_matrix_from_csr(ctx, *csr)
+    assert np.allclose(fd.fd_spectral_bounds(ctx, A, 20, 1), (-1.0, 2.0), rtol=0, atol=1e-12)
