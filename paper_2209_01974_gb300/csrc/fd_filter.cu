@@ -191,10 +191,6 @@ template <typename T>
 fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, int n,
                    const double* mu, double alpha, double beta, T* W1, T* W2, int64_t ldw,
                    double* bytes_out) {
-  const double Sx = sizeof(T), Sv = sizeof(T);
-  const double mat_bytes = (double)M->nnz * (Sv + 4.0);
-  const double vec = (double)nb * M->D * Sx;
-  double bytes = 0;
   const bool ident = M->identity != 0;
   StepArgs<T> s{};
   // x0 location
@@ -210,7 +206,6 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
   s.X = x0; s.ldx = ld0; s.Y = x1; s.ldy = ldw;
   s.c_ax = (T)alpha; s.c_x = (T)beta;
   FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_SPMMV, s));
-  bytes += mat_bytes + 2 * vec;
   // step 2: x2 = 2 A~ x1 - x0; acc = mu0 x0 + mu1 x1 + mu2 x2
   T* acc = V;          // accumulator storage (SELL order when not identity)
   int64_t lda = ldv;
@@ -228,7 +223,6 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
     else { s.Vout = W1; s.ldvo = ldw; }   // final result in SELL order, unpermuted below
   }
   FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_SECOND, s));
-  bytes += mat_bytes + (n > 2 ? 4 : 3) * vec;
   // generic steps: xk = 2 A~ x_{k-1} - x_{k-2}; acc += mu_k xk, three terms at a
   // time.  The reported bytes stay those of Eq. EstimateT (kappa = 5), the
   // algorithm's own count; what a step moves is less (step_terms).
@@ -249,10 +243,8 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
     }
     if (k < n) {
       s.Y = xpp; s.ldy = ldw;
-      bytes += mat_bytes + 5 * vec;
-    } else {
-      if (!ident) { s.Vout = xpp; s.ldvo = ldw; final_buf = xpp; }
-      bytes += mat_bytes + 4 * vec;
+    } else if (!ident) {
+      s.Vout = xpp; s.ldvo = ldw; final_buf = xpp;
     }
     FD_TRY(step_dispatch<T>(ctx, M, nb, s.nacc ? MODE_GENERIC : MODE_PLAIN, s));
     T* t = xp; xp = xpp; xpp = t;
@@ -261,7 +253,7 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
     if (n == 2) final_buf = W1;
     FD_TRY(permute<T>(ctx, M, final_buf, ldw, V, ldv, nb, false));
   }
-  if (bytes_out) *bytes_out += bytes;
+  if (bytes_out) *bytes_out += filter_bytes(M, nb, n, sizeof(T));
   return FD_OK;
 }
 
@@ -439,6 +431,13 @@ fd_status debug_check_matrix(fd_ctx* ctx, const fd_matrix* M) {
   return FD_OK;
 }
 
+double filter_bytes(const fd_matrix* M, int nb, int n, double elem) {
+  const double mat = (double)M->nnz * (elem + 4.0), vec = (double)nb * M->D * elem;
+  double bytes = (mat + 2 * vec) + (mat + (n > 2 ? 4 : 3) * vec);
+  if (n >= 3) bytes += (n - 3) * (mat + 5 * vec) + (mat + 4 * vec);
+  return bytes;
+}
+
 fd_status filter(fd_ctx* ctx, const fd_matrix* M, fd_prec prec, void* V, int64_t ldv, int nb,
                  int degree, const double* mu, double alpha, double beta, void* W1, void* W2,
                  int64_t ldw, double* bytes_out) {
@@ -446,6 +445,9 @@ fd_status filter(fd_ctx* ctx, const fd_matrix* M, fd_prec prec, void* V, int64_t
   // (the FP64 step is bound by GB300's FP64 rate; it keeps the row-major kernel)
   if (M->kron && prec == FD_F32)
     return kron_filter(ctx, M, prec, V, ldv, nb, degree, mu, alpha, beta, W1, W2, ldw, bytes_out);
+  bool used = false;
+  FD_TRY(filter_small(ctx, M, prec, V, ldv, nb, degree, mu, alpha, beta, W1, W2, ldw, bytes_out, &used));
+  if (used) return FD_OK;
   if (prec == FD_F64)
     return filter_t<double>(ctx, M, (double*)V, ldv, nb, degree, mu, alpha, beta, (double*)W1,
                             (double*)W2, ldw, bytes_out);

@@ -150,6 +150,22 @@ fd_status spmmv(fd_ctx* ctx, const fd_matrix* A, fd_prec prec, const void* X,
 fd_status filter(fd_ctx* ctx, const fd_matrix* A, fd_prec prec, void* V, int64_t ldv,
                  int nb, int degree, const double* mu, double alpha, double beta,
                  void* W1, void* W2, int64_t ldw, double* bytes_out);
+// the filter of a matrix small enough to stay in shared memory, in one launch
+// (fd_small.cu); *used = false when the launched steps are the better choice
+struct SmallPlan {
+  int cluster = 0;  // CTAs per cluster (0: does not fit)
+  int pw = 1;       // 8-byte columns per panel
+  int threads = 0;
+  size_t smem = 0;
+  double clocks = 0;  // estimated SM clocks of a step
+};
+SmallPlan small_plan(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int units);
+bool filter_small_pays(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int nb);
+fd_status filter_small(fd_ctx* ctx, const fd_matrix* M, fd_prec prec, void* V, int64_t ldv, int nb, int degree,
+                       const double* mu, double alpha, double beta, void* W1, void* W2, int64_t ldw,
+                       double* bytes_out, bool* used);
+// algorithmic bytes of a degree-n filter on nb columns (Eq. EstimateT, kappa = 5)
+double filter_bytes(const fd_matrix* M, int nb, int n, double elem);
 // the same filter for a matrix-free Hubbard operator: the block in 16-byte
 // column panels, slabs in korder (fd_kron.cu)
 fd_status kron_filter(fd_ctx* ctx, const fd_matrix* A, fd_prec prec, void* V, int64_t ldv,

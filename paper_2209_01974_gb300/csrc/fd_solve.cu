@@ -198,24 +198,42 @@ static fd_status solve_impl(fd_ctx* ctx, const fd_matrix* A, double a, double b,
   Timer tm(st), ttot(st);
   ttot.start();
 
-  // workspaces: V, AV (D x ns FP64), W1, W2 (D x nb FP64); FP32 bundle buffers
+  // Columns filtered per call: nb, or the whole block where the matrix is small
+  // enough for the one-launch filter (its panels of columns then fill the chip
+  // together instead of one bundle after the other).
+  const bool f64_sweeps = opt.precision == FD_F64 || (opt.precision == FD_F32 && !ff_sweeps);
+  int w32 = filter_small_pays(ctx, A, FD_F32, ns) ? ns : nb;
+  int w64 = filter_small_pays(ctx, A, ff_sweeps ? FD_FF : FD_F64, ns) ? ns : nb;
+  // workspaces: V, AV (D x ns FP64), W1, W2 (D x w64 FP64); FP32 bundle buffers
   void* p;
   FD_TRY(workspace(ctx, "solve_V", sizeof(double) * D * ns, &p)); double* V = (double*)p;
   FD_TRY(workspace(ctx, "solve_AV", sizeof(double) * D * ns, &p)); double* AV = (double*)p;
-  FD_TRY(workspace(ctx, "solve_W", sizeof(double) * 2 * D * nb, &p));
-  double* W1 = (double*)p;
-  double* W2 = W1 + D * nb;
+  double *W1 = nullptr, *W2 = nullptr;
   float *V32 = nullptr, *W132 = nullptr, *W232 = nullptr;
-  if (opt.precision == FD_F32) {
-    FD_TRY(workspace(ctx, "solve_W32", sizeof(float) * 3 * D * nb, &p));
-    V32 = (float*)p; W132 = V32 + D * nb; W232 = W132 + D * nb;
+  float* Vff = nullptr;  // float-float bundle (2 floats per element); its recurrence vectors reuse W1, W2
+  auto filter_buffers = [&]() -> fd_status {
+    if (f64_sweeps || ff_sweeps) {
+      FD_TRY(workspace(ctx, "solve_W", sizeof(double) * 2 * D * w64, &p));
+      W1 = (double*)p;
+      W2 = W1 + D * w64;
+    }
+    if (opt.precision == FD_F32) {
+      FD_TRY(workspace(ctx, "solve_W32", sizeof(float) * 3 * D * w32, &p));
+      V32 = (float*)p; W132 = V32 + D * w32; W232 = W132 + D * w32;
+    }
+    if (ff_sweeps) {
+      FD_TRY(workspace(ctx, "solve_Wff", sizeof(float) * 2 * D * w64, &p));
+      Vff = (float*)p;
+    }
+    return FD_OK;
+  };
+  fd_status ws = filter_buffers();
+  if (ws == FD_ERR_OOM && (w32 > nb || w64 > nb)) {  // a tight workspace limit: bundle by bundle
+    ctx->err.clear();
+    w32 = w64 = nb;
+    ws = filter_buffers();
   }
-  // float-float bundle (2 floats per element); its recurrence vectors reuse W1, W2
-  float* Vff = nullptr;
-  if (ff_sweeps) {
-    FD_TRY(workspace(ctx, "solve_Wff", sizeof(float) * 2 * D * nb, &p));
-    Vff = (float*)p;
-  }
+  FD_TRY(ws);
   FD_TRY(workspace(ctx, "solve_small", sizeof(double) * 2 * ns + sizeof(int) * ns + 64, &p));
   double* th_dev = (double*)p;
   double* rho_dev = th_dev + ns;
@@ -326,17 +344,18 @@ static fd_status solve_impl(fd_ctx* ctx, const fd_matrix* A, double a, double b,
     std::vector<double> mu = filter_coeffs(alpha * wl + beta, alpha * wr + beta, n);
     tm.start();
     double bytes = 0;
-    for (int j = 0; j < ns; j += nb) {
+    const int wd = use_f32 ? w32 : w64;
+    for (int j = 0; j < ns; j += wd) {
       if (use_f32) {
-        FD_TRY(copy_cols_f64_to_f32(ctx, V + j, ns, V32, nb, D, nb));
-        FD_TRY(filter(ctx, A, FD_F32, V32, nb, nb, n, mu.data(), alpha, beta, W132, W232, nb, &bytes));
-        FD_TRY(copy_cols_f32_to_f64(ctx, V32, nb, V + j, ns, D, nb));
+        FD_TRY(copy_cols_f64_to_f32(ctx, V + j, ns, V32, wd, D, wd));
+        FD_TRY(filter(ctx, A, FD_F32, V32, wd, wd, n, mu.data(), alpha, beta, W132, W232, wd, &bytes));
+        FD_TRY(copy_cols_f32_to_f64(ctx, V32, wd, V + j, ns, D, wd));
       } else if (ff_sweeps) {
-        FD_TRY(copy_cols_f64_to_ff(ctx, V + j, ns, Vff, nb, D, nb));
-        FD_TRY(filter(ctx, A, FD_FF, Vff, nb, nb, n, mu.data(), alpha, beta, W1, W2, nb, &bytes));
-        FD_TRY(copy_cols_ff_to_f64(ctx, Vff, nb, V + j, ns, D, nb));
+        FD_TRY(copy_cols_f64_to_ff(ctx, V + j, ns, Vff, wd, D, wd));
+        FD_TRY(filter(ctx, A, FD_FF, Vff, wd, wd, n, mu.data(), alpha, beta, W1, W2, wd, &bytes));
+        FD_TRY(copy_cols_ff_to_f64(ctx, Vff, wd, V + j, ns, D, wd));
       } else {
-        FD_TRY(filter(ctx, A, FD_F64, V + j, ns, nb, n, mu.data(), alpha, beta, W1, W2, nb, &bytes));
+        FD_TRY(filter(ctx, A, FD_F64, V + j, ns, wd, n, mu.data(), alpha, beta, W1, W2, wd, &bytes));
       }
     }
     res->t_filter += tm.stop_s();

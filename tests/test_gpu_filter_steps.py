@@ -46,3 +46,71 @@ def test_accumulation_remainders(spec, C, sigma, prec, n):
     ref = ch.cheb_filter(mat.to_scipy(csr), V0, mu, alpha, beta)
     u = {"f64": U64, "f32": U32, "ff": 2.0 ** -45}[prec]
     assert np.all(np.abs(out.cpu().numpy() - ref) <= filter_tolerance(csr, mu, alpha, beta, V0, u))
+
+
+def _random_ragged(D, seed):
+    return fd_inputs.random_symmetric_csr(D, 9, seed, max_row=40)
+
+
+# rows around the splits of the one-launch filter (clusters of 1, 2, 4, 8 CTAs, rows
+# in fours) and, from 40,000 on, the launched steps
+@pytest.mark.parametrize("D", [3, 31, 33, 130, 1023, 1500, 4999, 40001])
+@pytest.mark.parametrize("nb,prec", [(2, "f64"), (4, "f32"), (8, "ff"), (16, "f64"), (32, "f32"), (64, "f64"),
+                                     (64, "ff"), (128, "f32")])
+@pytest.mark.parametrize("sigma", [1, 64])
+def test_sizes(D, nb, prec, sigma):
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    csr = _random_ragged(D, D + nb)
+    A = fd.fd_matrix_from_csr(ctx, *csr, C=32, sigma=sigma)
+    n = 7
+    V0 = fd_inputs.random_block(D, nb, n).astype(np.float32).astype(np.float64)
+    lo, hi = lanczos.gershgorin(csr)
+    alpha, beta = ch.scale_params(lo - 0.01, hi + 0.01)
+    mu = np.random.default_rng(n).uniform(0.5, 1.0, n + 1)
+    ld = 2 * nb                                   # a bundle of a wider block
+    big = torch.zeros((D, ld), dtype=torch.float64, device="cuda")
+    big[:, nb:] = torch.from_numpy(V0)
+    shape, dtype = ((D, nb), torch.float64) if prec == "f64" else ((D, nb), torch.float32)
+    if prec == "ff":
+        shape = (D, nb, 2)
+    W1, W2 = (torch.empty(shape, dtype=dtype, device="cuda") for _ in range(2))
+    if prec == "f64":
+        fd.fd_filter(ctx, A, big[:, nb:], mu, alpha, beta, W1, W2)
+    else:
+        V = torch.empty(shape, dtype=dtype, device="cuda")
+        fd.fd_copy_block(ctx, big[:, nb:], V)
+        fd.fd_filter(ctx, A, V, mu, alpha, beta, W1, W2)
+        fd.fd_copy_block(ctx, V, big[:, nb:])
+    out = big.cpu().numpy()
+    assert np.all(out[:, :nb] == 0.0)
+    ref = ch.cheb_filter(mat.to_scipy(csr), V0, mu, alpha, beta)
+    # two roundings more per row: the scaled entries and the scaled diagonal
+    u = {"f64": U64, "f32": U32, "ff": 2.0 ** -45}[prec]
+    assert np.all(np.abs(out[:, nb:] - ref) <= filter_tolerance(csr, mu, alpha, beta, V0, u))
+
+
+@pytest.mark.parametrize("n", [998, 999, 1000, 1001, 2500])
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_steps_split_over_launches(n, prec):
+    """The one-launch filter takes at most 999 steps at a time."""
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    spec = "anderson3d:L=7,W=3,seed=5"
+    csr = mat.build(spec)
+    A = fd.fd_build_matrix(ctx, spec)
+    lo, hi = lanczos.gershgorin(csr)
+    alpha, beta = ch.scale_params(lo - 0.01, hi + 0.01)
+    mu = ch.filter_coeffs(0.1, 0.15, n)
+    V0 = fd_inputs.random_block(343, 8, n).astype(np.float32).astype(np.float64)
+    dtype = torch.float64 if prec == "f64" else torch.float32
+    V = torch.from_numpy(V0).to(dtype).cuda()
+    fd.fd_filter(ctx, A, V, mu, alpha, beta, torch.empty_like(V), torch.empty_like(V))
+    ref = ch.cheb_filter(mat.to_scipy(csr), V0, mu, alpha, beta)
+    # the errors of the steps add up like sqrt(n) (their signs vary); 40 sqrt(n) u |ref|
+    u = U64 if prec == "f64" else U32
+    assert np.linalg.norm(V.cpu().numpy() - ref) <= 40 * np.sqrt(n) * u * np.linalg.norm(V0)
