@@ -26,8 +26,8 @@
 // a 128 x 64 output tile, the 8 level accumulators in TMEM: 8 x 64 FP32
 // columns = all 512) is a pure Blackwell pipeline: one thread streams the
 // digit blocks of each K step into a four-stage shared-memory ring with
-// cp.async.bulk (mbarrier complete_tx), one thread issues the step's 36
-// tcgen05.mma (one per digit pair; M 128, N 64, K 16) and commits them to the
+// cp.async.bulk (mbarrier complete_tx), one thread issues the step's 12
+// tcgen05.mma (36 digit pairs; M 128, N up to 256, K 16) and commits them to the
 // stage's "empty" mbarrier, and every eighth step (K = 128) all threads read
 // the levels back with tcgen05.ld, convert them to 32-bit integers, combine
 // adjacent levels exactly in 32 bits and add them, scaled by 2^(7 (7 - l)),
@@ -70,8 +70,9 @@ constexpr int M_THREAD = 32;                          // MMA issuer (warp 1)
 // instruction descriptor of tcgen05.mma kind::f16: D FP32 (bits 4-5 = 1),
 // A and B bf16 (bits 7-9, 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4
 // at bit 24
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                           ((uint32_t)(TM >> 4) << 24);
+__host__ __device__ constexpr uint32_t idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -125,11 +126,12 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+template <int N>
 __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(IDESC), "r"(accumulate));
+      "l"(a), "l"(b), "r"(idesc(N)), "r"(accumulate));
 }
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -204,19 +206,31 @@ struct Acc {
   long long hi, lo;
 };
 
-// One K step's tensor-core work (issued by one thread): level l collects the
-// pairs (s, l - s) in its TMEM columns l * 64 ..; the first MMA of a level in
-// a K chunk overwrites, the rest accumulate.  Fully unrolled: the descriptor
-// of slice s is the base descriptor plus s * slice bytes / 16 in its address
-// field, an immediate.
-template <bool FIRST>
+// One K step's tensor-core work (issued by one thread).  Level l = s + t collects
+// the pairs (s, t) in its TMEM columns l * 64 .., so the products of one slice s of
+// A with consecutive slices t of B belong in consecutive columns, and consecutive
+// slices of B are consecutive rows of its shared-memory tile: one MMA takes up to
+// four of them as one operand of N = 256 (12 MMAs a step instead of 36 of N = 64,
+// which are bound by re-reading A from shared memory: 6 KB per 32 clocks of tensor
+// work).  Slice 0 of A starts every level of a K chunk, the others accumulate.
+template <int S, int T, int CNT>
+__device__ __forceinline__ void issue_run(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+  umma<CNT * TN>(tmem + (uint32_t)((S + T) * TN), adesc + (uint64_t)((S * A_SLICE) >> 4),
+                 bdesc + (uint64_t)((T * B_SLICE) >> 4), accumulate);
+}
+template <bool FIRST, int S = 0>
 __device__ __forceinline__ void issue_step(uint32_t tmem, uint64_t adesc, uint64_t bdesc) {
-#pragma unroll
-  for (int l = 0; l < OZ_S; ++l)
-#pragma unroll
-    for (int s = 0; s <= l; ++s)
-      umma(tmem + (uint32_t)(l * TN), adesc + (uint64_t)((s * A_SLICE) >> 4),
-           bdesc + (uint64_t)(((l - s) * B_SLICE) >> 4), (FIRST && s == 0) ? 0u : 1u);
+  if constexpr (S < OZ_S) {
+    constexpr int CNT = OZ_S - S;  // slices of B that meet slice S of A
+    constexpr uint32_t ACC = FIRST && S == 0 ? 0u : 1u;
+    if constexpr (CNT > 4) {
+      issue_run<S, 0, 4>(tmem, adesc, bdesc, ACC);
+      issue_run<S, 4, CNT - 4>(tmem, adesc, bdesc, ACC);
+    } else {
+      issue_run<S, 0, CNT>(tmem, adesc, bdesc, ACC);
+    }
+    issue_step<FIRST, S + 1>(tmem, adesc, bdesc);
+  }
 }
 
 // Read the 8 levels of this thread's 16 outputs (TMEM lane = tile row
@@ -409,33 +423,72 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 // ---------------------------------------------------------------------------
 // scales: exponent e with max |x| < 2^e (frexp); flag non-finite input
 // ---------------------------------------------------------------------------
-__global__ void k_col_maxabs(const double* X, int64_t ld, int64_t D, int n, double* part, int* bad) {
-  // grid (n_blocks_rows); each thread owns columns c = tid, tid + 256, ...
-  // maxima of |x| as 64-bit integers (the bit patterns of non-negative doubles
-  // order like their values, NaN above inf): integer instructions instead of
-  // GB300's slow FP64 ones
-  for (int c = threadIdx.x; c < n; c += blockDim.x) {
-    unsigned long long m[4] = {0, 0, 0, 0};  // four independent loads in flight
-    const int64_t g = gridDim.x;
-    int64_t r = blockIdx.x;
-    for (; r + 3 * g < D; r += 4 * g) {
+// One CTA takes 128 columns (blockIdx.y) over a slice of the rows: 64 threads
+// along the columns, two columns each, times four along the rows, eight rows in
+// flight per thread.  Maxima of |x| as 64-bit integers (the bit patterns of
+// non-negative doubles order like their values, NaN above inf): integer
+// instructions instead of GB300's slow FP64 ones.
+constexpr int CM_COLS = 128, CM_ROWS = 4, CM_UNROLL = 8;
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_col_maxabs(const double* __restrict__ X, int64_t ld, int64_t D, int n,
+                                                    double* part, int* bad) {
+  __shared__ unsigned long long red[CM_ROWS][CM_COLS];
+  const int cx = threadIdx.x & 63, ry = threadIdx.x >> 6;
+  const int c = blockIdx.y * CM_COLS + 2 * cx;
+  const int64_t per = (D + gridDim.x - 1) / gridDim.x;
+  const int64_t r0 = per * blockIdx.x, r1 = min(D, r0 + per);
+  const bool two = c + 1 < n;
+  unsigned long long m0 = 0, m1 = 0;
+  if (c < n) {
+    for (int64_t r = r0 + ry; r < r1; r += CM_ROWS * CM_UNROLL) {
+      double2 v[CM_UNROLL];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) m[u] = max(m[u], abs_bits(X[(r + u * g) * ld + c]));
+      for (int u = 0; u < CM_UNROLL; ++u) {
+        const int64_t ru = r + u * CM_ROWS;
+        v[u] = make_double2(0.0, 0.0);
+        if (ru < r1) {
+          const double* p = X + ru * ld + c;
+          if (VEC && two) {
+            v[u] = __ldg(reinterpret_cast<const double2*>(p));
+          } else {
+            v[u].x = __ldg(p);
+            if (two) v[u].y = __ldg(p + 1);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < CM_UNROLL; ++u) {
+        m0 = max(m0, abs_bits(v[u].x));
+        m1 = max(m1, abs_bits(v[u].y));
+      }
     }
-    for (; r < D; r += g) m[0] = max(m[0], abs_bits(X[r * ld + c]));
-    const unsigned long long mm = max(max(m[0], m[1]), max(m[2], m[3]));
-    if (mm >= 0x7FF0000000000000ull) *bad = 1;  // NaN or inf
-    part[(int64_t)blockIdx.x * n + c] = __longlong_as_double((long long)mm);
+  }
+  red[ry][2 * cx] = m0;
+  red[ry][2 * cx + 1] = m1;
+  __syncthreads();
+  if (threadIdx.x < CM_COLS) {
+    const int cc = blockIdx.y * CM_COLS + threadIdx.x;
+    const unsigned long long m = max(max(red[0][threadIdx.x], red[1][threadIdx.x]),
+                                     max(red[2][threadIdx.x], red[3][threadIdx.x]));
+    if (cc < n) {
+      if (m >= 0x7FF0000000000000ull) *bad = 1;  // NaN or inf
+      part[(int64_t)blockIdx.x * n + cc] = __longlong_as_double((long long)m);
+    }
   }
 }
+// one warp per column
 __global__ void k_col_exp(const double* part, int nb, int n, int* ex) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (c >= n) return;
-  double m = 0.0;
-  for (int b = 0; b < nb; ++b) m = fmax(m, part[(int64_t)b * n + c]);
-  int e = 0;
-  if (m > 0.0) frexp(m, &e);
-  ex[c] = e;
+  unsigned long long m = 0;
+  for (int b = lane; b < nb; b += 32) m = max(m, abs_bits(part[(int64_t)b * n + c]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) {
+    int e = 0;
+    if (m > 0) frexp(__longlong_as_double((long long)m), &e);
+    ex[c] = e;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -464,47 +517,62 @@ __global__ void k_digits_cols(const double* __restrict__ X, int64_t ld, int64_t 
   });
 }
 
-// one warp per row: the row's exponent (max |v| over the row, written to
-// er[r]; a non-finite value raises *bad), then its digit blocks
-__global__ void k_digits_rows(const double* __restrict__ V, int64_t ldv, int64_t D, int n, int64_t Dpad,
-                              int npad, int vec, int* er, int* bad, __nv_bfloat16* __restrict__ Vd) {
-  const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (r >= Dpad) return;
-  const bool live = r < D;
-  const double* row = V + r * ldv;
+// Eight rows per CTA: each warp brings one row into shared memory and finds its
+// exponent (max |v|, written to er[r]; a non-finite value raises *bad), then eight
+// threads side by side cut the same eight columns of the eight rows, so a slice's
+// stores are whole core matrices (128 consecutive bytes, 256 with the K-adjacent
+// one).  One warp per row storing 16 bytes here and there ran at 40 % of the copy
+// bandwidth (2,097,152 x 384: 7.3 ms).
+constexpr int DR_ROWS = 8;
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_digits_rows(const double* __restrict__ V, int64_t ldv, int64_t D, int n,
+                                                     int64_t Dpad, int npad, int* er, int* bad,
+                                                     __nv_bfloat16* __restrict__ Vd) {
+  extern __shared__ __align__(16) double rows_sm[];  // 8 x (npad + 2)
+  __shared__ int exps[DR_ROWS];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t rb = (int64_t)blockIdx.x * DR_ROWS, r = rb + w;
+  const int stride = npad + 2;  // 16 bytes apart in the banks
+  double* row = rows_sm + w * stride;
   unsigned long long mb = 0;  // max |v| as integer bits (see k_col_maxabs)
-  if (live)
-    for (int c = lane; c < n; c += 32) mb = max(mb, abs_bits(row[c]));
+  for (int c = 2 * lane; c < npad; c += 64) {
+    double2 v = make_double2(0.0, 0.0);
+    if (r < D) {
+      const double* p = V + r * ldv + c;
+      if (VEC && c + 1 < n) {
+        v = __ldg(reinterpret_cast<const double2*>(p));
+      } else {
+        if (c < n) v.x = __ldg(p);
+        if (c + 1 < n) v.y = __ldg(p + 1);
+      }
+    }
+    mb = max(mb, max(abs_bits(v.x), abs_bits(v.y)));
+    *reinterpret_cast<double2*>(row + c) = v;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-  if (mb >= 0x7FF0000000000000ull) {  // NaN or inf
-    if (lane == 0) *bad = 1;
-    mb = 0;
-  }
-  int e = 0;
-  const double m = __longlong_as_double((long long)mb);
-  if (m > 0.0) frexp(m, &e);
-  if (live && lane == 0) er[r] = e;
-  const int64_t nkc = npad / KS;
-  for (int g = lane; g < npad / 8; g += 32) {  // groups of 8 consecutive k (L1-resident row)
-    const int k0 = 8 * g;
-    double x[8];
-    if (vec && live && k0 + 8 <= n) {  // 16-byte aligned rows: four 16-byte loads
-      const double2* p = reinterpret_cast<const double2*>(row + k0);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double2 t = __ldg(p + q);
-        x[2 * q] = t.x;
-        x[2 * q + 1] = t.y;
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) x[q] = (live && k0 + q < n) ? row[k0 + q] : 0.0;
+  if (lane == 0) {
+    if (mb >= 0x7FF0000000000000ull) {  // NaN or inf
+      *bad = 1;
+      mb = 0;
     }
-    unsigned char* blk = reinterpret_cast<unsigned char*>(Vd + ((r >> 7) * nkc + (k0 >> 4)) * 8 * A_ELEMS);
-    const int off = core_offset((int)(r & 127), k0 & 15);
-    cut8(x, e, [&](int s, uint4 v) { *reinterpret_cast<uint4*>(blk + (size_t)s * A_SLICE + off) = v; });
+    int e = 0;
+    if (mb > 0) frexp(__longlong_as_double((long long)mb), &e);
+    if (r < D) er[r] = e;
+    exps[w] = e;
+  }
+  __syncthreads();
+  const int64_t nkc = npad / KS;
+  for (int item = threadIdx.x; item < npad; item += 256) {  // npad / 8 column groups x 8 rows
+    const int q = item & 7, k0 = (item >> 3) * 8;
+    const double* src = rows_sm + q * stride + k0;
+    double x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = src[u];
+    const int64_t rr = rb + q;
+    unsigned char* blk = reinterpret_cast<unsigned char*>(Vd + ((rr >> 7) * nkc + (k0 >> 4)) * 8 * A_ELEMS);
+    const int off = core_offset((int)(rr & 127), k0 & 15);
+    cut8(x, exps[q], [&](int s, uint4 v) { *reinterpret_cast<uint4*>(blk + (size_t)s * A_SLICE + off) = v; });
   }
 }
 
@@ -639,6 +707,9 @@ fd_status set_attrs(fd_ctx* ctx) {
   if (bit && (attrs_set.load() & bit)) return FD_OK;
   FD_CUDA(ctx, cudaFuncSetAttribute(k_oz_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
   FD_CUDA(ctx, cudaFuncSetAttribute(k_oz_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
+  const int rows_smem = (int)(sizeof(double) * DR_ROWS * (1024 + 2));
+  FD_CUDA(ctx, cudaFuncSetAttribute(k_digits_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem));
+  FD_CUDA(ctx, cudaFuncSetAttribute(k_digits_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem));
   attrs_set.fetch_or(bit);
   return FD_OK;
 }
@@ -679,12 +750,17 @@ fd_status cut_cols(fd_ctx* ctx, const double* X, int64_t ld, int64_t D, int w, c
 // Column exponents of X (n columns over D rows); non-finite values raise *bad.
 static fd_status col_exponents(fd_ctx* ctx, const double* X, int64_t ld, int64_t D, int n, int* ex,
                                int* bad) {
-  const int nb = (int)std::min<int64_t>(ctx->num_sms * 4, std::max<int64_t>(1, D));
+  // about eight CTAs per SM, at least one unrolled run of rows each
+  const int ct = (int)cdiv(n, CM_COLS);
+  const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(8LL * ctx->num_sms, ct), D / (CM_ROWS * CM_UNROLL)));
   void* p;
   FD_TRY(workspace(ctx, "oz_colmax", sizeof(double) * (size_t)nb * n, &p));
-  k_col_maxabs<<<nb, 256, 0, ctx->stream>>>(X, ld, D, n, (double*)p, bad);
+  if (((uintptr_t)X & 15) == 0 && ld % 2 == 0)
+    k_col_maxabs<true><<<dim3(nb, ct), 256, 0, ctx->stream>>>(X, ld, D, n, (double*)p, bad);
+  else
+    k_col_maxabs<false><<<dim3(nb, ct), 256, 0, ctx->stream>>>(X, ld, D, n, (double*)p, bad);
   FD_LAUNCHED(ctx);
-  k_col_exp<<<(unsigned)cdiv(n, 256), 256, 0, ctx->stream>>>((double*)p, nb, n, ex);
+  k_col_exp<<<(unsigned)cdiv(n, 8), 256, 0, ctx->stream>>>((double*)p, nb, n, ex);
   FD_LAUNCHED(ctx);
   return FD_OK;
 }
@@ -766,21 +842,19 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   FD_CUDA(ctx, cudaMemsetAsync(bad, 0, 2 * sizeof(int), ctx->stream));
   FD_TRY(col_exponents(ctx, M, n, n, n, em, bad));
   FD_TRY(cut_cols(ctx, M, n, n, n, em, Md, npad / KS));
-  const int vec = (((uintptr_t)V & 15) == 0 && (ldv & 1) == 0) ? 1 : 0;
-  k_digits_rows<<<(unsigned)cdiv(Dpad, 8), 256, 0, ctx->stream>>>(V, ldv, D, n, Dpad, npad, vec, er, bad, Vd);
+  const size_t rows_smem = sizeof(double) * DR_ROWS * (npad + 2);  // 65.7 KB at the widest, n = 1024
+  auto cut_rows = ((uintptr_t)V & 15) == 0 && (ldv & 1) == 0 ? k_digits_rows<true> : k_digits_rows<false>;
+  cut_rows<<<(unsigned)(Dpad / DR_ROWS), 256, rows_smem, ctx->stream>>>(V, ldv, D, n, Dpad, npad, er, bad, Vd);
   FD_LAUNCHED(ctx);
   int hbad = 0;
   FD_CUDA(ctx, cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   FD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   if (hbad) return FD_OK;  // non-finite input: the FP64 path propagates it
-  FD_TRY(workspace(ctx, "oz_rot_out", sizeof(double) * (size_t)D * n, &p));
-  double* Out = (double*)p;
+  // V is no longer read (its digits are): the product goes straight into it
   k_oz_rotate<<<(unsigned)((Dpad / TM) * (npad / TN)), OZ_THREADS, OZ_SMEM, ctx->stream>>>(
-      Vd, Md, ncbm, D, n, npad, upper ? 1 : 0, er, em, Out, n, err);
+      Vd, Md, ncbm, D, n, npad, upper ? 1 : 0, er, em, V, ldv, err);
   FD_LAUNCHED(ctx);
   FD_TRY(check_wait_flag(ctx, err));
-  FD_CUDA(ctx, cudaMemcpy2DAsync(V, ldv * sizeof(double), Out, n * sizeof(double), n * sizeof(double), D,
-                                 cudaMemcpyDeviceToDevice, ctx->stream));
   *used = true;
   return FD_OK;
 }
