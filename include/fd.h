@@ -208,7 +208,7 @@ fd_status fd_spmmv(fd_ctx* ctx, const fd_matrix* A, fd_prec prec,
  *   FD_GEMM_OZAKI  exact splitting into 7-bit integer digits on the tcgen05
  *                  tensor cores (Ozaki scheme, 8 bf16 digits per operand
  *                  relative to each row / column maximum, FP32 level sums in
- *                  TMEM exact over K chunks of 128, 2 x 64-bit integer
+ *                  TMEM exact over K chunks of 512, 2 x 64-bit integer
  *                  accumulation): FP64 accuracy at tensor-core speed.  Uses a
  *                  grow-only device workspace of 16 bytes per operand element
  *                  for the digit tiles

@@ -7,16 +7,19 @@
 // Rump, "Error-free transformations of matrix multiplication", Numer.
 // Algorithms 2012; Mukunoki et al. 2020 on tensor cores):
 //
-//   a_ik = 2^{e_i} sum_{s<8} d^a_{s,ik} 2^{-7(s+1)},  |d| <= 127 (7-bit digits)
-//   b_kj = 2^{f_j} sum_{t<8} d^b_{t,kj} 2^{-7(t+1)}
-//   (AB)_ij = 2^{e_i + f_j} sum_{l<8} 2^{-7(l+2)} sum_{s+t=l} sum_k d^a_s d^b_t
+//   a_ik = 2^{e_i} sum_{s<8} d^a_{s,ik} 2^{-(6+7s)},  -64 <= d <= 64 (7-bit digits)
+//   b_kj = 2^{f_j} sum_{t<8} d^b_{t,kj} 2^{-(6+7t)}
+//   (AB)_ij = 2^{e_i + f_j} sum_{l<8} 2^{-(12+7l)} sum_{s+t=l} sum_k d^a_s d^b_t
 //
 // with e_i (f_j) the exponent of the largest |a_ik| over k (|b_kj| over k), so
-// each operand is cut to 56 bits relative to its row (column) maximum, and the
-// pairs s + t >= 8 (weight <= 2^-63 relative) are dropped.  Every digit is an
-// integer of magnitude below 2^7, exact in bf16.  A level l sums at most 8
-// digit pairs; over a K chunk of 128 every partial sum stays below
-// 8 * 128 * 127^2 < 2^24, so the FP32 accumulation of the tensor core is exact.
+// each operand is rounded to 55 bits below its row (column) maximum, error at most
+// 2^-56, and the pairs s + t >= 8 are dropped.  The digits are balanced (in
+// [-64, 63], the first up to 64): every one is exact in bf16, and a product is at
+// most 2^12.  A level l sums at most 8 digit pairs; over a K chunk of 512 every
+// partial sum stays within 8 * 512 * 2^12 = 2^24, so the FP32 accumulation of the
+// tensor core is exact.  (Digits of magnitude and sign up to 127 allow chunks of
+// 128 only, and the levels' read-back after each chunk, which the tensor core
+// waits for, took a third of the time.)
 //
 // Two kernels per product.  A streaming kernel cuts each FP64 operand once
 // into its 8 bf16 digit slices and writes them to HBM already in the tensor
@@ -28,7 +31,7 @@
 // digit blocks of each K step into a four-stage shared-memory ring with
 // cp.async.bulk (mbarrier complete_tx), one thread issues the step's 12
 // tcgen05.mma (36 digit pairs; M 128, N up to 256, K 16) and commits them to the
-// stage's "empty" mbarrier, and every eighth step (K = 128) all threads read
+// stage's "empty" mbarrier, and every 32nd step (K = 512) all threads read
 // the levels back with tcgen05.ld, convert them to 32-bit integers, combine
 // adjacent levels exactly in 32 bits and add them, scaled by 2^(7 (7 - l)),
 // into two 64-bit integer accumulators per output (levels 0-3 and 4-7; value
@@ -48,11 +51,12 @@ namespace {
 
 constexpr int OZ_S = 8;             // digits per operand
 constexpr int OZ_B = 7;             // bits per digit
-constexpr int OZ_F = OZ_S * OZ_B;   // 56 fraction bits
+constexpr int OZ_F = OZ_S * OZ_B - 1;  // 55 fraction bits
+constexpr int OZ_UNIT = OZ_B * (OZ_S - 1) + 2 * (OZ_B - 1);  // accumulator unit 2^-61
 constexpr int TM = 128;             // output tile rows (tcgen05 M)
 constexpr int TN = 64;              // output tile columns (tcgen05 N)
 constexpr int KS = 16;              // K step (one tcgen05.mma)
-constexpr int SUBS = 8;             // K steps per exact FP32 chunk (K = 128)
+constexpr int SUBS = 32;            // K steps per exact FP32 chunk (K = 512)
 constexpr int NST = 4;              // shared-memory ring stages
 constexpr int OZ_THREADS = 512;
 constexpr int A_SLICE = TM * KS * 2;                  // 4096 bytes per digit block
@@ -139,33 +143,39 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+// 16 columns each of two levels, and the wait for both in the same statement (no
+// use of the registers can be scheduled before it)
+__device__ __forceinline__ void tmem_ld16x2(uint32_t t0, uint32_t t1, uint32_t (&r0)[16], uint32_t (&r1)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-      "[%16];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(r0[0]), "=r"(r0[1]), "=r"(r0[2]), "=r"(r0[3]), "=r"(r0[4]), "=r"(r0[5]), "=r"(r0[6]), "=r"(r0[7]), "=r"(r0[8]), "=r"(r0[9]), "=r"(r0[10]), "=r"(r0[11]), "=r"(r0[12]), "=r"(r0[13]), "=r"(r0[14]), "=r"(r0[15]),
+        "=r"(r1[0]), "=r"(r1[1]), "=r"(r1[2]), "=r"(r1[3]), "=r"(r1[4]), "=r"(r1[5]), "=r"(r1[6]), "=r"(r1[7]), "=r"(r1[8]), "=r"(r1[9]), "=r"(r1[10]), "=r"(r1[11]), "=r"(r1[12]), "=r"(r1[13]), "=r"(r1[14]), "=r"(r1[15])
+      : "r"(t0), "r"(t1)
+      : "memory");
 }
 
-// fixed-point magnitude y = |x| 2^(56 - e) (< 2^56 for |x| < 2^e) and sign of x
-__device__ __forceinline__ unsigned long long fixed56(double x, int e, uint32_t* sign) {
+// x 2^(55 - e) rounded to an integer (|x| < 2^e: magnitude at most 2^55), with 64
+// added to each of its 8 base-128 digits, so that every field holds its balanced
+// digit plus 64
+__device__ __forceinline__ unsigned long long biased_fixed(double x, int e) {
+  constexpr unsigned long long BIAS = 64ull * (((1ull << 56) - 1) / 127);
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((bits >> 52) & 0x7FF);
   unsigned long long m = bits & 0xFFFFFFFFFFFFFull;
   if (ex) m |= 1ull << 52;
-  const int sh = (ex ? ex : 1) - 1075 - e + OZ_F;  // |x| 2^(F - e) = m 2^sh < 2^56
-  *sign = (uint32_t)(bits >> 63);
-  if (m == 0 || sh <= -64) return 0;
-  return sh >= 0 ? m << sh : m >> (-sh);
+  const int sh = (ex ? ex : 1) - 1075 - e + OZ_F;  // |x| 2^(F - e) = m 2^sh
+  unsigned long long y = 0;
+  if (sh >= 0) y = m << sh;
+  else if (sh > -64) y = (m + (1ull << (-sh - 1))) >> (-sh);
+  return BIAS + ((bits >> 63) ? 0ull - y : y);
 }
 
-// bf16 bit pattern of the digit v in [0, 127]: the float v is built exactly by
+// bf16 bit pattern of the digit v - 64, v in [0, 128]: the float is built exactly by
 // the 2^23 bias trick and its upper half is the bf16 value (8 significant bits)
 __device__ __forceinline__ uint32_t bf16_of_digit(uint32_t v) {
-  return __float_as_uint(__uint_as_float(0x4B000000u | v) - 8388608.0f) >> 16;
+  return __float_as_uint(__uint_as_float(0x4B000000u | v) - 8388672.0f) >> 16;
 }
 
 // the 8 digit slices of 8 consecutive K values of one operand row (or
@@ -174,21 +184,18 @@ __device__ __forceinline__ uint32_t bf16_of_digit(uint32_t v) {
 template <typename Put>
 __device__ __forceinline__ void cut8(const double (&x)[8], int e, Put&& put) {
   unsigned long long y[8];
-  uint32_t sg[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) y[q] = fixed56(x[q], e, &sg[q]);
-  uint32_t smask[4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p) smask[p] = (sg[2 * p] << 15) | (sg[2 * p + 1] << 31);
+  for (int q = 0; q < 8; ++q) y[q] = biased_fixed(x[q], e);
 #pragma unroll
   for (int s = 0; s < OZ_S; ++s) {
-    const int sh = OZ_F - OZ_B * (s + 1);
+    const int sh = OZ_B * (OZ_S - 1 - s);
+    const uint32_t mask = s == 0 ? 0xFFu : 0x7Fu;  // the first digit may be 64
     uint32_t w[4];
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
-      const uint32_t lo = bf16_of_digit((uint32_t)(y[2 * p] >> sh) & 0x7Fu);
-      const uint32_t hi = bf16_of_digit((uint32_t)(y[2 * p + 1] >> sh) & 0x7Fu);
-      w[p] = (lo | (hi << 16)) | smask[p];
+      const uint32_t lo = bf16_of_digit((uint32_t)(y[2 * p] >> sh) & mask);
+      const uint32_t hi = bf16_of_digit((uint32_t)(y[2 * p + 1] >> sh) & mask);
+      w[p] = lo | (hi << 16);
     }
     put(s, make_uint4(w[0], w[1], w[2], w[3]));
   }
@@ -201,7 +208,7 @@ __device__ __forceinline__ int core_offset(int row, int k) {
 }
 
 // Exact accumulator of one output: value = hi 2^28 + lo in units of
-// 2^-63 2^(e_i + f_j); level l carries the weight 2^(7 (7 - l)).
+// 2^-61 2^(e_i + f_j); level l carries the weight 2^(7 (7 - l)).
 struct Acc {
   long long hi, lo;
 };
@@ -235,18 +242,17 @@ __device__ __forceinline__ void issue_step(uint32_t tmem, uint64_t adesc, uint64
 
 // Read the 8 levels of this thread's 16 outputs (TMEM lane = tile row
 // 32 (warp & 3) + lane, columns 16 (warp >> 2) ..) into the accumulators.
-// Level sums are integers below 2^24 (l + 1 pairs x 128 x 127^2), so two
-// adjacent levels combine exactly in 32 bits (c_l 2^7 + c_{l+1} < 2^31) and
-// only 32-bit conversions are needed (64-bit ones run on GB300's slow FP64
-// units).
+// Level sums are integers of at most (l + 1) 2^21 (l + 1 pairs x 512 x 2^12), so
+// two adjacent levels combine exactly in 32 bits (c_l 2^7 + c_{l+1} <= 7 2^28 + 2^24
+// < 2^31 for even l <= 6) and only 32-bit conversions are needed (64-bit ones run
+// on GB300's slow FP64 units).
 __device__ __forceinline__ void flush(uint32_t tmem, Acc (&acc)[16]) {
   const int w = threadIdx.x >> 5;
   const uint32_t base = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(16 * (w >> 2));
 #pragma unroll 1
   for (int pr = 0; pr < OZ_S / 2; ++pr) {  // level pairs (0,1) (2,3) (4,5) (6,7)
     uint32_t r0[16], r1[16];
-    tmem_ld16(base + (uint32_t)(2 * pr * TN), r0);
-    tmem_ld16(base + (uint32_t)((2 * pr + 1) * TN), r1);
+    tmem_ld16x2(base + (uint32_t)(2 * pr * TN), base + (uint32_t)((2 * pr + 1) * TN), r0, r1);
     const int sh = (pr & 1) ? 0 : 14;  // pairs (0,1), (4,5) carry 2^14 within hi / lo
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
@@ -619,7 +625,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         smem, acc,
         [&](int i, int j) {
           const int gi = i0 + i, gj = j0 + j;
-          return (gi < m && gj < n) ? ex[gi] + ey[gj] - 63 : 0;
+          return (gi < m && gj < n) ? ex[gi] + ey[gj] - OZ_UNIT : 0;
         },
         [&](int i, int j, double v) {
           const int gi = i0 + i, gj = j0 + j;
@@ -675,7 +681,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         [&](int i, int j) {
           const int64_t gr = r0 + i;
           const int gj = j0 + j;
-          return (gr < D && gj < n) ? er[gr] + em[gj] - 63 : 0;
+          return (gr < D && gj < n) ? er[gr] + em[gj] - OZ_UNIT : 0;
         },
         [&](int i, int j, double v) {
           const int64_t gr = r0 + i;
