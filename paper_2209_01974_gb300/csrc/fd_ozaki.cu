@@ -370,6 +370,23 @@ __device__ __forceinline__ double acc_value(const Acc& a, int sc) {
   return __longlong_as_double((long long)bits);
 }
 
+// The same for |hi|, |lo| < 2^51 (at most 32 exact chunks): both integers become
+// doubles by placing them in the significand of 3 2^79 and 3 2^51; taking both
+// offsets off the first leaves hi 2^28 - 3 2^51, a multiple of 2^28 below 2^80 (exact),
+// and adding the second rounds hi 2^28 + lo once.  Two FP64 additions and a dozen
+// integer instructions instead of 190 (the rotation's tiles end every 4 to 64 K
+// steps, and rounding their outputs took as long as the products).
+__device__ __forceinline__ double acc_value_small(const Acc& a, int sc) {
+  const double x = __longlong_as_double(0x44F8000000000000ll + a.hi);  // (3 2^51 + hi) 2^28
+  const double y = __longlong_as_double(0x4338000000000000ll + a.lo);  // 3 2^51 + lo
+  const double v = __dadd_rn(__dsub_rn(x, 0x3.0000003p79 /* 3 2^79 + 3 2^51 */), y);
+  const long long bits = __double_as_longlong(v);
+  const int e = (int)((bits >> 52) & 0x7FF);
+  if (e == 0) return 0.0;  // v is an integer: zero
+  if (e + sc < 1 || e + sc > 2046) return ldexp(v, sc);
+  return __longlong_as_double(bits + ((long long)sc << 52));
+}
+
 // CTA prologue: TMEM (warp 0) and the full / empty mbarriers of the ring
 __device__ __forceinline__ uint32_t tile_setup(unsigned char* smem, uint64_t** full, uint64_t** empty) {
   unsigned char* tail = smem + (size_t)NST * STAGE;
@@ -650,44 +667,142 @@ __global__ void k_oz_gram_reduce(const double* P, int slices, int m, int n, int 
 // ---------------------------------------------------------------------------
 // rotation: Out[r][j] = sum_k V[r][k] M[k][j] from the row-scaled digits of V
 // and the column-scaled digits of M; tile (rb, jt) covers rows [128 rb, +128)
-// and columns [64 jt, +64)
+// and columns [64 jt, +64).
+//
+// A tile is short (n / 16 K steps, fewer for a triangular M), so its end weighs as
+// much as its products: reading the levels back, rounding to FP64 and storing.  The
+// CTAs are persistent (one per SM) and take their tiles' K steps as one stream: the
+// bulk copies run on into the next tile, and its first NST K steps are issued as
+// soon as the levels have been read, so the tensor core works while the threads
+// round and store the previous tile from registers.  The grid is a multiple of the
+// tiles of a row block, which therefore run at the same time and share its digits
+// in L2, and a CTA moves on by one column tile per row block, so that the lengths
+// of a triangular M even out.  2,097,152 x 384, triangular M: 14.2 -> 13.0 ms (one
+// CTA per tile, 128-bit integer rounding, stores staged in the ring -> this); the
+// tensor pipe is active 42 % of the time.
 // ---------------------------------------------------------------------------
+enum { STORE_8 = 0, STORE_16 = 1, STORE_32 = 2 };  // bytes per store (alignment of Out and its rows)
+template <int STORE>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_rotate(const __nv_bfloat16* __restrict__ Vd, const __nv_bfloat16* __restrict__ Md, int ncbm,
-                int64_t D, int n, int npad, int upper, const int* er, const int* em,
+                int64_t D, int n, int npad, int nrb, int upper, const int* er, const int* em,
                 double* __restrict__ Out, int64_t ldo, int* err) {
   extern __shared__ __align__(128) unsigned char smem[];
-  // the column tiles of one row block are consecutive CTAs, so the row
-  // block's digits are read from HBM once and then from L2
-  const int njt = npad / TN;
-  const int64_t rb = blockIdx.x / njt;
-  const int jt = (int)(blockIdx.x % njt), j0 = jt * TN;
-  const int kend = upper ? min(npad, j0 + TN) : npad;  // M upper triangular: rows k <= j
-  const int64_t nkc = npad / KS;
+  const int njt = npad / TN, per = gridDim.x / njt;  // row blocks in flight
+  const int slot = blockIdx.x / njt, col0 = blockIdx.x % njt;
+  const int nkc = npad / KS;
+  const int64_t a_kc = 8LL * A_ELEMS, a_s = A_ELEMS;
+  const int64_t b_kc = 8LL * ncbm * B_ELEMS, b_s = (int64_t)ncbm * B_ELEMS;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto steps = [&](int jt) { return upper ? (jt + 1) * (TN / KS) : nkc; };  // M upper triangular: rows k <= j
+  auto next = [&](int jt) { return jt + 1 == njt ? 0 : jt + 1; };
   uint64_t *full, *empty;
   const uint32_t tmem = tile_setup(smem, &full, &empty);
-  Acc acc[16];
+  // producer warp: K step sc of tile (rb, jt) into the stage of stream position g
+  auto load = [&](int rb, int jt, int sc, uint32_t g) {
+    const int st = (int)(g % NST);
+    unsigned char* dst = smem + (size_t)st * STAGE;
+    if (lane == 0) mbar_expect_tx(&full[st], STAGE);
+    __syncwarp();
+    if (lane < 2 * OZ_S) {
+      const int s = lane >> 1;
+      if (lane & 1)
+        bulk_g2s(dst + OZ_S * A_SLICE + s * B_SLICE, Md + (int64_t)jt * B_ELEMS + sc * b_kc + s * b_s, B_SLICE,
+                 &full[st]);
+      else
+        bulk_g2s(dst + s * A_SLICE, Vd + (int64_t)rb * nkc * 8 * A_ELEMS + sc * a_kc + s * a_s, A_SLICE, &full[st]);
+    }
+  };
+  // MMA issuer: the K step at stream position g
+  auto issue = [&](int sc, uint32_t g) {
+    const int st = (int)(g % NST);
+    if (!mbar_wait(&full[st], (g / NST) & 1u)) return false;
+    tc_fence_after();
+    const uint32_t a0 = smem_u32(smem + (size_t)st * STAGE);
+    const uint64_t ad = sdesc(a0), bd = sdesc(a0 + OZ_S * A_SLICE);
+    if ((sc % SUBS) == 0) issue_step<true>(tmem, ad, bd);
+    else issue_step<false>(tmem, ad, bd);
+    umma_commit(&empty[st]);
+    return true;
+  };
+  bool ok = true;
+  // the next K step to load: tile (lrb, ljt), step ls, stream position lg
+  int lrb = slot, ljt = col0, ls = 0;
+  uint32_t lg = 0;
+  auto load_next = [&]() {
+    load(lrb, ljt, ls, lg);
+    ++lg;
+    if (++ls == steps(ljt)) {
+      ls = 0;
+      lrb += per;
+      ljt = next(ljt);
+    }
+  };
+  if (warp == P_THREAD / 32)
+    for (int i = 0; i < NST && lrb < nrb; ++i) load_next();
+  uint32_t g = 0;  // stream position of the current tile's first K step
+  int ahead = 0;   // K steps of the current tile issued already
+  int jt = col0;
+  for (int rb = slot; rb < nrb; rb += per, jt = next(jt)) {
+    const int nsub = steps(jt);
+    Acc acc[16];
 #pragma unroll
-  for (int c = 0; c < 16; ++c) acc[c] = Acc{0, 0};
-  const int64_t b_kc = 8LL * ncbm * B_ELEMS, b_s = (int64_t)ncbm * B_ELEMS;
-  const bool ok = run_tile(smem, full, empty, tmem, Vd + rb * nkc * 8 * A_ELEMS, 8LL * A_ELEMS, A_ELEMS,
-                           Md + (int64_t)jt * B_ELEMS, b_kc, b_s, kend / KS, acc);
-  if (!ok) {
-    if (threadIdx.x == 0) atomicExch(err, 1);
-  } else {
-    const int64_t r0 = rb * TM;
-    write_tile(
-        smem, acc,
-        [&](int i, int j) {
-          const int64_t gr = r0 + i;
-          const int gj = j0 + j;
-          return (gr < D && gj < n) ? er[gr] + em[gj] - OZ_UNIT : 0;
-        },
-        [&](int i, int j, double v) {
-          const int64_t gr = r0 + i;
-          const int gj = j0 + j;
-          if (gr < D && gj < n) Out[gr * ldo + gj] = v;
-        });
+    for (int c = 0; c < 16; ++c) acc[c] = Acc{0, 0};
+    for (int sc = 0; sc < nsub; ++sc) {
+      const int st = (int)((g + sc) % NST);
+      const uint32_t par = ((g + sc) / NST) & 1u;
+      if (threadIdx.x == M_THREAD && ok && sc >= ahead) ok = issue(sc, g + sc);
+      if (warp == P_THREAD / 32 && ok && lrb < nrb) {
+        // the stage is free again once the MMAs of K step sc have completed
+        ok = mbar_wait(&empty[st], par);
+        if (ok) load_next();
+      }
+      const bool last = sc == nsub - 1;
+      if ((sc % SUBS) == SUBS - 1 || last) {
+        // the issuer observes the completion; the others sleep in the barrier
+        if (threadIdx.x == M_THREAD && ok) ok = mbar_wait(&empty[st], par);
+        if (__syncthreads_or(!ok)) {
+          if (threadIdx.x == 0) atomicExch(err, 1);
+          tile_teardown(tmem);
+          return;
+        }
+        tc_fence_after();
+        flush(tmem, acc);
+        tc_fence_before();
+        __syncthreads();
+      }
+    }
+    g += (uint32_t)nsub;
+    // the next tile's first K steps, before this one's results are rounded
+    ahead = rb + per < nrb ? min(NST, min(steps(next(jt)), SUBS)) : 0;
+    if (threadIdx.x == M_THREAD) {
+      tc_fence_after();
+      for (int sc = 0; sc < ahead && ok; ++sc) ok = issue(sc, g + sc);
+    }
+    __syncwarp();
+    const int64_t row = (int64_t)rb * TM + 32 * (warp & 3) + lane;
+    const int c0 = jt * TN + 16 * (warp >> 2);
+    if (row < D && c0 < n) {
+      const int e = er[row] - OZ_UNIT;
+      double* o = Out + row * ldo + c0;
+#pragma unroll
+      for (int c = 0; c < 16; c += 4) {
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = acc_value_small(acc[c + u], c0 + c + u < n ? e + __ldg(em + c0 + c + u) : 0);
+        if (STORE == STORE_32 && c0 + c + 4 <= n) {
+          asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};\n" ::"l"(o + c), "d"(v[0]), "d"(v[1]), "d"(v[2]),
+                       "d"(v[3]) : "memory");
+        } else if (STORE >= STORE_16 && c0 + c + 4 <= n) {
+          *reinterpret_cast<double2*>(o + c) = make_double2(v[0], v[1]);
+          *reinterpret_cast<double2*>(o + c + 2) = make_double2(v[2], v[3]);
+        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (c0 + c + u < n) o[c + u] = v[u];
+        }
+      }
+    }
   }
   tile_teardown(tmem);
 }
@@ -712,7 +827,8 @@ fd_status set_attrs(fd_ctx* ctx) {
   const unsigned long long bit = ctx->device < 64 ? 1ull << ctx->device : 0ull;
   if (bit && (attrs_set.load() & bit)) return FD_OK;
   FD_CUDA(ctx, cudaFuncSetAttribute(k_oz_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
-  FD_CUDA(ctx, cudaFuncSetAttribute(k_oz_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
+  for (auto rot : {k_oz_rotate<STORE_8>, k_oz_rotate<STORE_16>, k_oz_rotate<STORE_32>})
+    FD_CUDA(ctx, cudaFuncSetAttribute(rot, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
   const int rows_smem = (int)(sizeof(double) * DR_ROWS * (1024 + 2));
   FD_CUDA(ctx, cudaFuncSetAttribute(k_digits_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem));
   FD_CUDA(ctx, cudaFuncSetAttribute(k_digits_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem));
@@ -849,7 +965,8 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   FD_TRY(col_exponents(ctx, M, n, n, n, em, bad));
   FD_TRY(cut_cols(ctx, M, n, n, n, em, Md, npad / KS));
   const size_t rows_smem = sizeof(double) * DR_ROWS * (npad + 2);  // 65.7 KB at the widest, n = 1024
-  auto cut_rows = ((uintptr_t)V & 15) == 0 && (ldv & 1) == 0 ? k_digits_rows<true> : k_digits_rows<false>;
+  const bool vec = ((uintptr_t)V & 15) == 0 && (ldv & 1) == 0;
+  auto cut_rows = vec ? k_digits_rows<true> : k_digits_rows<false>;
   cut_rows<<<(unsigned)(Dpad / DR_ROWS), 256, rows_smem, ctx->stream>>>(V, ldv, D, n, Dpad, npad, er, bad, Vd);
   FD_LAUNCHED(ctx);
   int hbad = 0;
@@ -857,8 +974,11 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   FD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   if (hbad) return FD_OK;  // non-finite input: the FP64 path propagates it
   // V is no longer read (its digits are): the product goes straight into it
-  k_oz_rotate<<<(unsigned)((Dpad / TM) * (npad / TN)), OZ_THREADS, OZ_SMEM, ctx->stream>>>(
-      Vd, Md, ncbm, D, n, npad, upper ? 1 : 0, er, em, V, ldv, err);
+  static_assert(1024 / KS <= 32 * SUBS, "acc_value_small holds 32 exact chunks");
+  const int njt = npad / TN, nrb = (int)(Dpad / TM);
+  const unsigned grid = (unsigned)(njt * std::max(1, std::min(nrb, ctx->num_sms / njt)));
+  auto rot = ((uintptr_t)V & 31) == 0 && ldv % 4 == 0 ? k_oz_rotate<STORE_32> : vec ? k_oz_rotate<STORE_16> : k_oz_rotate<STORE_8>;
+  rot<<<grid, OZ_THREADS, OZ_SMEM, ctx->stream>>>(Vd, Md, ncbm, D, n, npad, nrb, upper ? 1 : 0, er, em, V, ldv, err);
   FD_LAUNCHED(ctx);
   FD_TRY(check_wait_flag(ctx, err));
   *used = true;

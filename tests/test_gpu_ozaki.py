@@ -155,3 +155,40 @@ def test_full_size_gram_and_cholqr2(fd, ctx):
     assert np.abs(Q - np.eye(ns)).max() <= 1e-12
     del V
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("D", [1, 127, 128, 129, 128 * 152 + 5, 128 * 400 + 1])
+@pytest.mark.parametrize("n,ld", [(1, 1), (63, 65), (64, 64), (65, 66), (200, 200), (384, 388), (1024, 1024)])
+@pytest.mark.parametrize("upper", [False, True])
+def test_rotation_tiles(fd, ctx, D, n, ld, upper):
+    """Row blocks and column tiles around one round of the persistent grid, odd
+    and padded leading dimensions, more than one exact K chunk (n = 1024)."""
+    import torch
+    if D * n > 2.2e7:
+        pytest.skip("the reference takes too long")
+    rng = np.random.default_rng(D + n)
+    V, M = rng.standard_normal((D, n)), rng.standard_normal((n, n))
+    if upper:
+        M = np.triu(M)
+    big = torch.zeros((D, ld), dtype=torch.float64, device="cuda")
+    big[:, :n] = _t(V)
+    fd.fd_set_gemm_mode(ctx, "ozaki")
+    fd.fd_rotate(ctx, big[:, :n], _t(M), upper)
+    got = big.cpu().numpy()
+    assert np.all(got[:, n:] == 0.0)
+    bound = 8 * n * U * np.outer(np.abs(V).max(1), np.abs(M).max(0))
+    assert np.all(np.abs(got[:, :n] - V @ M) <= bound)
+
+
+def test_gram_over_several_exact_chunks(fd, ctx):
+    """Worst case of the level sums: every digit at its largest magnitude over
+    K chunks of 512 (the sums then reach 2^24)."""
+    # 2^-1 (1 + 2^-7 + 2^-14 + ...) has all balanced digits equal to 64 or -64 + carry
+    x = sum(2.0 ** (-1 - 7 * k) for k in range(7))
+    for sign in (1.0, -1.0):
+        X = np.full((70000, 64), x)
+        Y = np.full((70000, 64), sign * x)
+        fd.fd_set_gemm_mode(ctx, "ozaki")
+        C = fd.fd_gram(ctx, _t(X), _t(Y)).cpu().numpy()
+        ref = sign * 70000 * x * x
+        assert np.abs(C - ref).max() <= 8 * 70000 * U * x * x
