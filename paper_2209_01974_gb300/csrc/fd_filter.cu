@@ -6,9 +6,10 @@
 // three terms (step_terms), so a step moves 11/3 vectors on average, and the
 // steps follow each other by programmatic dependent launch (step_wait).
 // Measured: 2.1M-row stencil, nb = 64, FP32, degree 40 with its two conversions
-// 21.1 -> 17.6 ms; 1.4M-row road graph, nb = 32, FP32 6.95 -> 5.53 ms; 110,592-row
-// Anderson, nb = 32, float-float 19.1 -> 15.8 ms, FP64 (bound by the FP64 pipe)
-// 32.9 -> 31.3 ms.
+// 21.1 -> 17.6 ms; 1.4M-row road graph, nb = 32, FP32 6.95 -> 5.53 ms.  FP64 and
+// float-float filters scale the matrix once (scale_matrix): 110,592-row Anderson,
+// nb = 32, 4 x 100 steps, float-float 19.1 -> 14.9 ms (15.8 unscaled), FP64, bound by
+// the FP64 pipe, 32.9 -> 26.0 ms (31.3 unscaled).
 //
 // Work mapping: a group of G lanes owns one SELL row; each lane holds CPL
 // 16-byte vectors of the row (G * CPL * 16 bytes = nb * sizeof(T)), so every
@@ -78,6 +79,24 @@ __global__ void k_scan_packed(const uint32_t* ent, int64_t n, uint32_t mask, int
     if ((int64_t)(ent[i] & mask) >= bound) atomicExch(bad, 1);
 }
 
+// out = a2 val (+ b2 on the diagonals, entry 0 of every SELL row): the matrix a
+// filter's steps use.  One thread per SELL row.
+template <typename T>
+__global__ void k_scale_sell(const int64_t* chunk_ptr, const double* val, int64_t rows, int C, double a2, double b2,
+                             T* out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= rows) return;
+  const uint32_t chunk = (uint32_t)i / (uint32_t)C, r = (uint32_t)i - chunk * (uint32_t)C;
+  const int64_t e0 = chunk_ptr[chunk], e1 = chunk_ptr[chunk + 1];
+  for (int64_t e = e0 + r; e < e1; e += C) out[e] = T(e == e0 + r ? ::fma(a2, val[e], b2) : a2 * val[e]);
+}
+// the same for one table of the matrix-free operator
+template <typename T>
+__global__ void k_scale_table(const double* val, int64_t n, double a2, double b2, T* out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = T(::fma(a2, val[i], b2));
+}
+
 // dst[i] = src[perm[i]] (to SELL order) or dst[perm[i]] = src[i] (back)
 template <typename T>
 __global__ void k_permute_rows(const T* src, int64_t lds, T* dst, int64_t ldd,
@@ -97,8 +116,16 @@ bool dependent_step(const fd_ctx* ctx, unsigned grid, unsigned wave) {
   return !std::is_same_v<T, double> || grid * 2 <= (unsigned)ctx->num_sms || grid >= wave;
 }
 
+// the scaled matrix of a filter (nullptr: the matrix as it is)
+template <typename T>
+struct Scaled {
+  const T* val = nullptr;                                 // stored matrix
+  const T *up = nullptr, *dn = nullptr, *diag = nullptr;  // matrix-free tables
+  bool on() const { return val || diag; }
+};
+
 template <typename T, int NB>
-fd_status launch_kron_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<T>& s) {
+fd_status launch_kron_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<T>& s, const Scaled<T>& sc) {
   using L = Layout<T, NB>;
   KronArgs<T> K;
   K.D = M->D;
@@ -122,6 +149,11 @@ fd_status launch_kron_step(fd_ctx* ctx, const fd_matrix* M, int mode, const Step
     K.val_dn = reinterpret_cast<const ff*>(M->kvalff[1]);
     K.diag = reinterpret_cast<const ff*>(M->kdiagff);
   }
+  if (sc.diag) {
+    K.val_up = sc.up;
+    K.val_dn = sc.dn;
+    K.diag = sc.diag;
+  }
   const unsigned grid = (unsigned)cdiv(M->D, (int64_t)WARPS * L::RPW);
   const bool dep = dependent_step<T>(ctx, grid, (unsigned)ctx->num_sms * MIN_BLOCKS_F64);  // see launch_step
   if (mode == MODE_SPMMV) return launch_step_kernel(ctx, k_kron_step<T, NB, MODE_SPMMV>, grid, WARPS * 32, 0, false, K, s);
@@ -131,14 +163,15 @@ fd_status launch_kron_step(fd_ctx* ctx, const fd_matrix* M, int mode, const Step
 }
 
 template <typename T, int NB>
-fd_status launch_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<T>& s) {
-  if (M->kron) return launch_kron_step<T, NB>(ctx, M, mode, s);
+fd_status launch_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<T>& s, const Scaled<T>& sc) {
+  if (M->kron) return launch_kron_step<T, NB>(ctx, M, mode, s, sc);
   using L = Layout<T, NB>;
   SellArgs<T> A;
   A.chunk_ptr = M->chunk_ptr; A.row_len = M->row_len; A.col = M->col; A.D = M->D; A.C = M->C;
   if constexpr (std::is_same_v<T, double>) A.val = M->val;
   else if constexpr (std::is_same_v<T, float>) A.val = M->val32;
   else A.val = reinterpret_cast<const ff*>(M->valff);
+  if (sc.val) A.val = sc.val;
   constexpr int SW = step_warps<T>();
   const int64_t rows_per_block = (int64_t)SW * L::RPW;
   const unsigned grid = (unsigned)cdiv(M->D, rows_per_block);
@@ -158,15 +191,16 @@ fd_status launch_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<
 }
 
 template <typename T>
-fd_status step_dispatch(fd_ctx* ctx, const fd_matrix* M, int nb, int mode, const StepArgs<T>& s) {
+fd_status step_dispatch(fd_ctx* ctx, const fd_matrix* M, int nb, int mode, const StepArgs<T>& s,
+                        const Scaled<T>& sc = {}) {
   switch (nb) {
-    case 2: if constexpr (sizeof(T) == 8) return launch_step<T, 2>(ctx, M, mode, s); break;
-    case 4: return launch_step<T, 4>(ctx, M, mode, s);
-    case 8: return launch_step<T, 8>(ctx, M, mode, s);
-    case 16: return launch_step<T, 16>(ctx, M, mode, s);
-    case 32: return launch_step<T, 32>(ctx, M, mode, s);
-    case 64: return launch_step<T, 64>(ctx, M, mode, s);
-    case 128: return launch_step<T, 128>(ctx, M, mode, s);
+    case 2: if constexpr (sizeof(T) == 8) return launch_step<T, 2>(ctx, M, mode, s, sc); break;
+    case 4: return launch_step<T, 4>(ctx, M, mode, s, sc);
+    case 8: return launch_step<T, 8>(ctx, M, mode, s, sc);
+    case 16: return launch_step<T, 16>(ctx, M, mode, s, sc);
+    case 32: return launch_step<T, 32>(ctx, M, mode, s, sc);
+    case 64: return launch_step<T, 64>(ctx, M, mode, s, sc);
+    case 128: return launch_step<T, 128>(ctx, M, mode, s, sc);
     default: break;
   }
   return set_err(ctx, FD_ERR_ARG, "unsupported nb %d", nb);
@@ -187,11 +221,68 @@ fd_status permute(fd_ctx* ctx, const fd_matrix* M, const T* src, int64_t lds, T*
   return FD_OK;
 }
 
+// Shortest filter whose matrix is scaled first: the pass over the entries costs
+// about 5 us on a small matrix, a step gains 1 us there and a fifth of its time on
+// a large one.
+constexpr int SCALE_MIN_DEGREE = 12;
+
+// A' = 2 (alpha A + beta) in a buffer of the context, for FP64 and float-float
+// filters; left empty (the steps then scale their sums) for short ones, where the
+// buffer is refused, and under stream capture (a graph replays after the buffer has
+// been rewritten or has grown).  The buffer outlives the call: one on another stream
+// first waits for the steps that still read it (scale_done).
+template <typename T>
+fd_status scale_matrix(fd_ctx* ctx, const fd_matrix* M, int n, double alpha, double beta, Scaled<T>* out) {
+  if (sizeof(T) != 8 || n < SCALE_MIN_DEGREE) return FD_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return FD_OK;
+  }
+  const double a2 = 2 * alpha, b2 = 2 * beta;
+  void* p;
+  const int64_t count = M->kron ? M->khops[0] + M->khops[1] + 25 : M->nnz_sell;
+  if (workspace(ctx, "filter_scaled", sizeof(T) * (size_t)count, &p) != FD_OK) {
+    ctx->err.clear();
+    return FD_OK;
+  }
+  if (!ctx->scaled_read) FD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->scaled_read, cudaEventDisableTiming));
+  else if (ctx->scaled_stream != ctx->stream) FD_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->scaled_read, 0));
+  T* v = (T*)p;
+  if (!M->kron) {
+    const int64_t rows = M->n_chunks * M->C;
+    k_scale_sell<T><<<(unsigned)cdiv(rows, 256), 256, 0, ctx->stream>>>(M->chunk_ptr, M->val, rows, M->C, a2, b2, v);
+    FD_LAUNCHED(ctx);
+    out->val = v;
+    return FD_OK;
+  }
+  T* dst[3] = {v, v + M->khops[0], v + M->khops[0] + M->khops[1]};
+  const double* src[3] = {M->kval[0], M->kval[1], M->kdiag};
+  const int64_t len[3] = {M->khops[0], M->khops[1], 25};
+  for (int i = 0; i < 3; ++i) {
+    if (!len[i]) continue;
+    k_scale_table<T><<<(unsigned)cdiv(len[i], 256), 256, 0, ctx->stream>>>(src[i], len[i], a2, i == 2 ? b2 : 0.0, dst[i]);
+    FD_LAUNCHED(ctx);
+  }
+  out->up = dst[0];
+  out->dn = dst[1];
+  out->diag = dst[2];
+  return FD_OK;
+}
+fd_status scale_done(fd_ctx* ctx) {
+  ctx->scaled_stream = ctx->stream;
+  FD_CUDA(ctx, cudaEventRecord(ctx->scaled_read, ctx->stream));
+  return FD_OK;
+}
+
 template <typename T>
 fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, int n,
                    const double* mu, double alpha, double beta, T* W1, T* W2, int64_t ldw,
                    double* bytes_out) {
   const bool ident = M->identity != 0;
+  Scaled<T> sc;
+  FD_TRY(scale_matrix<T>(ctx, M, n, alpha, beta, &sc));
+  const int scaled = sc.on() ? 1 : 0;
   StepArgs<T> s{};
   // x0 location
   T* x0 = V;
@@ -204,8 +295,8 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
   // step 1: x1 = A~ x0
   T* x1 = ident ? W1 : W2;
   s.X = x0; s.ldx = ld0; s.Y = x1; s.ldy = ldw;
-  s.c_ax = (T)alpha; s.c_x = (T)beta;
-  FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_SPMMV, s));
+  s.c_ax = (T)(scaled ? 0.5 : alpha); s.c_x = (T)(scaled ? 0.0 : beta);
+  FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_SPMMV, s, sc));
   // step 2: x2 = 2 A~ x1 - x0; acc = mu0 x0 + mu1 x1 + mu2 x2
   T* acc = V;          // accumulator storage (SELL order when not identity)
   int64_t lda = ldv;
@@ -222,7 +313,8 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
     if (ident) { s.Vout = V; s.ldvo = ldv; }
     else { s.Vout = W1; s.ldvo = ldw; }   // final result in SELL order, unpermuted below
   }
-  FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_SECOND, s));
+  s.scaled = scaled;
+  FD_TRY(step_dispatch<T>(ctx, M, nb, MODE_SECOND, s, sc));
   // generic steps: xk = 2 A~ x_{k-1} - x_{k-2}; acc += mu_k xk, three terms at a
   // time.  The reported bytes stay those of Eq. EstimateT (kappa = 5), the
   // algorithm's own count; what a step moves is less (step_terms).
@@ -246,9 +338,11 @@ fd_status filter_t(fd_ctx* ctx, const fd_matrix* M, T* V, int64_t ldv, int nb, i
     } else if (!ident) {
       s.Vout = xpp; s.ldvo = ldw; final_buf = xpp;
     }
-    FD_TRY(step_dispatch<T>(ctx, M, nb, s.nacc ? MODE_GENERIC : MODE_PLAIN, s));
+    s.scaled = scaled;
+    FD_TRY(step_dispatch<T>(ctx, M, nb, s.nacc ? MODE_GENERIC : MODE_PLAIN, s, sc));
     T* t = xp; xp = xpp; xpp = t;
   }
+  if (scaled) FD_TRY(scale_done(ctx));
   if (!ident) {
     if (n == 2) final_buf = W1;
     FD_TRY(permute<T>(ctx, M, final_buf, ldw, V, ldv, nb, false));

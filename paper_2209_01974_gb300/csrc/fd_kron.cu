@@ -531,6 +531,8 @@ fd_status kron_panel_tables(fd_ctx* ctx, fd_matrix* A, double t) {
   for (int64_t u = 0; u < du; ++u) kmax = std::max<int>(kmax, (int)(pu[u + 1] - pu[u]));
   if (kmax > KP_MAX_HOPS) return set_err(ctx, FD_ERR_ARG, "%d up-spin hops exceed %d", kmax, KP_MAX_HOPS);
   A->kmax_up = kmax;
+  A->khops[0] = pu[du];
+  A->khops[1] = pd[dd];
   // hop values: -t for fermion sign +1, +t for -1 (compared as bit patterns)
   const double v0 = -t * 1.0, v1 = -t * -1.0;
   std::vector<uint32_t> ptr32(dd + 1), ent(std::max<int64_t>(pd[dd], 1));

@@ -783,6 +783,7 @@ fd_status fd_destroy(fd_ctx* ctx) {
   for (auto& e : ctx->ws)
     if (e.second.first) cudaFree(e.second.first);
   if (ctx->host_stage) cudaFreeHost(ctx->host_stage);
+  if (ctx->scaled_read) cudaEventDestroy(ctx->scaled_read);
   delete ctx;
   return FD_OK;
 }

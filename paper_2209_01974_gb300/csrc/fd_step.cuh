@@ -128,6 +128,8 @@ struct StepArgs {
   T mu0, mu1, mu2;           // SECOND: Vout = mu0 z + mu1 x + mu2 y; GENERIC: Vout = Vin + [mu0 z +]
                              // [mu1 x +] mu2 y, the last nacc (1 .. 3) of the terms, or no accumulation (0)
   int nacc;
+  int scaled;                // the matrix is A' = c_ax A + c_x I: c_ax, c_x are not applied again
+
 };
 
 template <int MODE, typename S>
@@ -206,14 +208,21 @@ struct RowHead {
   }
 };
 
-// Gather-accumulate s = sum_j a_ij x_j over the SELL row, returning the row's
-// own vector xi (entry 0 is the diagonal).  Entries are taken BATCH at a time:
+// FP64 and float-float steps sum a row as (sum_{j > 0} a_ij x_j) + (a_ii x_i - z):
+// with the matrix scaled beforehand that is the whole of x_k, in nnz + 1 operations
+// instead of nnz + 4 on the pipes that bound these steps, at the same rounding
+// error (see fd_small.cuh).
+template <typename T, int MODE>
+__host__ __device__ constexpr bool split_diagonal() { return sizeof(T) == 8 && MODE != MODE_SPMMV; }
+
+// Gather-accumulate s = sum_j a_ij x_j over the SELL row (SPLIT: without the
+// diagonal), returning the row's own vector xi (entry 0 is the diagonal).  Entries are taken BATCH at a time:
 // the matrix loads of a batch, then all its gathers, so a row of up to BATCH
 // entries costs one round trip of dependent loads.  Chunk lengths are padded to
 // a multiple of BATCH with (0, own row) entries, so the matrix loads need no
 // bounds; the gathers and FMAs of entries past the row's own length are
 // skipped (FP64 arithmetic, not memory, bounds the FP64 step on GB300).
-template <typename T, int NB>
+template <typename T, int NB, bool SPLIT = false>
 __device__ __forceinline__ void row_product(const RowHead<T>& h, const T* X, int64_t ldx, int len, int wlen,
                                             int gl, V16<T> (&acc)[Layout<T, NB>::CPL],
                                             V16<T> (&xi)[Layout<T, NB>::CPL]) {
@@ -225,7 +234,7 @@ __device__ __forceinline__ void row_product(const RowHead<T>& h, const T* X, int
   for (int v = 0; v < L::CPL; ++v) {
     xi[v].ld(xl + (uint64_t)(uint32_t)h.c[0] * ld + v * L::G * E);
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[v].v[e] = h.a[0] * xi[v].v[e];
+    for (int e = 0; e < E; ++e) acc[v].v[e] = SPLIT ? T(0) : h.a[0] * xi[v].v[e];
   }
 #pragma unroll
   for (int u = 1; u < BATCH; ++u) {
@@ -302,9 +311,9 @@ __device__ __forceinline__ void prefetch_rows(const SellArgs<T>& A, const StepAr
   }
 }
 
-// x_k of one row from its product, and the accumulator
+// x_k of one row from its product (and its diagonal entry a0), and the accumulator
 template <typename T, int NB, int MODE>
-__device__ __forceinline__ void step_epilogue(const StepArgs<T>& s, int64_t row, int gl,
+__device__ __forceinline__ void step_epilogue(const StepArgs<T>& s, int64_t row, int gl, T a0,
                                               const V16<T> (&acc)[Layout<T, NB>::CPL],
                                               const V16<T> (&xi)[Layout<T, NB>::CPL],
                                               const V16<T> (&z)[Layout<T, NB>::CPL],
@@ -321,7 +330,18 @@ __device__ __forceinline__ void step_epilogue(const StepArgs<T>& s, int64_t row,
       y.st(s.Y + row * s.ldy + off);
     } else {
 #pragma unroll
-      for (int e = 0; e < E; ++e) y.v[e] = s.c_ax * acc[v].v[e] + s.c_x * xi[v].v[e] - z[v].v[e];
+      for (int e = 0; e < E; ++e) {
+        if constexpr (split_diagonal<T, MODE>()) {
+          if (s.scaled) {
+            y.v[e] = acc[v].v[e] + fma(a0, xi[v].v[e], -z[v].v[e]);
+          } else {
+            const T ax = acc[v].v[e] + a0 * xi[v].v[e];
+            y.v[e] = s.c_ax * ax + s.c_x * xi[v].v[e] - z[v].v[e];
+          }
+        } else {
+          y.v[e] = s.c_ax * acc[v].v[e] + s.c_x * xi[v].v[e] - z[v].v[e];
+        }
+      }
       if (accumulates<MODE>(s)) {
         V16<T> o;
         if (MODE == MODE_SECOND) {
@@ -374,10 +394,10 @@ __device__ __forceinline__ void cheb_rows(const SellArgs<T>& A, const StepArgs<T
     }
   }
   V16<T> acc[L::CPL], xi[L::CPL];
-  row_product<T, NB>(h, s.X, s.ldx, len, wlen, gl, acc, xi);
+  row_product<T, NB, split_diagonal<T, MODE>()>(h, s.X, s.ldx, len, wlen, gl, acc, xi);
   if (!active) return;
 
-  step_epilogue<T, NB, MODE>(s, row, gl, acc, xi, z, vin);
+  step_epilogue<T, NB, MODE>(s, row, gl, h.a[0], acc, xi, z, vin);
 }
 
 // ---------------------------------------------------------------------------
@@ -408,10 +428,10 @@ struct KronArgs {
 // down hops, the up hops to u' > u), so the sums round as in the SELL kernel.
 // Hops are taken BATCH at a time, as in row_product: the table loads of a
 // batch, then its gathers.
-template <typename T, int NB>
+template <typename T, int NB, bool SPLIT>
 __device__ __forceinline__ void kron_row_product(const KronArgs<T>& K, const T* X, int64_t ldx,
                                                  int64_t row, int gl, V16<T> (&acc)[Layout<T, NB>::CPL],
-                                                 V16<T> (&xi)[Layout<T, NB>::CPL]) {
+                                                 V16<T> (&xi)[Layout<T, NB>::CPL], T* diag) {
   using L = Layout<T, NB>;
   constexpr int E = L::E;
   const T* xl = X + gl * E;
@@ -423,8 +443,9 @@ __device__ __forceinline__ void kron_row_product(const KronArgs<T>& K, const T* 
   for (int v = 0; v < L::CPL; ++v) {
     xi[v].ld(xl + row * ldx + v * L::G * E);
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[v].v[e] = dg * xi[v].v[e];
+    for (int e = 0; e < E; ++e) acc[v].v[e] = SPLIT ? T(0) : dg * xi[v].v[e];
   }
+  *diag = dg;
   // entries [k, ke) of one table
   auto hops = [&](const int32_t* col, const T* val, int64_t k, int64_t ke, int64_t r0, int64_t rs) {
     for (; k < ke; k += BATCH) {
@@ -483,8 +504,9 @@ __device__ __forceinline__ void kron_rows(const KronArgs<T>& K, const StepArgs<T
     }
   }
   V16<T> acc[L::CPL], xi[L::CPL];
-  kron_row_product<T, NB>(K, s.X, s.ldx, row, gl, acc, xi);
-  step_epilogue<T, NB, MODE>(s, row, gl, acc, xi, z, vin);
+  T dg;
+  kron_row_product<T, NB, split_diagonal<T, MODE>()>(K, s.X, s.ldx, row, gl, acc, xi, &dg);
+  step_epilogue<T, NB, MODE>(s, row, gl, dg, acc, xi, z, vin);
 }
 
 }  // namespace step

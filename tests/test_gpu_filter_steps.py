@@ -114,3 +114,68 @@ def test_steps_split_over_launches(n, prec):
     # the errors of the steps add up like sqrt(n) (their signs vary); 40 sqrt(n) u |ref|
     u = U64 if prec == "f64" else U32
     assert np.linalg.norm(V.cpu().numpy() - ref) <= 40 * np.sqrt(n) * u * np.linalg.norm(V0)
+
+
+def _filter_case(fd, ctx, spec, n, dtype, seed, alpha=None):
+    import torch
+    A = fd.fd_build_matrix(ctx, spec)
+    csr = mat.build(spec.replace(",kron=1", ""))
+    lo, hi = lanczos.gershgorin(csr)
+    alpha, beta = ch.scale_params(lo - 0.01, hi + 0.01)
+    mu = np.random.default_rng(seed).uniform(0.5, 1.0, n + 1) / (n + 1)
+    V0 = fd_inputs.random_block(len(csr[0]) - 1, 8, seed)
+    V = torch.from_numpy(V0).cuda()
+    ref = ch.cheb_filter(mat.to_scipy(csr), V0, mu, alpha, beta)
+    return A, V, mu, alpha, beta, torch.empty_like(V), torch.empty_like(V), ref, \
+        filter_tolerance(csr, mu, alpha, beta, V0, U64)
+
+
+LARGE = "anderson3d:L=34,W=3,seed=5"     # 39,304 rows: launched steps
+
+
+@pytest.mark.parametrize("spec", [LARGE, "hubbard:n_sites=7,n_up=3,n_dn=4,t=1,U=4,bc=periodic,kron=1"])
+def test_scaled_matrix_refused_or_captured(spec):
+    """A filter without its scaled-matrix buffer (workspace cap, stream capture)
+    gives the same result to rounding."""
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    A, V, mu, alpha, beta, W1, W2, ref, tol = _filter_case(fd, ctx, spec, 14, torch.float64, 3)
+    V0 = V.clone()
+    fd.fd_filter(ctx, A, V, mu, alpha, beta, W1, W2)
+    assert np.all(np.abs(V.cpu().numpy() - ref) <= tol)
+    ctx2 = fd.fd_create(0)
+    fd.fd_set_workspace_limit(ctx2, 8)
+    V.copy_(V0)
+    fd.fd_filter(ctx2, A, V, mu, alpha, beta, W1, W2)
+    assert np.all(np.abs(V.cpu().numpy() - ref) <= tol)
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        fd.fd_set_stream(ctx, s.cuda_stream)
+        V.copy_(V0)
+        with torch.cuda.graph(g, stream=s):
+            fd.fd_filter(ctx, A, V, mu, alpha, beta, W1, W2)
+        g.replay()
+    torch.cuda.synchronize()
+    assert np.all(np.abs(V.cpu().numpy() - ref) <= tol)
+
+
+def test_filters_of_one_context_on_two_streams():
+    """Two matrices and scalings through one context, its stream changed between
+    the calls without waiting: the scaled-matrix buffer is not overwritten early."""
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    a = _filter_case(fd, ctx, LARGE, 60, torch.float64, 1)
+    b = _filter_case(fd, ctx, "anderson3d:L=33,W=9,seed=8", 60, torch.float64, 2)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    for (A, V, mu, alpha, beta, W1, W2, _, _), s in zip((a, b), streams):
+        fd.fd_set_stream(ctx, s.cuda_stream)
+        fd.fd_filter(ctx, A, V, mu, alpha, beta, W1, W2)
+    torch.cuda.synchronize()
+    for c in (a, b):
+        assert np.all(np.abs(c[1].cpu().numpy() - c[7]) <= c[8])
