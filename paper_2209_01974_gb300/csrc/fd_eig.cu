@@ -7,8 +7,8 @@
 // result of the one before it.  Elementwise rounds pay a grid barrier, two L2 round
 // trips and the slow FP64 division and square roots of the angles n - 1 times a
 // sweep (7 us a round).  Here a round pairs blocks instead of columns:
-//   phase 1  one group of 128 threads per pair of blocks loads its 16 x 16
-//            principal submatrix, rotates the 64 pairs across the two blocks in 8
+//   phase 1  one CTA per pair of blocks loads its 16 x 16 principal submatrix,
+//            rotates the 64 pairs across the two blocks in 8
 //            inner rounds in shared memory (in the first round of a sweep all 120
 //            pairs in 15), and leaves the product J of the rotations;
 //   phase 2  A <- J^T A J block by block (upper half, mirrored) and Q <- Q J as
@@ -23,8 +23,9 @@
 // sum is within 2e-7 of 1, the third term below 1e-20), which makes the rotation
 // orthogonal to FP64 rounding.
 // Measured (device time, Rayleigh quotients, elementwise cyclic Jacobi -> this):
-// n = 128 7.06 -> 2.6 ms, n = 96 4.14 -> 1.67 ms, n = 20 0.79 -> 0.47 ms; twelve
-// instances of n = 64 in a batch 6.17 (one CTA each) -> 1.5 ms.
+// n = 128 7.06 -> 2.1 ms, n = 96 4.14 -> 1.6 ms, n = 32 0.38 ms; twelve instances
+// of n = 64 in a batch 6.17 (one CTA each) -> 1.3 ms.  Of the 14 us of a round
+// (n = 128) the eight inner rounds take 7, phase 2 and its loads 3, the barriers 3.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -44,6 +45,7 @@ constexpr int BB = 2 * B;         // pair width
 constexpr int GROUP = 128;        // threads of a task group
 constexpr int GROUPS = 2;         // groups per CTA
 constexpr int EIG_THREADS = GROUP * GROUPS;
+static_assert(EIG_THREADS == BB * BB && GROUPS == 2, "phase 1 gives each thread one element");
 
 struct EigArgs {
   EigTask one;           // n_inst = 1 and many = nullptr: this matrix
@@ -80,6 +82,17 @@ __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;\n" ::"r"(g + 1), "n"(GROUP) : "memory");
 }
 
+__device__ __forceinline__ float approx_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float approx_rsqrt(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // rotation that (nearly) annihilates a_pq: (c, s) orthogonal to FP64 rounding
 __device__ __forceinline__ void angle(double app, double aqq, double apq, double* c, double* s) {
   const float d = (float)(aqq - app), o = 2.0f * (float)apq;
@@ -92,11 +105,11 @@ __device__ __forceinline__ void angle(double app, double aqq, double apq, double
     return;
   }
   // t = tan(phi) = sgn(d o) |o| / (|d| + sqrt(d^2 + o^2)); scaled against underflow of the squares
-  const float big = fmaxf(fabsf(d), fabsf(o)), rb = 1.0f / big;
-  const float dd = fabsf(d) * rb, oo = o * rb;
-  float t = oo / (dd + sqrtf(fmaf(dd, dd, oo * oo)));
+  const float rb = approx_rcp(fmaxf(fabsf(d), fabsf(o)));
+  const float dd = fabsf(d) * rb, oo = o * rb, h = fmaf(dd, dd, oo * oo);  // h in [1, 2]
+  float t = oo * approx_rcp(fmaf(h, approx_rsqrt(h), dd));
   if (d < 0.0f) t = -t;
-  const float cf = rsqrtf(fmaf(t, t, 1.0f)), sf = t * cf;
+  const float cf = approx_rsqrt(fmaf(t, t, 1.0f)), sf = t * cf;
   const double c0 = (double)cf, s0 = (double)sf;
   const double e = fma(s0, s0, fma(c0, c0, -1.0));           // exact to 1e-16
   const double f = fma(e, fma(e, 0.375, -0.5), 1.0);          // (1 + e)^(-1/2)
@@ -118,7 +131,9 @@ __global__ void __launch_bounds__(EIG_THREADS) k_block_jacobi(EigArgs a) {
   unsigned char* done = dyn;
   unsigned char* cur = dyn + a.n_inst;
   const int g = threadIdx.x / GROUP, t = threadIdx.x % GROUP;
-  const int gid = blockIdx.x * GROUPS + g, ngroups = gridDim.x * GROUPS;
+  // a group's first task: all CTAs get one before any gets a second (the FP64
+  // pipes of an SM are shared by its groups)
+  const int spread = blockIdx.x + g * gridDim.x, ngroups = gridDim.x * GROUPS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t gt = (int64_t)blockIdx.x * EIG_THREADS + threadIdx.x, gn = (int64_t)gridDim.x * EIG_THREADS;
   for (int i = threadIdx.x; i < a.n_inst; i += EIG_THREADS) {
@@ -233,9 +248,11 @@ __global__ void __launch_bounds__(EIG_THREADS) k_block_jacobi(EigArgs a) {
     }
     if (!__syncthreads_or(left)) break;
     for (int r = 0; r < a.m_max - 1; ++r) {
-      // phase 1: rotations of every pair of blocks
+      // phase 1: rotations of every pair of blocks, one pair per CTA.  The first group
+      // finds the angles and rotates A; the second accumulates J from the angles of
+      // the inner round while the first is at the next one's.
       const int half_max = a.m_max / 2;
-      for (int w = gid; w < half_max * a.n_inst; w += ngroups) {
+      for (int w = blockIdx.x; w < half_max * a.n_inst; w += gridDim.x) {
         const int i = w % a.n_inst, k = w / a.n_inst;
         if (done[i]) continue;
         const EigTask& T = task(a, i);
@@ -244,58 +261,64 @@ __global__ void __launch_bounds__(EIG_THREADS) k_block_jacobi(EigArgs a) {
         const double* A = cur[i] ? T.A1 : T.A0;
         int bp, bq;
         pair_of(r, k, m, &bp, &bq);
-        group_sync(g);  // the previous task's reads are done
-        for (int e = t; e < BB * BB; e += GROUP) {
-          const int x = e / BB, y = e % BB;
+        __syncthreads();  // the previous task's reads are done
+        {
+          const int x = threadIdx.x / BB, y = threadIdx.x % BB;
           const int gx = x < B ? bp * B + x : bq * B + x - B, gy = y < B ? bp * B + y : bq * B + y - B;
-          sA[g][0][x][y] = __ldcg(A + (int64_t)gx * np + gy);
-          sJ[g][x][y] = x == y ? 1.0 : 0.0;
+          sA[0][0][x][y] = __ldcg(A + (int64_t)gx * np + gy);
+          sJ[0][x][y] = x == y ? 1.0 : 0.0;
         }
-        group_sync(g);
+        __syncthreads();
         const int rounds = r == 0 ? BB - 1 : B;
+        // pair j of inner round q
+        auto inner = [&](int q, int j, int* x, int* y) {
+          if (r == 0) {
+            pair_of(q, j, BB, x, y);
+          } else {
+            *x = j;
+            *y = B + ((j + q) & (B - 1));
+          }
+        };
+        const int l = t & (B - 1), rr = t >> 3;  // column pair, row (of 16; for A in pair order)
         int c = 0;
         for (int q = 0; q < rounds; ++q, c ^= 1) {
-          // pair j of this inner round
-          auto inner = [&](int j, int* x, int* y) {
-            if (r == 0) {
-              pair_of(q, j, BB, x, y);
-            } else {
-              *x = j;
-              *y = B + ((j + q) & (B - 1));
-            }
-          };
-          if (t < B) {
+          double* cs = sCS[c];
+          if (threadIdx.x < B) {
             int x, y;
-            inner(t, &x, &y);
-            angle(sA[g][c][x][x], sA[g][c][y][y], sA[g][c][x][y], &sCS[g][2 * t], &sCS[g][2 * t + 1]);
+            inner(q, threadIdx.x, &x, &y);
+            angle(sA[0][c][x][x], sA[0][c][y][y], sA[0][c][x][y], cs + 2 * threadIdx.x, cs + 2 * threadIdx.x + 1);
           }
-          group_sync(g);
-          const int l = t & (B - 1), rr = t >> 3;  // column pair, row (of 16) in pair order
-          int px, py, qx, qy;
-          inner(rr >> 1, &px, &py);
-          inner(l, &qx, &qy);
-          const double ck = sCS[g][2 * (rr >> 1)], sk = sCS[g][2 * (rr >> 1) + 1];
-          const double cl = sCS[g][2 * l], sl = sCS[g][2 * l + 1];
-          const double u0 = sA[g][c][px][qx], u1 = sA[g][c][px][qy];
-          const double v0 = sA[g][c][py][qx], v1 = sA[g][c][py][qy];
-          const bool second = rr & 1;
-          const double x0 = second ? sk : ck, x1 = second ? ck : -sk;
-          const double m0 = fma(x1, v0, x0 * u0), m1 = fma(x1, v1, x0 * u1);
-          const int row = second ? py : px;
-          sA[g][c ^ 1][row][qx] = fma(-sl, m1, cl * m0);
-          sA[g][c ^ 1][row][qy] = fma(sl, m0, cl * m1);
-          const double j0 = sJ[g][rr][qx], j1 = sJ[g][rr][qy];
-          sJ[g][rr][qx] = fma(-sl, j1, cl * j0);
-          sJ[g][rr][qy] = fma(sl, j0, cl * j1);
-          group_sync(g);
+          __syncthreads();
+          int qx, qy;
+          inner(q, l, &qx, &qy);
+          const double cl = cs[2 * l], sl = cs[2 * l + 1];
+          if (g == 0) {
+            int px, py;
+            inner(q, rr >> 1, &px, &py);
+            const double ck = cs[2 * (rr >> 1)], sk = cs[2 * (rr >> 1) + 1];
+            const double u0 = sA[0][c][px][qx], u1 = sA[0][c][px][qy];
+            const double v0 = sA[0][c][py][qx], v1 = sA[0][c][py][qy];
+            const bool second = rr & 1;
+            const double x0 = second ? sk : ck, x1 = second ? ck : -sk;
+            const double m0 = fma(x1, v0, x0 * u0), m1 = fma(x1, v1, x0 * u1);
+            const int row = second ? py : px;
+            sA[0][c ^ 1][row][qx] = fma(-sl, m1, cl * m0);
+            sA[0][c ^ 1][row][qy] = fma(sl, m0, cl * m1);
+            group_sync(0);
+          } else {
+            const double j0 = sJ[0][rr][qx], j1 = sJ[0][rr][qy];
+            sJ[0][rr][qx] = fma(-sl, j1, cl * j0);
+            sJ[0][rr][qy] = fma(sl, j0, cl * j1);
+            group_sync(1);
+          }
         }
-        for (int e = t; e < BB * BB; e += GROUP)
-          __stcg(T.J + (int64_t)k * BB * BB + e, sJ[g][e / BB][e % BB]);
+        __syncthreads();
+        __stcg(T.J + (int64_t)k * BB * BB + threadIdx.x, sJ[0][threadIdx.x / BB][threadIdx.x % BB]);
       }
       grid.sync();
       // phase 2: A <- J^T A J (half a 16 x 16 block per task) and Q <- Q J (8 rows)
       const int a_max = half_max * (half_max + 1), q_max = a.m_max * half_max;
-      for (int64_t w = gid; w < (int64_t)(a_max + q_max) * a.n_inst; w += ngroups) {
+      for (int64_t w = spread; w < (int64_t)(a_max + q_max) * a.n_inst; w += ngroups) {
         const int i = (int)(w % a.n_inst);
         int k = (int)(w / a.n_inst);
         if (done[i]) continue;
@@ -405,7 +428,7 @@ __global__ void __launch_bounds__(EIG_THREADS) k_block_jacobi(EigArgs a) {
 
 int eig_grid(const fd_ctx* ctx, int n_inst, int m_max) {
   const int64_t half = m_max / 2, tasks = (half * (half + 1) + m_max * half) * n_inst;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(tasks, GROUPS), ctx->num_sms));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(tasks, ctx->num_sms));
 }
 
 fd_status launch(fd_ctx* ctx, EigArgs& a, int grid) {
