@@ -23,6 +23,7 @@
 #include "fd_step.cuh"
 #include "fd_ff.cuh"
 #include "fd_eig.cuh"
+#include "fd_small.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -51,7 +52,7 @@ struct BInst {
   double* resid;  // ns
   double* rpart;  // residual partials: RBLK x ns
   int ns;
-  int pad;
+  int max_row;    // longest row of the matrix
 };
 
 struct BParams {  // rewritten by the host before every outer iteration
@@ -297,6 +298,51 @@ __global__ void __launch_bounds__(FF ? BF_FF_WARPS * 32 : WARPS * 32, FF ? BF_FF
       }
     }
     if (!b.spmmv_only) grid.sync();
+  }
+}
+
+// The filter of a batch whose matrices are small (fd_small.cuh): a cluster per
+// column panel (one 8-byte unit) takes it through all steps of its own instance's
+// degree, so no step waits for another instance and a late iteration with one
+// instance left costs what that instance costs.  Panels are listed bundle by bundle,
+// largest degree first.
+template <typename T, typename Mu>
+__device__ __forceinline__ void batched_panel(const BInst& I, const BParams& P, T* V, int unit, uint32_t rank,
+                                              uint32_t ranks, unsigned char* smem, Mu&& mu) {
+  small::Block<T> b;
+  b.chunk_ptr = I.A.chunk_ptr; b.row_len = I.A.row_len; b.col = I.A.col; b.val = I.A.val; b.perm = nullptr;
+  b.D = (int)I.A.D; b.C = I.A.C; b.max_row = I.max_row;
+  b.V = V; b.ldv = I.ns;
+  b.X[0] = b.X[1] = nullptr; b.ldw = 0;  // one launch takes all steps
+  b.a2 = 2 * P.alpha; b.b2 = 2 * P.beta;
+  b.n = P.degree; b.k0 = 1; b.k1 = P.degree;
+  small::filter_panel<T, 1, true>(b, unit, rank, ranks, smem, mu);
+}
+__global__ void __launch_bounds__(1024, 1) k_batched_small(BatchArgs b) {
+  extern __shared__ __align__(16) unsigned char bs_smem[];
+  uint32_t rank, ranks;
+  asm("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(ranks));
+  const int panel = (int)(blockIdx.x / ranks), t = panel / b.nb, u = panel % b.nb;
+  // the whole cluster leaves together
+  if (t >= *b.n_tasks) return;
+  const BTask tk = b.task[t];
+  const BInst& I = b.inst[tk.inst];
+  const BParams& P = b.par[tk.inst];
+  if (!P.active || P.degree == 0) return;
+  const double* mu = b.mu + P.mu_off;
+  if (P.f32) {
+    if (u >= b.nb / 2) return;
+    const float2* m = reinterpret_cast<const float2*>(mu);
+    batched_panel<float>(I, P, I.V32, tk.bundle * b.nb / 2 + u, rank, ranks, bs_smem, [&](int k) { return __ldg(m + k).x; });
+  } else if (P.ff) {
+    const float2* m = reinterpret_cast<const float2*>(mu);
+    batched_panel<ff>(I, P, reinterpret_cast<ff*>(I.V), tk.bundle * b.nb + u, rank, ranks, bs_smem, [&](int k) {
+      const float2 v = __ldg(m + k);
+      return ff(v.x, v.y);
+    });
+  } else {
+    batched_panel<double>(I, P, I.V, tk.bundle * b.nb + u, rank, ranks, bs_smem, [&](int k) { return __ldg(mu + k); });
   }
 }
 
@@ -583,6 +629,9 @@ struct Batch {
   int grid = 0;
   int grid_rr = 0, warps_rr = WARPS;  // the Rayleigh-Ritz SpMMV launch (FP64 rows)
   size_t smem_filter = 0;
+  // the one-launch filter of small matrices: CTAs per cluster (0: not used), threads, shared memory
+  int small_cluster = 0, small_threads = 0;
+  size_t small_smem = 0;
   cudaGraphExec_t exec = nullptr;
   int64_t max_D = 0;
 
@@ -672,6 +721,7 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
     I.Aff.chunk_ptr = M->chunk_ptr; I.Aff.row_len = M->row_len; I.Aff.col = M->col;
     I.Aff.val = reinterpret_cast<const ff*>(M->valff); I.Aff.D = M->D; I.Aff.C = M->C;
     I.ns = ns[i];
+    I.max_row = M->max_row;
     const int64_t D = M->D;
     const size_t nn = (size_t)ns[i] * ns[i];
     double* p = (double*)((char*)B.arena + off[i]);
@@ -762,6 +812,27 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
   FD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, B.warps * 32, B.smem_filter));
   if (per_sm < 1) return set_err(ctx, FD_ERR_ARG, "batched filter does not fit on an SM");
   B.grid = per_sm * ctx->num_sms;
+  // Every matrix small enough for a cluster's shared memory: panels instead of
+  // grid-wide steps.  Two CTAs per panel at least: with one, a late iteration with
+  // one instance left takes twice as long, while the full batch gains a tenth
+  // (12 instances of L = 10 .. 14, N_s = 64: 82 ms of filter per solve with the
+  // persistent kernel, 18 us a step with one instance left).
+  for (int cl = 2; cl <= 8 && !B.small_cluster; cl *= 2) {
+    bool fits = true;
+    int rows = 0;
+    size_t smem = 0;
+    for (int i = 0; i < n && fits; ++i) {
+      fits = A[i]->D <= small::MAX_ROWS && A[i]->max_row <= small::MAX_ROWS;
+      const int R = fits ? small::cta_rows((int)A[i]->D, cl) : 0;
+      rows = std::max(rows, R);
+      if (fits) smem = std::max(smem, small::cta_smem<double>((int)A[i]->D, R, 1, A[i]->max_row));
+    }
+    if (!fits || smem > ctx->smem_optin - 1024) continue;
+    B.small_cluster = cl;
+    B.small_smem = smem;
+    B.small_threads = std::min(1024, (rows + 31) & ~31);
+    FD_CUDA(ctx, cudaFuncSetAttribute(k_batched_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin));
+  }
   // the SpMMV of the Rayleigh-Ritz step always takes FP64 rows: the FP64
   // instantiation in the tuner's CTA shape
   const void* kr = filter_kernel_for(nb, false);
@@ -796,6 +867,19 @@ fd_status launch_filter(fd_ctx* ctx, Batch& B, int spmmv_only) {
   if (spmmv_only) {
     FD_CUDA(ctx, cudaLaunchKernel(filter_kernel_for(B.nb, false), B.grid_rr, B.warps_rr * 32, args,
                                   B.smem_filter, ctx->stream));
+  } else if (B.small_cluster) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)B.small_cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B.n_tasks_all * B.nb * B.small_cluster));
+    cfg.blockDim = dim3((unsigned)B.small_threads);
+    cfg.dynamicSmemBytes = B.small_smem;
+    cfg.stream = ctx->stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    FD_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_batched_small, a));
   } else {
     FD_CUDA(ctx, cudaLaunchCooperativeKernel(kf, B.grid, B.warps * 32, args, B.smem_filter, ctx->stream));
   }
