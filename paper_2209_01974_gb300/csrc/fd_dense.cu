@@ -176,15 +176,41 @@ __global__ void __launch_bounds__(1024) k_cholesky(const double* G, int n, doubl
   if (threadIdx.x == 0) *ok = fail ? 0 : 1;
 }
 
-// Cooperative version (one CTA per SM): the same right-looking elimination,
-// each step's trailing update spread over the CTAs by rows, one grid barrier
-// per column.  Row k is read unscaled during step k (the update uses
-// R_kj R_ki / d) and scaled by its owner after the barrier, when no CTA reads it
-// any more.  Reads of R bypass L1 (other CTAs wrote them).
-__global__ void __launch_bounds__(256) k_cholesky_coop(const double* G, int n, double coeff, double* R,
-                                                       int* ok) {
+// ---------------------------------------------------------------------------
+// Cooperative blocked version: panels of 8 rows, one grid barrier per panel.
+//
+// The chain of pivots bounds it (an FP64 reciprocal square root and an update per
+// column, 0.4 us), so what a panel adds to it is kept short: every CTA loads the
+// panel's rows, factors the 8 x 8 diagonal block in one warp's registers and solves
+// the panel into its shared memory by itself (the same values everywhere), and
+// only the trailing update is divided (rows over CTAs).  The panel's finished rows
+// are written after the barrier, when no CTA reads the unfinished ones any more.
+// One barrier per column instead took 440 us at n = 128, 1.61 ms at n = 384;
+// this takes 122 us and 0.47 ms.
+// ---------------------------------------------------------------------------
+constexpr int CB = 8;  // panel rows
+
+// 1 / sqrt(d), d > 0 finite: an FP32 estimate of the scaled value and one
+// third-order step in FP64
+__device__ __forceinline__ double rsqrt64(double d) {
+  const long long bits = __double_as_longlong(d);
+  int ex = (int)((bits >> 52) & 0x7FF) - 1023;
+  if (ex == -1023) return 1.0 / sqrt(d);  // subnormal
+  ex &= ~1;
+  const double m = __longlong_as_double(bits - ((long long)ex << 52));  // in [1, 4)
+  const double y = (double)rsqrtf((float)m);
+  const double e = fma(-m * y, y, 1.0);
+  const double r = fma(y * e, fma(0.375, e, 0.5), y);
+  return __longlong_as_double(__double_as_longlong(r) - ((long long)(ex / 2) << 52));
+}
+
+__global__ void __launch_bounds__(256) k_cholesky_coop(const double* G, int n, double coeff, double* R, int* ok) {
   cg::grid_group grid = cg::this_grid();
+  extern __shared__ double sP[];  // 2 x CB x n: the panel's finished rows, by panel parity
   __shared__ double red[256];
+  __shared__ double sD[CB][CB + 1], sR[CB];
+  __shared__ int sfail;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double tr = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) tr += G[(int64_t)i * n + i];
   red[threadIdx.x] = tr;
@@ -196,51 +222,129 @@ __global__ void __launch_bounds__(256) k_cholesky_coop(const double* G, int n, d
   const double shift = coeff * red[0];
   for (int i = blockIdx.x; i < n; i += gridDim.x)
     for (int j = threadIdx.x; j < n; j += blockDim.x)
-      R[(int64_t)i * n + j] = j >= i ? G[(int64_t)i * n + j] + (i == j ? shift : 0.0) : 0.0;
+      __stcg(R + (int64_t)i * n + j, j >= i ? G[(int64_t)i * n + j] + (i == j ? shift : 0.0) : 0.0);
   grid.sync();
   bool fail = false;
-  for (int k = 0; k < n; ++k) {
-    const double d = __ldcg(R + (int64_t)k * n + k);
-    if (!(d > 0.0) || !isfinite(d)) {  // the same value in every CTA: all stop here
+  for (int k0 = 0, panel = 0; k0 < n; k0 += CB, ++panel) {
+    const int kb = min(CB, n - k0);
+    double* P = sP + (panel & 1) * CB * n;
+    // the diagonal block: lane (i, j) of warp 0 holds elements (i, j) and (i + 4, j)
+    if (warp == 0) {
+      const int i = lane >> 3, j = lane & 7;
+      double v[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = i + 4 * h;
+        v[h] = r < kb && j < kb && j >= r ? __ldcg(R + (int64_t)(k0 + r) * n + k0 + j) : (r == j ? 1.0 : 0.0);
+      }
+      bool bad = false;
+#pragma unroll
+      for (int p = 0; p < CB; ++p) {
+        const double d = __shfl_sync(0xffffffffu, v[p >> 2], (p & 3) * 8 + p);
+        if (!(d > 0.0) || !isfinite(d)) bad = true;
+        const double ri = rsqrt64(bad ? 1.0 : d);
+        if (i == (p & 3)) v[p >> 2] = j == p ? d * ri : v[p >> 2] * ri;
+        const double rj = __shfl_sync(0xffffffffu, v[p >> 2], (p & 3) * 8 + j);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const double rr = __shfl_sync(0xffffffffu, v[p >> 2], (p & 3) * 8 + i + 4 * h);
+          if (i + 4 * h > p && j >= i + 4 * h) v[h] = fma(-rr, rj, v[h]);
+        }
+        if (lane == 0) sR[p] = ri;
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) sD[i + 4 * h][j] = v[h];
+      if (lane == 0) sfail = bad;
+    }
+    __syncthreads();
+    if (sfail) {  // the same in every CTA: all stop here
       fail = true;
       break;
     }
-    const double inv = 1.0 / d;
-    const double* rk = R + (int64_t)k * n;
-    for (int i = k + 1 + blockIdx.x; i < n; i += gridDim.x) {
-      const double a = __ldcg(rk + i) * inv;
+    // the panel's other columns: R_kk^T x = g
+    for (int j = k0 + threadIdx.x; j < n; j += blockDim.x) {
+      double x[CB];
+#pragma unroll
+      for (int p = 0; p < CB; ++p) x[p] = p < kb && j >= k0 + CB ? __ldcg(R + (int64_t)(k0 + p) * n + j) : 0.0;
+#pragma unroll
+      for (int p = 0; p < CB; ++p) {
+#pragma unroll
+        for (int q = 0; q < p; ++q) x[p] = fma(-sD[q][p], x[q], x[p]);
+        x[p] *= sR[p];
+      }
+#pragma unroll
+      for (int p = 0; p < CB; ++p) P[p * n + j] = j < k0 + CB ? (j - k0 >= p ? sD[p][j - k0] : 0.0) : x[p];
+    }
+    __syncthreads();
+    // trailing rows of this CTA
+    for (int i = k0 + CB + blockIdx.x; i < n; i += gridDim.x) {
       double* ri = R + (int64_t)i * n;
-      for (int j = i + threadIdx.x; j < n; j += blockDim.x) ri[j] -= a * __ldcg(rk + j);
+      for (int j = i + threadIdx.x; j < n; j += blockDim.x) {
+        double v = __ldcg(ri + j);
+#pragma unroll
+        for (int p = 0; p < CB; ++p) v = fma(-P[p * n + i], P[p * n + j], v);
+        __stcg(ri + j, v);
+      }
     }
     grid.sync();
-    if (k % gridDim.x == blockIdx.x) {
-      const double r = sqrt(d), rinv = 1.0 / r;
-      double* rw = R + (int64_t)k * n;
-      for (int j = k + 1 + threadIdx.x; j < n; j += blockDim.x) rw[j] *= rinv;
-      if (threadIdx.x == 0) rw[k] = r;
-    }
+    if (panel % gridDim.x == blockIdx.x)
+      for (int e = threadIdx.x; e < kb * (n - k0); e += blockDim.x) {
+        const int p = e / (n - k0), j = k0 + e % (n - k0);
+        if (j >= k0 + p) R[(int64_t)(k0 + p) * n + j] = P[p * n + j];
+      }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *ok = fail ? 0 : 1;
 }
 
 // ---------------------------------------------------------------------------
-// triangular inverse: X = R^-1 (upper), one warp per column
+// triangular inverse: X = R^-1 (upper).  One CTA takes 8 columns from their
+// diagonal block upwards in blocks of 8 rows: S = I - R X over the rows below (64
+// sums, split four ways over the row index), then back substitution inside the
+// block.  A warp per column, one row at a time with a warp-wide FP64 reduction
+// each, took 184 us at n = 128 and 0.70 ms at n = 384; this takes 66 us and 0.36 ms.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_tri_inverse(const double* R, int n, double* X) {
-  extern __shared__ double xs[];  // 8 warps x n
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j = blockIdx.x * 8 + w;
-  if (j >= n) return;
-  double* x = xs + (int64_t)w * n;
-  for (int i = j; i >= 0; --i) {
+  extern __shared__ double xs[];  // n x 8: the finished rows of the 8 columns
+  __shared__ double part[4][64];
+  __shared__ double S[CB][CB + 1], inv[CB];
+  const int c0 = blockIdx.x * CB;
+  const int i = (threadIdx.x >> 3) & 7, c = threadIdx.x & 7, slice = threadIdx.x >> 6;
+  const int last = min(n, c0 + CB);  // rows at or beyond `last` are zero
+  for (int r0 = c0; r0 >= 0; r0 -= CB) {
     double s = 0.0;
-    for (int k = i + 1 + lane; k <= j; k += 32) s = fma(R[(int64_t)i * n + k], x[k], s);
+    if (r0 + i < n)
+      for (int k = r0 + CB + slice; k < last; k += 4) s = fma(__ldg(R + (int64_t)(r0 + i) * n + k), xs[k * CB + c], s);
+    part[slice][i * CB + c] = s;
+    __syncthreads();
+    if (slice == 0) {
+      const int e = i * CB + c;
+      S[i][c] = (r0 + i == c0 + c ? 1.0 : 0.0) - ((part[0][e] + part[1][e]) + (part[2][e] + part[3][e]));
+    } else if (threadIdx.x < 64 + CB && r0 + threadIdx.x - 64 < n) {  // an FP64 division takes as long as the rest of a row
+      inv[threadIdx.x - 64] = 1.0 / __ldg(R + (int64_t)(r0 + threadIdx.x - 64) * n + r0 + threadIdx.x - 64);
+    }
+    __syncthreads();
+    if (threadIdx.x < CB) {  // one column per thread
+      const int col = threadIdx.x, rows = min(CB, n - r0);
+      double x[CB];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) x[i] = ((i == j ? 1.0 : 0.0) - s) / R[(int64_t)i * n + i];
-    __syncwarp();
+      for (int p = CB - 1; p >= 0; --p) {
+        x[p] = 0.0;
+        if (p < rows) {
+          double v = S[p][col];
+#pragma unroll
+          for (int q = p + 1; q < CB; ++q)
+            if (q < rows) v = fma(-__ldg(R + (int64_t)(r0 + p) * n + r0 + q), x[q], v);
+          x[p] = v * inv[p];
+          xs[(r0 + p) * CB + col] = x[p];
+        }
+      }
+    }
+    __syncthreads();
   }
-  for (int i = lane; i < n; i += 32) X[(int64_t)i * n + j] = i <= j ? x[i] : 0.0;
+  for (int e = threadIdx.x; e < n * CB; e += 256) {
+    const int r = e / CB, q = c0 + e % CB;
+    if (q < n) X[(int64_t)r * n + q] = r <= q ? xs[e] : 0.0;
+  }
 }
 
 // C = A * B, n x n (small)
@@ -282,38 +386,68 @@ __global__ void k_resid_reduce(const double* P, int nb, int n, double* out) {
   out[c] = sqrt(s);
 }
 
-__global__ void k_f64_to_f32(const double* s, int64_t lds, float* d, int64_t ldd, int64_t D, int n) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= D * n) return;
-  int64_t i = t / n;
-  int j = (int)(t % n);
-  d[i * ldd + j] = (float)s[i * lds + j];
+// Copies of D x n blocks with a change of type, W elements per thread and row (16
+// or 32 bytes on the wider side) and four rows in flight.  FP64 -> float-float: hi
+// the nearest float, lo the nearest float to the exact FP64 remainder; back, hi +
+// lo is exact in FP64.  One element per thread with a 64-bit division for its row
+// ran at half the copy bandwidth (11.8M x 32, FP64 -> FP32: 1.32 ms, now 0.65).
+struct pair_f { float hi, lo; };
+__device__ __forceinline__ void convert(double v, float& o) { o = __double2float_rn(v); }
+__device__ __forceinline__ void convert(float v, double& o) { o = (double)v; }
+__device__ __forceinline__ void convert(double v, pair_f& o) {
+  o.hi = __double2float_rn(v);
+  o.lo = __double2float_rn(v - (double)o.hi);
 }
-__global__ void k_f32_to_f64(const float* s, int64_t lds, double* d, int64_t ldd, int64_t D, int n) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= D * n) return;
-  int64_t i = t / n;
-  int j = (int)(t % n);
-  d[i * ldd + j] = (double)s[i * lds + j];
+__device__ __forceinline__ void convert(pair_f v, double& o) { o = (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ void convert(double v, double& o) { o = v; }
+__device__ __forceinline__ void convert(float v, float& o) { o = v; }
+
+template <typename T, int W>
+struct alignas(sizeof(T) * W < 16 ? sizeof(T) * W : 16) Pack { T v[W]; };
+
+template <typename S, typename T, int W>
+__global__ void __launch_bounds__(256) k_convert(const S* s, int64_t lds, T* d, int64_t ldd, int64_t D, int n) {
+  constexpr int UNROLL = 4;
+  const unsigned q = (unsigned)n / W, per = q < 256 ? 256 / q : 1;  // threads of a row, rows at once
+  const unsigned r = threadIdx.x / q, c0 = q < 256 ? threadIdx.x - r * q : threadIdx.x;
+  if (q < 256 && r >= per) return;
+  const int64_t row0 = (int64_t)blockIdx.x * per * UNROLL + (q < 256 ? r : 0);
+  for (unsigned c = c0; c < q; c += 256) {
+    Pack<S, W> in[UNROLL];
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      const int64_t row = row0 + (int64_t)u * per;
+      if (row < D) in[u] = *reinterpret_cast<const Pack<S, W>*>(s + row * lds + (int64_t)c * W);
+    }
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      const int64_t row = row0 + (int64_t)u * per;
+      if (row < D) {
+        Pack<T, W> out;
+#pragma unroll
+        for (int e = 0; e < W; ++e) convert(in[u].v[e], out.v[e]);
+        *reinterpret_cast<Pack<T, W>*>(d + row * ldd + (int64_t)c * W) = out;
+      }
+    }
+  }
 }
-// FP64 <-> float-float (element = 2 floats): hi the nearest float, lo the
-// nearest float to the exact FP64 remainder; back, hi + lo is exact in FP64
-__global__ void k_f64_to_ff(const double* s, int64_t lds, float* d, int64_t ldd, int64_t D, int n) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= D * n) return;
-  int64_t i = t / n;
-  int j = (int)(t % n);
-  const double v = s[i * lds + j];
-  const float hi = __double2float_rn(v);
-  *reinterpret_cast<float2*>(d + 2 * (i * ldd + j)) = make_float2(hi, __double2float_rn(v - (double)hi));
+
+template <typename S, typename T, int W>
+bool packs(const S* s, int64_t lds, const T* d, int64_t ldd, int n) {
+  return n % W == 0 && lds % W == 0 && ldd % W == 0 && (uintptr_t)s % alignof(Pack<S, W>) == 0 &&
+         (uintptr_t)d % alignof(Pack<T, W>) == 0;
 }
-__global__ void k_ff_to_f64(const float* s, int64_t lds, double* d, int64_t ldd, int64_t D, int n) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= D * n) return;
-  int64_t i = t / n;
-  int j = (int)(t % n);
-  const float2 v = *reinterpret_cast<const float2*>(s + 2 * (i * lds + j));
-  d[i * ldd + j] = (double)v.x + (double)v.y;
+
+template <typename S, typename T>
+fd_status convert_block(fd_ctx* ctx, const S* s, int64_t lds, T* d, int64_t ldd, int64_t D, int n) {
+  constexpr int W = sizeof(S) == 4 || sizeof(T) == 4 ? 4 : 2;
+  const int w = packs<S, T, W>(s, lds, d, ldd, n) ? W : 1;
+  const int64_t q = n / w, per = q < 256 ? 256 / q : 1;
+  const unsigned grid = (unsigned)cdiv(D, per * 4);
+  if (w == W) k_convert<S, T, W><<<grid, 256, 0, ctx->stream>>>(s, lds, d, ldd, D, n);
+  else k_convert<S, T, 1><<<grid, 256, 0, ctx->stream>>>(s, lds, d, ldd, D, n);
+  FD_LAUNCHED(ctx);
+  return FD_OK;
 }
 
 }  // namespace
@@ -402,19 +536,20 @@ fd_status rotate_fp64(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, con
 }
 
 fd_status cholesky(fd_ctx* ctx, const double* G, int n, double coeff, double* R, int* ok_dev) {
-  if (n >= 64) {  // one CTA per SM, co-resident (cooperative launch)
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cholesky_coop, 256, 0);
-    if (per_sm >= 1) {
-      const int grid = std::min(ctx->num_sms, n);
-      void* args[] = {(void*)&G, (void*)&n, (void*)&coeff, (void*)&R, (void*)&ok_dev};
-      if (cudaLaunchCooperativeKernel((const void*)k_cholesky_coop, grid, 256, args, 0, ctx->stream) ==
-          cudaSuccess) {
-        ctx->launches++;
-        return FD_OK;
-      }
-      cudaGetLastError();  // cooperative launch unavailable: the one-CTA kernel below
+  // two panels or more: one CTA per SM, co-resident (cooperative launch), no more
+  // than there are rows to update
+  const size_t smem = sizeof(double) * 2 * CB * n;
+  if (n > CB && smem <= ctx->smem_optin) {
+    if (smem > 32 * 1024)
+      FD_CUDA(ctx, cudaFuncSetAttribute(k_cholesky_coop, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)(sizeof(double) * 2 * CB * 1024)));
+    const int grid = std::min(ctx->num_sms, n);
+    void* args[] = {(void*)&G, (void*)&n, (void*)&coeff, (void*)&R, (void*)&ok_dev};
+    if (cudaLaunchCooperativeKernel((const void*)k_cholesky_coop, grid, 256, args, smem, ctx->stream) == cudaSuccess) {
+      ctx->launches++;
+      return FD_OK;
     }
+    cudaGetLastError();  // cooperative launch unavailable: the one-CTA kernel below
   }
   k_cholesky<<<1, 1024, 0, ctx->stream>>>(G, n, coeff, R, ok_dev);
   FD_LAUNCHED(ctx);
@@ -422,10 +557,11 @@ fd_status cholesky(fd_ctx* ctx, const double* G, int n, double coeff, double* R,
 }
 
 fd_status tri_inverse(fd_ctx* ctx, const double* R, int n, double* Rinv) {
-  const size_t smem = sizeof(double) * 8 * n;
+  const size_t smem = sizeof(double) * CB * n;
   if (smem > 48 * 1024)
-    FD_CUDA(ctx, cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_tri_inverse<<<(unsigned)cdiv(n, 8), 256, smem, ctx->stream>>>(R, n, Rinv);
+    FD_CUDA(ctx, cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(sizeof(double) * CB * 1024)));
+  k_tri_inverse<<<(unsigned)cdiv(n, CB), 256, smem, ctx->stream>>>(R, n, Rinv);
   FD_LAUNCHED(ctx);
   return FD_OK;
 }
@@ -538,27 +674,19 @@ fd_status rayleigh_ritz_dev(fd_ctx* ctx, const fd_matrix* A, double* V, double* 
 
 fd_status copy_cols_f64_to_f32(fd_ctx* ctx, const double* src, int64_t lds, float* dst, int64_t ldd,
                                int64_t D, int n) {
-  k_f64_to_f32<<<(unsigned)cdiv(D * n, 256), 256, 0, ctx->stream>>>(src, lds, dst, ldd, D, n);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
+  return convert_block(ctx, src, lds, dst, ldd, D, n);
 }
 fd_status copy_cols_f32_to_f64(fd_ctx* ctx, const float* src, int64_t lds, double* dst, int64_t ldd,
                                int64_t D, int n) {
-  k_f32_to_f64<<<(unsigned)cdiv(D * n, 256), 256, 0, ctx->stream>>>(src, lds, dst, ldd, D, n);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
+  return convert_block(ctx, src, lds, dst, ldd, D, n);
 }
 fd_status copy_cols_f64_to_ff(fd_ctx* ctx, const double* src, int64_t lds, float* dst, int64_t ldd,
                               int64_t D, int n) {
-  k_f64_to_ff<<<(unsigned)cdiv(D * n, 256), 256, 0, ctx->stream>>>(src, lds, dst, ldd, D, n);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
+  return convert_block(ctx, src, lds, reinterpret_cast<pair_f*>(dst), ldd, D, n);
 }
 fd_status copy_cols_ff_to_f64(fd_ctx* ctx, const float* src, int64_t lds, double* dst, int64_t ldd,
                               int64_t D, int n) {
-  k_ff_to_f64<<<(unsigned)cdiv(D * n, 256), 256, 0, ctx->stream>>>(src, lds, dst, ldd, D, n);
-  FD_LAUNCHED(ctx);
-  return FD_OK;
+  return convert_block(ctx, reinterpret_cast<const pair_f*>(src), lds, dst, ldd, D, n);
 }
 
 }  // namespace fdi
@@ -622,10 +750,8 @@ fd_status fd_copy_block(fd_ctx* ctx, const void* src, fd_prec sp, int64_t lds, v
     return copy_cols_f64_to_ff(ctx, (const double*)src, lds, (float*)dst, ldd, D, n);
   if (sp == FD_FF && dp == FD_F64)
     return copy_cols_ff_to_f64(ctx, (const float*)src, lds, (double*)dst, ldd, D, n);
-  const size_t es = sp == FD_F32 ? 4 : 8;
-  FD_CUDA(ctx, cudaMemcpy2DAsync(dst, ldd * es, src, lds * es, n * es, D, cudaMemcpyDeviceToDevice,
-                                 ctx->stream));
-  return FD_OK;
+  if (sp == FD_F32) return convert_block(ctx, (const float*)src, lds, (float*)dst, ldd, D, n);
+  return convert_block(ctx, (const double*)src, lds, (double*)dst, ldd, D, n);  // float-float pairs: 8 bytes too
 }
 
 fd_status fd_rayleigh_ritz(fd_ctx* ctx, const fd_matrix* A, double* V, double* AV, int64_t D, int ns,

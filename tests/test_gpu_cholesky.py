@@ -1,0 +1,61 @@
+"""Cholesky and triangular inverse through Cholesky-QR: orders around the 8-row
+panels and the grid, graded blocks; block copies at every width and alignment."""
+import numpy as np
+import pytest
+
+import fd_inputs
+pytestmark = pytest.mark.gpu
+
+
+def _qr(V0):
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    V = torch.from_numpy(V0).cuda()
+    R = torch.empty((V0.shape[1],) * 2, dtype=torch.float64, device="cuda")
+    passes = fd.fd_orthonormalize(ctx, V, R)
+    return V.cpu().numpy(), R.cpu().numpy(), passes
+
+
+@pytest.mark.parametrize("ns", [1, 2, 7, 8, 9, 15, 16, 17, 63, 65, 127, 153, 161, 200, 305, 600])
+@pytest.mark.parametrize("spread", [0, 6])
+def test_orders(ns, spread):
+    D = 2 * ns + 37
+    V0 = fd_inputs.random_block(D, ns, ns) * np.logspace(0, -spread, ns)[None, :]
+    Q, R, passes = _qr(V0)
+    assert passes == 2
+    assert np.abs(Q.T @ Q - np.eye(ns)).max() <= 1e-14 * max(1.0, ns / 100)
+    assert np.all(np.tril(R, -1) == 0.0)
+    # R against LAPACK's up to row signs, column by column: each column's size sets its scale
+    ref = np.linalg.qr(V0, mode="r")
+    ref *= np.sign(np.diag(ref))[:, None]
+    scale = np.linalg.norm(V0, axis=0)
+    assert np.all(np.abs(R - ref) <= 1e-12 * np.sqrt(ns) * scale[None, :])
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 6, 255, 256, 257, 1030])
+@pytest.mark.parametrize("pad,shift", [(0, 0), (2, 2), (3, 1), (4, 0)])
+def test_copy_block_widths(n, pad, shift):
+    """Type conversions at widths and alignments with and without wide accesses."""
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    D = 67
+    src = torch.from_numpy(fd_inputs.random_block(D, n, n)).cuda()
+    big = torch.zeros((D, n + pad + shift), dtype=torch.float64, device="cuda")
+    v64 = big[:, shift:shift + n]
+    fd.fd_copy_block(ctx, src, v64)
+    assert torch.equal(v64, src) and int((big != 0).sum()) == D * n
+    v32 = torch.zeros((D, n + pad + shift), dtype=torch.float32, device="cuda")[:, shift:shift + n]
+    fd.fd_copy_block(ctx, v64, v32)
+    assert torch.equal(v32, src.float())
+    fd.fd_copy_block(ctx, v32, v64)
+    assert torch.equal(v64, src.float().double())
+    vff = torch.zeros((D, n + pad + shift, 2), dtype=torch.float32, device="cuda")[:, shift:shift + n]
+    fd.fd_copy_block(ctx, src, vff)
+    hi = src.float()
+    assert torch.equal(vff[..., 0], hi) and torch.equal(vff[..., 1], (src - hi.double()).float())
+    fd.fd_copy_block(ctx, vff, v64)
+    assert torch.equal(v64, hi.double() + (src - hi.double()).float().double())
