@@ -63,24 +63,13 @@ __global__ void k_extract(const double* V, int64_t ldv, int64_t D, const int* se
 
 // ---- host-side filter coefficients (Sec. 2: Chebyshev expansion of a window,
 // Jackson-damped as in the kernel polynomial method the paper cites) --------
-// cos(k th), sin(k th) for k = 0, 1, 2, ...: from the library up to k = 63 and every
-// 16th k after that, in between by rotation.  The argument k th is itself rounded
-// (by up to k th u, 100 u from k = 64 on), so the 15 rotations in between (under 24 u)
-// stay inside the error that evaluating every term has.
-struct Rotor {
-  double th, c1, s1, c = 1.0, s = 0.0;
-  explicit Rotor(double t) : th(t), c1(std::cos(t)), s1(std::sin(t)) {}
-  void to(int k) {
-    if (k < 64 || k % 16 == 0) {
-      c = std::cos((double)k * th);
-      s = std::sin((double)k * th);
-    } else {
-      const double cn = c * c1 - s * s1;
-      s = s * c1 + c * s1;
-      c = cn;
-    }
-  }
-};
+double cheb_eval(const std::vector<double>& mu, double x) {
+  x = std::min(1.0, std::max(-1.0, x));
+  const double th = std::acos(x);
+  double s = 0.0;
+  for (size_t k = 0; k < mu.size(); ++k) s += mu[k] * std::cos((double)k * th);
+  return s;
+}
 
 }  // namespace
 
@@ -88,22 +77,16 @@ std::vector<double> filter_coeffs(double x_l, double x_r, int n) {
   x_l = std::max(-1.0, x_l);
   x_r = std::min(1.0, x_r);
   const double th_l = std::acos(x_l), th_r = std::acos(x_r);
-  const double th_c = std::acos(std::min(1.0, std::max(-1.0, 0.5 * (x_l + x_r))));
   const int N = n + 1;
-  const double a = M_PI / (N + 1), cot = 1.0 / std::tan(a);
+  const double a = M_PI / (N + 1);
   std::vector<double> mu(n + 1);
-  Rotor ra(a), rl(th_l), rr(th_r), rc(th_c);
-  double p = 0.0;  // the filter at the window's centre
   for (int k = 0; k <= n; ++k) {
-    ra.to(k);
-    rl.to(k);
-    rr.to(k);
-    rc.to(k);
-    const double g = ((N - k + 1) * ra.c + ra.s * cot) / (N + 1);
-    const double c = k == 0 ? (th_l - th_r) / M_PI : 2.0 * (rl.s - rr.s) / (k * M_PI);
+    const double g = ((N - k + 1) * std::cos(a * k) + std::sin(a * k) / std::tan(a)) / (N + 1);
+    const double c = k == 0 ? (th_l - th_r) / M_PI
+                            : 2.0 * (std::sin(k * th_l) - std::sin(k * th_r)) / (k * M_PI);
     mu[k] = g * c;
-    p += mu[k] * rc.c;
   }
+  const double p = cheb_eval(mu, 0.5 * (x_l + x_r));
   for (auto& m : mu) m /= p;
   return mu;
 }
