@@ -101,6 +101,7 @@ struct V16<ffa::ff> {
   __device__ __forceinline__ void set(const float4& t) { v[0] = ff(t.x, t.y); v[1] = ff(t.z, t.w); }
   __device__ __forceinline__ float4 get() const { return make_float4(v[0].hi, v[0].lo, v[1].hi, v[1].lo); }
   __device__ __forceinline__ void ldg(const ff* p) { set(__ldg(reinterpret_cast<const float4*>(p))); }
+  __device__ __forceinline__ void ldm(const ff* p) { set(*reinterpret_cast<const float4*>(p)); }
   __device__ __forceinline__ void ld(const ff* p) {
     float4 t;
     asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n"
