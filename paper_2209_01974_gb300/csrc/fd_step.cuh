@@ -167,15 +167,16 @@ __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;
 constexpr int WARPS = 8;
 constexpr int BATCH = 4;   // entries per batch; SELL chunk lengths are multiples of 8
 constexpr int MIN_BLOCKS = 12;     // FP32 steps: 4-warp CTAs, 48 resident warps per SM (<= 40 registers)
-constexpr int MIN_BLOCKS_F64 = 4;  // FP64 steps: 8-warp CTAs with 64 registers (FP64-ALU bound anyway)
+constexpr int MIN_BLOCKS_F64 = 4;  // matrix-free and batched FP64 steps: 8-warp CTAs with 64 registers
 // CTA shape of the fused step (k_cheb_step): warps per CTA and resident CTAs
-// per SM (the launch bounds).  Smaller CTAs for FP32 (more of them in flight, a
-// finer L2 prefetch granule), 8 warps for FP64; other arithmetic types may
-// specialise it.
+// per SM (the launch bounds).  FP32: 48 warps per SM (more spill, fewer hide less
+// latency: 14 CTAs 28 % slower); FP64, bound by its pipe, 32 warps with 64 registers,
+// in 4-warp CTAs because the last wave then ends more evenly (8-warp CTAs 1 to 3 %
+// slower); other arithmetic types may specialise it.
 template <typename T>
 struct StepShape {
-  static constexpr int warps = sizeof(T) == 4 ? 4 : WARPS;
-  static constexpr int min_blocks = sizeof(T) == 4 ? MIN_BLOCKS : MIN_BLOCKS_F64;
+  static constexpr int warps = 4;
+  static constexpr int min_blocks = sizeof(T) == 4 ? MIN_BLOCKS : 8;
 };
 template <typename T>
 __host__ __device__ constexpr int step_warps() { return StepShape<T>::warps; }
