@@ -107,7 +107,7 @@ struct BatchArgs {
   int spmmv_only;           // 1: AV = A V for all listed bundles, one pass, no barrier
 };
 
-constexpr int GSLICES = 8;   // Gram row slices per instance
+constexpr int GSLICES = 32;  // Gram row slices per instance (8: 262 us a Gram of 2,744 x 64)
 constexpr int RBLK = 16;     // residual partial blocks per instance
 
 // ---------------------------------------------------------------------------

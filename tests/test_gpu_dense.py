@@ -131,3 +131,42 @@ def test_kpm_moments_match_oracle(fd, ctx, R):
     mu = fd.fd_kpm_moments(ctx, A, 48, R, 7, alpha, beta)
     muo = kpm.kpm_moments(mat.to_scipy(csr), 48, R, 7, alpha, beta)
     assert np.abs(mu - muo).max() < 1e-11
+
+
+@pytest.mark.parametrize("D", [1, 3, 4, 5, 3647, 3648, 3653, 7295, 7296, 7311])
+@pytest.mark.parametrize("n,ld", [(1, 1), (3, 3), (63, 66), (64, 64), (65, 65), (130, 131)])
+@pytest.mark.parametrize("upper", [False, True])
+def test_fp64_rotation_row_splits(fd, ctx, D, n, ld, upper):
+    """4, 8 and 16 rows per thread block, with remainders of rows, columns and of
+    the unrolled sum; the padding columns stay as they are."""
+    import torch
+    rng = np.random.default_rng(D + n)
+    V, M = rng.standard_normal((D, n)), rng.standard_normal((n, n))
+    if upper:
+        M = np.triu(M)
+    big = torch.full((D, ld), 7.0, dtype=torch.float64, device="cuda")
+    big[:, :n] = _t(V)
+    fd.fd_set_gemm_mode(ctx, "fp64")
+    try:
+        fd.fd_rotate(ctx, big[:, :n], _t(M), upper)
+    finally:
+        fd.fd_set_gemm_mode(ctx, "auto")
+    got = big.cpu().numpy()
+    assert np.all(got[:, n:] == 7.0)
+    # two sums of n products, each within n u of its sum of magnitudes
+    bound = 2 * (n + 1) * 2.0 ** -53 * (np.abs(V) @ np.abs(M))
+    assert np.all(np.abs(got[:, :n] - V @ M) <= bound)
+
+
+@pytest.mark.parametrize("D", [1, 15, 16, 17, 33, 609, 1728])
+@pytest.mark.parametrize("n", [1, 33, 96])
+def test_fp64_gram_of_few_rows(fd, ctx, D, n):
+    """Row slices down to one shared-memory stage and fewer rows than that."""
+    rng = np.random.default_rng(D + n)
+    V = rng.standard_normal((D, n))
+    fd.fd_set_gemm_mode(ctx, "fp64")
+    try:
+        G = fd.fd_gram(ctx, _t(V), _t(V)).cpu().numpy()
+    finally:
+        fd.fd_set_gemm_mode(ctx, "auto")
+    assert np.all(np.abs(G - V.T @ V) <= 2 * (D + 1) * 2.0 ** -53 * (np.abs(V).T @ np.abs(V)))
