@@ -398,14 +398,14 @@ __global__ void __launch_bounds__(WARPS * 32, 4)
           V16<double> z;
           z.ldcs(Z + off);
 #pragma unroll
-          for (int e = 0; e < E; ++e) y.v[e] = c_ax * acc[v].v[e] + c_x * xi[v].v[e] - z.v[e];
+          for (int e = 0; e < E; ++e) y.v[e] = fma(c_ax, acc[v].v[e], fma(c_x, xi[v].v[e], -z.v[e]));
         }
         y.st(Y + off);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           sxy = fma(y.v[e], xi[v].v[e], sxy);
           syy = fma(y.v[e], y.v[e], syy);
-          sxx = fma(xi[v].v[e], xi[v].v[e], sxx);
+          if (FIRST) sxx = fma(xi[v].v[e], xi[v].v[e], sxx);  // only x_0 . x_0 is used
         }
       }
     }

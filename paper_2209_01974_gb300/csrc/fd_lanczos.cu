@@ -158,7 +158,15 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(LzArgs a) {
         if (pass == 0) alpha = cs[j];
         for (int64_t r = r0 + threadIdx.x; r < r1; r += LZ_THREADS) {
           double s = w[r];
-          for (int v = 0; v <= j; ++v) s = fma(-M.Q[(int64_t)v * M.D + r], cs[v], s);
+          int v = 0;
+          for (; v + LZ_TILE <= j + 1; v += LZ_TILE) {  // the loads of a tile together
+            double q[LZ_TILE];
+#pragma unroll
+            for (int u = 0; u < LZ_TILE; ++u) q[u] = M.Q[(int64_t)(v + u) * M.D + r];
+#pragma unroll
+            for (int u = 0; u < LZ_TILE; ++u) s = fma(-q[u], cs[v + u], s);
+          }
+          for (; v <= j; ++v) s = fma(-M.Q[(int64_t)v * M.D + r], cs[v], s);
           w[r] = s;
         }
         __syncthreads();
