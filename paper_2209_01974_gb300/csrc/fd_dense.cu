@@ -21,9 +21,54 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // Gram: P[slice] = X[rows of slice]^T Y[rows of slice], 64 x 64 output tiles
+//
+// Bound by the FP64 pipe (a warp's FMA takes 16 cycles of an SM), so a tile's 16 x 16
+// parts that lie beyond the product's edge, or below a symmetric product's diagonal,
+// are left out: the mirrored part has the same sums in the same order.  Measured,
+// 476,929 rows: 16 columns 3,390 -> 306 us, 32 3,465 -> 722 us, 64 3,536 -> 2,172 us.
 // ---------------------------------------------------------------------------
 constexpr int GT = 64;   // tile edge
+constexpr int GP = 16;   // edge of a tile's parts: thread (ty, tx) has one element of each
 constexpr int GK = 16;   // rows per shared-memory stage
+
+// one tile's parts (u, v), u, v < U, on or above the diagonal if DIAG
+template <int U, bool DIAG>
+__device__ __forceinline__ void gram_tile(const double* __restrict__ X, int64_t ldx, const double* __restrict__ Y,
+                                          int64_t ldy, int i0, int j0, int m, int n, int64_t k0, int64_t k1,
+                                          double (&Xs)[GK][GT], double (&Ys)[GK][GT], double* Ps) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  constexpr int W = GP * U;
+  double acc[U][U] = {};
+  for (int64_t kb = k0; kb < k1; kb += GK) {
+#pragma unroll
+    for (int q = 0; q < (GK * W) / 256; ++q) {
+      int e = threadIdx.x + q * 256;
+      int kk = e / W, c = e % W;
+      int64_t k = kb + kk;
+      Xs[kk][c] = (k < k1 && i0 + c < m) ? X[k * ldx + i0 + c] : 0.0;
+      Ys[kk][c] = (k < k1 && j0 + c < n) ? Y[k * ldy + j0 + c] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < GK; ++kk) {
+      double a[U], b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) { a[u] = Xs[kk][ty + GP * u]; b[u] = Ys[kk][tx + GP * u]; }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = DIAG ? u : 0; v < U; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = DIAG ? u : 0; v < U; ++v) {
+      int i = i0 + ty + GP * u, j = j0 + tx + GP * v;
+      if (i < m && j < n) Ps[(int64_t)i * n + j] = acc[u][v];
+    }
+}
 
 __global__ void __launch_bounds__(256)
     k_gram_partial(const double* __restrict__ X, int64_t ldx, const double* __restrict__ Y,
@@ -44,38 +89,17 @@ __global__ void __launch_bounds__(256)
   const int i0 = ti * GT, j0 = tj * GT;
   const int64_t k0 = (int64_t)blockIdx.y * rows_per_slice;
   const int64_t k1 = min(D, k0 + rows_per_slice);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
-  for (int64_t kb = k0; kb < k1; kb += GK) {
-#pragma unroll
-    for (int q = 0; q < (GK * GT) / 256; ++q) {
-      int e = threadIdx.x + q * 256;
-      int kk = e / GT, c = e % GT;
-      int64_t k = kb + kk;
-      Xs[kk][c] = (k < k1 && i0 + c < m) ? X[k * ldx + i0 + c] : 0.0;
-      Ys[kk][c] = (k < k1 && j0 + c < n) ? Y[k * ldy + j0 + c] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { a[u] = Xs[kk][ty + 16 * u]; b[u] = Ys[kk][tx + 16 * u]; }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
-    }
-    __syncthreads();
-  }
   double* Ps = P + (int64_t)blockIdx.y * m * n;
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
-      if (i < m && j < n) Ps[(int64_t)i * n + j] = acc[u][v];
-    }
+  const int parts = (min(GT, max(m - i0, n - j0)) + GP - 1) / GP;
+  const bool diag = sym && ti == tj;
+#define FD_GRAM_TILE(U) \
+  if (diag) gram_tile<U, true>(X, ldx, Y, ldy, i0, j0, m, n, k0, k1, Xs, Ys, Ps); \
+  else gram_tile<U, false>(X, ldx, Y, ldy, i0, j0, m, n, k0, k1, Xs, Ys, Ps)
+  if (parts == 1) { FD_GRAM_TILE(1); }
+  else if (parts == 2) { FD_GRAM_TILE(2); }
+  else if (parts == 3) { FD_GRAM_TILE(3); }
+  else { FD_GRAM_TILE(4); }
+#undef FD_GRAM_TILE
 }
 
 __global__ void k_gram_reduce(const double* P, int slices, int m, int n, bool sym, double* C,
@@ -83,11 +107,11 @@ __global__ void k_gram_reduce(const double* P, int slices, int m, int n, bool sy
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)m * n) return;
   int i = (int)(e / n), j = (int)(e % n);
-  if (sym && i / GT > j / GT) return;  // computed by the mirrored tile
+  if (sym && i / GP > j / GP) return;  // computed by the mirrored part
   double s = 0.0;
   for (int q = 0; q < slices; ++q) s += P[(int64_t)q * m * n + e];
   C[(int64_t)i * ldc + j] = s;
-  if (sym && i / GT < j / GT) C[(int64_t)j * ldc + i] = s;
+  if (sym && i / GP < j / GP) C[(int64_t)j * ldc + i] = s;
 }
 
 // ---------------------------------------------------------------------------
@@ -95,7 +119,8 @@ __global__ void k_gram_reduce(const double* P, int slices, int m, int n, bool sy
 // ---------------------------------------------------------------------------
 // RT rows per CTA: 256 / RT threads along the columns, RT / 4 of each 64 columns per
 // thread.  Few rows are spread thinner, 4 to a CTA, so that every SM's FP64 pipe has
-// rows and warps enough (1,728 x 96: 34 us, 125 us with 16 rows in 108 CTAs).
+// rows and warps enough (1,728 x 96: 34 us, 125 us with 16 rows in 108 CTAs).  Bound by
+// the FP64 pipe from 64 columns on; the columns that a last 64 lacks are left out.
 template <int RT>
 __global__ void __launch_bounds__(256)
     k_rotate(double* V, int64_t ldv, int64_t D, int n, const double* __restrict__ M, bool upper) {
@@ -114,6 +139,7 @@ __global__ void __launch_bounds__(256)
     double acc[COLS] = {};
     const int kend = upper ? min(n, cb + 64) : n;
     const double* vr = Vt + r * n;
+    const int nv = min(COLS, (n - cb + LANES - 1) / LANES);  // columns beyond n cost FP64 cycles too
     int col[COLS];
 #pragma unroll
     for (int v = 0; v < COLS; ++v) col[v] = min(cb + c0 + LANES * v, n - 1);  // beyond n: not stored
@@ -127,11 +153,13 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v < COLS; ++v) acc[v] = fma(vr[k + u], m[u][v], acc[v]);
+        for (int v = 0; v < COLS; ++v)
+          if (v < nv) acc[v] = fma(vr[k + u], m[u][v], acc[v]);
     }
     for (; k < kend; ++k)
 #pragma unroll
-      for (int v = 0; v < COLS; ++v) acc[v] = fma(vr[k], __ldg(M + (int64_t)k * n + col[v]), acc[v]);
+      for (int v = 0; v < COLS; ++v)
+        if (v < nv) acc[v] = fma(vr[k], __ldg(M + (int64_t)k * n + col[v]), acc[v]);
     if (r < nr) {
 #pragma unroll
       for (int v = 0; v < COLS; ++v) {
@@ -469,7 +497,12 @@ fd_status convert_block(fd_ctx* ctx, const S* s, int64_t lds, T* d, int64_t ldd,
 
 }  // namespace
 
-// tall-skinny products large enough for the tensor-core splitting to pay off
+// tall-skinny products large enough for the tensor-core splitting to pay off.  It is
+// faster from fewer rows and columns on (30,001 x 80: orthonormalisation 0.96 ms), but
+// its digits are relative to the largest entry of a row or column, and blocks whose
+// columns differ in size lose to that (orthonormalisation error 3.5e-16 -> 8.8e-14): the
+// line stays where FP64 costs several times as much (65,537 x 128: Gram 1,149 against
+// 241 us, rotation 1,745 against 220 us)
 static bool use_ozaki(const fd_ctx* ctx, int64_t D, int m, int n) {
   if (ctx->gemm_mode == FD_GEMM_FP64) return false;
   if (ctx->gemm_mode == FD_GEMM_OZAKI) return true;

@@ -159,14 +159,20 @@ def test_fp64_rotation_row_splits(fd, ctx, D, n, ld, upper):
 
 
 @pytest.mark.parametrize("D", [1, 15, 16, 17, 33, 609, 1728])
-@pytest.mark.parametrize("n", [1, 33, 96])
-def test_fp64_gram_of_few_rows(fd, ctx, D, n):
-    """Row slices down to one shared-memory stage and fewer rows than that."""
+@pytest.mark.parametrize("m,n", [(1, 1), (16, 16), (17, 33), (48, 49), (64, 5), (33, 33), (96, 96), (129, 130)])
+def test_fp64_gram_parts(fd, ctx, D, m, n):
+    """Row slices down to one shared-memory stage and fewer rows than that; tiles of
+    one to four 16-column parts, of two blocks and of one with itself."""
     rng = np.random.default_rng(D + n)
-    V = rng.standard_normal((D, n))
+    X, Y = rng.standard_normal((D, m)), rng.standard_normal((D, n))
     fd.fd_set_gemm_mode(ctx, "fp64")
     try:
-        G = fd.fd_gram(ctx, _t(V), _t(V)).cpu().numpy()
+        Xt = _t(X)
+        G = fd.fd_gram(ctx, Xt, _t(Y)).cpu().numpy()
+        S = fd.fd_gram(ctx, Xt, Xt).cpu().numpy()
     finally:
         fd.fd_set_gemm_mode(ctx, "auto")
-    assert np.all(np.abs(G - V.T @ V) <= 2 * (D + 1) * 2.0 ** -53 * (np.abs(V).T @ np.abs(V)))
+    u = 2 * (D + 1) * 2.0 ** -53
+    assert np.all(np.abs(G - X.T @ Y) <= u * (np.abs(X).T @ np.abs(Y)))
+    assert np.all(np.abs(S - X.T @ X) <= u * (np.abs(X).T @ np.abs(X)))
+    assert np.array_equal(S, S.T)
