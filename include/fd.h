@@ -171,7 +171,10 @@ fd_status fd_spectral_bounds(fd_ctx* ctx, const fd_matrix* A, int steps,
  * D x nb block V (device, leading dimension ldv).  One fused kernel per
  * degree step computes the SpMMV W2 <- 2 A~ W1 - W2 together with
  * V <- V + mu_k W2 (Alg. 2 fuses the SpMV with the vector update so that W2 is
- * not read twice).
+ * not read twice; the terms of three steps are added to V at a time).  A matrix
+ * whose panels fit the shared memory of a few SMs takes all steps in one launch.
+ * FP64 and float-float filters of degree 12 and more scale the matrix once into a
+ * workspace of the context, unless it is refused or the stream is capturing.
  *   prec    FD_F64: V, W1, W2 are double and H's FP64 values are used;
  *           FD_F32: V, W1, W2 are float, H's FP32 copy, FP32 accumulation;
  *           FD_FF: V, W1, W2 hold float-float pairs (2 floats per element,
@@ -247,7 +250,8 @@ fd_status fd_check_bounded_wait(fd_ctx* ctx, int limit_us);
 fd_status fd_gram(fd_ctx* ctx, const double* X, int64_t ldx, const double* Y, int64_t ldy,
                   int64_t D, int m, int n, double* C, int ldc);
 /* In-place rotation V <- V M (device; V: D x n with ldv, M: n x n row-major;
- * upper != 0: M is upper triangular and its lower part is not read). */
+ * upper != 0: M is upper triangular and its lower part is not read).  After
+ * FD_ERR_TIMEOUT V holds old and new rows. */
 fd_status fd_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const double* M,
                     int upper);
 
@@ -447,7 +451,8 @@ typedef struct {
  * instance, instances of different sizes).  Each outer iteration of all
  * unconverged instances runs as one CUDA graph: one persistent cooperative
  * kernel applies the Chebyshev filters of every bundle of every instance (all
- * degree steps, a grid-wide barrier between steps), batched Cholesky-QR and
+ * degree steps, a grid-wide barrier between steps; instances whose panels fit the
+ * shared memory of a few SMs take one cluster per panel), batched Cholesky-QR and
  * Rayleigh-Ritz kernels cover all instances per launch, and all Ritz values
  * and residuals are copied to the host once.  Instances drop out when they
  * converge.  The per-instance intervals and degrees follow fd_solve's

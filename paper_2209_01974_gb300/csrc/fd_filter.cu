@@ -6,10 +6,10 @@
 // three terms (step_terms), so a step moves 11/3 vectors on average, and the
 // steps follow each other by programmatic dependent launch (step_wait).
 // Measured: 2.1M-row stencil, nb = 64, FP32, degree 40 with its two conversions
-// 21.1 -> 17.6 ms; 1.4M-row road graph, nb = 32, FP32 6.95 -> 5.53 ms.  FP64 and
+// 21.1 -> 17.2 ms; 1.4M-row road graph, nb = 32, FP32 6.95 -> 5.40 ms.  FP64 and
 // float-float filters scale the matrix once (scale_matrix): 110,592-row Anderson,
 // nb = 32, 4 x 100 steps, float-float 19.1 -> 14.9 ms (15.8 unscaled), FP64, bound by
-// the FP64 pipe, 32.9 -> 26.0 ms (31.3 unscaled).
+// the FP64 pipe, 32.9 -> 25.7 ms (31.3 unscaled).
 //
 // Work mapping: a group of G lanes owns one SELL row; each lane holds CPL
 // 16-byte vectors of the row (G * CPL * 16 bytes = nb * sizeof(T)), so every
@@ -180,9 +180,9 @@ fd_status launch_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<
   // Dependent launch, but for the first step (MODE_SPMMV), which follows a
   // kernel that is not a step, and for FP64 grids between half the SMs and one
   // wave: their CTAs would be placed beside the previous step's, unevenly over
-  // the SMs, and the FP64 pipe of the fuller ones sets the time (nb = 16, 4,900
-  // rows in 154 CTAs: 9.2 us a step against 8.2 us; 1,728 rows in 54 CTAs:
-  // 3.4 us against 4.1 us).
+  // the SMs, and the FP64 pipe of the fuller ones sets the time (8-warp CTAs,
+  // nb = 16, 4,900 rows in 154 CTAs: 9.2 us a step against 8.2 us; 1,728 rows in 54
+  // CTAs: 3.4 us against 4.1 us).
   const bool dep = dependent_step<T>(ctx, grid, pf);
   if (mode == MODE_SPMMV) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SPMMV>, grid, SW * 32, 0, false, A, s, pf);
   if (mode == MODE_SECOND) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SECOND>, grid, SW * 32, 0, dep, A, s, pf);

@@ -138,7 +138,6 @@ struct StepArgs {
                              // [mu1 x +] mu2 y, the last nacc (1 .. 3) of the terms, or no accumulation (0)
   int nacc;
   int scaled;                // the matrix is A' = c_ax A + c_x I: c_ax, c_x are not applied again
-
 };
 
 template <int MODE, typename S>
