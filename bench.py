@@ -13,7 +13,9 @@ Rayleigh-Ritz (SpMMV, Gram, Jacobi, rotations) and the residual norms run in
 FP64 and are read back to the host.
 value = algorithmic filter bytes per step (Eq. EstimateT, kappa = 5) / step
 time: the sweep's HBM throughput with the orthogonalisation and Rayleigh-Ritz
-time charged to it.  The all-FP64 form of the same step is reported under
+time charged to it.  The steps move less than the algorithm counts (they visit the
+accumulator every third time: 11/3 vectors instead of 5), which roofline.moved
+states beside it, with its own fraction of the peak.  The all-FP64 form of the same step is reported under
 "f64_form"; its fused step is bound by GB300's FP64 rate, not by HBM.  The
 inputs (6.4 GB block, 0.5 GB matrix) exceed the 129 MB L2, so no flush is
 needed between steps.
@@ -49,13 +51,13 @@ WORKLOAD = {"workload": "anderson3d L=128 (2,097,152 rows) stencil, nb=64, degre
 
 # GB300 FP64 peak (nominal 1.25 TFLOP/s; an FMA-loop probe on this machine measured 1.20)
 FP64_TFLOPS = 1.25
-# DRAM bytes (read + write) of one generic FP32 step of this workload, from one ncu
+# DRAM bytes (read + write) of one accumulating FP32 step of this workload, from one ncu
 # capture of `bench.py --kernel-only f32` (profiles/k_cheb_step_f32_stencil_L128_nb64.md),
 # with the kernel shape it was taken on and the SHA-256 of the step kernel's sources
 # at that time: when the sources differ, the figure is stale and is reported as null
-TRAFFIC_F32 = {"bytes": 1.762341888e9 + 1.0270528e9, "kernel": "k_cheb_step<float,64,GENERIC>",
+TRAFFIC_F32 = {"bytes": 1.762509824e9 + 1.024038912e9, "kernel": "k_cheb_step<float,64,GENERIC>",
                "rows": 2097152, "nnz": 14680064, "nb": 64,
-               "sources_sha256": "ca2c354e272c5d65b724693c96f91916002584102c602b2b76fa213a5c67b8c7"}
+               "sources_sha256": "a90517f3460c50989d836af93009b6c6009781f69d1537b704f85c9a2bcbbb92"}
 STEP_SOURCES = ["paper_2209_01974_gb300/csrc/fd_step.cuh", "paper_2209_01974_gb300/csrc/fd_filter.cu"]
 
 
@@ -92,6 +94,13 @@ def filter_bytes(D, nnz, nb, n, Sx):
 
 def generic_step_bytes(D, nnz, nb, Sx):
     return nnz * (Sx + 4.0) + 5 * nb * D * Sx
+
+
+def moved_filter_bytes(D, nnz, nb, n, Sx):
+    """Bytes that the steps of a degree-n filter move, n >= 3: as filter_bytes, but a
+    step that leaves the accumulator alone reads two vectors and writes one."""
+    plain = sum(1 for k in range(3, n) if (k - 2) % 3)
+    return filter_bytes(D, nnz, nb, n, Sx) - plain * 2 * nb * D * Sx
 
 
 # --------------------------------------------------------------------------- clocks
@@ -420,6 +429,8 @@ def run_gpu(args):
                          f"L=128 stencil, columns split over {cores} spawned processes: {dt:.2f} s",
                "one_core": {"value": gbs1, "unit": UNIT, "seconds": dt1}}
     traffic, traffic_note = traffic_record(D, nnz, NB)
+    # GB/s that the filter phase really moves
+    moved = achieved * moved_filter_bytes(D, nnz, NB, DEGREE, 4.0) / filter_bytes(D, nnz, NB, DEGREE, 4.0)
     if rank == 0:
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
@@ -428,6 +439,7 @@ def run_gpu(args):
                 "data": "synthetic", "config": WORKLOAD,
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                              "frac": achieved / peak, "traffic": traffic, "traffic_source": traffic_note,
+                             "moved": moved, "moved_frac": moved / peak,
                              "peak_source": peak_note,
                              "kernel": "k_cheb_step<float,64> (fused SpMMV + recurrence + "
                                        "accumulation), averaged over the filter phase",
