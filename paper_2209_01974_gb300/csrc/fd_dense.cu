@@ -621,7 +621,8 @@ fd_status cholesky(fd_ctx* ctx, const double* G, int n, double coeff, double* R,
 
 fd_status tri_inverse(fd_ctx* ctx, const double* R, int n, double* Rinv) {
   const size_t smem = sizeof(double) * CB * n;
-  if (smem > 48 * 1024)
+  // the default limit of 48 KB covers the kernel's static arrays too (2.7 KB)
+  if (smem > 32 * 1024)
     FD_CUDA(ctx, cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(sizeof(double) * CB * 1024)));
   k_tri_inverse<<<(unsigned)cdiv(n, CB), 256, smem, ctx->stream>>>(R, n, Rinv);

@@ -1,5 +1,9 @@
 """Cholesky and triangular inverse through Cholesky-QR: orders around the 8-row
 panels and the grid, graded blocks; block copies at every width and alignment."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -32,6 +36,25 @@ def test_orders(ns, spread):
     ref *= np.sign(np.diag(ref))[:, None]
     scale = np.linalg.norm(V0, axis=0)
     assert np.all(np.abs(R - ref) <= 1e-12 * np.sqrt(ns) * scale[None, :])
+
+
+def test_orders_whose_shared_memory_is_just_above_the_default():
+    """From 727 on the triangular inverse's shared memory, static and dynamic, exceeds
+    the 48 KB that a launch gets unasked.  In a process of its own: the larger limit
+    stays with a kernel once a wider block has asked for it."""
+    code = """
+import numpy as np, torch
+import fd_inputs, paper_2209_01974_gb300 as fd
+ctx = fd.fd_create(0)
+for ns in (726, 727, 768, 769, 1024):
+    V = torch.from_numpy(fd_inputs.random_block(ns + 37, ns, ns)).cuda()
+    assert fd.fd_orthonormalize(ctx, V) == 2
+    Q = V.cpu().numpy()
+    assert np.abs(Q.T @ Q - np.eye(ns)).max() <= 1e-14 * ns / 100, ns
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
 
 
 @pytest.mark.parametrize("n", [1, 3, 4, 6, 255, 256, 257, 1030])
