@@ -436,7 +436,8 @@ __global__ void k_resid_reduce(const double* P, int nb, int n, double* out) {
 // the nearest float, lo the nearest float to the exact FP64 remainder; back, hi +
 // lo is exact in FP64.  One element per thread with a 64-bit division for its row
 // ran at half the copy bandwidth (11.8M x 32, FP64 -> FP32: 1.32 ms, now 0.65).
-struct pair_f { float hi, lo; };
+struct alignas(8) pair_f { float hi, lo; };
+struct pair_u { float hi, lo; };  // the same at a 4-byte boundary
 __device__ __forceinline__ void convert(double v, float& o) { o = __double2float_rn(v); }
 __device__ __forceinline__ void convert(float v, double& o) { o = (double)v; }
 __device__ __forceinline__ void convert(double v, pair_f& o) {
@@ -444,11 +445,18 @@ __device__ __forceinline__ void convert(double v, pair_f& o) {
   o.lo = __double2float_rn(v - (double)o.hi);
 }
 __device__ __forceinline__ void convert(pair_f v, double& o) { o = (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ void convert(double v, pair_u& o) {
+  pair_f p;
+  convert(v, p);
+  o = pair_u{p.hi, p.lo};
+}
+__device__ __forceinline__ void convert(pair_u v, double& o) { o = (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ void convert(pair_u v, pair_u& o) { o = v; }
 __device__ __forceinline__ void convert(double v, double& o) { o = v; }
 __device__ __forceinline__ void convert(float v, float& o) { o = v; }
 
 template <typename T, int W>
-struct alignas(sizeof(T) * W < 16 ? sizeof(T) * W : 16) Pack { T v[W]; };
+struct alignas(W == 1 ? alignof(T) : sizeof(T) * W < 16 ? sizeof(T) * W : 16) Pack { T v[W]; };
 
 template <typename S, typename T, int W>
 __global__ void __launch_bounds__(256) k_convert(const S* s, int64_t lds, T* d, int64_t ldd, int64_t D, int n) {
@@ -746,10 +754,12 @@ fd_status copy_cols_f32_to_f64(fd_ctx* ctx, const float* src, int64_t lds, doubl
 }
 fd_status copy_cols_f64_to_ff(fd_ctx* ctx, const double* src, int64_t lds, float* dst, int64_t ldd,
                               int64_t D, int n) {
+  if ((uintptr_t)dst & 7) return convert_block(ctx, src, lds, reinterpret_cast<pair_u*>(dst), ldd, D, n);
   return convert_block(ctx, src, lds, reinterpret_cast<pair_f*>(dst), ldd, D, n);
 }
 fd_status copy_cols_ff_to_f64(fd_ctx* ctx, const float* src, int64_t lds, double* dst, int64_t ldd,
                               int64_t D, int n) {
+  if ((uintptr_t)src & 7) return convert_block(ctx, reinterpret_cast<const pair_u*>(src), lds, dst, ldd, D, n);
   return convert_block(ctx, reinterpret_cast<const pair_f*>(src), lds, dst, ldd, D, n);
 }
 
@@ -815,6 +825,9 @@ fd_status fd_copy_block(fd_ctx* ctx, const void* src, fd_prec sp, int64_t lds, v
   if (sp == FD_FF && dp == FD_F64)
     return copy_cols_ff_to_f64(ctx, (const float*)src, lds, (double*)dst, ldd, D, n);
   if (sp == FD_F32) return convert_block(ctx, (const float*)src, lds, (float*)dst, ldd, D, n);
+  // a float-float block may start at any float, between the 8-byte boundaries too
+  if (((uintptr_t)src | (uintptr_t)dst) & 7)
+    return convert_block(ctx, (const pair_u*)src, lds, (pair_u*)dst, ldd, D, n);
   return convert_block(ctx, (const double*)src, lds, (double*)dst, ldd, D, n);  // float-float pairs: 8 bytes too
 }
 

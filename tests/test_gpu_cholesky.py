@@ -82,3 +82,28 @@ def test_copy_block_widths(n, pad, shift):
     assert torch.equal(vff[..., 0], hi) and torch.equal(vff[..., 1], (src - hi.double()).float())
     fd.fd_copy_block(ctx, vff, v64)
     assert torch.equal(v64, hi.double() + (src - hi.double()).float().double())
+
+
+@pytest.mark.parametrize("n", [1, 4, 5, 256, 1030])
+@pytest.mark.parametrize("so,do", [(0, 1), (1, 0), (1, 1)])
+def test_copy_block_pairs_between_8_byte_boundaries(n, so, do):
+    """Float-float blocks that start at an odd float."""
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    D = 67
+
+    def block(off):
+        return torch.zeros(2 * D * n + 1, dtype=torch.float32, device="cuda")[off:off + 2 * D * n].view(D, n, 2)
+    src = torch.from_numpy(fd_inputs.random_block(D, n, n)).cuda()
+    a, b = block(so), block(do)
+    assert a.data_ptr() % 8 == 4 * so and b.data_ptr() % 8 == 4 * do
+    fd.fd_copy_block(ctx, src, a)
+    hi = src.float()
+    assert torch.equal(a[..., 0], hi) and torch.equal(a[..., 1], (src - hi.double()).float())
+    fd.fd_copy_block(ctx, a, b)
+    assert torch.equal(a, b)
+    back = torch.empty_like(src)
+    fd.fd_copy_block(ctx, b, back)
+    assert torch.equal(back, b[..., 0].double() + b[..., 1].double())
