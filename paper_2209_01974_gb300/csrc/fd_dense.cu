@@ -431,41 +431,38 @@ __global__ void k_resid_reduce(const double* P, int nb, int n, double* out) {
   if (lane == 0) out[c] = sqrt(s);
 }
 
-// Copies of D x n blocks with a change of type, W elements per thread and row (16
-// or 32 bytes on the wider side) and four rows in flight.  FP64 -> float-float: hi
-// the nearest float, lo the nearest float to the exact FP64 remainder; back, hi +
-// lo is exact in FP64.  One element per thread with a 64-bit division for its row
-// ran at half the copy bandwidth (11.8M x 32, FP64 -> FP32: 1.32 ms, now 0.65).
+// Copies of D x n blocks with a change of type.  FP64 -> float-float: hi the nearest
+// float, lo the nearest float to the exact FP64 remainder; back, hi + lo is exact in
+// FP64.
 struct alignas(8) pair_f { float hi, lo; };
 struct pair_u { float hi, lo; };  // the same at a 4-byte boundary
 __device__ __forceinline__ void convert(double v, float& o) { o = __double2float_rn(v); }
 __device__ __forceinline__ void convert(float v, double& o) { o = (double)v; }
-__device__ __forceinline__ void convert(double v, pair_f& o) {
+template <typename P>
+__device__ __forceinline__ void convert(double v, P& o) {
   o.hi = __double2float_rn(v);
   o.lo = __double2float_rn(v - (double)o.hi);
 }
-__device__ __forceinline__ void convert(pair_f v, double& o) { o = (double)v.hi + (double)v.lo; }
-__device__ __forceinline__ void convert(double v, pair_u& o) {
-  pair_f p;
-  convert(v, p);
-  o = pair_u{p.hi, p.lo};
-}
-__device__ __forceinline__ void convert(pair_u v, double& o) { o = (double)v.hi + (double)v.lo; }
-__device__ __forceinline__ void convert(pair_u v, pair_u& o) { o = v; }
 __device__ __forceinline__ void convert(double v, double& o) { o = v; }
 __device__ __forceinline__ void convert(float v, float& o) { o = v; }
+__device__ __forceinline__ void convert(pair_f v, double& o) { o = (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ void convert(pair_u v, double& o) { o = (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ void convert(pair_u v, pair_u& o) { o = v; }
 
 template <typename T, int W>
-struct alignas(W == 1 ? alignof(T) : sizeof(T) * W < 16 ? sizeof(T) * W : 16) Pack { T v[W]; };
+struct alignas(sizeof(T) * W < 16 ? sizeof(T) * W : 16) Pack { T v[W]; };
 
-template <typename S, typename T, int W>
+// FP64 and FP32 blocks, bound by memory: W elements per thread and row (16 or 32
+// bytes on the wider side) and UNROLL rows in flight.  One element per thread with a
+// 64-bit division for its row ran at half the copy bandwidth (11.8M x 32, FP64 ->
+// FP32: 1.32 ms, now 0.65).
+template <typename S, typename T, int W, int UNROLL>
 __global__ void __launch_bounds__(256) k_convert(const S* s, int64_t lds, T* d, int64_t ldd, int64_t D, int n) {
-  constexpr int UNROLL = 4;
   const unsigned q = (unsigned)n / W, per = q < 256 ? 256 / q : 1;  // threads of a row, rows at once
-  const unsigned r = threadIdx.x / q, c0 = q < 256 ? threadIdx.x - r * q : threadIdx.x;
+  const unsigned r = threadIdx.x / q, c0 = q < 256 ? threadIdx.x - r * q : blockIdx.y * 256 + threadIdx.x;
   if (q < 256 && r >= per) return;
   const int64_t row0 = (int64_t)blockIdx.x * per * UNROLL + (q < 256 ? r : 0);
-  for (unsigned c = c0; c < q; c += 256) {
+  for (unsigned c = c0; c < q; c += gridDim.y * 256) {
     Pack<S, W> in[UNROLL];
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
@@ -485,6 +482,20 @@ __global__ void __launch_bounds__(256) k_convert(const S* s, int64_t lds, T* d, 
   }
 }
 
+// Float-float blocks: the conversions are bound by the FP64 pipe, so a thread takes
+// one element and none is idle at the end of a row (rows of packs as above, 3,000,000
+// x 33: 788 us to float-float, 590 back, against 709 and 533).
+template <typename S, typename T>
+__global__ void __launch_bounds__(256) k_convert_each(const S* s, int64_t lds, T* d, int64_t ldd, int64_t D, int n) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= D * n) return;
+  const int64_t i = t / n;
+  const int j = (int)(t % n);
+  T o;
+  convert(s[i * lds + j], o);
+  d[i * ldd + j] = o;
+}
+
 template <typename S, typename T, int W>
 bool packs(const S* s, int64_t lds, const T* d, int64_t ldd, int n) {
   return n % W == 0 && lds % W == 0 && ldd % W == 0 && (uintptr_t)s % alignof(Pack<S, W>) == 0 &&
@@ -496,9 +507,21 @@ fd_status convert_block(fd_ctx* ctx, const S* s, int64_t lds, T* d, int64_t ldd,
   constexpr int W = sizeof(S) == 4 || sizeof(T) == 4 ? 4 : 2;
   const int w = packs<S, T, W>(s, lds, d, ldd, n) ? W : 1;
   const int64_t q = n / w, per = q < 256 ? 256 / q : 1;
-  const unsigned grid = (unsigned)cdiv(D, per * 4);
-  if (w == W) k_convert<S, T, W><<<grid, 256, 0, ctx->stream>>>(s, lds, d, ldd, D, n);
-  else k_convert<S, T, 1><<<grid, 256, 0, ctx->stream>>>(s, lds, d, ldd, D, n);
+  const unsigned wide = q < 256 ? 1 : (unsigned)std::min<int64_t>(cdiv(q, 256), 65535);  // CTAs along a row
+  // four rows per thread where that leaves every SM eight CTAs; small blocks are
+  // spread over more of them (50 x 5,000, FP64 -> FP32: 8.3 -> 4.2 us)
+  const bool deep = cdiv(D, per * 4) * wide >= 8LL * ctx->num_sms;
+  const dim3 grid((unsigned)cdiv(D, per * (deep ? 4 : 1)), wide);
+  auto kernel = w == W ? deep ? k_convert<S, T, W, 4> : k_convert<S, T, W, 1>
+                       : deep ? k_convert<S, T, 1, 4> : k_convert<S, T, 1, 1>;
+  kernel<<<grid, 256, 0, ctx->stream>>>(s, lds, d, ldd, D, n);
+  FD_LAUNCHED(ctx);
+  return FD_OK;
+}
+
+template <typename S, typename T>
+fd_status convert_each(fd_ctx* ctx, const S* s, int64_t lds, T* d, int64_t ldd, int64_t D, int n) {
+  k_convert_each<<<(unsigned)cdiv(D * n, 256), 256, 0, ctx->stream>>>(s, lds, d, ldd, D, n);
   FD_LAUNCHED(ctx);
   return FD_OK;
 }
@@ -754,13 +777,13 @@ fd_status copy_cols_f32_to_f64(fd_ctx* ctx, const float* src, int64_t lds, doubl
 }
 fd_status copy_cols_f64_to_ff(fd_ctx* ctx, const double* src, int64_t lds, float* dst, int64_t ldd,
                               int64_t D, int n) {
-  if ((uintptr_t)dst & 7) return convert_block(ctx, src, lds, reinterpret_cast<pair_u*>(dst), ldd, D, n);
-  return convert_block(ctx, src, lds, reinterpret_cast<pair_f*>(dst), ldd, D, n);
+  if ((uintptr_t)dst & 7) return convert_each(ctx, src, lds, reinterpret_cast<pair_u*>(dst), ldd, D, n);
+  return convert_each(ctx, src, lds, reinterpret_cast<pair_f*>(dst), ldd, D, n);
 }
 fd_status copy_cols_ff_to_f64(fd_ctx* ctx, const float* src, int64_t lds, double* dst, int64_t ldd,
                               int64_t D, int n) {
-  if ((uintptr_t)src & 7) return convert_block(ctx, reinterpret_cast<const pair_u*>(src), lds, dst, ldd, D, n);
-  return convert_block(ctx, reinterpret_cast<const pair_f*>(src), lds, dst, ldd, D, n);
+  if ((uintptr_t)src & 7) return convert_each(ctx, reinterpret_cast<const pair_u*>(src), lds, dst, ldd, D, n);
+  return convert_each(ctx, reinterpret_cast<const pair_f*>(src), lds, dst, ldd, D, n);
 }
 
 }  // namespace fdi
@@ -827,7 +850,7 @@ fd_status fd_copy_block(fd_ctx* ctx, const void* src, fd_prec sp, int64_t lds, v
   if (sp == FD_F32) return convert_block(ctx, (const float*)src, lds, (float*)dst, ldd, D, n);
   // a float-float block may start at any float, between the 8-byte boundaries too
   if (((uintptr_t)src | (uintptr_t)dst) & 7)
-    return convert_block(ctx, (const pair_u*)src, lds, (pair_u*)dst, ldd, D, n);
+    return convert_each(ctx, (const pair_u*)src, lds, (pair_u*)dst, ldd, D, n);
   return convert_block(ctx, (const double*)src, lds, (double*)dst, ldd, D, n);  // float-float pairs: 8 bytes too
 }
 

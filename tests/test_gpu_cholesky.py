@@ -61,11 +61,20 @@ for ns in (726, 727, 768, 769, 1024):
 @pytest.mark.parametrize("pad,shift", [(0, 0), (2, 2), (3, 1), (4, 0)])
 def test_copy_block_widths(n, pad, shift):
     """Type conversions at widths and alignments with and without wide accesses."""
+    _copies(67, n, pad, shift)
+
+
+@pytest.mark.parametrize("D,n", [(1, 1), (3, 5000), (50, 1021), (20011, 7), (9731, 130), (3000, 1025)])
+def test_copy_block_splits(D, n):
+    """One and four rows per thread, several thread blocks along a row."""
+    _copies(D, n, 1, 0)
+
+
+def _copies(D, n, pad, shift):
     import torch
 
     import paper_2209_01974_gb300 as fd
     ctx = fd.fd_create(0)
-    D = 67
     src = torch.from_numpy(fd_inputs.random_block(D, n, n)).cuda()
     big = torch.zeros((D, n + pad + shift), dtype=torch.float64, device="cuda")
     v64 = big[:, shift:shift + n]
