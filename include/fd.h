@@ -250,8 +250,8 @@ fd_status fd_check_bounded_wait(fd_ctx* ctx, int limit_us);
 fd_status fd_gram(fd_ctx* ctx, const double* X, int64_t ldx, const double* Y, int64_t ldy,
                   int64_t D, int m, int n, double* C, int ldc);
 /* In-place rotation V <- V M (device; V: D x n with ldv, M: n x n row-major;
- * upper != 0: M is upper triangular and its lower part is not read).  After
- * FD_ERR_TIMEOUT V holds old and new rows. */
+ * upper != 0: M is upper triangular and its lower part is not used, whatever
+ * it holds).  After FD_ERR_TIMEOUT V holds old and new rows. */
 fd_status fd_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const double* M,
                     int upper);
 

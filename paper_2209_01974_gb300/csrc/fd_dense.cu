@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "fd_internal.cuh"
@@ -143,23 +144,33 @@ __global__ void __launch_bounds__(256)
     int col[COLS];
 #pragma unroll
     for (int v = 0; v < COLS; ++v) col[v] = min(cb + c0 + LANES * v, n - 1);  // beyond n: not stored
-    int k = 0;
-    for (; k + 4 <= kend; k += 4) {
-      double m[4][COLS];
+    // rows k0 .. k1 of M; TRI: the diagonal block of an upper M, of which what is stored
+    // below the diagonal does not enter
+    auto add_rows = [&](auto tri, int k, int k1) {
+      constexpr bool TRI = decltype(tri)::value;
+      for (; k + 4 <= k1; k += 4) {
+        double m[4][COLS];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v < COLS; ++v) m[u][v] = __ldg(M + (int64_t)(k + u) * n + col[v]);
+          for (int v = 0; v < COLS; ++v) m[u][v] = TRI && k + u > col[v] ? 0.0 : __ldg(M + (int64_t)(k + u) * n + col[v]);
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < COLS; ++v)
+            if (v < nv) acc[v] = fma(vr[k + u], m[u][v], acc[v]);
+      }
+      for (; k < k1; ++k)
 #pragma unroll
         for (int v = 0; v < COLS; ++v)
-          if (v < nv) acc[v] = fma(vr[k + u], m[u][v], acc[v]);
+          if (v < nv) acc[v] = fma(vr[k], TRI && k > col[v] ? 0.0 : __ldg(M + (int64_t)k * n + col[v]), acc[v]);
+    };
+    if (upper) {
+      add_rows(std::false_type{}, 0, cb);
+      add_rows(std::true_type{}, cb, kend);
+    } else {
+      add_rows(std::false_type{}, 0, kend);
     }
-    for (; k < kend; ++k)
-#pragma unroll
-      for (int v = 0; v < COLS; ++v)
-        if (v < nv) acc[v] = fma(vr[k], __ldg(M + (int64_t)k * n + col[v]), acc[v]);
     if (r < nr) {
 #pragma unroll
       for (int v = 0; v < COLS; ++v) {

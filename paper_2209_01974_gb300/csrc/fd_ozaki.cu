@@ -451,8 +451,9 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 // flight per thread.  Maxima of |x| as 64-bit integers (the bit patterns of
 // non-negative doubles order like their values, NaN above inf): integer
 // instructions instead of GB300's slow FP64 ones.
+// UPPER: X is upper triangular, and what is stored below its diagonal does not enter.
 constexpr int CM_COLS = 128, CM_ROWS = 4, CM_UNROLL = 8;
-template <bool VEC>
+template <bool VEC, bool UPPER>
 __global__ void __launch_bounds__(256) k_col_maxabs(const double* __restrict__ X, int64_t ld, int64_t D, int n,
                                                     double* part, int* bad) {
   __shared__ unsigned long long red[CM_ROWS][CM_COLS];
@@ -477,6 +478,8 @@ __global__ void __launch_bounds__(256) k_col_maxabs(const double* __restrict__ X
             v[u].x = __ldg(p);
             if (two) v[u].y = __ldg(p + 1);
           }
+          if (UPPER && ru > c) v[u].x = 0.0;
+          if (UPPER && ru > c + 1) v[u].y = 0.0;
         }
       }
 #pragma unroll
@@ -522,6 +525,7 @@ __global__ void k_col_exp(const double* part, int nb, int n, int* ex) {
 //   row-scaled operand (rotation V), D rows over K = n columns:
 //     block (rb, kc, s) of 128 rows x 16 k at ((rb * nkc + kc) * 8 + s) * 2048
 // ---------------------------------------------------------------------------
+template <bool UPPER>
 __global__ void k_digits_cols(const double* __restrict__ X, int64_t ld, int64_t D, int w, int wpad,
                               const int* ex, int64_t nkc, __nv_bfloat16* __restrict__ Xd) {
   const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -531,7 +535,7 @@ __global__ void k_digits_cols(const double* __restrict__ X, int64_t ld, int64_t 
   const int64_t k0 = 8 * g, kc = g >> 1;
   double x[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) x[q] = (c < w && k0 + q < D) ? X[(k0 + q) * ld + c] : 0.0;
+  for (int q = 0; q < 8; ++q) x[q] = (c < w && k0 + q < D && !(UPPER && k0 + q > c)) ? X[(k0 + q) * ld + c] : 0.0;
   const int ncb = wpad / 64;
   unsigned char* blk = reinterpret_cast<unsigned char*>(Xd + (kc * 8 * ncb + (c >> 6)) * B_ELEMS);
   const int off = core_offset(c & 63, (int)(k0 & 15));
@@ -857,30 +861,33 @@ bool digit_workspace(fd_ctx* ctx, const char* name, size_t bytes, __nv_bfloat16*
   return true;
 }
 
-// column-scaled digits of a D x w operand (K = D rows, padded to 16)
+// column-scaled digits of a D x w operand (K = D rows, padded to 16; upper: of its
+// upper triangle)
 fd_status cut_cols(fd_ctx* ctx, const double* X, int64_t ld, int64_t D, int w, const int* ex,
-                   __nv_bfloat16* Xd, int64_t nkc) {
+                   __nv_bfloat16* Xd, int64_t nkc, bool upper = false) {
   const int wpad = (int)cdiv(w, TM) * TM;
   const int64_t items = nkc * 2 * wpad;
-  k_digits_cols<<<(unsigned)cdiv(items, 256), 256, 0, ctx->stream>>>(X, ld, D, w, wpad, ex, nkc, Xd);
+  auto kernel = upper ? k_digits_cols<true> : k_digits_cols<false>;
+  kernel<<<(unsigned)cdiv(items, 256), 256, 0, ctx->stream>>>(X, ld, D, w, wpad, ex, nkc, Xd);
   FD_LAUNCHED(ctx);
   return FD_OK;
 }
 
 }  // namespace
 
-// Column exponents of X (n columns over D rows); non-finite values raise *bad.
+// Column exponents of X (n columns over D rows; upper: of its upper triangle);
+// non-finite values raise *bad.
 static fd_status col_exponents(fd_ctx* ctx, const double* X, int64_t ld, int64_t D, int n, int* ex,
-                               int* bad) {
+                               int* bad, bool upper = false) {
   // about eight CTAs per SM, at least one unrolled run of rows each
   const int ct = (int)cdiv(n, CM_COLS);
   const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(8LL * ctx->num_sms, ct), D / (CM_ROWS * CM_UNROLL)));
   void* p;
   FD_TRY(workspace(ctx, "oz_colmax", sizeof(double) * (size_t)nb * n, &p));
-  if (((uintptr_t)X & 15) == 0 && ld % 2 == 0)
-    k_col_maxabs<true><<<dim3(nb, ct), 256, 0, ctx->stream>>>(X, ld, D, n, (double*)p, bad);
-  else
-    k_col_maxabs<false><<<dim3(nb, ct), 256, 0, ctx->stream>>>(X, ld, D, n, (double*)p, bad);
+  const bool vec = ((uintptr_t)X & 15) == 0 && ld % 2 == 0;
+  auto kernel = upper ? vec ? k_col_maxabs<true, true> : k_col_maxabs<false, true>
+                      : vec ? k_col_maxabs<true, false> : k_col_maxabs<false, false>;
+  kernel<<<dim3(nb, ct), 256, 0, ctx->stream>>>(X, ld, D, n, (double*)p, bad);
   FD_LAUNCHED(ctx);
   k_col_exp<<<(unsigned)cdiv(n, 8), 256, 0, ctx->stream>>>((double*)p, nb, n, ex);
   FD_LAUNCHED(ctx);
@@ -962,8 +969,8 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   int* bad = er + D;
   int* err = bad + 1;
   FD_CUDA(ctx, cudaMemsetAsync(bad, 0, 2 * sizeof(int), ctx->stream));
-  FD_TRY(col_exponents(ctx, M, n, n, n, em, bad));
-  FD_TRY(cut_cols(ctx, M, n, n, n, em, Md, npad / KS));
+  FD_TRY(col_exponents(ctx, M, n, n, n, em, bad, upper));
+  FD_TRY(cut_cols(ctx, M, n, n, n, em, Md, npad / KS, upper));
   const size_t rows_smem = sizeof(double) * DR_ROWS * (npad + 2);  // 65.7 KB at the widest, n = 1024
   const bool vec = ((uintptr_t)V & 15) == 0 && (ldv & 1) == 0;
   auto cut_rows = vec ? k_digits_rows<true> : k_digits_rows<false>;

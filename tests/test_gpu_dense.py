@@ -158,6 +158,27 @@ def test_fp64_rotation_row_splits(fd, ctx, D, n, ld, upper):
     assert np.all(np.abs(got[:, :n] - V @ M) <= bound)
 
 
+@pytest.mark.parametrize("mode", ["fp64", "ozaki"])
+@pytest.mark.parametrize("D,n", [(700, 33), (300, 65), (4000, 130), (8000, 64)])
+@pytest.mark.parametrize("below", [1.0, 1e200, np.nan])
+def test_upper_rotation_leaves_the_lower_part_out(fd, ctx, mode, D, n, below):
+    """An in-place factor: whatever is stored below the diagonal, the product is that of
+    the upper triangle, to the last bit."""
+    rng = np.random.default_rng(n)
+    V, M = rng.standard_normal((D, n)), np.triu(rng.standard_normal((n, n)))
+    full = M + np.tril(np.full((n, n), below), -1)
+    got = []
+    fd.fd_set_gemm_mode(ctx, mode)
+    try:
+        for m in (M, full):
+            v = _t(V)
+            fd.fd_rotate(ctx, v, _t(m), True)
+            got.append(v.cpu().numpy())
+    finally:
+        fd.fd_set_gemm_mode(ctx, "auto")
+    assert np.array_equal(got[0], got[1])
+
+
 @pytest.mark.parametrize("D", [1, 15, 16, 17, 33, 609, 1728])
 @pytest.mark.parametrize("m,n", [(1, 1), (16, 16), (17, 33), (48, 49), (64, 5), (33, 33), (96, 96), (129, 130)])
 def test_fp64_gram_parts(fd, ctx, D, m, n):
