@@ -242,6 +242,11 @@ fd_status fd_debug_set_sell_column(fd_ctx* ctx, fd_matrix* A, int64_t entry, int
  * left behind and the context still usable; the GPU does not fault or hang.
  * Synchronises. */
 fd_status fd_check_bounded_wait(fd_ctx* ctx, int limit_us);
+/* Test hook of the same path inside the products: with from_row_block >= 0, the
+ * rotation's waits for its operands give up at once from that block of 128 rows on,
+ * and all of the Gram product's do (-1: off, the default).  Nothing hangs: the
+ * kernels wait for their own copies in flight, free what they hold and return. */
+fd_status fd_debug_give_up(fd_ctx* ctx, int from_row_block);
 
 /* Gram product C = X^T Y (device; X: D x m with ldx, Y: D x n with ldy, C: m x n
  * row-major with ldc), the tall-skinny contraction of Cholesky-QR and

@@ -93,6 +93,7 @@ _SIGS = {
     "fd_spmmv": (_i32, [_vp, _vp, _i32, _vp, _i64, _vp, _i64, _i32]),
     "fd_set_gemm_mode": (_i32, [_vp, _i32]),
     "fd_check_bounded_wait": (_i32, [_vp, _i32]),
+    "fd_debug_give_up": (_i32, [_vp, _i32]),
     "fd_comm_metrics": (_i32, [_vp, _vp, _i32, ctypes.POINTER(ctypes.c_int64),
                                ctypes.POINTER(ctypes.c_int64), _pd]),
     "fd_gram": (_i32, [_vp, _vp, _i64, _vp, _i64, _i64, _i32, _i32, _vp, _i32]),
@@ -337,6 +338,11 @@ def fd_check_bounded_wait(ctx, limit_us=100000):
     """The bounded-wait diagnostic; returns its fd_status (FD_ERR_TIMEOUT when the
     wait gave up as designed) instead of raising."""
     return _lib.fd_check_bounded_wait(ctx.handle, int(limit_us))
+
+
+def fd_debug_give_up(ctx, from_row_block=-1):
+    """Test hook: waits of the tensor-core products give up from this row block on (-1: off)."""
+    _check(ctx, _lib.fd_debug_give_up(ctx.handle, int(from_row_block)))
 
 
 def fd_comm_metrics(ctx, A, n_p):

@@ -19,6 +19,7 @@ struct fd_ctx {
   size_t smem_optin = 0;
   std::string err;
   int64_t launches = 0;
+  int give_up_from = -1;  // fd_debug_give_up
   int gemm_mode = 0;  // fd_gemm_mode: 0 auto, 1 FP64 arithmetic, 2 bf16 tensor-core splitting
   // grow-only device workspaces keyed by purpose
   std::unordered_map<std::string, std::pair<void*, size_t>> ws;

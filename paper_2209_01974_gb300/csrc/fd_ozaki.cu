@@ -42,6 +42,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 
 #include "fd_internal.cuh"
@@ -66,6 +67,7 @@ constexpr int STAGE = OZ_S * (A_SLICE + B_SLICE);     // 49,152 bytes
 constexpr int CM_K = 128;                             // K-adjacent core matrices (LBO)
 constexpr int CM_MN = (KS / 8) * 128;                 // MN-adjacent 8-row groups (SBO) = 256
 constexpr size_t OZ_SMEM = (size_t)NST * STAGE + 2 * NST * 8 + 16;  // + barriers, TMEM address
+constexpr size_t LEAVE_BAR = OZ_SMEM - 8;             // barrier of the exit after a timeout
 constexpr int64_t OZ_MAX_CHUNKS = 1 << 16;            // per CTA, keeps the accumulators exact
 constexpr unsigned TMEM_COLS = 512;                   // 8 levels x 64 columns
 constexpr int P_THREAD = 0;                           // bulk-copy producer (warp 0, lanes 0-15)
@@ -93,9 +95,12 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)));
 }
 
+constexpr long long WAIT_CYCLES = 4000000000ll;  // about 2 s at 2 GHz
+constexpr long long DRAIN_CYCLES = 200000000ll;  // 0.1 s
+
 // bounded wait for the completion of the barrier phase with the given parity;
-// gives up after `limit` SM clock cycles (default about 2 s at 2 GHz)
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = 4000000000ll) {
+// gives up after `limit` SM clock cycles
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = WAIT_CYCLES) {
   const long long t0 = clock64();
   for (;;) {
     uint32_t done;
@@ -264,13 +269,31 @@ __device__ __forceinline__ void flush(uint32_t tmem, Acc (&acc)[16]) {
   }
 }
 
+// Before a CTA leaves after a wait that gave up: wait (again with a limit) for the bulk
+// copies that it has posted (`loaded` K steps since the ring began), which would otherwise
+// arrive in the shared memory of the next CTA, and for the MMAs that it has issued,
+// which write TMEM.
+__device__ __forceinline__ void drain(unsigned char* smem, uint64_t* full, uint32_t loaded) {
+  if (threadIdx.x == P_THREAD)
+    for (uint32_t i = loaded > NST ? loaded - NST : 0; i < loaded; ++i)
+      mbar_wait(&full[i % NST], (i / NST) & 1u, DRAIN_CYCLES);
+  if (threadIdx.x == M_THREAD) {
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + LEAVE_BAR);
+    mbar_init(bar);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    umma_commit(bar);  // all MMAs before it
+    mbar_wait(bar, 0, DRAIN_CYCLES);
+  }
+  __syncthreads();
+}
+
 // The product pipeline of one CTA.  K step sc reads digit block (sc, s) of A
 // at A + sc a_kc + s a_s and of B likewise (bf16 elements).  Returns false if
 // a bounded wait gave up (the same answer in every thread).
 __device__ __forceinline__ bool run_tile(unsigned char* smem, uint64_t* full, uint64_t* empty, uint32_t tmem,
                                          const __nv_bfloat16* A, int64_t a_kc, int64_t a_s,
                                          const __nv_bfloat16* B, int64_t b_kc, int64_t b_s, int nsub,
-                                         Acc (&acc)[16]) {
+                                         bool give_up, Acc (&acc)[16]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // producer warp: lane 0 posts the stage's byte count, lanes 0-15 issue one
   // bulk copy each (slice lane / 2 of A or B)
@@ -287,9 +310,10 @@ __device__ __forceinline__ bool run_tile(unsigned char* smem, uint64_t* full, ui
         bulk_g2s(dst + s * A_SLICE, A + sc * a_kc + s * a_s, A_SLICE, &full[st]);
     }
   };
-  bool ok = true;
+  bool ok = !give_up;
+  uint32_t loaded = 0;  // K steps posted by the producer warp
   if (warp == P_THREAD / 32)
-    for (int sc = 0; sc < nsub && sc < NST; ++sc) load(sc);
+    for (; loaded < (uint32_t)nsub && loaded < NST; ++loaded) load((int)loaded);
   for (int sc = 0; sc < nsub; ++sc) {
     const int st = sc % NST;
     const uint32_t par = (uint32_t)(sc / NST) & 1u;
@@ -307,12 +331,18 @@ __device__ __forceinline__ bool run_tile(unsigned char* smem, uint64_t* full, ui
     if (warp == P_THREAD / 32 && ok && sc + NST < nsub) {
       // the stage is free again once the MMAs of K step sc have completed
       ok = mbar_wait(&empty[st], par);
-      if (ok) load(sc + NST);
+      if (ok) {
+        load(sc + NST);
+        ++loaded;
+      }
     }
     if ((sc % SUBS) == SUBS - 1 || sc == nsub - 1) {
       // the issuer observes the completion; the others sleep in the barrier
       if (threadIdx.x == M_THREAD && ok) ok = mbar_wait(&empty[st], par);
-      if (__syncthreads_or(!ok)) return false;
+      if (__syncthreads_or(!ok)) {
+        drain(smem, full, loaded);
+        return false;
+      }
       tc_fence_after();
       flush(tmem, acc);
       tc_fence_before();
@@ -611,7 +641,7 @@ __global__ void __launch_bounds__(256) k_digits_rows(const double* __restrict__ 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gram(const __nv_bfloat16* __restrict__ Xd, int ncbx, const __nv_bfloat16* __restrict__ Yd, int ncby,
               int64_t nkc, int m, int n, int ntj, int sym, int64_t kc_per_slice, const int* ex,
-              const int* ey, double* __restrict__ P, int* err) {
+              const int* ey, double* __restrict__ P, bool give_up, int* err) {
   extern __shared__ __align__(128) unsigned char smem[];
   int t = blockIdx.x, ti = 0, tj;
   if (sym) {
@@ -637,7 +667,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   const int64_t a_kc = 8LL * ncbx * B_ELEMS, a_s = (int64_t)ncbx * B_ELEMS;
   const int64_t b_kc = 8LL * ncby * B_ELEMS, b_s = (int64_t)ncby * B_ELEMS;
   const bool ok = run_tile(smem, full, empty, tmem, Xd + kc0 * a_kc + (int64_t)(2 * ti) * B_ELEMS, a_kc, a_s,
-                           Yd + kc0 * b_kc + (int64_t)tj * B_ELEMS, b_kc, b_s, nsub, acc);
+                           Yd + kc0 * b_kc + (int64_t)tj * B_ELEMS, b_kc, b_s, nsub, give_up, acc);
   if (!ok) {
     if (threadIdx.x == 0) atomicExch(err, 1);
   } else {
@@ -690,7 +720,7 @@ template <int STORE>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_rotate(const __nv_bfloat16* __restrict__ Vd, const __nv_bfloat16* __restrict__ Md, int ncbm,
                 int64_t D, int n, int npad, int nrb, int upper, const int* er, const int* em,
-                double* __restrict__ Out, int64_t ldo, int* err) {
+                double* __restrict__ Out, int64_t ldo, int give_up_from, int* err) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int njt = npad / TN, per = gridDim.x / njt;  // row blocks in flight
   const int slot = blockIdx.x / njt, col0 = blockIdx.x % njt;
@@ -729,7 +759,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     umma_commit(&empty[st]);
     return true;
   };
-  bool ok = true;
+  bool ok = slot < give_up_from;
   // the next K step to load: tile (lrb, ljt), step ls, stream position lg
   int lrb = slot, ljt = col0, ls = 0;
   uint32_t lg = 0;
@@ -767,6 +797,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         if (threadIdx.x == M_THREAD && ok) ok = mbar_wait(&empty[st], par);
         if (__syncthreads_or(!ok)) {
           if (threadIdx.x == 0) atomicExch(err, 1);
+          drain(smem, full, lg);
           tile_teardown(tmem);
           return;
         }
@@ -777,6 +808,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       }
     }
     g += (uint32_t)nsub;
+    if (rb + per >= give_up_from) ok = false;  // fd_debug_give_up; in the waits themselves it costs 1.5 %
     // the next tile's first K steps, before this one's results are rounded
     ahead = rb + per < nrb ? min(NST, min(steps(next(jt)), SUBS)) : 0;
     if (threadIdx.x == M_THREAD) {
@@ -940,7 +972,8 @@ fd_status oz_gram(fd_ctx* ctx, const double* X, int64_t ldx, const double* Y, in
   FD_TRY(workspace(ctx, "oz_gram_partial", sizeof(double) * slices * m * n, &p));
   double* P = (double*)p;
   k_oz_gram<<<dim3(tiles, (unsigned)slices), OZ_THREADS, OZ_SMEM, ctx->stream>>>(
-      Xd, ncbx, Yd, ncby, nkc, m, n, ntj, sym ? 1 : 0, kps, ex, ey, P, err);
+      Xd, ncbx, Yd, ncby, nkc, m, n, ntj, sym ? 1 : 0, kps, ex, ey, P,
+      ctx->give_up_from >= 0, err);
   FD_LAUNCHED(ctx);
   FD_TRY(check_wait_flag(ctx, err));
   k_oz_gram_reduce<<<(unsigned)cdiv((int64_t)m * n, 256), 256, 0, ctx->stream>>>(P, (int)slices, m, n,
@@ -985,7 +1018,8 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   const int njt = npad / TN, nrb = (int)(Dpad / TM);
   const unsigned grid = (unsigned)(njt * std::max(1, std::min(nrb, ctx->num_sms / njt)));
   auto rot = ((uintptr_t)V & 31) == 0 && ldv % 4 == 0 ? k_oz_rotate<STORE_32> : vec ? k_oz_rotate<STORE_16> : k_oz_rotate<STORE_8>;
-  rot<<<grid, OZ_THREADS, OZ_SMEM, ctx->stream>>>(Vd, Md, ncbm, D, n, npad, nrb, upper ? 1 : 0, er, em, V, ldv, err);
+  rot<<<grid, OZ_THREADS, OZ_SMEM, ctx->stream>>>(Vd, Md, ncbm, D, n, npad, nrb, upper ? 1 : 0, er, em, V, ldv,
+                                              ctx->give_up_from >= 0 ? ctx->give_up_from : INT_MAX, err);
   FD_LAUNCHED(ctx);
   FD_TRY(check_wait_flag(ctx, err));
   *used = true;
@@ -995,6 +1029,13 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
 }  // namespace fdi
 
 using namespace fdi;
+
+extern "C" fd_status fd_debug_give_up(fd_ctx* ctx, int from_row_block) {
+  if (!ctx) return FD_ERR_ARG;
+  ctx->err.clear();
+  ctx->give_up_from = std::max(from_row_block, -1);
+  return FD_OK;
+}
 
 extern "C" fd_status fd_check_bounded_wait(fd_ctx* ctx, int limit_us) {
   if (!ctx) return FD_ERR_ARG;

@@ -129,6 +129,32 @@ def test_bounded_wait_gives_up_and_context_stays_usable(fd, ctx):
     assert np.all(np.abs(C - X.T @ X) <= _bound(X, X))
 
 
+def test_products_whose_waits_give_up_leave_the_gpu_usable(fd, ctx):
+    """Waits that give up in the first tiles, in later ones and in the last: every CTA
+    leaves after its own copies and MMAs, the call reports FD_ERR_TIMEOUT, and the next
+    product is right."""
+    D, n = 128 * 400, 130
+    V, M = _block(D, n, 3, 1), np.random.default_rng(4).standard_normal((n, n))
+    X = _block(20000, 96, 5)
+    fd.fd_set_gemm_mode(ctx, "ozaki")
+    bound = 8 * n * U * np.outer(np.abs(V).max(1), np.abs(M).max(0))
+    for start in (0, 60, 170, 399):
+        Vt, Xt = _t(V), _t(X)
+        fd.fd_debug_give_up(ctx, start)
+        try:
+            for call in (lambda: fd.fd_rotate(ctx, Vt, _t(M)), lambda: fd.fd_gram(ctx, Xt, Xt)):
+                with pytest.raises(fd.FDError) as e:
+                    call()
+                assert e.value.status == fd.FD_ERR_TIMEOUT
+        finally:
+            fd.fd_debug_give_up(ctx, -1)
+        Vt = _t(V)
+        fd.fd_rotate(ctx, Vt, _t(M))
+        assert np.all(np.abs(Vt.cpu().numpy() - V @ M) <= bound)
+        C = fd.fd_gram(ctx, Xt, Xt).cpu().numpy()
+        assert np.all(np.abs(C - X.T @ X) <= _bound(X, X))
+
+
 def test_full_size_gram_and_cholqr2(fd, ctx):
     # the bench's block, 2,097,152 x 384: sampled Gram entries against CPU dot
     # products, then the orthonormality of CholQR2 (tensor-core products) checked
