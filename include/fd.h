@@ -212,13 +212,16 @@ fd_status fd_spmmv(fd_ctx* ctx, const fd_matrix* A, fd_prec prec,
  *                  tensor cores (Ozaki scheme, 8 bf16 digits per operand
  *                  relative to each row / column maximum, FP32 level sums in
  *                  TMEM exact over K chunks of 512, 2 x 64-bit integer
- *                  accumulation): FP64 accuracy at tensor-core speed.  Uses a
- *                  grow-only device workspace of 16 bytes per operand element
- *                  for the digit tiles
+ *                  accumulation): FP64 accuracy at tensor-core speed.  Uses
+ *                  grow-only device workspaces of 16 bytes per operand element
+ *                  for the digit tiles and, in rotations, 8 bytes per element
+ *                  of V for its rows
  *   FD_GEMM_AUTO   Ozaki for D >= 65536 and at least 64 columns, else FP64
  * Inputs holding NaN or infinity always take the FP64 path, and so does a
- * product whose digit workspace cannot be allocated.  A bounded device-side
- * wait that gives up in a tensor-core product returns FD_ERR_TIMEOUT. */
+ * product whose workspaces cannot be allocated.  A bounded device-side wait
+ * that gives up in a tensor-core product returns FD_ERR_TIMEOUT; that product's
+ * block is then as it was before (an orthonormalisation or Rayleigh-Ritz step
+ * may have passed earlier products: V still spans the same space). */
 typedef enum { FD_GEMM_AUTO = 0, FD_GEMM_FP64 = 1, FD_GEMM_OZAKI = 2 } fd_gemm_mode;
 fd_status fd_set_gemm_mode(fd_ctx* ctx, fd_gemm_mode mode);
 
@@ -256,7 +259,7 @@ fd_status fd_gram(fd_ctx* ctx, const double* X, int64_t ldx, const double* Y, in
                   int64_t D, int m, int n, double* C, int ldc);
 /* In-place rotation V <- V M (device; V: D x n with ldv, M: n x n row-major;
  * upper != 0: M is upper triangular and its lower part is not used, whatever
- * it holds).  After FD_ERR_TIMEOUT V holds old and new rows. */
+ * it holds).  FD_ERR_TIMEOUT leaves V as it was. */
 fd_status fd_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const double* M,
                     int upper);
 

@@ -579,12 +579,14 @@ __global__ void k_digits_cols(const double* __restrict__ X, int64_t ld, int64_t 
 // threads side by side cut the same eight columns of the eight rows, so a slice's
 // stores are whole core matrices (128 consecutive bytes, 256 with the K-adjacent
 // one).  One warp per row storing 16 bytes here and there ran at 40 % of the copy
-// bandwidth (2,097,152 x 384: 7.3 ms).
+// bandwidth (2,097,152 x 384: 7.3 ms).  The rows go to `keep` as well (D x ldk, ldk
+// even): the product overwrites V, and a wait that gives up must leave V as it was.
 constexpr int DR_ROWS = 8;
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_digits_rows(const double* __restrict__ V, int64_t ldv, int64_t D, int n,
                                                      int64_t Dpad, int npad, int* er, int* bad,
-                                                     __nv_bfloat16* __restrict__ Vd) {
+                                                     __nv_bfloat16* __restrict__ Vd, double* __restrict__ keep,
+                                                     int64_t ldk) {
   extern __shared__ __align__(16) double rows_sm[];  // 8 x (npad + 2)
   __shared__ int exps[DR_ROWS];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -602,6 +604,7 @@ __global__ void __launch_bounds__(256) k_digits_rows(const double* __restrict__ 
         if (c < n) v.x = __ldg(p);
         if (c + 1 < n) v.y = __ldg(p + 1);
       }
+      if (c < n) __stcs(reinterpret_cast<double2*>(keep + r * ldk + c), v);
     }
     mb = max(mb, max(abs_bits(v.x), abs_bits(v.y)));
     *reinterpret_cast<double2*>(row + c) = v;
@@ -996,6 +999,12 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   if (!digit_workspace(ctx, "oz_digits_m", sizeof(__nv_bfloat16) * (size_t)npad * ncbm * 64 * OZ_S, &Md))
     return FD_OK;
   void* p;
+  const int64_t ldk = n + (n & 1);
+  if (workspace(ctx, "oz_rot_keep", sizeof(double) * (size_t)D * ldk, &p) != FD_OK) {
+    ctx->err.clear();
+    return FD_OK;
+  }
+  double* keep = (double*)p;
   FD_TRY(workspace(ctx, "oz_rot_small", sizeof(int) * ((size_t)n + D + 8), &p));
   int* em = (int*)p;
   int* er = em + n;
@@ -1007,13 +1016,14 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   const size_t rows_smem = sizeof(double) * DR_ROWS * (npad + 2);  // 65.7 KB at the widest, n = 1024
   const bool vec = ((uintptr_t)V & 15) == 0 && (ldv & 1) == 0;
   auto cut_rows = vec ? k_digits_rows<true> : k_digits_rows<false>;
-  cut_rows<<<(unsigned)(Dpad / DR_ROWS), 256, rows_smem, ctx->stream>>>(V, ldv, D, n, Dpad, npad, er, bad, Vd);
+  cut_rows<<<(unsigned)(Dpad / DR_ROWS), 256, rows_smem, ctx->stream>>>(V, ldv, D, n, Dpad, npad, er, bad, Vd, keep, ldk);
   FD_LAUNCHED(ctx);
   int hbad = 0;
   FD_CUDA(ctx, cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   FD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   if (hbad) return FD_OK;  // non-finite input: the FP64 path propagates it
-  // V is no longer read (its digits are): the product goes straight into it
+  // V is no longer read (its digits are): the product goes straight into it.  On a
+  // timeout V gets its rows back from `keep`.
   static_assert(1024 / KS <= 32 * SUBS, "acc_value_small holds 32 exact chunks");
   const int njt = npad / TN, nrb = (int)(Dpad / TM);
   const unsigned grid = (unsigned)(njt * std::max(1, std::min(nrb, ctx->num_sms / njt)));
@@ -1021,7 +1031,11 @@ fd_status oz_rotate(fd_ctx* ctx, double* V, int64_t ldv, int64_t D, int n, const
   rot<<<grid, OZ_THREADS, OZ_SMEM, ctx->stream>>>(Vd, Md, ncbm, D, n, npad, nrb, upper ? 1 : 0, er, em, V, ldv,
                                               ctx->give_up_from >= 0 ? ctx->give_up_from : INT_MAX, err);
   FD_LAUNCHED(ctx);
-  FD_TRY(check_wait_flag(ctx, err));
+  const fd_status done = check_wait_flag(ctx, err);
+  if (done == FD_ERR_TIMEOUT)
+    FD_CUDA(ctx, cudaMemcpy2DAsync(V, sizeof(double) * ldv, keep, sizeof(double) * ldk, sizeof(double) * n, D,
+                                   cudaMemcpyDeviceToDevice, ctx->stream));
+  FD_TRY(done);
   *used = true;
   return FD_OK;
 }

@@ -155,6 +155,27 @@ def test_products_whose_waits_give_up_leave_the_gpu_usable(fd, ctx):
         assert np.all(np.abs(C - X.T @ X) <= _bound(X, X))
 
 
+@pytest.mark.parametrize("n,ld", [(64, 64), (130, 130), (129, 131), (200, 204)])
+@pytest.mark.parametrize("start", [0, 100, 290])
+def test_block_is_kept_when_a_wait_gives_up(fd, ctx, n, ld, start):
+    """A rotation that times out part of the way leaves V, and the columns beside it, as
+    they were."""
+    import torch
+    D = 128 * 300 - 5
+    big = torch.randn((D, ld), dtype=torch.float64, device="cuda")
+    ref = big.clone()
+    M = _t(np.random.default_rng(4).standard_normal((n, n)))
+    fd.fd_set_gemm_mode(ctx, "ozaki")
+    fd.fd_debug_give_up(ctx, start)
+    try:
+        with pytest.raises(fd.FDError) as e:
+            fd.fd_rotate(ctx, big[:, :n], M)
+    finally:
+        fd.fd_debug_give_up(ctx, -1)
+    assert e.value.status == fd.FD_ERR_TIMEOUT
+    assert torch.equal(big, ref)
+
+
 def test_full_size_gram_and_cholqr2(fd, ctx):
     # the bench's block, 2,097,152 x 384: sampled Gram entries against CPU dot
     # products, then the orthonormality of CholQR2 (tensor-core products) checked
