@@ -6,14 +6,15 @@
 // all matrices run in one cooperative kernel: the CTAs are divided among the
 // matrices, each owns a run of rows, and a step has four grid barriers (two
 // passes of dot products, the norm, the next vector) and no host round trip.  64
-// threads of a CTA go along the rows and four such sets along the vectors: FP64
-// adds issue at one warp in 64 clocks, so a CTA's sums are combined by a
-// halving exchange (9 adds for 8 sums over a warp instead of 40).
+// threads of a CTA go along the rows and four such sets along the vectors (along the
+// rows too while there are fewer tiles of vectors than sets): FP64 adds issue at one
+// warp in 64 clocks, so a CTA's sums are combined by a halving exchange (9 adds for 8
+// sums over a warp instead of 40).
 // The tridiagonal matrix (at most 1000 x 1000) is diagonalised on the host by
 // implicit QL with the last components of the eigenvectors alone carried along.
-// Measured: 20 steps on 110,592 rows 4.4 -> 1.1 ms; 50 steps on each of twelve
-// matrices of 1,000 to 2,744 rows 89 (device time, without the 600 host round
-// trips) -> 2.1 ms.
+// Measured against a kernel per operation: 20 steps on 110,592 rows 4.6 -> 0.9 ms, on
+// 2,097,152 11.6 -> 8.8; 50 steps on each of twelve matrices of 1,000 to 2,744 rows 89
+// (device time, without the 600 host round trips) -> 2.1 ms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -31,6 +32,11 @@ namespace {
 constexpr int LZ_THREADS = 256;
 constexpr int LZ_ROWS = 64;                       // threads along the rows
 constexpr int LZ_SETS = LZ_THREADS / LZ_ROWS;     // sets along the vectors
+// CTAs per SM for many rows, and the rows per SM of each: one CTA has too few loads
+// under way to stream the vectors (2.1M rows, 20 steps: 24.1 ms with one per SM, 8.7 with
+// four), but more cost barriers and registers (110,592 rows: 0.98 ms with one, 1.9 with
+// four; 262,144 rows 1.79, 1.57 with two, 2.35 with four)
+constexpr int LZ_PER_SM = 4, LZ_SM_ROWS = 1024;
 constexpr int LZ_TILE = 8;                        // vectors of a set at a time
 constexpr size_t LZ_CHUNK_BYTES = 256u << 20;     // workspace of one launch of several matrices
 
@@ -54,7 +60,9 @@ struct LzArgs {
   double* part;    // 2 x gridDim.x x m_max
 };
 
-__global__ void __launch_bounds__(LZ_THREADS) k_lanczos(LzArgs a) {
+// PER_SM: CTAs that must fit an SM (4: 64 registers)
+template <int PER_SM>
+__global__ void __launch_bounds__(LZ_THREADS, PER_SM) k_lanczos(LzArgs a) {
   cg::grid_group grid = cg::this_grid();
   extern __shared__ double cs[];  // m_max coefficients
   __shared__ double red[LZ_THREADS / 32][LZ_TILE];
@@ -73,11 +81,13 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(LzArgs a) {
     double* P = a.part + ((int64_t)buf * gridDim.x + blockIdx.x) * a.m_max;
     const int tiles = nv ? (nv + LZ_TILE - 1) / LZ_TILE : 1;
     for (int t0 = 0; t0 < tiles; t0 += LZ_SETS) {
-      const int tile = t0 + set;
+      // fewer tiles than sets left: several sets share a tile, each with its own rows
+      const int share = tiles - t0 > 2 ? 1 : tiles - t0 == 2 ? 2 : 4;
+      const int tile = t0 + set / share, part = set % share;
       double x[LZ_TILE] = {};
       if (tile < tiles) {
         const int v0 = tile * LZ_TILE;
-        for (int64_t r = r0 + rt; r < r1; r += LZ_ROWS) {
+        for (int64_t r = r0 + part * LZ_ROWS + rt; r < r1; r += LZ_ROWS * share) {
           const double wr = w[r];
           if (nv) {
 #pragma unroll
@@ -102,9 +112,11 @@ __global__ void __launch_bounds__(LZ_THREADS) k_lanczos(LzArgs a) {
       x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
       if ((lane & 3) == 0) red[warp][lane >> 2] = x[0];
       __syncthreads();
-      if (rt < LZ_TILE && tile < tiles) {
+      if (rt < LZ_TILE && tile < tiles && part == 0) {
         const int v = tile * LZ_TILE + rt;
-        if (v < max(nv, 1)) __stcg(P + v, red[2 * set][rt] + red[2 * set + 1][rt]);
+        double sum = red[2 * set][rt] + red[2 * set + 1][rt];
+        for (int q = 1; q < share; ++q) sum += red[2 * (set + q)][rt] + red[2 * (set + q) + 1][rt];
+        if (v < max(nv, 1)) __stcg(P + v, sum);
       }
       __syncthreads();
     }
@@ -258,7 +270,7 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
            (n == 0 || (total + doubles(first + n)) * sizeof(double) <= LZ_CHUNK_BYTES))
       total += doubles(first + n++);
     auto bytes = [&](int k, size_t t) {
-      return sizeof(double) * (t + 2 * (size_t)ctx->num_sms * steps) + sizeof(LzMatrix) * k + 64;
+      return sizeof(double) * (t + 2 * (size_t)LZ_PER_SM * ctx->num_sms * steps) + sizeof(LzMatrix) * k + 64;
     };
     void* p = nullptr;
     fd_status ws = workspace(ctx, "lanczos", bytes(n, total), &p);
@@ -273,7 +285,7 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
     double* base = (double*)(((uintptr_t)(dm + n) + 15) & ~(uintptr_t)15);
     std::vector<LzMatrix> h(n);
     size_t outs = 0;
-    int64_t rows = 0;
+    int64_t rows = 0, all_rows = 0;
     double* q = base;
     int m_max = 0;
     for (int i = 0; i < n; ++i) {
@@ -287,7 +299,10 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
       m_max = std::max(m_max, L.m);
       outs += 2 * (size_t)L.m + 2;
       rows = std::max(rows, M->D);
+      all_rows += M->D;
     }
+    const int per_sm = (int)std::min<int64_t>(LZ_PER_SM, cdiv(all_rows, (int64_t)LZ_SM_ROWS * ctx->num_sms));
+    const void* kernel = per_sm > 1 ? (const void*)k_lanczos<LZ_PER_SM> : (const void*)k_lanczos<1>;
     double* out = q;  // all outputs together, then the vectors
     q += outs;
     double* o = out;
@@ -303,12 +318,12 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
     a.mat = dm;
     a.n = n;
     a.m_max = m_max;
-    // one CTA per SM at most (co-resident), no more than one per 64 rows
-    a.cpi = (int)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms / n, cdiv(rows, LZ_ROWS)));
+    // co-resident, no more than one CTA per 64 rows
+    a.cpi = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * ctx->num_sms / n, cdiv(rows, LZ_ROWS)));
     a.part = q;
     FD_CUDA(ctx, cudaMemcpyAsync(dm, h.data(), sizeof(LzMatrix) * n, cudaMemcpyHostToDevice, st));
     void* args[] = {&a};
-    FD_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_lanczos, a.cpi * n, LZ_THREADS, args,
+    FD_CUDA(ctx, cudaLaunchCooperativeKernel(kernel, a.cpi * n, LZ_THREADS, args,
                                              sizeof(double) * (size_t)m_max, st));
     FD_LAUNCHED(ctx);
     std::vector<double> ho(outs);

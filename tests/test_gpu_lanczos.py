@@ -27,6 +27,18 @@ def test_bounds_match_oracle(spec, C, sigma, steps):
     assert max(abs(lo - olo), abs(hi - ohi)) <= 1e-9 * (ohi - olo)
 
 
+@pytest.mark.parametrize("spec,steps", [("chain:n=155649,t=1", 9), ("anderson3d:L=56,W=5,seed=1", 20),
+                                        ("chain:n=500003,t=1", 17), ("anderson3d:L=90,W=5,seed=2", 20)])
+def test_many_rows_match_oracle(spec, steps):
+    """Two to four CTAs per SM, with one to three tiles of vectors."""
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    csr = mat.build(spec)
+    lo, hi = fd.fd_spectral_bounds(ctx, fd.fd_build_matrix(ctx, spec), steps, 3)
+    olo, ohi = lanczos.inclusion_interval(csr, steps, 3)
+    assert max(abs(lo - olo), abs(hi - ohi)) <= 1e-9 * (ohi - olo)
+
+
 def test_early_stop_on_an_invariant_subspace():
     import paper_2209_01974_gb300 as fd
     ctx = fd.fd_create(0)
