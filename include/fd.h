@@ -319,7 +319,7 @@ typedef struct {
   int ns;            /* search vectors N_s [nb * ceil(4 N_t / nb)] (Sec. 2: N_s/N_t ~ 4) */
   int max_outer;     /* outer iterations before FD_ERR_NOCONV [60] */
   int n_max;         /* largest filter degree [100000] */
-  int lanczos_steps; /* [20] */
+  int lanczos_steps; /* at most 28,000 (a coefficient per step in shared memory) [20] */
   uint64_t seed;     /* start block: SplitMix64 stream 2 (Lanczos: stream 3) [0] */
   int precision;     /* FD_F64: all-FP64 sweeps; FD_F32: FP32 sweeps until the
                         largest wanted residual reaches 100 u32 |H| or fails to

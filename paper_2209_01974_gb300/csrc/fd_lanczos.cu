@@ -10,8 +10,8 @@
 // rows too while there are fewer tiles of vectors than sets): FP64 adds issue at one
 // warp in 64 clocks, so a CTA's sums are combined by a halving exchange (9 adds for 8
 // sums over a warp instead of 40).
-// The tridiagonal matrix (at most 1000 x 1000) is diagonalised on the host by
-// implicit QL with the last components of the eigenvectors alone carried along.
+// The tridiagonal matrix is diagonalised on the host by implicit QL with the last
+// components of the eigenvectors alone carried along.
 // Measured against a kernel per operation: 20 steps on 110,592 rows 4.6 -> 0.9 ms, on
 // 2,097,152 11.6 -> 8.8; 50 steps on each of twelve matrices of 1,000 to 2,744 rows 89
 // (device time, without the 600 host round trips) -> 2.1 ms.
@@ -258,6 +258,10 @@ bool tridiagonal_ql(std::vector<double>& d, std::vector<double>& e, std::vector<
 fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const* A, int steps,
                                 const uint64_t* seeds, double* lam_l, double* lam_r) {
   cudaStream_t st = ctx->stream;
+  const int64_t step_limit = (int64_t)((ctx->smem_optin - 1024) / sizeof(double));
+  for (int i = 0; i < n_inst; ++i)
+    if (std::min<int64_t>(steps, A[i]->D) > step_limit)
+      return set_err(ctx, FD_ERR_ARG, "more than %lld Lanczos steps", (long long)step_limit);
   for (int first = 0; first < n_inst;) {
     // as many matrices as the workspace chunk holds (at least one)
     auto doubles = [&](int i) {
@@ -301,8 +305,16 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
       rows = std::max(rows, M->D);
       all_rows += M->D;
     }
-    const int per_sm = (int)std::min<int64_t>(LZ_PER_SM, cdiv(all_rows, (int64_t)LZ_SM_ROWS * ctx->num_sms));
+    int per_sm = (int)std::min<int64_t>(LZ_PER_SM, cdiv(all_rows, (int64_t)LZ_SM_ROWS * ctx->num_sms));
     const void* kernel = per_sm > 1 ? (const void*)k_lanczos<LZ_PER_SM> : (const void*)k_lanczos<1>;
+    // a coefficient per step in shared memory
+    const size_t smem = sizeof(double) * (size_t)m_max;
+    if (smem > 32 * 1024) {
+      FD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin - 1024));
+      int fit = 0;
+      FD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, LZ_THREADS, smem));
+      per_sm = std::max(1, std::min(per_sm, fit));
+    }
     double* out = q;  // all outputs together, then the vectors
     q += outs;
     double* o = out;
@@ -323,8 +335,7 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
     a.part = q;
     FD_CUDA(ctx, cudaMemcpyAsync(dm, h.data(), sizeof(LzMatrix) * n, cudaMemcpyHostToDevice, st));
     void* args[] = {&a};
-    FD_CUDA(ctx, cudaLaunchCooperativeKernel(kernel, a.cpi * n, LZ_THREADS, args,
-                                             sizeof(double) * (size_t)m_max, st));
+    FD_CUDA(ctx, cudaLaunchCooperativeKernel(kernel, a.cpi * n, LZ_THREADS, args, smem, st));
     FD_LAUNCHED(ctx);
     std::vector<double> ho(outs);
     FD_CUDA(ctx, cudaMemcpyAsync(ho.data(), out, sizeof(double) * outs, cudaMemcpyDeviceToHost, st));

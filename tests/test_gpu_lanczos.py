@@ -39,6 +39,24 @@ def test_many_rows_match_oracle(spec, steps):
     assert max(abs(lo - olo), abs(hi - ohi)) <= 1e-9 * (ohi - olo)
 
 
+def test_more_steps_than_the_default_shared_memory_holds():
+    """A solve may ask for thousands of steps: 6,200 coefficients are 48.4 KB.  (Two
+    eigenvalues, so that the recurrence itself ends after two steps.)"""
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+
+    def solve(D, steps):
+        csr = (np.arange(D + 1, dtype=np.int64), np.arange(D, dtype=np.int32), np.where(np.arange(D) % 3, 2.0, -1.0))
+        A = fd.fd_matrix_from_csr(ctx, *csr)
+        return fd.fd_solve(ctx, A, 1.9, 2.1, 1, 8, 10, 1e-9, raise_noconv=False, max_outer=1, lanczos_steps=steps)[2]
+    for D in (7000, 200000):    # one and two CTAs per SM
+        res = solve(D, 6200)
+        assert np.allclose((res["lam_l"], res["lam_r"]), (-1.0, 2.0), rtol=0, atol=1e-12)
+    with pytest.raises(fd.FDError) as e:
+        solve(40000, 40000)
+    assert e.value.status == fd.FD_ERR_ARG
+
+
 def test_early_stop_on_an_invariant_subspace():
     import paper_2209_01974_gb300 as fd
     ctx = fd.fd_create(0)
