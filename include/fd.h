@@ -85,11 +85,12 @@ int64_t fd_kernel_launches(const fd_ctx* ctx);
 fd_status fd_workspace_info(const fd_ctx* ctx, size_t* bytes_held, int64_t* allocations);
 /* Cap the bytes the context's workspaces may hold together (0 = no cap, the
  * default).  A workspace that would grow beyond the cap is refused before
- * anything is freed or allocated and the call needing it returns FD_ERR_OOM,
- * exactly as when cudaMalloc fails; the tensor-core products instead fall
- * back to FP64 arithmetic when their digit workspace is refused.  Lets a
- * caller bound the library's memory (and tests inject an allocation failure
- * from the host). */
+ * anything is freed or allocated, exactly as when cudaMalloc fails.  Scratch
+ * that other calls have left behind is then given back, what can do with less
+ * takes less, and the tensor-core products fall back to FP64 arithmetic; a
+ * call that still lacks a workspace returns FD_ERR_OOM.  Lets a caller bound
+ * the library's memory (and tests inject an allocation failure from the
+ * host). */
 fd_status fd_set_workspace_limit(fd_ctx* ctx, size_t limit_bytes);
 
 /* ------------------------------------------------------------------ matrices */

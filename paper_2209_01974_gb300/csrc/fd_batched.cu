@@ -708,6 +708,8 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
     B.ns_max = std::max(B.ns_max, ns[i]);
     B.max_D = std::max<int64_t>(B.max_D, D);
   }
+  const size_t eig_off = (bytes + 255) & ~(size_t)255;  // the eigensolver's tasks and partial sums
+  bytes = eig_off + sizeof(EigTask) * n + sizeof(float) * eig_part_floats(ctx, n);
   FD_CUDA(ctx, cudaMalloc(&B.arena, bytes));
   B.h_inst.resize(n);
   B.h_eig.assign(n, EigTask{});
@@ -775,9 +777,7 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
   B.d_off = (int64_t*)c; c += sizeof(int64_t) * (nta + 1);
   B.d_tdeg = (int*)c; c += sizeof(int) * nta;
   B.d_ntask = (int*)c;
-  void* pe;
-  FD_TRY(workspace(ctx, "batch_eig", sizeof(EigTask) * n + sizeof(float) * eig_part_floats(ctx, n), &pe));
-  B.d_eig = (EigTask*)pe;
+  B.d_eig = (EigTask*)((char*)B.arena + eig_off);
   B.d_eig_part = (float*)(B.d_eig + n);
   FD_CUDA(ctx, cudaMemcpyAsync(B.d_eig, B.h_eig.data(), sizeof(EigTask) * n, cudaMemcpyHostToDevice, ctx->stream));
   B.mu_cap = mu_cap;

@@ -564,10 +564,17 @@ fd_status gram(fd_ctx* ctx, const double* X, int64_t ldx, const double* Y, int64
   // (1,728 x 96 with its reduction: 51 us, 70 us with 64 rows per slice)
   int64_t slices = std::max<int64_t>(1, cdiv(4LL * ctx->num_sms, tiles));
   slices = std::min<int64_t>(slices, std::max<int64_t>(1, cdiv(D, GK)));
-  const int64_t rps = cdiv(cdiv(D, slices), GK) * GK;
+  int64_t rps = cdiv(cdiv(D, slices), GK) * GK;
   slices = std::max<int64_t>(1, cdiv(D, rps));
   void* p;
-  FD_TRY(workspace(ctx, "gram_partial", sizeof(double) * slices * m * n, &p));
+  if (workspace(ctx, "gram_partial", sizeof(double) * slices * m * n, &p, true) != FD_OK) {
+    // refused: slices of four stages or more
+    ctx->err.clear();
+    slices = std::min<int64_t>(slices, std::max<int64_t>(1, cdiv(D, 4 * GK)));
+    rps = cdiv(cdiv(D, slices), GK) * GK;
+    slices = std::max<int64_t>(1, cdiv(D, rps));
+    FD_TRY(workspace(ctx, "gram_partial", sizeof(double) * slices * m * n, &p));
+  }
   double* P = (double*)p;
   dim3 grid(tiles, (unsigned)slices);
   k_gram_partial<<<grid, 256, 0, ctx->stream>>>(X, ldx, Y, ldy, D, m, n, ntj, sym, rps, P);

@@ -242,7 +242,7 @@ fd_status scale_matrix(fd_ctx* ctx, const fd_matrix* M, int n, double alpha, dou
   const double a2 = 2 * alpha, b2 = 2 * beta;
   void* p;
   const int64_t count = M->kron ? M->khops[0] + M->khops[1] + 25 : M->nnz_sell;
-  if (workspace(ctx, "filter_scaled", sizeof(T) * (size_t)count, &p) != FD_OK) {
+  if (workspace(ctx, "filter_scaled", sizeof(T) * (size_t)count, &p, true) != FD_OK) {
     ctx->err.clear();
     return FD_OK;
   }

@@ -113,8 +113,11 @@ fd_status set_err(fd_ctx* ctx, fd_status st, const char* fmt, ...);
     if (s_ != FD_OK) return s_;      \
   } while (0)
 
-// grow-only workspace of at least `bytes` bytes under `name`
-fd_status workspace(fd_ctx* ctx, const char* name, size_t bytes, void** out);
+// Grow-only workspace of at least `bytes` bytes under `name`.  When it is refused,
+// scratch that outlives its call is given back first (trim_workspaces: nobody may
+// hold a pointer into such scratch across another call of this), unless the request
+// is optional: the caller can do with less then.
+fd_status workspace(fd_ctx* ctx, const char* name, size_t bytes, void** out, bool optional = false);
 fd_status host_stage(fd_ctx* ctx, size_t bytes, void** out);
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }

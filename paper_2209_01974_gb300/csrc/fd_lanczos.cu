@@ -273,15 +273,42 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
     while (first + n < n_inst && n < ctx->num_sms &&
            (n == 0 || (total + doubles(first + n)) * sizeof(double) <= LZ_CHUNK_BYTES))
       total += doubles(first + n++);
+    // the launch of the first k of them: co-resident CTAs, no more than one per 64 rows
+    int64_t rows = 0, all_rows = 0;
+    int m_max = 0, cpi = 0;
+    size_t smem = 0;
+    const void* kernel = nullptr;
+    auto plan = [&](int k) -> fd_status {
+      rows = all_rows = 0;
+      m_max = 0;
+      for (int i = first; i < first + k; ++i) {
+        rows = std::max(rows, A[i]->D);
+        all_rows += A[i]->D;
+        m_max = std::max(m_max, (int)std::min<int64_t>(steps, A[i]->D));
+      }
+      int per_sm = (int)std::min<int64_t>(LZ_PER_SM, cdiv(all_rows, (int64_t)LZ_SM_ROWS * ctx->num_sms));
+      kernel = per_sm > 1 ? (const void*)k_lanczos<LZ_PER_SM> : (const void*)k_lanczos<1>;
+      smem = sizeof(double) * (size_t)m_max;  // a coefficient per step
+      if (smem > 32 * 1024) {
+        FD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin - 1024));
+        int fit = 0;
+        FD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, LZ_THREADS, smem));
+        per_sm = std::max(1, std::min(per_sm, fit));
+      }
+      cpi = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * ctx->num_sms / k, cdiv(rows, LZ_ROWS)));
+      return FD_OK;
+    };
     auto bytes = [&](int k, size_t t) {
-      return sizeof(double) * (t + 2 * (size_t)LZ_PER_SM * ctx->num_sms * steps) + sizeof(LzMatrix) * k + 64;
+      return sizeof(double) * (t + 2 * (size_t)cpi * k * m_max) + sizeof(LzMatrix) * k + 64;
     };
     void* p = nullptr;
-    fd_status ws = workspace(ctx, "lanczos", bytes(n, total), &p);
+    FD_TRY(plan(n));
+    fd_status ws = workspace(ctx, "lanczos", bytes(n, total), &p, n > 1);
     if (ws == FD_ERR_OOM && n > 1) {  // a tight workspace limit: one matrix at a time
       n = 1;
       total = doubles(first);
       ctx->err.clear();
+      FD_TRY(plan(n));
       ws = workspace(ctx, "lanczos", bytes(n, total), &p);
     }
     FD_TRY(ws);
@@ -289,9 +316,7 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
     double* base = (double*)(((uintptr_t)(dm + n) + 15) & ~(uintptr_t)15);
     std::vector<LzMatrix> h(n);
     size_t outs = 0;
-    int64_t rows = 0, all_rows = 0;
     double* q = base;
-    int m_max = 0;
     for (int i = 0; i < n; ++i) {
       const fd_matrix* M = A[first + i];
       LzMatrix& L = h[i];
@@ -300,20 +325,7 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
       L.C = M->C;
       L.m = (int)std::min<int64_t>(steps, M->D);
       L.key = fdrng::key(seeds[first + i], fdrng::STREAM_LANCZOS);
-      m_max = std::max(m_max, L.m);
       outs += 2 * (size_t)L.m + 2;
-      rows = std::max(rows, M->D);
-      all_rows += M->D;
-    }
-    int per_sm = (int)std::min<int64_t>(LZ_PER_SM, cdiv(all_rows, (int64_t)LZ_SM_ROWS * ctx->num_sms));
-    const void* kernel = per_sm > 1 ? (const void*)k_lanczos<LZ_PER_SM> : (const void*)k_lanczos<1>;
-    // a coefficient per step in shared memory
-    const size_t smem = sizeof(double) * (size_t)m_max;
-    if (smem > 32 * 1024) {
-      FD_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin - 1024));
-      int fit = 0;
-      FD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, LZ_THREADS, smem));
-      per_sm = std::max(1, std::min(per_sm, fit));
     }
     double* out = q;  // all outputs together, then the vectors
     q += outs;
@@ -330,8 +342,7 @@ fd_status spectral_bounds_batch(fd_ctx* ctx, int n_inst, const fd_matrix* const*
     a.mat = dm;
     a.n = n;
     a.m_max = m_max;
-    // co-resident, no more than one CTA per 64 rows
-    a.cpi = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * ctx->num_sms / n, cdiv(rows, LZ_ROWS)));
+    a.cpi = cpi;
     a.part = q;
     FD_CUDA(ctx, cudaMemcpyAsync(dm, h.data(), sizeof(LzMatrix) * n, cudaMemcpyHostToDevice, st));
     void* args[] = {&a};

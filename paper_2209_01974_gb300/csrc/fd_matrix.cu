@@ -27,15 +27,39 @@ fd_status set_err(fd_ctx* ctx, fd_status st, const char* fmt, ...) {
   return st;
 }
 
-fd_status workspace(fd_ctx* ctx, const char* name, size_t bytes, void** out) {
+// Scratch that no call needs any more once its kernels have run: given back when
+// another workspace is refused
+static bool trim_workspaces(fd_ctx* ctx, const char* except) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  bool any = false;
+  for (const char* name : {"filter_scaled", "solve_wide", "gram_partial", "jacobi", "lanczos", "resid_partial",
+                           "oz_colmax", "oz_gram_partial"}) {
+    auto it = ctx->ws.find(name);
+    if (it == ctx->ws.end() || !it->second.first || it->first == except) continue;
+    if (!any) cudaStreamSynchronize(ctx->stream);  // queued work may use it
+    cudaFree(it->second.first);                    // waits for other streams
+    ctx->ws_bytes -= it->second.second;
+    it->second = {nullptr, 0};
+    any = true;
+  }
+  return any;
+}
+
+fd_status workspace(fd_ctx* ctx, const char* name, size_t bytes, void** out, bool optional) {
   auto& e = ctx->ws[name];
   if (e.second < bytes) {
     size_t b = std::max<size_t>(bytes, 256);
     // a context-level cap (fd_set_workspace_limit) refuses the growth before
     // anything is freed or allocated, exactly like a failed cudaMalloc
-    if (ctx->ws_limit && ctx->ws_bytes - e.second + b > ctx->ws_limit)
+    if (ctx->ws_limit && ctx->ws_bytes - e.second + b > ctx->ws_limit) {
+      if (!optional && trim_workspaces(ctx, name)) return workspace(ctx, name, bytes, out, true);
       return set_err(ctx, FD_ERR_OOM, "workspace '%s' of %zu bytes exceeds the context's limit of %zu bytes",
                      name, b, ctx->ws_limit);
+    }
     if (e.first) {
       // the old buffer may still be used by queued work on the stream
       FD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -49,6 +73,7 @@ fd_status workspace(fd_ctx* ctx, const char* name, size_t bytes, void** out) {
     ctx->ws_allocs++;
     if (err != cudaSuccess) {
       cudaGetLastError();
+      if (!optional && trim_workspaces(ctx, name)) return workspace(ctx, name, bytes, out, true);
       return set_err(ctx, FD_ERR_OOM, "cudaMalloc of %zu bytes for workspace '%s' failed: %s",
                      b, name, cudaGetErrorString(err));
     }

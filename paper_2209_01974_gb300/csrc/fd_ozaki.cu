@@ -916,9 +916,13 @@ static fd_status col_exponents(fd_ctx* ctx, const double* X, int64_t ld, int64_t
                                int* bad, bool upper = false) {
   // about eight CTAs per SM, at least one unrolled run of rows each
   const int ct = (int)cdiv(n, CM_COLS);
-  const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(8LL * ctx->num_sms, ct), D / (CM_ROWS * CM_UNROLL)));
+  int nb = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(8LL * ctx->num_sms, ct), D / (CM_ROWS * CM_UNROLL)));
   void* p;
-  FD_TRY(workspace(ctx, "oz_colmax", sizeof(double) * (size_t)nb * n, &p));
+  if (workspace(ctx, "oz_colmax", sizeof(double) * (size_t)nb * n, &p, true) != FD_OK) {
+    ctx->err.clear();
+    nb = std::min(nb, 4 * ctx->num_sms);
+    FD_TRY(workspace(ctx, "oz_colmax", sizeof(double) * (size_t)nb * n, &p));
+  }
   const bool vec = ((uintptr_t)X & 15) == 0 && ld % 2 == 0;
   auto kernel = upper ? vec ? k_col_maxabs<true, true> : k_col_maxabs<false, true>
                       : vec ? k_col_maxabs<true, false> : k_col_maxabs<false, false>;

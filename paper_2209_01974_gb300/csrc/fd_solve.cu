@@ -198,42 +198,21 @@ static fd_status solve_impl(fd_ctx* ctx, const fd_matrix* A, double a, double b,
   Timer tm(st), ttot(st);
   ttot.start();
 
-  // Columns filtered per call: nb, or the whole block where the matrix is small
-  // enough for the one-launch filter (its panels of columns then fill the chip
-  // together instead of one bundle after the other).
-  const bool f64_sweeps = opt.precision == FD_F64 || (opt.precision == FD_F32 && !ff_sweeps);
-  int w32 = filter_small_pays(ctx, A, FD_F32, ns) ? ns : nb;
-  int w64 = filter_small_pays(ctx, A, ff_sweeps ? FD_FF : FD_F64, ns) ? ns : nb;
-  // workspaces: V, AV (D x ns FP64), W1, W2 (D x w64 FP64); FP32 bundle buffers
+  // workspaces: V, AV (D x ns FP64), W1, W2 (D x nb FP64); FP32 and float-float bundle buffers
   void* p;
   FD_TRY(workspace(ctx, "solve_V", sizeof(double) * D * ns, &p)); double* V = (double*)p;
   FD_TRY(workspace(ctx, "solve_AV", sizeof(double) * D * ns, &p)); double* AV = (double*)p;
-  double *W1 = nullptr, *W2 = nullptr;
-  float *V32 = nullptr, *W132 = nullptr, *W232 = nullptr;
-  float* Vff = nullptr;  // float-float bundle (2 floats per element); its recurrence vectors reuse W1, W2
-  auto filter_buffers = [&]() -> fd_status {
-    if (f64_sweeps || ff_sweeps) {
-      FD_TRY(workspace(ctx, "solve_W", sizeof(double) * 2 * D * w64, &p));
-      W1 = (double*)p;
-      W2 = W1 + D * w64;
-    }
-    if (opt.precision == FD_F32) {
-      FD_TRY(workspace(ctx, "solve_W32", sizeof(float) * 3 * D * w32, &p));
-      V32 = (float*)p; W132 = V32 + D * w32; W232 = W132 + D * w32;
-    }
-    if (ff_sweeps) {
-      FD_TRY(workspace(ctx, "solve_Wff", sizeof(float) * 2 * D * w64, &p));
-      Vff = (float*)p;
-    }
-    return FD_OK;
-  };
-  fd_status ws = filter_buffers();
-  if (ws == FD_ERR_OOM && (w32 > nb || w64 > nb)) {  // a tight workspace limit: bundle by bundle
-    ctx->err.clear();
-    w32 = w64 = nb;
-    ws = filter_buffers();
+  FD_TRY(workspace(ctx, "solve_W", sizeof(double) * 2 * D * nb, &p)); double* W = (double*)p;
+  float *W32 = nullptr, *Wff = nullptr;
+  if (opt.precision == FD_F32) {
+    FD_TRY(workspace(ctx, "solve_W32", sizeof(float) * 3 * D * nb, &p));
+    W32 = (float*)p;
   }
-  FD_TRY(ws);
+  // float-float bundle (2 floats per element); its recurrence vectors take solve_W
+  if (ff_sweeps) {
+    FD_TRY(workspace(ctx, "solve_Wff", sizeof(float) * 2 * D * nb, &p));
+    Wff = (float*)p;
+  }
   FD_TRY(workspace(ctx, "solve_small", sizeof(double) * 2 * ns + sizeof(int) * ns + 64, &p));
   double* th_dev = (double*)p;
   double* rho_dev = th_dev + ns;
@@ -344,18 +323,40 @@ static fd_status solve_impl(fd_ctx* ctx, const fd_matrix* A, double a, double b,
     std::vector<double> mu = filter_coeffs(alpha * wl + beta, alpha * wr + beta, n);
     tm.start();
     double bytes = 0;
-    const int wd = use_f32 ? w32 : w64;
+    // Columns filtered per call: nb, or the whole block where the matrix is small
+    // enough for the one-launch filter (its panels of columns then fill the chip
+    // together instead of one bundle after the other) and a workspace for it is left:
+    // one that another call can take back, so it is asked for before every filter
+    const fd_prec prec = use_f32 ? FD_F32 : ff_sweeps ? FD_FF : FD_F64;
+    int wd = nb;
+    float* Vs = use_f32 ? W32 : Wff;  // the sweep's copy of the bundle
+    void *W1 = W, *W2 = W + D * nb;
+    if (use_f32) {
+      W1 = W32 + D * nb;
+      W2 = W32 + 2 * D * nb;
+    }
+    if (ns > nb && filter_small_pays(ctx, A, prec, ns)) {
+      const size_t blk = (size_t)D * ns * (use_f32 ? 4 : 8);
+      if (workspace(ctx, "solve_wide", (prec == FD_F64 ? 2 : 3) * blk, &p, true) == FD_OK) {
+        wd = ns;
+        W1 = p;
+        W2 = (char*)p + blk;
+        Vs = (float*)((char*)p + 2 * blk);
+      } else {
+        ctx->err.clear();
+      }
+    }
     for (int j = 0; j < ns; j += wd) {
       if (use_f32) {
-        FD_TRY(copy_cols_f64_to_f32(ctx, V + j, ns, V32, wd, D, wd));
-        FD_TRY(filter(ctx, A, FD_F32, V32, wd, wd, n, mu.data(), alpha, beta, W132, W232, wd, &bytes));
-        FD_TRY(copy_cols_f32_to_f64(ctx, V32, wd, V + j, ns, D, wd));
+        FD_TRY(copy_cols_f64_to_f32(ctx, V + j, ns, Vs, wd, D, wd));
+        FD_TRY(filter(ctx, A, prec, Vs, wd, wd, n, mu.data(), alpha, beta, W1, W2, wd, &bytes));
+        FD_TRY(copy_cols_f32_to_f64(ctx, Vs, wd, V + j, ns, D, wd));
       } else if (ff_sweeps) {
-        FD_TRY(copy_cols_f64_to_ff(ctx, V + j, ns, Vff, wd, D, wd));
-        FD_TRY(filter(ctx, A, FD_FF, Vff, wd, wd, n, mu.data(), alpha, beta, W1, W2, wd, &bytes));
-        FD_TRY(copy_cols_ff_to_f64(ctx, Vff, wd, V + j, ns, D, wd));
+        FD_TRY(copy_cols_f64_to_ff(ctx, V + j, ns, Vs, wd, D, wd));
+        FD_TRY(filter(ctx, A, prec, Vs, wd, wd, n, mu.data(), alpha, beta, W1, W2, wd, &bytes));
+        FD_TRY(copy_cols_ff_to_f64(ctx, Vs, wd, V + j, ns, D, wd));
       } else {
-        FD_TRY(filter(ctx, A, FD_F64, V + j, ns, wd, n, mu.data(), alpha, beta, W1, W2, wd, &bytes));
+        FD_TRY(filter(ctx, A, prec, V + j, ns, wd, n, mu.data(), alpha, beta, W1, W2, wd, &bytes));
       }
     }
     res->t_filter += tm.stop_s();

@@ -61,6 +61,83 @@ def test_refused_digit_workspace_falls_back_to_fp64(fd):
     assert np.abs(Q - Qo).max() <= 1e-10
 
 
+# Bytes of workspace that each call needs beside the matrix's own (152 SMs): what it held
+# when every buffer was as small as it can be.  Larger buffers are taken where there
+# is room for them.
+TIGHT = [("solve", "anderson3d:L=8,W=8,seed=1", dict(precision="f64"), 1613184),
+         ("solve", "anderson3d:L=16,W=8,seed=1", dict(precision="f64"), 8717888),
+         ("solve", "anderson3d:L=16,W=8,seed=1", dict(precision="f32", finish="ff"), 10028608),
+         ("solve", "anderson3d:L=20,W=8,seed=1", dict(precision="ff"), 17427520),
+         ("solve", "anderson3d:L=20,W=8,seed=1", dict(precision="f32"), 17939520),
+         ("solve", "anderson3d:L=32,W=8,seed=1", dict(precision="ff"), 69356608),
+         ("solve", "anderson3d:L=44,W=8,seed=1", dict(precision="f64"), 523515008),
+         ("solve", "hubbard:n_sites=10,n_up=5,n_dn=5,t=1,U=4,bc=periodic,kron=1", dict(precision="ff"), 119864032),
+         ("solve", "roadgraph:side=100,q=0.3,seed=1", dict(precision="f64"), 20365376),
+         ("bounds", "anderson3d:L=8,W=8,seed=1", 20, 146816), ("bounds", "anderson3d:L=64,W=8,seed=1", 20, 46242368),
+         ("bounds", "anderson3d:L=8,W=8,seed=1", 200, 3110336), ("bounds", "anderson3d:L=24,W=8,seed=1", 200, 24705728),
+         ("ortho", "anderson3d:L=12,W=8,seed=1", 64, 1015872), ("ortho", "anderson3d:L=48,W=8,seed=1", 128, 369903232),
+         ("ritz", "anderson3d:L=8,W=8,seed=1", 16, 125248), ("ritz", "anderson3d:L=12,W=8,seed=1", 64, 1393728),
+         ("ritz", "anderson3d:L=16,W=8,seed=1", 96, 5588544), ("ritz", "anderson3d:L=48,W=8,seed=1", 128, 597184128),
+         ("ritz", "anderson3d:L=64,W=8,seed=1", 256, 2744556672), ("lehmann", "anderson3d:L=16,W=8,seed=1", 96, 11634304),
+         ("lehmann", "anderson3d:L=64,W=8,seed=1", 256, 3279657120),
+         ("batch", "anderson3d:L=8,W=8,seed=1", 3, 150484), ("batch", "anderson3d:L=24,W=8,seed=1", 3, 2501716)]
+
+
+@pytest.mark.parametrize("call,spec,arg,room", TIGHT)
+def test_calls_within_the_least_workspace(fd, call, spec, arg, room):
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the figures are those of 152 SMs")
+    ctx = fd.fd_create(0)
+    A = fd.fd_build_matrix(ctx, spec)
+    if call in ("ortho", "ritz", "lehmann"):
+        V0 = torch.linalg.qr(torch.randn((A.D, arg), dtype=torch.float64, device="cuda"))[0].contiguous()
+    limit = ctx.workspace[0] + room
+    fd.fd_set_workspace_limit(ctx, limit)
+    for _ in range(2):
+        if call == "solve":
+            fd.fd_solve(ctx, A, 0.9, 1.1, 16, 16, 60, 1e-9, raise_noconv=False, max_outer=3, n_max=300, **arg)
+        elif call == "bounds":
+            fd.fd_spectral_bounds(ctx, A, arg, 0)
+        elif call == "ortho":
+            assert fd.fd_orthonormalize(ctx, V0.clone()) == 2
+        elif call == "ritz":
+            fd.fd_rayleigh_ritz(ctx, A, V0.clone(), torch.empty_like(V0))
+        elif call == "lehmann":
+            fd.fd_lehmann_bounds(ctx, A, V0, 0.1)
+        else:
+            fd.fd_solve_batched(ctx, [A] * arg, [(-0.01, 0.01, 8, i) for i in range(arg)], 8, 60, 1e-9,
+                                raise_noconv=False, max_outer=3, n_max=100)
+        assert ctx.workspace[0] <= limit
+
+
+def test_scratch_of_one_call_makes_room_for_another(fd):
+    """The scaled matrix of a filter and the buffers of a solve's whole-block filter are
+    extras: the orthonormalisation after them has the workspace that it has without."""
+    import torch
+    ctx = fd.fd_create(0)
+    A = fd.fd_build_matrix(ctx, "anderson3d:L=48,W=8,seed=1")     # 110,592 rows
+    B = fd.fd_build_matrix(ctx, "anderson3d:L=12,W=8,seed=1")
+    V = _t(fd_inputs.random_block(20000, 96, 1))
+    fd.fd_orthonormalize(ctx, V)
+    plain = ctx.workspace[0]
+    X = torch.randn((A.D, 8), dtype=torch.float64, device="cuda")
+    W1, W2 = torch.empty_like(X), torch.empty_like(X)
+    mu = fd.fd_filter_coeffs(-0.1, 0.1, 20)
+
+    c2 = fd.fd_create(0)
+    fd.fd_set_workspace_limit(c2, plain)
+    Y, Z = X.clone(), X.clone()
+    fd.fd_filter(c2, A, Y, mu, 0.1, 0.0, W1, W2)
+    held = c2.workspace[0]
+    assert held > 0                                              # the scaled matrix
+    fd.fd_orthonormalize(c2, _t(fd_inputs.random_block(20000, 96, 1)))
+    fd.fd_filter(c2, A, Z, mu, 0.1, 0.0, W1, W2)                 # with or without it
+    assert torch.linalg.norm(Y - Z) <= 1e-13 * torch.linalg.norm(Y)
+    fd.fd_solve(c2, B, 0.9, 1.1, 4, 8, 60, 1e-9, raise_noconv=False, max_outer=2)
+    assert c2.workspace[0] <= plain
+
+
 def test_too_narrow_inclusion_interval_is_widened(fd):
     # the 8-site chain's spectrum is [-4.2358, 20.2358]; starting from
     # [-4, 19] misses both ends: Ritz values outside widen the interval and the
