@@ -460,10 +460,12 @@ typedef struct {
  * instance, instances of different sizes).  Each outer iteration of all
  * unconverged instances runs as one CUDA graph: one persistent cooperative
  * kernel applies the Chebyshev filters of every bundle of every instance (all
- * degree steps, a grid-wide barrier between steps; instances whose panels fit the
- * shared memory of a few SMs take one cluster per panel), batched Cholesky-QR and
+ * degree steps, a grid-wide barrier between steps), batched Cholesky-QR and
  * Rayleigh-Ritz kernels cover all instances per launch, and all Ritz values
- * and residuals are copied to the host once.  Instances drop out when they
+ * and residuals are copied to the host once.  Where all matrices of the batch
+ * fit the shared memory of a cluster of up to eight SMs, iterations that are
+ * estimated to be faster that way take one cluster per column panel through
+ * all its steps instead.  Instances drop out when they
  * converge.  The per-instance intervals and degrees follow fd_solve's
  * heuristic.  Matrices must be built with sigma = 1; N_s per instance (opt->ns
  * or nb ceil(4 n_target / nb)) must be at most 96; nb in {2, ..., 64}.
@@ -481,10 +483,11 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
                            double* resid);
 
 /* Autotuner of the batched filter: for the matrices given by n_inst spec
- * strings, times the persistent batched filter (degree `probe_degree`, FP64)
- * for every combination of block width nb in {8, 16, 32, 64} (with N_s =
+ * strings, times the batched filter (degree `probe_degree`, FP64) for every
+ * combination of block width nb in {8, 16, 32, 64} (with N_s =
  * nb ceil(4 n_target / nb) <= 96), SELL chunk height C in {32, 64, 128} and
- * CTA shape (4 or 8 warps), and returns the fastest with its throughput in
+ * CTA shape of the persistent kernel (4 or 8 warps; 8 where the filter runs as
+ * column panels), and returns the fastest with its throughput in
  * algorithmic GB/s (Eq. EstimateT bytes).  Builds and frees its own matrices. */
 fd_status fd_tune_batched(fd_ctx* ctx, int n_inst, const char* const* specs, int n_target,
                           int probe_degree, int* nb, int* C, int* cta_warps, double* gbs);

@@ -1,15 +1,21 @@
 // Batched filter diagonalization: many independent, unevenly sized problems
 // solved together.  Every outer iteration (Sec. 2, Alg. 1) of all unconverged
 // instances is one CUDA graph: the Chebyshev filters of every search-vector
-// bundle of every instance run in ONE persistent cooperative kernel (all
-// degree steps, a grid-wide barrier between steps), followed by batched
+// bundle of every instance run in ONE kernel, followed by batched
 // Cholesky-QR and Rayleigh-Ritz kernels that each cover all instances in one
 // launch, and one copy of all Ritz values and residuals to the host.  The host
 // then applies the same interval/degree heuristic as fd_solve per instance.
 //
-// An autotuner (fd_tune_batched) times the persistent filter over candidate
-// block widths nb, SELL chunk heights C and CTA shapes on the actual
-// instances and returns the fastest.
+// Two kernels can run the filters.  The persistent cooperative kernel
+// (k_batched_filter) takes all bundles through one degree step after the other,
+// with a grid-wide barrier between steps.  Where every matrix fits the shared
+// memory of a cluster, k_batched_small can take each column through all its
+// steps instead; the host picks one of the two before every iteration
+// (panels_pay).
+//
+// An autotuner (fd_tune_batched) times the filter over candidate block widths nb,
+// SELL chunk heights C and, where the persistent kernel runs, CTA shapes on the
+// actual instances and returns the fastest.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -102,7 +108,7 @@ struct BatchArgs {
   const int* task_deg;      // n_tasks filter degrees, non-increasing
   const int* n_tasks;       // tasks in the list this iteration
   const double* mu;
-  const int* kmax;          // largest degree this iteration
+  const int* kmax;          // steps of the persistent kernel this iteration; 1: panels instead (kmax[1])
   int nb;
   int spmmv_only;           // 1: AV = A V for all listed bundles, one pass, no barrier
 };
@@ -305,7 +311,7 @@ __global__ void __launch_bounds__(FF ? BF_FF_WARPS * 32 : WARPS * 32, FF ? BF_FF
 // column panel (one 8-byte unit) takes it through all steps of its own instance's
 // degree, so no step waits for another instance and a late iteration with one
 // instance left costs what that instance costs.  Panels are listed bundle by bundle,
-// largest degree first.
+// largest degree first.  Runs where panels_pay says so.
 template <typename T, typename Mu>
 __device__ __forceinline__ void batched_panel(const BInst& I, const BParams& P, T* V, int unit, uint32_t rank,
                                               uint32_t ranks, unsigned char* smem, Mu&& mu) {
@@ -325,7 +331,7 @@ __global__ void __launch_bounds__(1024, 1) k_batched_small(BatchArgs b) {
   asm("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(ranks));
   const int panel = (int)(blockIdx.x / ranks), t = panel / b.nb, u = panel % b.nb;
   // the whole cluster leaves together
-  if (t >= *b.n_tasks) return;
+  if (!b.kmax[1] || t >= *b.n_tasks) return;
   const BTask tk = b.task[t];
   const BInst& I = b.inst[tk.inst];
   const BParams& P = b.par[tk.inst];
@@ -632,6 +638,7 @@ struct Batch {
   // the one-launch filter of small matrices: CTAs per cluster (0: not used), threads, shared memory
   int small_cluster = 0, small_threads = 0;
   size_t small_smem = 0;
+  std::vector<double> nnz;    // entries per row
   cudaGraphExec_t exec = nullptr;
   int64_t max_D = 0;
 
@@ -789,7 +796,7 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
   FD_CUDA(ctx, cudaMemcpyAsync(B.d_off, B.h_off.data(), sizeof(int64_t) * B.h_off.size(), cudaMemcpyHostToDevice, ctx->stream));
   FD_CUDA(ctx, cudaMallocHost(&B.h_par, sizeof(BParams) * n));
   FD_CUDA(ctx, cudaMallocHost(&B.h_mu, sizeof(double) * mu_cap));
-  FD_CUDA(ctx, cudaMallocHost(&B.h_kmax, sizeof(int)));
+  FD_CUDA(ctx, cudaMallocHost(&B.h_kmax, 2 * sizeof(int)));
   FD_CUDA(ctx, cudaMallocHost(&B.h_out, sizeof(double) * 2 * n * B.ns_max + sizeof(BParams) * n));
   FD_CUDA(ctx, cudaMallocHost(&B.h_task_p, sizeof(BTask) * nta));
   FD_CUDA(ctx, cudaMallocHost(&B.h_off_p, sizeof(int64_t) * (nta + 1)));
@@ -812,11 +819,12 @@ fd_status batch_setup(fd_ctx* ctx, Batch& B, int n, const fd_matrix* const* A, c
   FD_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, B.warps * 32, B.smem_filter));
   if (per_sm < 1) return set_err(ctx, FD_ERR_ARG, "batched filter does not fit on an SM");
   B.grid = per_sm * ctx->num_sms;
+  B.nnz.resize(n);
+  for (int i = 0; i < n; ++i) B.nnz[i] = (double)A[i]->nnz / (double)A[i]->D;
   // Every matrix small enough for a cluster's shared memory: panels instead of
-  // grid-wide steps.  Two CTAs per panel at least: with one, a late iteration with
-  // one instance left takes twice as long, while the full batch gains a tenth
-  // (12 instances of L = 10 .. 14, N_s = 64: 82 ms of filter per solve with the
-  // persistent kernel, 18 us a step with one instance left).
+  // grid-wide steps are possible.  Two CTAs per panel at least: with one, a late
+  // iteration with one instance left takes twice as long, while the full batch gains
+  // a tenth (12 instances of L = 10 .. 14).
   for (int cl = 2; cl <= 8 && !B.small_cluster; cl *= 2) {
     bool fits = true;
     int rows = 0;
@@ -857,6 +865,58 @@ fd_status copy_tasks(fd_ctx* ctx, Batch& B) {
   return FD_OK;
 }
 
+// Whether this iteration's filters (the host's B.h_par) run as panels, and the
+// words that tell the kernels.  SM clocks of a panel's step: its rows, and the latency
+// of a step (the entries of the longest row one after another), which other CTAs of the
+// SM hide; the panels share the resident clusters.  Of the persistent kernel's step: the
+// barrier with its chain of loads per batch of entries, and the elements of all
+// columns.  Fitted to 336 batches (1 to 64 instances of 512 to 8,000 rows with 3 to 60
+// entries a row, N_s = 16 and 64, all three sweep types): the choice is the faster
+// one, or within 11 % of it.  12 instances with N_s = 64, 1,000 steps, panels / steps: 1,000
+// rows FP64 37 / 42 ms, float-float 23 / 34; 4,096 rows 119 / 106, 55 / 77; 8,000 rows 301 /
+// 195, 191 / 134; 1,000 rows of 59 entries 289 / 155, 348 / 109.
+bool panels_pay(const fd_ctx* ctx, const Batch& B) {
+  if (!B.small_cluster) return false;
+  double work = 0.0, longest = 0.0, steps = 0.0, barrier = 0.0;
+  int kmax = 0;
+  for (int i = 0; i < B.n; ++i) {
+    const BParams& P = B.h_par[i];
+    if (!P.active || P.degree == 0) continue;
+    const BInst& I = B.h_inst[i];
+    const int R = small::cta_rows((int)I.A.D, B.small_cluster), threads = std::min(1024, (R + 31) & ~31);
+    const size_t smem = small::cta_smem<double>((int)I.A.D, R, 1, I.max_row);
+    const double per_sm = std::max<double>(1, std::min<int>((int)(ctx->smem_optin / (smem + 1024)), 2048 / threads));
+    const double nnz = B.nnz[i], elems = (double)I.A.D * I.ns / ctx->num_sms, batches = std::ceil(I.max_row / 4.0);
+    const double wide = B.small_cluster == 8 ? 1.0 : 0.0;
+    double panel, element, step;
+    if (P.f32) {
+      panel = R * 0.10 * nnz + (3030 + 1300 * wide + 5 * I.max_row) / per_sm;
+      element = 0.23 * nnz + 1.17;
+      step = 12100 + 1600 * batches;
+    } else if (P.ff) {
+      panel = R * (0.10 * nnz + 1.41) + (4090 + 490 * wide + 62 * I.max_row) / per_sm;
+      element = 0.376 * nnz + 3.44;
+      step = 11600 + 3100 * batches;
+    } else {
+      panel = R * (0.307 * nnz + 5.56) + (3600 + 45 * I.max_row) / per_sm;
+      element = 0.674 * nnz + 4.47;
+      step = 10400 + 2300 * batches;
+    }
+    work += (double)(P.f32 ? I.ns / 2 : I.ns) * P.degree * panel;
+    longest = std::max(longest, P.degree * panel);
+    steps += P.degree * elems * element;
+    barrier = std::max(barrier, step);
+    kmax = std::max(kmax, P.degree);
+  }
+  const int resident = resident_clusters(ctx, B.small_cluster);
+  return resident > 0 && std::max(longest, work / resident + 0.5 * longest) < kmax * barrier + steps;
+}
+void set_route(const fd_ctx* ctx, Batch& B, int kmax) {
+  const bool panels = panels_pay(ctx, B);
+  B.h_kmax[0] = panels ? 0 : kmax;
+  B.h_kmax[1] = panels ? 1 : 0;
+}
+
 fd_status launch_filter(fd_ctx* ctx, Batch& B, int spmmv_only) {
   BatchArgs a;
   a.inst = B.d_inst; a.par = B.d_par; a.task = B.d_task; a.task_off = B.d_off; a.mu = B.d_mu;
@@ -867,7 +927,10 @@ fd_status launch_filter(fd_ctx* ctx, Batch& B, int spmmv_only) {
   if (spmmv_only) {
     FD_CUDA(ctx, cudaLaunchKernel(filter_kernel_for(B.nb, false), B.grid_rr, B.warps_rr * 32, args,
                                   B.smem_filter, ctx->stream));
-  } else if (B.small_cluster) {
+    FD_LAUNCHED(ctx);
+    return FD_OK;
+  }
+  if (B.small_cluster) {  // returns at once when the steps run
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)B.small_cluster;
@@ -880,9 +943,9 @@ fd_status launch_filter(fd_ctx* ctx, Batch& B, int spmmv_only) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     FD_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_batched_small, a));
-  } else {
-    FD_CUDA(ctx, cudaLaunchCooperativeKernel(kf, B.grid, B.warps * 32, args, B.smem_filter, ctx->stream));
+    FD_LAUNCHED(ctx);
   }
+  FD_CUDA(ctx, cudaLaunchCooperativeKernel(kf, B.grid, B.warps * 32, args, B.smem_filter, ctx->stream));
   FD_LAUNCHED(ctx);
   return FD_OK;
 }
@@ -937,7 +1000,7 @@ fd_status enqueue_iteration(fd_ctx* ctx, Batch& B) {
   cudaStream_t st = ctx->stream;
   FD_CUDA(ctx, cudaMemcpyAsync(B.d_par, B.h_par, sizeof(BParams) * B.n, cudaMemcpyHostToDevice, st));
   FD_CUDA(ctx, cudaMemcpyAsync(B.d_mu, B.h_mu, sizeof(double) * B.mu_cap, cudaMemcpyHostToDevice, st));
-  FD_CUDA(ctx, cudaMemcpyAsync(B.d_kmax, B.h_kmax, sizeof(int), cudaMemcpyHostToDevice, st));
+  FD_CUDA(ctx, cudaMemcpyAsync(B.d_kmax, B.h_kmax, 2 * sizeof(int), cudaMemcpyHostToDevice, st));
   FD_TRY(copy_tasks(ctx, B));
   const dim3 cgrid((unsigned)std::max(1, ctx->num_sms * 2), B.n);
   if (B.f32 || B.ff) {
@@ -1084,7 +1147,7 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
   }
   // first iteration: no filter, orthonormalise + Rayleigh-Ritz
   for (int i = 0; i < n_inst; ++i) B.h_par[i] = BParams{1};
-  *B.h_kmax = 0;
+  set_route(ctx, B, 0);
   B.list_tasks();
   // capture one iteration as a graph; replay it every outer iteration
   bool use_graph = true;
@@ -1104,7 +1167,7 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
     cudaGetLastError();
   }
   ctx->err.clear();
-  int it = 0;
+  int it = 0, kmax = 0;
   int n_left = n_inst;
   for (; it < max_outer && n_left > 0; ++it) {
     if (use_graph) {
@@ -1122,10 +1185,10 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
       float msv = 0;
       cudaEventElapsedTime(&msv, e0, e1);
       fprintf(stderr, "batched it %d: active %d (FP32 sweeps %d), top degree %d, elapsed %.2f s\n", it,
-              n_left, n32, *B.h_kmax, msv * 1e-3);
+              n_left, n32, kmax, msv * 1e-3);
     }
     const BParams* dev_par = (const BParams*)(B.h_out + (size_t)2 * n_inst * B.ns_max);
-    int kmax = 0;
+    kmax = 0;
     size_t mu_off = 0;
     for (int i = 0; i < n_inst; ++i) {
       BParams& P = B.h_par[i];
@@ -1202,7 +1265,7 @@ fd_status fd_solve_batched(fd_ctx* ctx, int n_inst, const fd_matrix* const* A,
       mu_off += n + 1;
       kmax = std::max(kmax, n);
     }
-    *B.h_kmax = kmax;
+    set_route(ctx, B, kmax);
     B.list_tasks();
   }
   cudaEventRecord(e1, st);
@@ -1282,13 +1345,17 @@ fd_status fd_tune_batched(fd_ctx* ctx, int n_inst, const char* const* specs, int
         std::vector<double> mu(probe_degree + 1);
         for (int k = 0; k <= probe_degree; ++k) mu[k] = 1.0 / (k + 1);
         std::copy(mu.begin(), mu.end(), B.h_mu);
-        *B.h_kmax = probe_degree;
+        set_route(ctx, B, probe_degree);
+        if (B.h_kmax[1] && w != WARPS) {  // the panels have no CTA shape to choose
+          B.release();
+          continue;
+        }
         B.list_tasks();
         s = copy_tasks(ctx, B);
         if (s != FD_OK) { B.release(); break; }
         FD_CUDA(ctx, cudaMemcpyAsync(B.d_par, B.h_par, sizeof(BParams) * n_inst, cudaMemcpyHostToDevice, st));
         FD_CUDA(ctx, cudaMemcpyAsync(B.d_mu, B.h_mu, sizeof(double) * (probe_degree + 1), cudaMemcpyHostToDevice, st));
-        FD_CUDA(ctx, cudaMemcpyAsync(B.d_kmax, B.h_kmax, sizeof(int), cudaMemcpyHostToDevice, st));
+        FD_CUDA(ctx, cudaMemcpyAsync(B.d_kmax, B.h_kmax, 2 * sizeof(int), cudaMemcpyHostToDevice, st));
         s = launch_filter(ctx, B, 0);  // warm-up
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);

@@ -65,7 +65,7 @@ fd_status launch_pw(fd_ctx* ctx, const Params<T>& p, int units, int cluster, siz
 
 // Clusters of a launch that are resident at once (cached per device and size:
 // they depend on the chip's groups of SMs, and every CTA here fills most of one)
-static int resident_clusters(const fd_ctx* ctx, int cluster) {
+int resident_clusters(const fd_ctx* ctx, int cluster) {
   static std::atomic<int> cache[64][9];
   if (cluster == 1) return ctx->num_sms;
   std::atomic<int>* slot = ctx->device < 64 ? &cache[ctx->device][cluster] : nullptr;

@@ -157,3 +157,33 @@ def test_uneven_anderson_batch_ff_finish_matches_sequential(fd, ctx):
         assert r["n_spmmv_ff"] > 0
         th1, rho1, r1 = fd.fd_solve(ctx, m, a, b, nt, 16, 200, 1e-9, seed=sd, precision="f32", finish="ff")
         assert np.abs(th - th1).max() <= 1e-10 * max(abs(r1["lam_l"]), abs(r1["lam_r"]))
+
+
+@pytest.mark.parametrize("form", [{}, {"precision": "ff"}, {"precision": "f32", "finish": "ff"}])
+def test_persistent_steps_of_every_form_match_sequential(fd, ctx, form):
+    """Instances too large for column panels (L = 21, 22): FP64, float-float and FP32 rows of
+    the persistent kernel's instantiations."""
+    specs = [(21, 9.7, 3), (22, 12.1, 5), (17, 11.3, 8)]
+    mats = [fd.fd_build_matrix(ctx, f"anderson3d:L={L},W={W},seed={s}") for L, W, s in specs]
+    probs = [(-0.02, 0.02, 6, s) for _, _, s in specs]
+    out, res = fd.fd_solve_batched(ctx, mats, probs, 8, 150, 1e-9, **form)
+    for m, (a, b, nt, sd), (th, rho), r in zip(mats, probs, out, res):
+        assert r["converged"] == 1 and rho.max() <= 1e-9
+        assert form.get("precision") != "f32" or r["n_spmmv_f32"] > 0
+        assert not form or r["n_spmmv_ff"] > 0
+        th1, _, r1 = fd.fd_solve(ctx, m, a, b, nt, 8, 150, 1e-9, seed=sd, **form)
+        assert np.abs(th - th1).max() <= 1e-10 * max(abs(r1["lam_l"]), abs(r1["lam_r"]))
+
+
+@pytest.mark.parametrize("form", [{}, {"precision": "ff"}, {"precision": "f32", "finish": "ff"}])
+def test_iterations_change_between_steps_and_panels(fd, ctx, form):
+    """Twelve matrices with long rows fit as panels, but run as steps while many are left
+    and as panels when few are; the eigenvalues are those of dense solves."""
+    import fd_inputs
+    csrs = [fd_inputs.random_symmetric_csr(600 + 40 * i, 40, i) for i in range(12)]
+    mats = [fd.fd_matrix_from_csr(ctx, *c) for c in csrs]
+    out, res = fd.fd_solve_batched(ctx, mats, [(-0.05, 0.05, 8, i) for i in range(12)], 8, 40, 1e-9, **form)
+    for c, (th, rho), r in zip(csrs, out, res):
+        ev = np.linalg.eigvalsh(mat.to_scipy(c).toarray())
+        assert r["converged"] == 1 and rho.max() <= 1e-9
+        assert np.abs(th - _nearest(ev, 0.0, 8)).max() <= 1e-10 * np.abs(ev).max()
