@@ -251,9 +251,12 @@ __device__ __forceinline__ void batched_row_group_ff(const BatchArgs& b, int t, 
 
 // FF: the instantiation with FP32 and float-float rows only, the filter of
 // solves that use float-float sweeps, in 4-warp CTAs.  Eight of them per SM (64
-// registers) rather than twelve: at 40 registers the two row types spill 420
-// bytes (12 instances of L = 10 .. 14, nb = 8: 125 ms of filter per solve against
-// 167 ms).
+// registers) rather than twelve, where the two row types spill 420 bytes.  FP32 steps
+// alone are faster with twelve (32 instances of 24^3 rows, 1,000 steps: 352 ms against
+// 404), float-float ones with eight (552 against 623); whole solves, eight against
+// twelve: 64 instances of 16^3 to 48^3 rows, seven iterations, FP32 with float-float finish
+// 53.0 / 55.1 s, float-float 66.6 / 71.3; eight of 22^3 to 29^3 6.15 / 6.51 and 7.45 / 8.32;
+// four of 30^3 to 33^3 6.41 / 6.20 and 8.45 / 8.85.
 constexpr int BF_FF_WARPS = 4, BF_FF_BLOCKS = 8;
 template <int NB, bool FF>
 __global__ void __launch_bounds__(FF ? BF_FF_WARPS * 32 : WARPS * 32, FF ? BF_FF_BLOCKS : 3)
