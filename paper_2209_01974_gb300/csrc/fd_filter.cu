@@ -36,8 +36,9 @@ namespace {
 using namespace step;
 using ffa::ff;
 
-template <typename T, int NB, int MODE>
-__global__ void __launch_bounds__(step_warps<T>() * 32, step_min_blocks<T>())
+// BLOCKS: resident CTAs per SM (the launch bounds)
+template <typename T, int NB, int MODE, int BLOCKS>
+__global__ void __launch_bounds__(step_warps<T>() * 32, BLOCKS)
     k_cheb_step(SellArgs<T> A, StepArgs<T> s, unsigned pf) {
   using L = Layout<T, NB>;
   constexpr int WARPS = step_warps<T>();
@@ -162,6 +163,24 @@ fd_status launch_kron_step(fd_ctx* ctx, const fd_matrix* M, int mode, const Step
   return launch_step_kernel(ctx, k_kron_step<T, NB, MODE_GENERIC>, grid, WARPS * 32, 0, dep, K, s);
 }
 
+template <typename T, int NB, int BLOCKS>
+fd_status launch_cheb_step(fd_ctx* ctx, unsigned grid, int mode, const SellArgs<T>& A, const StepArgs<T>& s) {
+  constexpr int SW = step_warps<T>();
+  // prefetch distance: one wave of resident CTAs
+  const unsigned pf = (unsigned)ctx->num_sms * BLOCKS;
+  // Dependent launch, but for the first step (MODE_SPMMV), which follows a
+  // kernel that is not a step, and for FP64 grids between half the SMs and one
+  // wave: their CTAs would be placed beside the previous step's, unevenly over
+  // the SMs, and the FP64 pipe of the fuller ones sets the time (8-warp CTAs,
+  // nb = 16, 4,900 rows in 154 CTAs: 9.2 us a step against 8.2 us; 1,728 rows in 54
+  // CTAs: 3.4 us against 4.1 us).
+  const bool dep = dependent_step<T>(ctx, grid, pf);
+  if (mode == MODE_SPMMV) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SPMMV, BLOCKS>, grid, SW * 32, 0, false, A, s, pf);
+  if (mode == MODE_SECOND) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SECOND, BLOCKS>, grid, SW * 32, 0, dep, A, s, pf);
+  if (mode == MODE_PLAIN) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_PLAIN, BLOCKS>, grid, SW * 32, 0, dep, A, s, pf);
+  return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_GENERIC, BLOCKS>, grid, SW * 32, 0, dep, A, s, pf);
+}
+
 template <typename T, int NB>
 fd_status launch_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<T>& s, const Scaled<T>& sc) {
   if (M->kron) return launch_kron_step<T, NB>(ctx, M, mode, s, sc);
@@ -175,21 +194,25 @@ fd_status launch_step(fd_ctx* ctx, const fd_matrix* M, int mode, const StepArgs<
   constexpr int SW = step_warps<T>();
   const int64_t rows_per_block = (int64_t)SW * L::RPW;
   const unsigned grid = (unsigned)cdiv(M->D, rows_per_block);
-  // prefetch distance: one wave of resident CTAs (the launch-bounds occupancy)
-  const unsigned pf = (unsigned)ctx->num_sms * step_min_blocks<T>();
-  // Dependent launch, but for the first step (MODE_SPMMV), which follows a
-  // kernel that is not a step, and for FP64 grids between half the SMs and one
-  // wave: their CTAs would be placed beside the previous step's, unevenly over
-  // the SMs, and the FP64 pipe of the fuller ones sets the time (8-warp CTAs,
-  // nb = 16, 4,900 rows in 154 CTAs: 9.2 us a step against 8.2 us; 1,728 rows in 54
-  // CTAs: 3.4 us against 4.1 us).
-  const bool dep = dependent_step<T>(ctx, grid, pf);
-  if (mode == MODE_SPMMV) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SPMMV>, grid, SW * 32, 0, false, A, s, pf);
-  if (mode == MODE_SECOND) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_SECOND>, grid, SW * 32, 0, dep, A, s, pf);
-  if (mode == MODE_PLAIN) return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_PLAIN>, grid, SW * 32, 0, dep, A, s, pf);
-  return launch_step_kernel(ctx, k_cheb_step<T, NB, MODE_GENERIC>, grid, SW * 32, 0, dep, A, s, pf);
+  // The shape of StepShape serves many short rows.  Long ones, or a few rows far longer
+  // than the rest, are a chain of loads that more registers shorten (the float-float
+  // loop over a row spills a little at 40 of them), and in a grid of one wave the
+  // registers are there for the taking.  us a step, default shape / this:
+  //   FP64 4,000 rows, some of 300 entries, nb = 32, 128: 47.3 / 44.2, 92.7 / 78.8;
+  //   float-float the same 86.2 / 77.4, 128 / 109; 40,000 rows of 41, nb = 8 31.5 / 25.1;
+  //   4,000 such rows, nb = 128 42.2 / 27.5; 4,900 rows of 8, nb = 128 13.1 / 10.7.
+  //   (262,144 rows of 7, nb = 64, float-float: 156 with 12 CTAs, 160 with 10, 176 with 8)
+  const unsigned sms = (unsigned)ctx->num_sms;
+  const bool long_rows = M->nnz >= 12 * M->D, few_long = M->max_row >= 64 && (int64_t)M->max_row * M->D > 4 * M->nnz;
+  if constexpr (std::is_same_v<T, ff>) {
+    if (grid <= 8 * sms || few_long) return launch_cheb_step<T, NB, 8>(ctx, grid, mode, A, s);
+    // a grid that is one wave with 12 keeps them (7,000 rows of 41, nb = 64: 26.9, with 10 30.0)
+    if (grid <= 10 * sms || (long_rows && grid > 12 * sms)) return launch_cheb_step<T, NB, 10>(ctx, grid, mode, A, s);
+  }
+  if constexpr (std::is_same_v<T, double>)
+    if (long_rows || few_long) return launch_cheb_step<T, NB, 6>(ctx, grid, mode, A, s);
+  return launch_cheb_step<T, NB, step_min_blocks<T>()>(ctx, grid, mode, A, s);
 }
-
 template <typename T>
 fd_status step_dispatch(fd_ctx* ctx, const fd_matrix* M, int nb, int mode, const StepArgs<T>& s,
                         const Scaled<T>& sc = {}) {

@@ -179,3 +179,26 @@ def test_filters_of_one_context_on_two_streams():
     torch.cuda.synchronize()
     for c in (a, b):
         assert np.all(np.abs(c[1].cpu().numpy() - c[7]) <= c[8])
+
+
+@pytest.mark.parametrize("D,nb", [(30000, 8), (28000, 16), (30000, 32), (9000, 128)])
+def test_float_float_long_rows(D, nb):
+    """The float-float step's CTAs per SM by the length of rows and the size of the grid."""
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    ctx = fd.fd_create(0)
+    csr = fd_inputs.random_symmetric_csr(D, 17, nb, max_row=60)
+    A = fd.fd_matrix_from_csr(ctx, *csr)
+    assert A.info["nnz"] >= 12 * D
+    V0 = fd_inputs.random_block(D, nb, 3).astype(np.float32).astype(np.float64)
+    lo, hi = lanczos.gershgorin(csr)
+    alpha, beta = ch.scale_params(lo - 0.01, hi + 0.01)
+    mu = np.random.default_rng(1).uniform(0.5, 1.0, 14)
+    out = torch.from_numpy(V0).cuda()
+    V = torch.empty((D, nb, 2), dtype=torch.float32, device="cuda")
+    fd.fd_copy_block(ctx, out, V)
+    fd.fd_filter(ctx, A, V, mu, alpha, beta, torch.empty_like(V), torch.empty_like(V))
+    fd.fd_copy_block(ctx, V, out)
+    ref = ch.cheb_filter(mat.to_scipy(csr), V0, mu, alpha, beta)
+    assert np.all(np.abs(out.cpu().numpy() - ref) <= filter_tolerance(csr, mu, alpha, beta, V0, 2.0 ** -45))
