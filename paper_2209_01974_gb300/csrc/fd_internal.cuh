@@ -169,7 +169,7 @@ struct SmallPlan {
 };
 SmallPlan small_plan(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int units);
 int resident_clusters(const fd_ctx* ctx, int cluster);  // clusters of one CTA per SM that run at once
-bool filter_small_pays(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int nb);
+bool filter_small_pays(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int nb, SmallPlan* chosen = nullptr);
 fd_status filter_small(fd_ctx* ctx, const fd_matrix* M, fd_prec prec, void* V, int64_t ldv, int nb, int degree,
                        const double* mu, double alpha, double beta, void* W1, void* W2, int64_t ldw,
                        double* bytes_out, bool* used);

@@ -99,12 +99,14 @@ int resident_clusters(const fd_ctx* ctx, int cluster) {
 // clocks (2 FMA a clock, at about 60 % with the few warps a CTA has) or, for FP32 and
 // float-float, the issue clocks of an entry; in a cluster the stores of its rows to
 // the other CTAs (about 16 clocks per warp); plus the barrier and the latency of a
-// step (about 1,500 clocks for a cluster, 800 for a single CTA).
+// step (about 1,500 clocks for a cluster, 800 for a single CTA, and 20 to 60 for every
+// further entry of a long row, which one thread takes one after the other).
 SmallPlan small_plan(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int units) {
   SmallPlan best;
   if (M->kron || M->D > MAX_ROWS || M->max_row > MAX_ROWS) return best;
   const double nnz = (double)M->nnz / (double)M->D;
   const double per_unit = prec == FD_F64 ? (nnz + 1.4) / 1.2 : prec == FD_F32 ? (6 * nnz + 30) / 80 : (20 * nnz + 70) / 80;
+  const double chain = prec == FD_F32 ? 0.0 : (prec == FD_FF ? 60.0 : 20.0) * std::max(0, M->max_row - 8);
   for (int pw : {1, 2, 4, 8}) {
     if (units % pw) continue;
     for (int cl = 1; cl <= 8; ++cl) {  // 8: the largest portable cluster
@@ -119,7 +121,7 @@ SmallPlan small_plan(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int un
       const int64_t panels = units / pw;
       const int64_t layers = cdiv(panels, resident);  // CTAs on the fullest SM
       const int64_t waves = cdiv(layers, per_sm);
-      double clocks = (double)layers * R * pw * (per_unit + (cl - 1) * 0.5) + (double)waves * (cl > 1 ? 1500 : 800);
+      double clocks = (double)layers * R * pw * (per_unit + (cl - 1) * 0.5) + (double)waves * ((cl > 1 ? 1500 : 800) + chain);
       if (cl > 1) clocks *= 1.15;  // near ties go to the smaller cluster
       if (best.cluster == 0 || clocks < best.clocks) {
         best.cluster = cl;
@@ -135,19 +137,26 @@ SmallPlan small_plan(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int un
 
 // SM clocks of a launched step over the same columns: the launch and the chain of
 // loads (per batch of entries), and the FP64 pipe (nnz + 4 operations) or the issue
-// of the entries.  Fitted to D = 4,900 .. 17,576 (FP64 6.5 us at nb = 8, 11.3 us at
-// nb = 64; FP32 2.5 to 4.7 us; float-float 6 to 8 us).
+// of the entries.  The launch costs less where steps overlap: dependent launches,
+// which FP64 grids below a wave do without, and in float-float a grid whose CTAs
+// have the registers of one wave.  Fitted to D = 4,096 .. 17,576, 375 filters of stencil,
+// Hubbard, road and random matrices with 3 to 100 entries a row: of launched steps and
+// panels the faster one is taken, or one within 10 % of it (21 % in FP32 from 2,744 rows
+// on one SM, 41 % in FP64 for 4,900 rows of 4 entries with nb = 64).
 static double launched_clocks(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int units) {
   const double nnz = (double)M->nnz / (double)M->D, elems = (double)M->D * units / ctx->num_sms;
   const double batches = std::ceil(std::min<double>(M->max_row, 2 * nnz) / step::BATCH);
-  if (prec == FD_F64) return 10000 + 1000 * batches + elems * (nnz + 4) / 2;
+  const int64_t rows = 4 * (32 / std::max(1, std::min(32, units / 2)));  // of a CTA, 8-byte elements
+  const int64_t grid = cdiv(M->D, rows);
+  if (prec == FD_F64) return (grid >= 8LL * ctx->num_sms ? 6600 : 10600) + 700 * batches + elems * (nnz + 4) / 2;
   if (prec == FD_F32) return 1800 + 1600 * batches + elems * (8 * nnz + 60) / 128;
-  return 9000 + 1000 * batches + elems * (25 * nnz + 130) / 128;
+  return (grid <= 10LL * ctx->num_sms ? 5000 : 9000) + 1400 * batches + elems * (25 * nnz + 130) / 128;
 }
 
-bool filter_small_pays(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int nb) {
+bool filter_small_pays(const fd_ctx* ctx, const fd_matrix* M, fd_prec prec, int nb, SmallPlan* chosen) {
   const int units = prec == FD_F32 ? nb / 2 : nb;
   const SmallPlan plan = small_plan(ctx, M, prec, units);
+  if (chosen) *chosen = plan;
   return plan.cluster > 0 && plan.clocks < launched_clocks(ctx, M, prec, units);
 }
 
@@ -185,9 +194,9 @@ fd_status filter_small(fd_ctx* ctx, const fd_matrix* M, fd_prec prec, void* V, i
                        const double* mu, double alpha, double beta, void* W1, void* W2, int64_t ldw,
                        double* bytes_out, bool* used) {
   *used = false;
-  if (!filter_small_pays(ctx, M, prec, nb)) return FD_OK;
+  SmallPlan plan;
+  if (!filter_small_pays(ctx, M, prec, nb, &plan)) return FD_OK;
   const int units = prec == FD_F32 ? nb / 2 : nb;
-  const SmallPlan plan = small_plan(ctx, M, prec, units);
   if (prec == FD_F64)
     FD_TRY(filter_small_t<double>(ctx, M, plan, (double*)V, ldv, units, degree, mu, alpha, beta, (double*)W1, (double*)W2, ldw));
   else if (prec == FD_FF)
