@@ -243,20 +243,6 @@ __global__ void __launch_bounds__(1024) k_cholesky(const double* G, int n, doubl
 // ---------------------------------------------------------------------------
 constexpr int CB = 8;  // panel rows
 
-// 1 / sqrt(d), d > 0 finite: an FP32 estimate of the scaled value and one
-// third-order step in FP64
-__device__ __forceinline__ double rsqrt64(double d) {
-  const long long bits = __double_as_longlong(d);
-  int ex = (int)((bits >> 52) & 0x7FF) - 1023;
-  if (ex == -1023) return 1.0 / sqrt(d);  // subnormal
-  ex &= ~1;
-  const double m = __longlong_as_double(bits - ((long long)ex << 52));  // in [1, 4)
-  const double y = (double)rsqrtf((float)m);
-  const double e = fma(-m * y, y, 1.0);
-  const double r = fma(y * e, fma(0.375, e, 0.5), y);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)(ex / 2) << 52));
-}
-
 __global__ void __launch_bounds__(256) k_cholesky_coop(const double* G, int n, double coeff, double* R, int* ok) {
   cg::grid_group grid = cg::this_grid();
   extern __shared__ double sP[];  // 2 x CB x n: the panel's finished rows, by panel parity
@@ -295,7 +281,7 @@ __global__ void __launch_bounds__(256) k_cholesky_coop(const double* G, int n, d
       for (int p = 0; p < CB; ++p) {
         const double d = __shfl_sync(0xffffffffu, v[p >> 2], (p & 3) * 8 + p);
         if (!(d > 0.0) || !isfinite(d)) bad = true;
-        const double ri = rsqrt64(bad ? 1.0 : d);
+        const double ri = rsqrt(bad ? 1.0 : d);
         if (i == (p & 3)) v[p >> 2] = j == p ? d * ri : v[p >> 2] * ri;
         const double rj = __shfl_sync(0xffffffffu, v[p >> 2], (p & 3) * 8 + j);
 #pragma unroll

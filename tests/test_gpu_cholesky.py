@@ -38,6 +38,21 @@ def test_orders(ns, spread):
     assert np.all(np.abs(R - ref) <= 1e-12 * np.sqrt(ns) * scale[None, :])
 
 
+@pytest.mark.parametrize("exponent", [-500, -333, -1, 0, 1, 400, 501])
+@pytest.mark.parametrize("ns", [3, 24, 40])
+def test_pivots_of_every_size(ns, exponent):
+    """Pivots down to 2^-1000 and up to 2^1002, even and odd powers of two side by side:
+    scaling columns by powers of two scales R's columns by them and leaves Q."""
+    D = 3 * ns + 50
+    V0 = fd_inputs.random_block(D, ns, ns)
+    scale = np.ldexp(1.0, exponent + np.arange(ns) % 3 - 1)
+    Q, R, passes = _qr(V0 * scale[None, :])
+    Q1, R1, _ = _qr(V0)
+    assert passes == 2
+    assert np.abs(Q - Q1).max() <= 1e-13 and np.abs(Q.T @ Q - np.eye(ns)).max() <= 1e-14
+    assert np.abs(R / scale[None, :] - R1).max() <= 1e-13 * np.abs(R1).max()
+
+
 def test_orders_whose_shared_memory_is_just_above_the_default():
     """From 727 on the triangular inverse's shared memory, static and dynamic, exceeds
     the 48 KB that a launch gets unasked.  In a process of its own: the larger limit
