@@ -433,6 +433,10 @@ int eig_grid(const fd_ctx* ctx, int n_inst, int m_max) {
 
 fd_status launch(fd_ctx* ctx, EigArgs& a, int grid) {
   void* args[] = {&a};
+  // two bytes per matrix beside 13 KB of static arrays: from 17,900 matrices on more than
+  // a launch gets unasked
+  if (a.n_inst > 8192)
+    FD_CUDA(ctx, cudaFuncSetAttribute(k_block_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
   FD_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_block_jacobi, grid, EIG_THREADS, args,
                                            (size_t)2 * a.n_inst, ctx->stream));
   FD_LAUNCHED(ctx);

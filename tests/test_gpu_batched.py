@@ -187,3 +187,16 @@ def test_iterations_change_between_steps_and_panels(fd, ctx, form):
         ev = np.linalg.eigvalsh(mat.to_scipy(c).toarray())
         assert r["converged"] == 1 and rho.max() <= 1e-9
         assert np.abs(th - _nearest(ev, 0.0, 8)).max() <= 1e-10 * np.abs(ev).max()
+
+
+def test_many_instances(fd, ctx):
+    """18,500 problems in one batch: the bookkeeping of every instance fits the kernels'
+    shared memory.  (The same 8-row matrix for all; N_s = D, so the first iteration is exact.)"""
+    A = fd.fd_build_matrix(ctx, "chain:n=8,t=1")
+    n = 18500
+    out, res = fd.fd_solve_batched(ctx, [A] * n, [(-0.2, 0.2, 2, i) for i in range(n)], 8, 10, 1e-9, n_max=10,
+                                   max_outer=2)
+    ev = 2.0 * np.cos(np.pi * np.arange(1, 9) / 9)
+    want = _nearest(ev, 0.0, 2)
+    assert all(r["converged"] == 1 for r in res)
+    assert max(np.abs(th - want).max() for th, _ in out) <= 1e-12
