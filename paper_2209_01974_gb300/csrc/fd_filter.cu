@@ -252,8 +252,9 @@ constexpr int SCALE_MIN_DEGREE = 12;
 // A' = 2 (alpha A + beta) in a buffer of the context, for FP64 and float-float
 // filters; left empty (the steps then scale their sums) for short ones, where the
 // buffer is refused, and under stream capture (a graph replays after the buffer has
-// been rewritten or has grown).  The buffer outlives the call: one on another stream
-// first waits for the steps that still read it (scale_done).
+// been rewritten or has grown).  The buffer outlives the call, so
+// the next one first waits for the steps that still read it (scale_done), whatever its
+// stream: a stream's handle may be that of one destroyed with work left.
 template <typename T>
 fd_status scale_matrix(fd_ctx* ctx, const fd_matrix* M, int n, double alpha, double beta, Scaled<T>* out) {
   if (sizeof(T) != 8 || n < SCALE_MIN_DEGREE) return FD_OK;
@@ -270,7 +271,7 @@ fd_status scale_matrix(fd_ctx* ctx, const fd_matrix* M, int n, double alpha, dou
     return FD_OK;
   }
   if (!ctx->scaled_read) FD_CUDA(ctx, cudaEventCreateWithFlags(&ctx->scaled_read, cudaEventDisableTiming));
-  else if (ctx->scaled_stream != ctx->stream) FD_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->scaled_read, 0));
+  else FD_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->scaled_read, 0));
   T* v = (T*)p;
   if (!M->kron) {
     const int64_t rows = M->n_chunks * M->C;
@@ -293,7 +294,6 @@ fd_status scale_matrix(fd_ctx* ctx, const fd_matrix* M, int n, double alpha, dou
   return FD_OK;
 }
 fd_status scale_done(fd_ctx* ctx) {
-  ctx->scaled_stream = ctx->stream;
   FD_CUDA(ctx, cudaEventRecord(ctx->scaled_read, ctx->stream));
   return FD_OK;
 }

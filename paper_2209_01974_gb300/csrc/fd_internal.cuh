@@ -27,9 +27,7 @@ struct fd_ctx {
   int64_t ws_allocs = 0;    // cudaMalloc calls made for workspaces
   size_t ws_limit = 0;      // cap on ws_bytes (0 = none): growth beyond it fails with FD_ERR_OOM
   int debug_checks = 0;     // scan matrix index arrays before step kernels (FD_ERR_BOUNDS)
-  // the scaled-matrix buffer of the last filter: its last reader and where it ran
-  cudaEvent_t scaled_read = nullptr;
-  cudaStream_t scaled_stream = nullptr;
+  cudaEvent_t scaled_read = nullptr;  // the last reader of the scaled-matrix buffer
   // pinned host staging
   void* host_stage = nullptr;
   size_t host_stage_bytes = 0;

@@ -202,3 +202,42 @@ def test_float_float_long_rows(D, nb):
     fd.fd_copy_block(ctx, V, out)
     ref = ch.cheb_filter(mat.to_scipy(csr), V0, mu, alpha, beta)
     assert np.all(np.abs(out.cpu().numpy() - ref) <= filter_tolerance(csr, mu, alpha, beta, V0, 2.0 ** -45))
+
+
+def test_scaled_matrix_across_destroyed_streams():
+    """The scaled matrix of one filter is not overwritten by the next one's while steps on
+    a stream that has since been destroyed still read it; the new stream may get the old
+    one's handle."""
+    import ctypes
+
+    import torch
+
+    import paper_2209_01974_gb300 as fd
+    rt = torch.cuda.cudart()
+    ctx = fd.fd_create(0)
+    specs = ["anderson3d:L=60,W=3,seed=5", "anderson3d:L=60,W=3,seed=6"]
+    mats = [fd.fd_build_matrix(ctx, s) for s in specs]
+    D, nb = 60 ** 3, 16
+    mu = np.random.default_rng(3).uniform(0.5, 1.0, 101)
+    V0 = torch.randn((D, nb), dtype=torch.float64, device="cuda")
+
+    def run(stream_of, sync):
+        out = []
+        for A in mats:
+            V, W1, W2 = V0.clone(), torch.empty_like(V0), torch.empty_like(V0)
+            torch.cuda.synchronize() if sync else torch.cuda.current_stream().synchronize()
+            s = stream_of()
+            fd.fd_set_stream(ctx, s.value)
+            fd.fd_filter(ctx, A, V, mu, 0.12, 0.01, W1, W2)
+            fd.fd_set_stream(ctx, None)
+            assert int(rt.cudaStreamDestroy(s.value)) == 0   # returns at once, the work goes on
+            out.append((V, W1, W2))
+        torch.cuda.synchronize()
+        return [o[0] for o in out]
+
+    def fresh():
+        s = ctypes.c_void_p()
+        assert int(rt.cudaStreamCreate(ctypes.addressof(s))) == 0
+        return s
+    apart, close = run(fresh, True), run(fresh, False)
+    assert all(torch.equal(a, b) for a, b in zip(apart, close))
