@@ -14,10 +14,11 @@ FP64 and are read back to the host.
 value = algorithmic filter bytes per step (Eq. EstimateT, kappa = 5) / step
 time: the sweep's HBM throughput with the orthogonalisation and Rayleigh-Ritz
 time charged to it.  The steps move less than the algorithm counts (they visit the
-accumulator every third time: 11/3 vectors instead of 5), which roofline.moved
-states beside it, with its own fraction of the peak.  The all-FP64 form of the same step is reported under
-"f64_form"; its fused step is bound by GB300's FP64 rate, not by HBM.  The
-inputs (6.4 GB block, 0.5 GB matrix) exceed the 129 MB L2, so no flush is
+accumulator every third time: 11/3 vectors instead of 5), so roofline.achieved and
+its fraction of the peak are those of the bytes moved, and roofline.algorithmic
+states the algorithm's rate beside them.  The all-FP64 form of the same step is
+reported under "f64_form"; its fused step is bound by GB300's FP64 rate, not by HBM,
+and its roofline counts the FP64 operations that the steps execute.  The inputs (6.4 GB block, 0.5 GB matrix) exceed the 129 MB L2, so no flush is
 needed between steps.
 
 `--impl reference` times the FP64 CPU oracle (scipy CSR SpMMV + NumPy) on a
@@ -55,9 +56,9 @@ FP64_TFLOPS = 1.25
 # capture of `bench.py --kernel-only f32` (profiles/k_cheb_step_f32_stencil_L128_nb64.md),
 # with the kernel shape it was taken on and the SHA-256 of the step kernel's sources
 # at that time: when the sources differ, the figure is stale and is reported as null
-TRAFFIC_F32 = {"bytes": 1.762509824e9 + 1.024038912e9, "kernel": "k_cheb_step<float,64,GENERIC>",
+TRAFFIC_F32 = {"bytes": 1.762473216e9 + 1.024061184e9, "kernel": "k_cheb_step<float,64,GENERIC>",
                "rows": 2097152, "nnz": 14680064, "nb": 64,
-               "sources_sha256": "a90517f3460c50989d836af93009b6c6009781f69d1537b704f85c9a2bcbbb92"}
+               "sources_sha256": "84add6152813e227f6af43ec9ce164346265c2bbf399b27f14195871a0b286f5"}
 STEP_SOURCES = ["paper_2209_01974_gb300/csrc/fd_step.cuh", "paper_2209_01974_gb300/csrc/fd_filter.cu"]
 
 
@@ -101,6 +102,21 @@ def moved_filter_bytes(D, nnz, nb, n, Sx):
     step that leaves the accumulator alone reads two vectors and writes one."""
     plain = sum(1 for k in range(3, n) if (k - 2) % 3)
     return filter_bytes(D, nnz, nb, n, Sx) - plain * 2 * nb * D * Sx
+
+
+def fp64_step_flops(D, nnz, nb):
+    """FP64 operations of a step on the scaled matrix, two flops each: one per entry, one
+    that joins the diagonal's part to the sum, and one per accumulated term (a term a
+    step on average)."""
+    return 2.0 * nb * (nnz + 2.0 * D)
+
+
+def hbm_roofline(algorithmic, moved_ratio, peak):
+    """Roofline entry of the filter phase: algorithmic GB/s, bytes moved per algorithmic
+    byte, peak GB/s."""
+    moved = algorithmic * moved_ratio
+    return {"bound": "hbm", "achieved": moved, "peak": peak, "unit": "GB/s", "frac": moved / peak,
+            "algorithmic": algorithmic}
 
 
 # --------------------------------------------------------------------------- clocks
@@ -371,7 +387,7 @@ def run_gpu(args):
     k64 = args.steps
     total64, times64, _, _ = timed("f64", k64, 1)
     filt64 = sum(t[0] for t in times64)
-    flops64 = (NS // NB) * DEGREE * (2.0 * nnz * NB + 6.0 * NB * D)
+    flops64 = (NS // NB) * DEGREE * fp64_step_flops(D, nnz, NB)
     f64_form = {"value": job_throughput(sweep_bytes64, k64, world, total64), "unit": UNIT,
                 "ms_per_step": total64 / k64, "steps": k64,
                 "filter_gbs": sweep_bytes64 * k64 / (filt64 * 1e-3) / 1e9,
@@ -429,17 +445,15 @@ def run_gpu(args):
                          f"L=128 stencil, columns split over {cores} spawned processes: {dt:.2f} s",
                "one_core": {"value": gbs1, "unit": UNIT, "seconds": dt1}}
     traffic, traffic_note = traffic_record(D, nnz, NB)
-    # GB/s that the filter phase really moves
-    moved = achieved * moved_filter_bytes(D, nnz, NB, DEGREE, 4.0) / filter_bytes(D, nnz, NB, DEGREE, 4.0)
+    moved_ratio = moved_filter_bytes(D, nnz, NB, DEGREE, 4.0) / filter_bytes(D, nnz, NB, DEGREE, 4.0)
     if rank == 0:
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32",
                 "dtype_detail": "FP32 filter sweeps; FP64 Cholesky-QR, Rayleigh-Ritz, residuals",
                 "data": "synthetic", "config": WORKLOAD,
-                "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                             "frac": achieved / peak, "traffic": traffic, "traffic_source": traffic_note,
-                             "moved": moved, "moved_frac": moved / peak,
+                "roofline": {**hbm_roofline(achieved, moved_ratio, peak),
+                             "traffic": traffic, "traffic_source": traffic_note,
                              "peak_source": peak_note,
                              "kernel": "k_cheb_step<float,64> (fused SpMMV + recurrence + "
                                        "accumulation), averaged over the filter phase",

@@ -30,6 +30,23 @@ def test_filter_bytes_sums_the_steps():
         assert bench.filter_bytes(D, NNZ, NB, n, 4.0) == want
 
 
+def test_roofline_counts_what_the_steps_move():
+    mat, vec = NNZ * 8.0, NB * D * 4.0
+    for n in (3, 4, 5, 12, 500):
+        # reads x_{k-1}, x_{k-2}, writes x_k (not in the last step); the accumulator is read
+        # and written every third step from the second on, and in the last step
+        want = mat + 2 * vec + (mat + 4 * vec)
+        for k in range(3, n + 1):
+            want += mat + (3 if k < n else 2) * vec + (2 * vec if (k - 2) % 3 == 0 or k == n else 0)
+        assert bench.moved_filter_bytes(D, NNZ, NB, n, 4.0) == want
+    ratio = bench.moved_filter_bytes(D, NNZ, NB, 500, 4.0) / bench.filter_bytes(D, NNZ, NB, 500, 4.0)
+    e = bench.hbm_roofline(6650.0, ratio, 6800.0)
+    assert e["algorithmic"] == 6650.0 and e["achieved"] == 6650.0 * ratio
+    assert e["frac"] == e["achieved"] / e["peak"] < 0.75
+    # 7 entries a row: 7 + 1 operations and one accumulated term, 2 flops each
+    assert bench.fp64_step_flops(D, NNZ, NB) == 2 * 9 * D * NB
+
+
 def test_traffic_record_belongs_to_the_committed_kernel():
     """roofline.traffic is an ncu capture of one generic FP32 step on this
     shape; it is only valid for the step sources it was taken on."""
