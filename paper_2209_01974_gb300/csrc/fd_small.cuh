@@ -13,7 +13,7 @@
 // before the cluster's hardware barrier.  (Gathering remotely instead, from the
 // other CTAs' shared memory or through L2, was 2 to 4 times slower: scattered
 // 8-byte reads cost several clocks each.)  Clusters never wait for one another.
-// Measured per step (launched steps of the start -> this): 400 rows 6.6 -> 1.4 us
+// Measured per step (launched steps then -> this): 400 rows 6.6 -> 1.4 us
 // (FP64), 0.76 (FP32); 1,728 rows, nb = 16, FP64 6.6 -> 1.8, FP32 5.3 -> 1.6,
 // float-float 6.6 -> 1.4; 4,900 rows of 8 entries, nb = 16, FP64 8.5 -> 5.6, FP32
 // 8.6 -> 2.1; 4,096 stencil rows, nb = 32, FP64 8.6 -> 4.8.

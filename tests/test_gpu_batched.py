@@ -1,5 +1,6 @@
-"""Batched FD (many uneven instances, one persistent filter launch per outer
-iteration, CUDA graph) against dense eigensolvers and against one-by-one solves."""
+"""Batched FD (many uneven instances, one filter launch per outer iteration, as
+column panels or as persistent steps, CUDA graph) against dense eigensolvers and
+against one-by-one solves."""
 import numpy as np
 import pytest
 
@@ -85,7 +86,7 @@ def test_batched_rejects_sigma_sorted_matrices(fd, ctx):
 
 @pytest.mark.parametrize("nb", [8, 16])
 def test_small_batch_fp32_form_matches_dense(fd, ctx, nb):
-    # FP32 sweeps with the FP64 finish in the persistent batched filter
+    # FP32 sweeps with the FP64 finish (column panels at these sizes)
     mats = [fd.fd_build_matrix(ctx, s) for s in SMALL]
     probs = [(-0.3, 0.3, 8, 0)] * 5 + [(7.5, 8.5, 8, 0)]
     probs[4], probs[5] = (7.5, 8.5, 8, 0), (-0.3, 0.3, 8, 0)
@@ -100,7 +101,7 @@ def test_small_batch_fp32_form_matches_dense(fd, ctx, nb):
 
 def test_uneven_anderson_batch_fp32_form_matches_sequential(fd, ctx):
     # the FP32 form batched and one by one: the same switch rule and the same
-    # fused FP32 step, so the same eigenvalues
+    # recurrence in FP32, so the same eigenvalues
     seeds = [0, 14, 22, 26, 53, 12]
     specs = []
     for s_ in seeds:
@@ -125,8 +126,8 @@ def test_batched_fp32_form_needs_nb_4(fd, ctx):
 
 @pytest.mark.parametrize("form", [{"precision": "ff"}, {"precision": "f32", "finish": "ff"}])
 def test_small_batch_ff_forms_match_dense(fd, ctx, form):
-    # float-float rows in the persistent batched filter (all sweeps, or the
-    # FP32 form's finish), the Rayleigh-Ritz SpMMV in the FP64 instantiation
+    # float-float sweeps (all of them, or the FP32 form's finish; column panels at
+    # these sizes), the Rayleigh-Ritz SpMMV in FP64
     mats = [fd.fd_build_matrix(ctx, s) for s in SMALL]
     probs = [(-0.3, 0.3, 8, 0)] * 5 + [(7.5, 8.5, 8, 0)]
     probs[4], probs[5] = (7.5, 8.5, 8, 0), (-0.3, 0.3, 8, 0)
@@ -143,7 +144,7 @@ def test_small_batch_ff_forms_match_dense(fd, ctx, form):
 
 def test_uneven_anderson_batch_ff_finish_matches_sequential(fd, ctx):
     # FP32 sweeps with the float-float finish, batched and one by one: the same
-    # switch rule and the same arithmetic per row, so the same eigenvalues
+    # switch rule and the same arithmetic, so the same eigenvalues
     seeds = [0, 14, 22, 53]
     specs = []
     for s_ in seeds:

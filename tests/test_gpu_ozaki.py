@@ -37,8 +37,8 @@ def _block(D, n, seed, spread=6):
 
 
 def _bound(X, Y):
-    # split error per term < (2^-55 truncation + 2^-53.2 dropped digit pairs) 2^(e+f)
-    # <= 2^-50.9 |X|max |Y|max, the reference's own rounding <= K u |X|max |Y|max:
+    # split error per term < (2^-55 rounding + 2^-53.1 dropped digit pairs) 2^(e+f)
+    # <= 2^-50.8 |X|max |Y|max, the reference's own rounding <= K u |X|max |Y|max:
     # together under 8 K u |X|max |Y|max = K 2^-50 |X|max |Y|max
     K = X.shape[0]
     return 8 * K * U * np.outer(np.abs(X).max(0), np.abs(Y).max(0))
