@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(EIG_THREADS) k_block_jacobi(EigArgs a) {
   // same in every CTA)
   unsigned char* done = dyn;
   unsigned char* cur = dyn + a.n_inst;
+  unsigned char* last = cur + a.n_inst;  // whether the sweep at hand is its last
   const int g = threadIdx.x / GROUP, t = threadIdx.x % GROUP;
   // a group's first task: all CTAs get one before any gets a second (the FP64
   // pipes of an SM are shared by its groups)
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(EIG_THREADS) k_block_jacobi(EigArgs a) {
   const int64_t gt = (int64_t)blockIdx.x * EIG_THREADS + threadIdx.x, gn = (int64_t)gridDim.x * EIG_THREADS;
   for (int i = threadIdx.x; i < a.n_inst; i += EIG_THREADS) {
     done[i] = !live(task(a, i));
-    cur[i] = 0;
+    cur[i] = last[i] = 0;
   }
   __syncthreads();
 
@@ -239,9 +240,14 @@ __global__ void __launch_bounds__(EIG_THREADS) k_block_jacobi(EigArgs a) {
       if (done[i]) continue;
       float off, all;
       gather(i, false, &off, &all);
-      if (off <= a.tol2 * all || !(all <= 3e38f)) {
+      // A rotation leaves 1e-7 of its entry, so what is left below the threshold may be
+      // far above the rounding: it gets one sweep more, which the eigenvectors of close
+      // pairs need.
+      const bool below = off <= a.tol2 * all, rounding = off <= 5e-32f * (float)task(a, i).n * all;
+      if (last[i] || rounding || !(all <= 3e38f)) {
         if (lane == 0) done[i] = 1;
       } else {
+        if (below && lane == 0) last[i] = 1;
         left = 1;
       }
       __syncwarp();
@@ -433,12 +439,12 @@ int eig_grid(const fd_ctx* ctx, int n_inst, int m_max) {
 
 fd_status launch(fd_ctx* ctx, EigArgs& a, int grid) {
   void* args[] = {&a};
-  // two bytes per matrix beside 13 KB of static arrays: from 17,900 matrices on more than
+  // three bytes per matrix beside 13 KB of static arrays: from 11,900 matrices on more than
   // a launch gets unasked
   if (a.n_inst > 8192)
     FD_CUDA(ctx, cudaFuncSetAttribute(k_block_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
   FD_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_block_jacobi, grid, EIG_THREADS, args,
-                                           (size_t)2 * a.n_inst, ctx->stream));
+                                           (size_t)3 * a.n_inst, ctx->stream));
   FD_LAUNCHED(ctx);
   return FD_OK;
 }
