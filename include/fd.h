@@ -30,7 +30,8 @@
  *     return after enqueueing work.
  *   - Matrices are library-owned and freed with fd_matrix_free.
  *   - The library allocates its internal workspaces with cudaMalloc and keeps
- *     them in the context until fd_destroy.
+ *     them in the context until fd_destroy (scratch between calls also until
+ *     another workspace is refused: fd_set_workspace_limit).
  */
 #ifndef FD_H
 #define FD_H
